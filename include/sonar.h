@@ -96,7 +96,7 @@ typedef struct {
                                the bounded cast visits fewer nodes. */
     int32_t accumulate;  /* 0: deterministic fold of each bin's returns in canonical
                                ray order (default; bitwise reproducible);
-                            1: warp-aggregated shared-memory atomics */
+                            1: any order (the same fold: it costs nothing more) */
     int32_t reserved;
 } sonar_params;
 
@@ -260,10 +260,10 @@ typedef struct {
     float* fan;
 } sonar_batch_outputs;
 
-/* Plans a batch: validates the items, splits every sensor into work units of
- * whole azimuth columns (shapes from the autotuner's cache when it has an
- * entry for the sensor shape, defaults otherwise), orders the units
- * largest-first for the persistent launch, and uploads the descriptors
+/* Plans a batch: validates the items, lists the blocks of every launch (ray-cast
+ * tiles, azimuth columns, bands of range rows, fan squares; launch shapes from
+ * the autotuner's cache when it has an entry for the sensor shape, defaults
+ * otherwise), allocates the batch's scratch and uploads the descriptors
  * (synchronous).  n_items >= 1. */
 sonar_status sonar_batch_create(sonar_ctx_t ctx, const sonar_batch_item* items,
                                 int32_t n_items, sonar_batch_t* out);
@@ -278,9 +278,9 @@ sonar_status sonar_batch_update(sonar_batch_t batch, const sonar_batch_item* ite
                                 int32_t n_items, void* stream);
 
 /* Renders every item of the batch: one launch builds the exact-ray sin/cos
- * tables, one casts every ray of every sensor, one persistent launch bins and
- * adds noise for all column work units (dynamic work list), one normalises
- * every range row, and the fans are resampled by one launch for the items
+ * tables, one casts every ray of every sensor, one folds every azimuth column's
+ * returns, one adds the noise and normalises every range row (a further one
+ * divides by the image maximum, normalise = 2), and the fans are resampled by one launch for the items
  * that share a fan geometry (after refreshing any coordinate table whose
  * geometry changed) and one for the others.  The first call for a given
  * (params, theta, outputs) captures the launches in a CUDA graph; later calls
@@ -288,7 +288,7 @@ sonar_status sonar_batch_update(sonar_batch_t batch, const sonar_batch_item* ite
  * no re-plan) since the last forward replays a second graph without the two
  * table launches, whose tables are then current (calls on one batch are
  * stream-ordered, as for a context).  Results per item equal sonar_render's
- * for the same item and tile shape (bitwise, in deterministic accumulation). */
+ * for the same item (bitwise). */
 sonar_status sonar_render_batch(sonar_batch_t batch, const sonar_params* params,
                                 const float* d_theta, int32_t n_mat,
                                 const sonar_batch_outputs* out, void* stream);
@@ -310,8 +310,8 @@ sonar_status sonar_render_batch_backward(sonar_batch_t batch, const sonar_params
  * writes d_dtheta [2 + n_mat], the adjoint of d_grad_polar (packed like the
  * polar output) through this forward's I~ and hit records (out->noised and
  * out->hits, or the batch's scratch when NULL).  The adjoint needs I~ and the
- * records only, so one CUDA graph runs it beside the normalisation and fan
- * launches.  Results equal sonar_render_batch followed by
+ * records only, so one CUDA graph runs it beside the fan launches (and the
+ * whole-image normalisation).  Results equal sonar_render_batch followed by
  * sonar_render_batch_backward with the same arguments (bitwise).  Captured once
  * per (params, theta, outputs, grad, dtheta) and replayed after. */
 sonar_status sonar_render_batch_step(sonar_batch_t batch, const sonar_params* params,
@@ -319,8 +319,8 @@ sonar_status sonar_render_batch_step(sonar_batch_t batch, const sonar_params* pa
                                      const sonar_batch_outputs* out, const float* d_grad_polar,
                                      float* d_dtheta, void* stream);
 
-/* Plan statistics: out[0] work units, out[1] total rays, out[2] persistent
- * grid size, out[3] block size, out[4] graphs captured so far. */
+/* Plan statistics: out[0] and out[2] blocks of the fold launch, out[1] total
+ * rays, out[3] its block size, out[4] graphs captured so far. */
 sonar_status sonar_batch_info(sonar_batch_t batch, int64_t out[5]);
 
 /* Kernel launches per replay: out[0] kernel nodes of the forward graph replayed
@@ -335,7 +335,8 @@ sonar_status sonar_batch_kernels(sonar_batch_t batch, int32_t out[2]);
  * branches of a sonar_render_batch_step replay, where ms[3] and ms[4] overlap
  * ms[2]), measured by CUDA
  * events captured inside their graphs: ms[0] the ray-cast launch, ms[1] the
- * binning/noise launch, ms[2] the normalisation and fan launches, ms[3] the
+ * fold and row launches (binning, noise, normalisation by rows), ms[2] the fan
+ * launches and the whole-image normalisation, ms[3] the
  * adjoint row-term launch, ms[4] the adjoint gather and final-reduction
  * launches.  Waits for those replays to finish; a phase not yet run reports
  * -1. */
@@ -349,10 +350,9 @@ sonar_status sonar_batch_destroy(sonar_batch_t batch);
  * fastest per sensor shape (n_beams, n_elev, n_range_bins, n_az_bins) in the
  * context's tuning cache; later sonar_batch_create and sonar_render calls use
  * it.  Stage 1 times the forward launches over the ray-cast warp tiles (beams
- * x elevations per warp) and register variants; stage 2 times the columns per
- * binning work unit and the block size, which also shape the adjoint, on the
- * forward launches plus, when `out` holds hit records and I~, the adjoint of
- * a constant upstream gradient.  Each candidate scores the best of 3 rounds
+ * x elevations per warp) and register variants; stage 2, when `out` holds hit
+ * records and I~, times the adjoint's block size on the forward launches plus
+ * the adjoint of a constant upstream gradient.  Each candidate scores the best of 3 rounds
  * of 3 passes.  Runs on `stream` and synchronises it; allocates and frees its
  * own scratch (a polar-sized gradient).  Outputs of `out` are overwritten. */
 sonar_status sonar_autotune(sonar_batch_t batch, const sonar_params* params,
@@ -360,8 +360,9 @@ sonar_status sonar_autotune(sonar_batch_t batch, const sonar_params* params,
                             const sonar_batch_outputs* out, void* stream);
 
 /* Tuning cache entries: writes up to `cap` rows of 8 int32
- * (n_beams, n_elev, n_range_bins, n_az_bins, cols, tb, block, occ), tb =
- * beams per ray-cast warp (a power of two <= 32; elevations = 32 / tb), occ =
+ * (n_beams, n_elev, n_range_bins, n_az_bins, cols, tb, block, occ), cols
+ * unused (kept so that saved rows stay valid; >= 1), block the adjoint's threads
+ * per block, tb = beams per ray-cast warp (a power of two <= 32; elevations = 32 / tb), occ =
  * the ray-cast variant, a sum of flags: 8 caps its registers at 64 (32
  * one-warp blocks per SM), 16 walks the 8-wide tree instead of the 4-wide one
  * (both are built per scene; the hit records are the same either way).  A

@@ -1,13 +1,12 @@
 // Sonar post-processing kernels (OceanSim, arXiv 2503.01074, Sec. III-A-2).
 //
-// k_bin               one work unit = whole azimuth columns of one sensor: the
-//                     units' hit records -> intensity (Eq. 2, two-way) -> polar
-//                     binning into a shared-memory column block -> Eq. 3-6 noise
-//                     per bin -> I~ to HBM.  A unit owns its columns, so every
-//                     polar bin is written exactly once: no global atomics, no
-//                     memset of the image.
-// k_norm_rows         range-wise normalisation: one warp per range row takes the
-//                     row maximum of I~ and writes N = I~ / max.
+// k_fold              one warp (or block) = one azimuth column of one sensor: the
+//                     column's hit records -> intensity (Eq. 2, two-way) -> the sums
+//                     of its bins with returns, compactly (a bitmap, ranks, values):
+//                     no global atomics, no memset and no dense image of P.
+// k_rows              one warp = one range row: Eq. 3-6 noise of every bin, the row
+//                     maximum and N = I~ / max; writes I~ and N, reads neither.
+// k_norm_rows         whole-image normalisation only: N = I~ / max.
 // k_fan_*             fan resample of the normalised image: per-pixel polar
 //                     coordinate tables, then bilinear gathers for up to 8
 //                     frames per table read.
@@ -26,481 +25,449 @@ namespace sonar {
 namespace {
 
 // ---------------------------------------------------------------------------
-// bin + noise: one work unit = whole azimuth columns of one sensor
+// fold: the rays of every azimuth column -> the column's bins with returns
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void load_unit(const BinArgs& a, int u, SensorDev* S, SceneDev* SC, Unit* U) {
-    if (a.units) {
-        *U = a.units[u];
-        *S = a.sensors[U->sensor];
-        *SC = a.scenes[S->scene];
+// The score of a hit record: s = mu[m] cos exp(-2 alpha r) gain (Eq. 2).
+__device__ __forceinline__ float score_of(const FoldArgs& a, const SceneDev& sc, uint4 h, float alpha, float gain) {
+    int m = __ldg(sc.mat_orig + h.y);
+    m = m < a.n_mat ? m : a.n_mat - 1;
+    return __ldg(a.theta + 2 + m) * __uint_as_float(h.w) * expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
+}
+
+// Range row of a record of azimuth column `col`, or -1: no return, or a
+// corrupt record (reported in the error word).
+__device__ __forceinline__ int row_of(const FoldArgs& a, const SensorDev& S, const SceneDev& sc, uint4 h, int col) {
+    if (h.x == kNoKey) return -1;
+    const uint32_t row = h.x / (uint32_t)S.naz;
+    if (row >= (uint32_t)S.nr || h.x - row * (uint32_t)S.naz != (uint32_t)col || h.y >= (uint32_t)sc.n_tris) {
+        atomicOr(a.err, SONAR_DEVERR_INDEX);
+        return -1;
+    }
+    return (int)row;
+}
+
+// Exclusive prefix of the set bits of bits[0..nwords) into pre (one warp); returns their number.
+__device__ __forceinline__ int bit_prefix(const uint32_t* bits, uint32_t* pre, int nwords, int lane) {
+    int total = 0;
+    for (int w0 = 0; w0 < nwords; w0 += 32) {
+        const int w = w0 + lane;
+        const int n = w < nwords ? __popc(bits[w]) : 0;
+        int x = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (w < nwords) pre[w] = (uint32_t)(total + x - n);
+        total += __shfl_sync(0xFFFFFFFFu, x, 31);
+    }
+    return total;
+}
+
+__device__ __forceinline__ int bit_rank(const uint32_t* bits, const uint32_t* pre, int row) {
+    return (int)pre[row >> 5] + __popc(bits[row >> 5] & ((1u << (row & 31)) - 1u));
+}
+
+// Adds each lane's score to acc[idx] (idx < 0: none), equal bins in lane
+// order onto the bin's running sum: with the rays taken 32 at a time in
+// canonical order, every bin is the sequential sum of its returns.  The lowest
+// lane of a bin reads its peers' scores from shared memory (32 words of the
+// warp's own): shuffles among the peers would run the bins one after another
+// (64 frames: 63 us with them).
+__device__ __forceinline__ void fold_step(float* acc, float* scores, int idx, float score, int lane) {
+    scores[lane] = score;
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, idx);
+    __syncwarp();
+    if (idx >= 0 && lane == __ffs(peers) - 1) {
+        float v = acc[idx] + score;
+        for (uint32_t m = peers & (peers - 1); m; m &= m - 1) v += scores[__ffs(m) - 1];
+        acc[idx] = v;
+    }
+    __syncwarp();
+}
+
+// A finished bin (rank k of its column): P and the speckle factor 0.5 + w_sm
+// of Eq. 3, compactly; or P into the image itself where no scratch holds them.
+__device__ __forceinline__ void put_bin(const FoldArgs& a, const SensorDev& S, const PhiloxKey& K, int64_t first, int k,
+                                        int row, int col, float P) {
+    const uint32_t b = (uint32_t)row * (uint32_t)S.naz + (uint32_t)col;
+    if (a.dense) {
+        a.dense[S.polar_off + b] = P;
     } else {
-        *S = a.one;
-        *SC = a.one_scene;
-        U->sensor = 0;
-        U->c0 = u * a.one.cols;
-        U->c1 = min(U->c0 + a.one.cols, a.one.naz);
-        U->rays = 0;
+        a.vals[S.val_off + first + k] = make_float2(P, 0.5f + gauss_of(bin_draws(b, S, K), a.sigma_sm));
     }
 }
 
-// The unit's rays are the contiguous hit records of its beams.  Their scores
-// s = mu[m] cos exp(-2 alpha r) gain are summed into a shared-memory column
-// block (DET: in canonical ray order, warps taking turns and each group of
-// equal bins folded by its leader in lane order; otherwise warp-aggregated
-// shared-memory atomics); then Eq. 3-6 noise per bin and I~ to HBM.
-// The additive term of Eq. 3 for range row `row` (centre r_c) and a column
-// whose beam-pattern factor 0.5 exp(-phi_c^2 / sigma_phi) is `pat`, from the
-// bin's uniform word of the additive stream: (r_c^2 / r_max^2)(1 + pat w_sa),
-// w_sa ~ Rayleigh(sigma_sa) (Eq. 4).
-struct AdditiveTerm {
-    float dr, rmin, inv_rmax2, sig_sa;
-    __device__ __forceinline__ float operator()(int row, float pat, uint32_t word) const {
-        const float w_sa = rayleigh_of(word, sig_sa);
-        const float rc = fmaf(small_u2f(row) + 0.5f, dr, rmin);
-        return rc * rc * inv_rmax2 * (1.0f + pat * w_sa);
-    }
-};
-
-template <int DET>
-__global__ void __launch_bounds__(512) k_bin(BinArgs a) {
-    extern __shared__ __align__(16) float acc[];
+// One warp per azimuth column (sensors with at most one beam per column, and
+// those whose per-beam rows do not fit in shared memory), or one block per
+// column with its warps on the column's beams (S.fold_beams).
+//
+// Only the bins that a ray lands in (about 6 % of them) are stored: pass 1 marks
+// the column's rows with returns in a bitmap, a prefix over its words ranks
+// them, pass 2 sums the scores at the ranks, and the bitmap with its ranks is
+// what the row kernel looks bins up in (a bit per bin plus 8 bytes per ray,
+// against the 8 bytes per bin of a dense image written and read back).  A
+// column's working set is so a few hundred words rather than a row of floats
+// per range bin, and no pass over all bins is left here.
+//
+// Bound by the latency of its dependent steps (record, material, rank, sum),
+// which the resident columns hide.  Measured, this kernel and k_rows against the
+// binning kernel over dense column blocks and the normalisation pass that they
+// replace: 64 frames of 512 x 64 rays into 1000 x 512 bins 48 + 98 us against
+// 231 + 43 us (132 + 43 us with hand-picked units); 32 frames of 1024 x 256
+// rays into 4000 x 1024 bins 148 + 410 us against 1122 + 153 us; one frame of
+// 3000 x 460 rays into 350 x 220 bins 42 + 6 us against 462 + 5 us.
+__global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a) {
+    extern __shared__ __align__(16) uint32_t fold_smem[];
     __shared__ SensorDev S;
     __shared__ SceneDev SC;
-    __shared__ Unit U;
-    __shared__ int s_unit, s_count;
-    __shared__ float s_red[32];
-    __shared__ float s_pat[kMaxCols];
-    __shared__ int s_b0[kMaxCols + 1];   // per-beam fold: first local beam of each column
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    const float alpha = __ldg(a.theta), gain = __ldg(a.theta + 1);
-    int clean_nbin = -1;   // block-uniform: the unit size whose accumulator and bitmap are known zero
-    int next_u = 0;   // thread 0: the unit taken ahead, while the block works on the current one
-    for (int iter = 0;; ++iter) {
-        int u;
-        if (a.work_counter) {
-            if (tid == 0) s_unit = iter == 0 ? atomicAdd(a.work_counter, 1) : next_u;
-            __syncthreads();
-            u = s_unit;
-            if (tid == 0 && u < a.n_units) next_u = atomicAdd(a.work_counter, 1);
+    __shared__ int s_col, s_n;
+    __shared__ float s_scores[16][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (warp == 0) {
+        if (a.sensors) {
+            const int4 m = __ldg(a.block_map + blockIdx.x);
+            copy_words(&S, a.sensors + m.x, lane);
+            copy_words(&SC, a.scenes + m.z, lane);
+            if (lane == 0) s_col = m.y;
         } else {
-            if (iter > 0) break;
-            u = blockIdx.x;
+            copy_param(&S, &a.one, lane);
+            copy_param(&SC, &a.one_scene, lane);
+            if (lane == 0) s_col = blockIdx.x * (a.one.fold_beams ? 1 : nw);
         }
-        if (u >= a.n_units) break;
-        if (a.units) {   // warp 0 fetches the unit, then its sensor and scene descriptors at once
-            if (warp == 0) {
-                const Unit un = a.units[u];
-                copy_words(&S, a.sensors + un.sensor, lane);
-                copy_words(&SC, a.scenes + un.scene, lane);
-                if (lane == 0) U = un;
-            }
-        } else if (tid == 0) {
-            load_unit(a, u, &S, &SC, &U);
-        }
-        __syncthreads();
-        const int cw = U.c1 - U.c0;
-        const int i0 = first_beam_of_col(U.c0, S.nb, S.naz), i1 = first_beam_of_col(U.c1, S.nb, S.naz);
-        const int64_t r0 = (int64_t)i0 * S.ne, r1 = (int64_t)i1 * S.ne;
-        const int nbin = S.nr * cw;
-        const sonar_hit* H = a.hits + S.hits_off;
-        // Deterministic fold, per-beam form: warp w owns beams w, w + nw, ... of the
-        // unit and folds each beam's rays in elevation order into that beam's own
-        // row accumulator (one writer: no barriers); a bin then adds its column's
-        // beams in beam order.  With one beam per column this is exactly the
-        // sequential canonical-order fold.
-        const int nbeam = i1 - i0;
-        const bool per_beam = DET && S.fold_beams;
-        float* accb = acc + nbin;
-        int* list = reinterpret_cast<int*>(acc + nbin + (per_beam ? nbeam * S.nr : 0));
-        // the list of bins with returns holds one entry per ray at most (only a
-        // bin that a ray lands in can be nonzero): the host sizes it so
-        const int lcap = (int)min((int64_t)nbin, r1 - r0);
-        // Noise first: with at most one beam per column and no whole-image
-        // maximum, a bin's additive term does not depend on the fold, so pass 1
-        // writes it for every bin before the rays are folded (the fold's record
-        // loads then meet a busy block rather than a barrier); the fold lists each
-        // bin at its first return (a shared bitmap), and pass 2 finishes and
-        // resets only the listed bins, which leaves the accumulator and bitmap
-        // zero for the next unit of the same size.
-        if (DET && !per_beam && S.nb <= S.naz && a.params.normalise != 2) {
-            uint32_t* bits = reinterpret_cast<uint32_t*>(acc + nbin);
-            const int nwords = (nbin + 31) >> 5;
-            int* flist = reinterpret_cast<int*>(bits + nwords);
-            if (clean_nbin != nbin)
-                for (int k = tid; k < nbin + nwords; k += nt) acc[k] = 0.0f;   // bitmap words too (0.0f is 0)
-            const float dr = (S.rmax - S.rmin) / (float)S.nr, da = S.hfov / (float)S.naz;
-            const float inv_rmax2 = 1.0f / (S.rmax * S.rmax);
-            const float inv_sphi = 1.0f / a.params.sigma_phi;
-            const float sig_sa = a.params.sigma_sa, sig_sm = a.params.sigma_sm;
-            for (int c = tid; c < cw; c += nt) {
-                const float pc = fmaf(small_u2f(U.c0 + c) + 0.5f, da, -0.5f * S.hfov);
-                s_pat[c] = 0.5f * expf(-pc * pc * inv_sphi);
-            }
-            if (tid == 0) s_count = 0;
-            __syncthreads();
-            const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
-            const uint32_t naz_r = (uint32_t)S.naz, c0_r = (uint32_t)U.c0, flo = S.frame_lo, fhi = S.frame_hi;
-            const float rmin_r = S.rmin;
-            const AdditiveTerm additive{dr, rmin_r, inv_rmax2, sig_sa};
-            float* const noised_r = a.noised + S.polar_off;
-            float* const binned_r = a.binned ? a.binned + S.polar_off : nullptr;
-            if (((naz_r | c0_r | (uint32_t)cw) & 3u) == 0) {
-                const int cq = cw >> 2, nquad = S.nr * cq;
-                const int dqr = nt / cq, dqc = nt - dqr * cq;
-                int row = tid / cq, qc = tid - row * cq;
-                const bool vec = ((reinterpret_cast<uintptr_t>(noised_r) |
-                                   reinterpret_cast<uintptr_t>(binned_r)) & 15u) == 0;
-                for (int g = tid; g < nquad; g += nt) {
-                    const uint32_t b0 = (uint32_t)row * naz_r + c0_r + 4u * (uint32_t)qc;
-                    const U4 x = additive_words(b0 >> 2, flo, fhi, K);
-                    const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-                    float add[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) add[j] = additive(row, s_pat[4 * qc + j], xw[j]);
-                    if (vec) {
-                        *reinterpret_cast<float4*>(noised_r + b0) = make_float4(add[0], add[1], add[2], add[3]);
-                        if (binned_r) *reinterpret_cast<float4*>(binned_r + b0) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            noised_r[b0 + j] = add[j];
-                            if (binned_r) binned_r[b0 + j] = 0.0f;
-                        }
-                    }
-                    row += dqr;
-                    qc += dqc;
-                    if (qc >= cq) { qc -= cq; ++row; }
-                }
-            } else {
-                const int drow = nt / cw, dcol = nt - drow * cw;
-                int row = tid / cw, col = tid - row * cw;
-                for (int k = tid; k < nbin; k += nt) {
-                    const uint32_t b = (uint32_t)row * naz_r + c0_r + (uint32_t)col;
-                    const U4 x = additive_words(b >> 2, flo, fhi, K);
-                    noised_r[b] = additive(row, s_pat[col], word_of(x, b & 3u));
-                    if (binned_r) binned_r[b] = 0.0f;
-                    row += drow;
-                    col += dcol;
-                    if (col >= cw) { col -= cw; ++row; }
-                }
-            }
-            // the fold: warp w takes beams w, w + nw, ... of the unit, each in
-            // elevation order (its column's canonical order)
-            for (int bb = warp; bb < nbeam; bb += nw) {
-                const sonar_hit* Hb = H + (int64_t)(i0 + bb) * S.ne;
-                for (int jb = 0; jb < S.ne; jb += 32) {
-                    const int j = jb + lane;
-                    uint32_t lkey = kNoKey;
-                    float score = 0.0f;
-                    if (j < S.ne) {
-                        const uint4 h = __ldg(reinterpret_cast<const uint4*>(Hb + j));
-                        if (h.x != kNoKey) {
-                            const uint32_t br = h.x / naz_r, ba = h.x - br * naz_r;
-                            lkey = br * (uint32_t)cw + (ba - c0_r);
-                            if (lkey >= (uint32_t)nbin || h.y >= (uint32_t)SC.n_tris) {   // not this unit's bin: a corrupt record
-                                atomicOr(a.err, SONAR_DEVERR_INDEX);
-                                lkey = kNoKey;
-                            }
-                            int m = lkey == kNoKey ? 0 : SC.mat_orig[h.y];
-                            m = m < a.n_mat ? m : a.n_mat - 1;
-                            score = __ldg(a.theta + 2 + m) * __uint_as_float(h.w) *
-                                    expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
-                        }
-                    }
-                    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, lkey);
-                    if (lkey != kNoKey) {
-                        const int leader = __ffs(peers) - 1;
-                        float v = lane == leader ? acc[lkey] : 0.0f;
-                        for (uint32_t m = peers; m; m &= m - 1) v += __shfl_sync(peers, score, __ffs(m) - 1);
-                        if (lane == leader) {
-                            acc[lkey] = v;
-                            const uint32_t bit = 1u << (lkey & 31u);
-                            if (!(atomicOr(&bits[lkey >> 5], bit) & bit)) {
-                                const int q = atomicAdd(&s_count, 1);
-                                if (q < lcap) flist[q] = (int)lkey;
-                                else atomicOr(a.err, SONAR_DEVERR_INDEX);
-                            }
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-            // pass 2: the listed bins get P (0.5 + w_sm) on top of the additive
-            // term written by pass 1 (visible after the barrier), then are reset
-            const int nl = min(s_count, lcap);
-            for (int q = tid; q < nl; q += nt) {
-                const int k = flist[q];
-                const int rw = k / cw, cl = k - rw * cw;
-                const uint32_t b = (uint32_t)rw * naz_r + c0_r + (uint32_t)cl;
-                const float P = acc[k];
-                acc[k] = 0.0f;
-                bits[k >> 5] = 0u;
-                if (binned_r) binned_r[b] = P;
-                if (P != 0.0f) {
-                    const float w_sm = gauss_of(bin_draws(b, S, K), sig_sm);
-                    noised_r[b] = P * (0.5f + w_sm) + noised_r[b];
-                }
-            }
-            clean_nbin = nbin;
-            __syncthreads();
-            continue;
-        }
-        clean_nbin = -1;   // the path below leaves its accumulator in use
-        if (per_beam) {
-            for (int k = tid; k < nbeam * S.nr; k += nt) accb[k] = 0.0f;
-            for (int c = tid; c <= cw; c += nt) s_b0[c] = first_beam_of_col(U.c0 + c, S.nb, S.naz) - i0;
-        } else {
-            for (int k = tid; k < nbin; k += nt) acc[k] = 0.0f;
-        }
-        __syncthreads();
-        if (per_beam) {
-            for (int bb = warp; bb < nbeam; bb += nw) {
-                const sonar_hit* Hb = H + (int64_t)(i0 + bb) * S.ne;
-                float* racc = accb + bb * S.nr;
-                for (int jb = 0; jb < S.ne; jb += 32) {
-                    const int j = jb + lane;
-                    uint32_t row = kNoKey;
-                    float score = 0.0f;
-                    if (j < S.ne) {
-                        const uint4 h = __ldg(reinterpret_cast<const uint4*>(Hb + j));
-                        if (h.x != kNoKey) {
-                            row = h.x / (uint32_t)S.naz;
-                            int m = SC.mat_orig[h.y];
-                            m = m < a.n_mat ? m : a.n_mat - 1;
-                            score = __ldg(a.theta + 2 + m) * __uint_as_float(h.w) *
-                                    expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
-                        }
-                    }
-                    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, row);
-                    if (row != kNoKey) {
-                        const int leader = __ffs(peers) - 1;
-                        float v = lane == leader ? racc[row] : 0.0f;
-                        for (uint32_t m = peers; m; m &= m - 1) v += __shfl_sync(peers, score, __ffs(m) - 1);
-                        if (lane == leader) racc[row] = v;
-                    }
-                }
-            }
-        }
-        // With at most one beam per column (n_beams <= n_az_bins) a beam's bins
-        // are its column's own: warp w folds beams w, w + nw, ... straight into
-        // the unit's accumulator, each in elevation order (the canonical order of
-        // that column's rays, so the same sums as the turn-taking fold below),
-        // with no barriers between warps.
-        const bool col_fold = DET && !per_beam && S.nb <= S.naz;
-        if (col_fold) {
-            const uint32_t naz = (uint32_t)S.naz;
-            for (int bb = warp; bb < nbeam; bb += nw) {
-                const sonar_hit* Hb = H + (int64_t)(i0 + bb) * S.ne;
-                for (int jb = 0; jb < S.ne; jb += 32) {
-                    const int j = jb + lane;
-                    uint32_t lkey = kNoKey;
-                    float score = 0.0f;
-                    if (j < S.ne) {
-                        const uint4 h = __ldg(reinterpret_cast<const uint4*>(Hb + j));
-                        if (h.x != kNoKey) {
-                            const uint32_t br = h.x / naz, ba = h.x - br * naz;
-                            lkey = br * (uint32_t)cw + (ba - (uint32_t)U.c0);
-                            int m = SC.mat_orig[h.y];
-                            m = m < a.n_mat ? m : a.n_mat - 1;
-                            score = __ldg(a.theta + 2 + m) * __uint_as_float(h.w) *
-                                    expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
-                        }
-                    }
-                    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, lkey);
-                    if (lkey != kNoKey) {
-                        const int leader = __ffs(peers) - 1;
-                        float v = lane == leader ? acc[lkey] : 0.0f;
-                        for (uint32_t m = peers; m; m &= m - 1) v += __shfl_sync(peers, score, __ffs(m) - 1);
-                        if (lane == leader) acc[lkey] = v;
-                    }
-                }
-            }
-        }
-        for (int64_t base = r0; base < (per_beam || col_fold ? r0 : r1); base += nt) {
-            const int64_t r = base + tid;
-            uint32_t lkey = kNoKey;
-            float score = 0.0f;
-            if (r < r1) {
-                const uint4 h = __ldg(reinterpret_cast<const uint4*>(H + r));
-                if (h.x != kNoKey) {
-                    const uint32_t br = h.x / (uint32_t)S.naz, ba = h.x - br * (uint32_t)S.naz;
-                    lkey = br * (uint32_t)cw + (ba - (uint32_t)U.c0);
-                    int m = SC.mat_orig[h.y];
-                    m = m < a.n_mat ? m : a.n_mat - 1;
-                    score = __ldg(a.theta + 2 + m) * __uint_as_float(h.w) *
-                            expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
-                }
-            }
-            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, lkey);
-            const int leader = __ffs(peers) - 1;
-            if (DET) {
-                for (int w = 0; w < nw; ++w) {
-                    if (warp == w && lkey != kNoKey) {
-                        float v = lane == leader ? acc[lkey] : 0.0f;
-                        for (uint32_t m = peers; m; m &= m - 1) {
-                            const float x = __shfl_sync(peers, score, __ffs(m) - 1);
-                            v += x;
-                        }
-                        if (lane == leader) acc[lkey] = v;
-                    }
-                    __syncthreads();
-                }
-            } else {
-                if (lkey != kNoKey) {
-                    float v = 0.0f;
-                    for (uint32_t m = peers; m; m &= m - 1) v += __shfl_sync(peers, score, __ffs(m) - 1);
-                    if (lane == leader) atomicAdd(&acc[lkey], v);
-                }
-            }
-        }
-        __syncthreads();
-        // Eq. 3-6 per bin.  Pass 1 visits every bin: the additive Rayleigh term,
-        // which is already the final value of a bin without returns (P = 0 makes
-        // the multiplicative term exactly 0); bins with returns are listed.  Pass 2
-        // finishes the listed bins with the Gaussian multiplicative term.  (row,
-        // col) advance incrementally: no division and no integer-to-float
-        // conversion instruction in pass 1.
-        const float dr = (S.rmax - S.rmin) / (float)S.nr, da = S.hfov / (float)S.naz;
-        const float inv_rmax2 = 1.0f / (S.rmax * S.rmax);
-        const float inv_sphi = 1.0f / a.params.sigma_phi;
-        const float sig_sa = a.params.sigma_sa, sig_sm = a.params.sigma_sm;
-        for (int c = tid; c < cw; c += nt) {
-            const float pc = fmaf(small_u2f(U.c0 + c) + 0.5f, da, -0.5f * S.hfov);
-            s_pat[c] = 0.5f * expf(-pc * pc * inv_sphi);
-        }
-        if (tid == 0) s_count = 0;
-        __syncthreads();
-        const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
-        // the sensor fields this loop reads, in registers (the loop's shared-memory
-        // stores would otherwise make the compiler reload them every bin)
-        const uint32_t naz_r = (uint32_t)S.naz, c0_r = (uint32_t)U.c0, flo = S.frame_lo, fhi = S.frame_hi;
-        const float rmin_r = S.rmin;
-        const AdditiveTerm additive{dr, rmin_r, inv_rmax2, sig_sa};
-        float* const noised_r = a.noised + S.polar_off;
-        float* const binned_r = a.binned ? a.binned + S.polar_off : nullptr;
-        // Pass 1 writes every bin's additive term to I~ (pass 2 adds the
-        // multiplicative term of the listed bins to it).  When the unit's bins
-        // come in aligned fours (row width, first column and unit width multiples
-        // of 4) a thread takes four neighbouring bins: one Philox block gives
-        // their four additive draws, and they move as 16-byte vectors.
-        if (((naz_r | c0_r | (uint32_t)cw) & 3u) == 0) {
-            const int cq = cw >> 2, nquad = S.nr * cq;
-            const int dqr = nt / cq, dqc = nt - dqr * cq;
-            int row = tid / cq, qc = tid - row * cq;
-            const bool vec = ((reinterpret_cast<uintptr_t>(noised_r) |
-                               reinterpret_cast<uintptr_t>(binned_r)) & 15u) == 0;
-            for (int g = tid; g < nquad; g += nt) {
-                const int k0 = row * cw + 4 * qc;
-                const uint32_t b0 = (uint32_t)row * naz_r + c0_r + 4u * (uint32_t)qc;
-                float P[4];
-                if (per_beam) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        P[j] = 0.0f;
-                        for (int bb = s_b0[4 * qc + j]; bb < s_b0[4 * qc + j + 1]; ++bb) P[j] += accb[bb * S.nr + row];
-                    }
-                } else {
-                    const float4 v = *reinterpret_cast<const float4*>(acc + k0);
-                    P[0] = v.x; P[1] = v.y; P[2] = v.z; P[3] = v.w;
-                }
-                const U4 x = additive_words(b0 >> 2, flo, fhi, K);
-                const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-                float add[4], keep[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    add[j] = additive(row, s_pat[4 * qc + j], xw[j]);
-                    keep[j] = add[j];
-                    if (P[j] != 0.0f) {
-                        keep[j] = P[j];
-                        const int q = atomicAdd(&s_count, 1);
-                        if (q < lcap) list[q] = k0 + j;
-                        else atomicOr(a.err, SONAR_DEVERR_INDEX);
-                    }
-                }
-                if (vec) {
-                    *reinterpret_cast<float4*>(noised_r + b0) = make_float4(add[0], add[1], add[2], add[3]);
-                    if (binned_r) *reinterpret_cast<float4*>(binned_r + b0) = make_float4(P[0], P[1], P[2], P[3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        noised_r[b0 + j] = add[j];
-                        if (binned_r) binned_r[b0 + j] = P[j];
-                    }
-                }
-                *reinterpret_cast<float4*>(acc + k0) = make_float4(keep[0], keep[1], keep[2], keep[3]);
-                row += dqr;
-                qc += dqc;
-                if (qc >= cq) { qc -= cq; ++row; }
-            }
-        } else {
-            const int drow = nt / cw, dcol = nt - drow * cw;
-            int row = tid / cw, col = tid - row * cw;
-            for (int k = tid; k < nbin; k += nt) {
-                const uint32_t b = (uint32_t)row * naz_r + c0_r + (uint32_t)col;
-                float P;
-                if (per_beam) {
-                    P = 0.0f;
-                    for (int bb = s_b0[col]; bb < s_b0[col + 1]; ++bb) P += accb[bb * S.nr + row];
-                } else {
-                    P = acc[k];
-                }
-                const U4 x = additive_words(b >> 2, flo, fhi, K);
-                const float add = additive(row, s_pat[col], word_of(x, b & 3u));
-                if (binned_r) binned_r[b] = P;
-                noised_r[b] = add;
-                if (P != 0.0f) {
-                    acc[k] = P;
-                    const int q = atomicAdd(&s_count, 1);
-                    if (q < lcap) list[q] = k;
-                    else atomicOr(a.err, SONAR_DEVERR_INDEX);
-                } else {
-                    acc[k] = add;
-                }
-                row += drow;
-                col += dcol;
-                if (col >= cw) { col -= cw; ++row; }
-            }
-        }
-        __syncthreads();
-        // Pass 2: the listed bins (P != 0) add P (0.5 + w_sm) to the additive
-        // term that pass 1 wrote (visible to the block after the barrier)
-        const int nlist = min(s_count, lcap);
-        for (int q = tid; q < nlist; q += nt) {
-            const int k = list[q];
-            const int rw = k / cw, cl = k - rw * cw;
-            const uint32_t b = (uint32_t)(rw * S.naz + U.c0 + cl);
-            const float P = acc[k];
-            const float w_sm = gauss_of(bin_draws(b, S, K), sig_sm);
-            const float In = P * (0.5f + w_sm) + noised_r[b];
-            noised_r[b] = In;
-            acc[k] = In;
-        }
-        __syncthreads();
-        if (a.params.normalise == 2) {
-            // one maximum per unit for the whole-image normalisation; range-row
-            // maxima are taken by the normalisation kernel from I~ itself
-            float m = -CUDART_INF_F;
-            for (int k = tid; k < nbin; k += nt) m = fmaxf(m, acc[k]);
-            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-            if (lane == 0) s_red[warp] = m;
-            __syncthreads();
-            if (tid == 0) {
-                for (int w = 1; w < nw; ++w) m = fmaxf(m, s_red[w]);
-                atomicMax(a.rowmax + S.rowmax_off, ord_enc(fmaxf(m, s_red[0])));
-            }
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    const float alpha = __ldg(a.theta), gain = __ldg(a.theta + 1);
+    const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
+    const int ne = S.ne, nwords = (S.nr + 31) >> 5;
+    const int col = s_col + (S.fold_beams ? 0 : warp);
+    if (col >= S.naz) return;   // whole warps only (the last block of a sensor)
+    const int i0 = first_beam_of_col(col, S.nb, S.naz), i1 = first_beam_of_col(col + 1, S.nb, S.naz);
+    const int64_t first = (int64_t)i0 * ne;          // the column's first ray, and its first value slot
+    const int64_t n = (int64_t)(i1 - i0) * ne;
+    const sonar_hit* H = a.hits + S.hits_off + first;
+    const int most = (int)min((int64_t)S.nr, n);     // bins with returns, at most
+    if (!S.fold_beams) {
+        uint32_t* bits = fold_smem + (int64_t)warp * a.words_per_warp;
+        uint32_t* pre = bits + nwords;
+        float* acc = reinterpret_cast<float*>(pre + nwords);
+        int* rows = reinterpret_cast<int*>(acc + most);
+        for (int w = lane; w < nwords; w += 32) bits[w] = 0u;
+        __syncwarp();
+        for (int64_t j = lane; j < n; j += 32) {
+            const int row = row_of(a, S, SC, __ldg(reinterpret_cast<const uint4*>(H + j)), col);
+            if (row >= 0) atomicOr(bits + (row >> 5), 1u << (row & 31));
+        }
+        __syncwarp();
+        const int nd = bit_prefix(bits, pre, nwords, lane);
+        for (int k = lane; k < nd; k += 32) acc[k] = 0.0f;
+        __syncwarp();
+        for (int64_t jb = 0; jb < n; jb += 32) {
+            int idx = -1;
+            float score = 0.0f;
+            if (jb + lane < n) {
+                const uint4 h = __ldg(reinterpret_cast<const uint4*>(H + jb + lane));
+                const int row = row_of(a, S, SC, h, col);
+                if (row >= 0) {
+                    idx = bit_rank(bits, pre, row);
+                    rows[idx] = row;
+                    score = score_of(a, SC, h, alpha, gain);
+                }
+            }
+            fold_step(acc, s_scores[warp], idx, score, lane);
+        }
+        for (int k = lane; k < nd; k += 32) put_bin(a, S, K, first, k, rows[k], col, acc[k]);
+        if (a.bands)
+            for (int w = lane; w < nwords; w += 32)
+                a.bands[S.band_off + (int64_t)w * S.naz + col] = make_uint2(bits[w], (uint32_t)first + pre[w]);
+        return;
+    }
+    // per-beam form: each beam sums its own rows in elevation order, a bin then
+    // adds its column's beams in beam order
+    const int nbeam = i1 - i0, nt = blockDim.x;
+    uint32_t* bits = fold_smem;
+    uint32_t* pre = bits + nwords;
+    int* rows = reinterpret_cast<int*>(pre + nwords);
+    float* acc = reinterpret_cast<float*>(rows + most);   // [nbeam][nd]
+    for (int w = tid; w < nwords; w += nt) bits[w] = 0u;
+    __syncthreads();
+    for (int64_t j = tid; j < n; j += nt) {
+        const int row = row_of(a, S, SC, __ldg(reinterpret_cast<const uint4*>(H + j)), col);
+        if (row >= 0) atomicOr(bits + (row >> 5), 1u << (row & 31));
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int total = bit_prefix(bits, pre, nwords, lane);
+        if (lane == 0) s_n = total;
+    }
+    __syncthreads();
+    const int nd = s_n;
+    for (int k = tid; k < nbeam * nd; k += nt) acc[k] = 0.0f;
+    __syncthreads();
+    for (int bb = warp; bb < nbeam; bb += nw) {
+        for (int jb = 0; jb < ne; jb += 32) {
+            int idx = -1;
+            float score = 0.0f;
+            if (jb + lane < ne) {
+                const uint4 h = __ldg(reinterpret_cast<const uint4*>(H + (int64_t)bb * ne + jb + lane));
+                const int row = row_of(a, S, SC, h, col);
+                if (row >= 0) {
+                    idx = bit_rank(bits, pre, row);
+                    rows[idx] = row;   // every writer of a rank writes the same row
+                    score = score_of(a, SC, h, alpha, gain);
+                }
+            }
+            fold_step(acc + bb * nd, s_scores[warp], idx, score, lane);
+        }
+    }
+    __syncthreads();
+    for (int k = tid; k < nd; k += nt) {
+        float P = 0.0f;
+        for (int bb = 0; bb < nbeam; ++bb) P += acc[bb * nd + k];
+        put_bin(a, S, K, first, k, rows[k], col, P);
+    }
+    if (a.bands)
+        for (int w = tid; w < nwords; w += nt)
+            a.bands[S.band_off + (int64_t)w * S.naz + col] = make_uint2(bits[w], (uint32_t)first + pre[w]);
 }
 
 // ---------------------------------------------------------------------------
-// phase 2a: range-wise normalisation, one warp per (sensor, range row)
+// rows: noise (Eq. 3-6) and range-wise normalisation, one warp per range row
 // ---------------------------------------------------------------------------
 
+// The additive term of Eq. 3 for a range row (`rc` its centre, squared over
+// r_max^2) and a column whose beam-pattern factor 0.5 exp(-phi_c^2 / sigma_phi)
+// is `pat`, from the bin's uniform word of the additive stream:
+// (r_c^2 / r_max^2)(1 + pat w_sa), w_sa ~ Rayleigh(sigma_sa) (Eq. 4).
+__device__ __forceinline__ float additive_term(float rc, float inv_rmax2, float pat, uint32_t word, float sig_sa) {
+    const float w_sa = rayleigh_of(word, sig_sa);
+    return rc * rc * inv_rmax2 * (1.0f + pat * w_sa);
+}
+
+__device__ __forceinline__ float pattern_of(const SensorDev& S, int col, float da, float inv_sphi) {
+    const float pc = fmaf(small_u2f((uint32_t)col) + 0.5f, da, -0.5f * S.hfov);
+    return 0.5f * expf(-pc * pc * inv_sphi);
+}
+
+__device__ __forceinline__ float norm_value(float In, float m, int mode) {
+    return (mode != 0 && m > 0.0f) ? In / m : In;
+}
+
+// v / m correctly rounded, given y = 1 / m correctly rounded, for v >= 2^-100
+// and 2^-60 <= m <= 2^60 (nothing under- or overflows): v y is within two ulp,
+// one residual step brings it within one, and a second one rounds correctly
+// (P. Markstein, IBM J. Res. Dev. 34(1), 1990).  Five FMA-pipe operations,
+// against nine and two on the quarter-rate unit for the general division.
+__device__ __forceinline__ float div_by(float v, float m, float y) {
+    float q = v * y;
+    q = fmaf(fmaf(-m, q, v), y, q);
+    return fmaf(fmaf(-m, q, v), y, q);
+}
+
+// Four neighbouring bins of one row share a Philox block (their index over
+// four), so a lane takes quads: q-th quad of the row, its columns
+// 4 q - sh + (0..3), sh = row * naz mod 4 (nonzero only where naz is not a
+// multiple of 4; the row's first and last quads then reach over its ends).
+//
+// A block takes a.rows_per_block rows of one band of 32, so the bitmap words of
+// its columns (and the columns' beam pattern) are read once into shared memory
+// and serve all its rows.  A bin with a return fetches P and the speckle factor
+// from its column's compact list; every other bin is the additive term alone.
+// REG > 0: a row of up to 128 REG bins stays in registers between its maximum
+// and the division, so I~ and N are written and nothing is read back; REG = 0
+// (wider rows, and the dense form of the fold's result): I~ is written, then read
+// back by the same lanes and divided.
+//
+// Bound by instruction issue (about 80 per bin, most of them the logarithm and a
+// quarter of a Philox block): 64 frames of 1000 x 512 bins in 98 us, 2.7 TB/s of
+// stores.  The 262 MB that it writes would take 39 us.
+template <int REG, bool VEC>
+__global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_constant__ RowsArgs a) {
+    extern __shared__ __align__(16) uint32_t rows_smem[];
+    __shared__ SensorDev S;
+    __shared__ int s_row0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp == 0) {
+        // the rows run from the last sensor back to the first, so that the first
+        // sensors' N is the last written and the fan finds it in L2
+        const int blk = gridDim.x - 1 - blockIdx.x;
+        if (a.sensors) {
+            const int2 m = __ldg(a.block_map + blk);
+            copy_words(&S, a.sensors + m.x, lane);
+            if (lane == 0) s_row0 = m.y;
+        } else {
+            copy_param(&S, &a.one, lane);
+            if (lane == 0) s_row0 = blk * a.rows_per_block;
+        }
+    }
+    __syncthreads();
+    const int naz = S.naz, nr = S.nr, row0 = s_row0;
+    const float dr = (S.rmax - S.rmin) / (float)nr, da = S.hfov / (float)naz;
+    const float inv_rmax2 = 1.0f / (S.rmax * S.rmax), inv_sphi = 1.0f / a.params.sigma_phi;
+    const float sig_sa = a.params.sigma_sa;
+    const int mode = a.params.normalise;
+    const bool dense = REG == 0 && a.dense;
+    const uint2* bands = a.bands + S.band_off + (int64_t)(row0 >> 5) * naz;
+    const bool staged = REG > 0 || naz <= kRowsStaged;
+    float* pat = reinterpret_cast<float*>(rows_smem);
+    uint2* mask = reinterpret_cast<uint2*>(rows_smem + ((naz + 3) & ~3));
+    if (staged) {
+        for (int c = tid; c < naz; c += blockDim.x) {
+            pat[c] = pattern_of(S, c, da, inv_sphi);
+            if (!dense) mask[c] = __ldg(bands + c);
+        }
+        __syncthreads();
+    }
+    const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
+    const uint32_t flo = S.frame_lo, fhi = S.frame_hi;
+    const float2* vals = a.vals + S.val_off;
+    float image_max = -CUDART_INF_F;
+    for (int r = warp; r < a.rows_per_block; r += 8) {
+        const int row = row0 + r;
+        if (row >= nr) break;
+        const uint32_t b0 = (uint32_t)row * (uint32_t)naz;
+        const int sh = VEC ? 0 : (int)(b0 & 3u), nq = (sh + naz + 3) >> 2;
+        const int64_t off = S.polar_off + (int64_t)b0 - sh;   // of the first quad's first bin
+        const float rc = fmaf(small_u2f((uint32_t)row) + 0.5f, dr, S.rmin);
+        const uint32_t bit = 1u << (row & 31);
+        // the four bins of quad q: I~ in v, P in p
+        auto quad = [&](int q, float (&v)[4], float (&p)[4]) {
+            float2 ret[4];
+            float pt[4];
+            uint2 w[4];
+            if (VEC && staged) {   // 16-byte shared-memory reads
+                const float4 p4 = *reinterpret_cast<const float4*>(pat + 4 * q);
+                pt[0] = p4.x; pt[1] = p4.y; pt[2] = p4.z; pt[3] = p4.w;
+                const uint4 w0 = *reinterpret_cast<const uint4*>(mask + 4 * q);
+                const uint4 w1 = *reinterpret_cast<const uint4*>(mask + 4 * q + 2);
+                w[0] = make_uint2(w0.x, w0.y); w[1] = make_uint2(w0.z, w0.w);
+                w[2] = make_uint2(w1.x, w1.y); w[3] = make_uint2(w1.z, w1.w);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 4 * q - sh + j;
+                ret[j] = make_float2(0.0f, 0.0f);
+                if (VEC || (c >= 0 && c < naz)) {
+                    if (!(VEC && staged)) pt[j] = staged ? pat[c] : pattern_of(S, c, da, inv_sphi);
+                    if (dense) {
+                        ret[j].x = a.dense[off + 4 * q + j];
+                        w[j].x = 0u;
+                    } else if (!(VEC && staged)) {
+                        w[j] = staged ? mask[c] : __ldg(bands + c);
+                    }
+                } else {
+                    w[j].x = 0u;
+                }
+            }
+            if ((w[0].x | w[1].x | w[2].x | w[3].x) & bit) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (w[j].x & bit) ret[j] = __ldg(vals + w[j].y + __popc(w[j].x & (bit - 1u)));
+            }
+            const U4 x = additive_words((b0 >> 2) + (uint32_t)q, flo, fhi, K);
+            const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 4 * q - sh + j;
+                v[j] = -CUDART_INF_F;
+                p[j] = ret[j].x;
+                if (VEC || (c >= 0 && c < naz)) {
+                    const float add = additive_term(rc, inv_rmax2, pt[j], xw[j], sig_sa);
+                    if (dense) {
+                        v[j] = add;
+                        if (ret[j].x != 0.0f)
+                            v[j] = fmaf(ret[j].x, 0.5f + gauss_of(bin_draws(b0 + (uint32_t)c, S, K), a.params.sigma_sm), add);
+                    } else {
+                        v[j] = fmaf(ret[j].x, ret[j].y, add);
+                    }
+                }
+            }
+            if (!VEC) {   // bins over the row's ends: no part in its maximum (nor in the least value)
+                const float most = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = v[j] == -CUDART_INF_F ? most : v[j];
+            }
+        };
+        auto store = [&](float* to, int q, const float (&v)[4]) {
+            if (VEC) {
+                *reinterpret_cast<float4*>(to + off + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c = 4 * q - sh + j;
+                    if (c >= 0 && c < naz) to[off + 4 * q + j] = v[j];
+                }
+            }
+        };
+        float m = -CUDART_INF_F;
+        if constexpr (REG > 0) {
+            float v[REG][4];
+#pragma unroll
+            for (int k = 0; k < REG; ++k) {
+                const int q = lane + 32 * k;
+                if (q < nq) {
+                    float p[4];
+                    quad(q, v[k], p);
+                    if (a.binned) store(a.binned, q, p);
+                    store(a.noised, q, v[k]);
+                } else {
+                    v[k][0] = v[k][1] = v[k][2] = v[k][3] = -CUDART_INF_F;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < REG; ++k) m = fmaxf(m, fmaxf(fmaxf(v[k][0], v[k][1]), fmaxf(v[k][2], v[k][3])));
+            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            if (mode != 2) {
+                // the row's values are the additive term (positive) and more unless a
+                // reflectivity is negative: the general division is the exception
+                bool plain = mode == 1 && m >= 0x1p-60f && m <= 0x1p60f;
+#pragma unroll
+                for (int k = 0; k < REG; ++k) {
+                    const float least = fminf(fminf(v[k][0], v[k][1]), fminf(v[k][2], v[k][3]));
+                    plain = plain && (least >= 0x1p-100f || lane + 32 * k >= nq);
+                }
+                const float y = 1.0f / m;
+#pragma unroll
+                for (int k = 0; k < REG; ++k) {
+                    const int q = lane + 32 * k;
+                    if (q < nq) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            v[k][j] = plain ? div_by(v[k][j], m, y) : norm_value(v[k][j], m, mode);
+                        store(a.polar, q, v[k]);
+                    }
+                }
+            }
+        } else {
+            for (int q = lane; q < nq; q += 32) {
+                float v[4], p[4];
+                quad(q, v, p);
+                if (a.binned) store(a.binned, q, p);
+                store(a.noised, q, v);
+                m = fmaxf(m, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+            }
+            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            if (mode != 2) {
+                for (int q = lane; q < nq; q += 32) {
+                    float v[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = 4 * q - sh + j;
+                        v[j] = VEC || (c >= 0 && c < naz) ? norm_value(a.noised[off + 4 * q + j], m, mode) : 0.0f;
+                    }
+                    store(a.polar, q, v);
+                }
+            }
+        }
+        image_max = fmaxf(image_max, m);
+    }
+    // whole-image normalisation: the maximum of the image, divided by in a launch of its own
+    if (mode == 2 && lane == 0) atomicMax(a.gmax + S.rowmax_off, ord_enc(image_max));
+}
+
 // The noise stream itself: Philox4x32-10 of n counters under one key, the
-// same round function the binning, adjoint and DVL kernels draw from.
+// same round function the fold, row, adjoint and DVL kernels draw from.
 __global__ void __launch_bounds__(256) k_philox_words(const uint4* ctr, int64_t n, uint32_t k0, uint32_t k1,
                                                       uint4* out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -510,9 +477,9 @@ __global__ void __launch_bounds__(256) k_philox_words(const uint4* ctr, int64_t 
     out[i] = make_uint4(x.x, x.y, x.z, x.w);
 }
 
-__device__ __forceinline__ float norm_value(float In, float m, int mode) {
-    return (mode != 0 && m > 0.0f) ? In / m : In;
-}
+// ---------------------------------------------------------------------------
+// phase 2a: range-wise normalisation, one warp per (sensor, range row)
+// ---------------------------------------------------------------------------
 
 // One row: its maximum over azimuth and N = I~ / max (any alignment and width).
 __device__ __forceinline__ void norm_row(const NormArgs& a, int64_t g, int lane) {
@@ -1065,22 +1032,36 @@ __global__ void __launch_bounds__(256) k_adj_final(const double* partials, int n
 // ---------------------------------------------------------------------------
 
 void set_kernel_attributes() {
-    cudaFuncSetAttribute(k_bin<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-    cudaFuncSetAttribute(k_bin<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    cudaFuncSetAttribute(k_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    cudaFuncSetAttribute(k_rows<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    cudaFuncSetAttribute(k_rows<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
     cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
 }
 
-cudaError_t launch_bin(const BinArgs& a, int det, int grid, int block, size_t smem, cudaStream_t st) {
-    if (det) k_bin<1><<<grid, block, smem, st>>>(a);
-    else k_bin<0><<<grid, block, smem, st>>>(a);
+cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
+    if (grid > 0) k_fold<<<grid, block, smem, st>>>(a);
     return cudaGetLastError();
 }
 
-int bin_blocks_per_sm(int det, int block, size_t smem) {
-    int n = 0;
-    const void* f = det ? (const void*)k_bin<1> : (const void*)k_bin<0>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, block, smem) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
+// The row kernel for rows of up to `naz` bins: in registers up to 512 and up to
+// 1024 bins, else written and read back.  `vec`: 16-byte stores (every row of
+// every sensor starts on a 16-byte boundary of each image).
+cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st) {
+    if (grid <= 0) return cudaSuccess;
+    // a row whose first bin is not a multiple of 4 may need one quad more
+    const int reach = vec ? naz : naz + 3;
+    const size_t smem = naz <= kRowsStaged ? ((size_t)((naz + 3) & ~3) + 2 * (size_t)naz) * sizeof(uint32_t) : 0;
+    if (reach <= 512 && !a.dense) {
+        if (vec) k_rows<4, true><<<grid, 256, smem, st>>>(a);
+        else k_rows<4, false><<<grid, 256, smem, st>>>(a);
+    } else if (reach <= 1024 && !a.dense) {
+        if (vec) k_rows<8, true><<<grid, 256, smem, st>>>(a);
+        else k_rows<8, false><<<grid, 256, smem, st>>>(a);
+    } else {
+        if (vec) k_rows<0, true><<<grid, 256, smem, st>>>(a);
+        else k_rows<0, false><<<grid, 256, smem, st>>>(a);
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, void* out, cudaStream_t st) {

@@ -21,9 +21,9 @@ using namespace sonar;
 namespace {
 
 struct Tune {
-    int cols = 0;     // binning: azimuth columns per work unit (0: derive)
+    int cols = 1;     // kept for saved rows: the fold takes one azimuth column per warp
     int tb = 0;       // tracing: beams per warp tile, elevations = 32 / tb (0: derive)
-    int block = 128;  // binning: threads per block
+    int block = 128;  // adjoint: threads per block (which also sets its ray chunks)
     int occ = 0;      // tracing variant: kTraceCap caps registers at 64 (32 one-warp blocks per SM),
                       // kTraceWide walks the 8-wide tree
 };
@@ -45,7 +45,7 @@ struct sonar_ctx {
     std::vector<bool> alive;
     std::string last_error;
     uint32_t* d_err = nullptr;
-    Scratch rowmax, noised, rowinfo, partials, counters, hits, trig;
+    Scratch rowmax, noised, rowinfo, partials, counters, hits, trig, vals, bands;
     // the exact-ray tables last built by a single-sensor call: their buffer and
     // the angular geometry they hold (beams, elevations, fields of view)
     const float4* trig_at = nullptr;
@@ -135,18 +135,11 @@ sonar_status check_nmat(sonar_ctx* ctx, int32_t scene, int32_t n_mat) {
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Tile shape for a sensor: the tuning cache entry, else one block-wide ray
-// tile per unit, bounded by the shared-memory column block.
+// Launch shapes for a sensor: the tuning cache entry, else the defaults.
 Tune tune_for(const sonar_ctx* ctx, const sonar_sensor& s) {
     Tune t;
     auto it = ctx->tune.find(ShapeKey{s.n_beams, s.n_elev, s.n_range_bins, s.n_az_bins});
     if (it != ctx->tune.end()) t = it->second;
-    const int bpc = std::max(1, s.n_beams / std::max(1, s.n_az_bins));
-    if (t.cols <= 0) t.cols = std::max(1, t.block / std::max(1, s.n_elev * bpc));
-    // a unit's column block, its bitmap (a bit per bin) and its list (at most a
-    // word per bin) fit the dynamic shared memory: bins * 65 / 32 words
-    const int max_cols_smem = std::max(1, (int)(kMaxDynSmem / 4 * 32 / 65) / s.n_range_bins);
-    t.cols = std::max(1, std::min({t.cols, s.n_az_bins, max_cols_smem, kMaxCols}));
     if (t.block < 32 || t.block > 512 || (t.block & 31)) t.block = 128;
     if (t.tb <= 0) t.tb = 8;
     if (t.tb > 32 || (t.tb & (t.tb - 1))) t.tb = 8;
@@ -172,31 +165,39 @@ int single_variant(const sonar_ctx* ctx, const sonar_sensor& s, int tb, int occ)
     return occ & ~kTraceWide;
 }
 
-// A single frame alone on the GPU: the tuned shapes, but binning units of
-// about two per SM (the batch tunes may favour few, large units) and at least
-// four columns wide, a multiple of 4 where the row allows, so that the noise
-// pass draws four bins per Philox block; and the ray-cast variant chosen by the
-// frame's own launch size.
+// A single frame alone on the GPU: the tuned shapes, and the ray-cast variant
+// chosen by the frame's own launch size.
 Tune single_tune(const sonar_ctx* ctx, const sonar_sensor& s) {
     Tune t = tune_for(ctx, s);
-    int cols = std::max(4, s.n_az_bins / (2 * ctx->sm_count));
-    if (s.n_az_bins % 4 == 0) cols &= ~3;
-    const int max_cols_smem = std::max(1, (int)(kMaxDynSmem / 4 * 32 / 65) / s.n_range_bins);
-    t.cols = std::max(1, std::min({cols, s.n_az_bins, max_cols_smem, kMaxCols}));
     t.occ = single_variant(ctx, s, t.tb, t.occ);
     return t;
 }
 
-// Most beams a binning unit of this sensor covers (its columns' beams).
-int64_t unit_beams_max(const SensorDev& s) {
-    int64_t most = 0;
-    for (int t = 0; t < s.n_tiles; ++t) {
-        const int64_t c0 = (int64_t)t * s.cols, c1 = std::min<int64_t>(c0 + s.cols, s.naz);
-        most = std::max<int64_t>(most, first_beam_of_col(c1, s.nb, s.naz) - first_beam_of_col(c0, s.nb, s.naz));
-    }
-    return most;
+// Most beams of an azimuth column (n_beams spread over n_az_bins columns).
+int64_t col_beams_max(const SensorDev& s) { return (s.nb + (int64_t)s.naz - 1) / s.naz; }
+
+int64_t band_count(const SensorDev& s) { return ((int64_t)s.nr + 31) / 32; }
+
+// Shared-memory words of a column in the fold: the rows' bitmap and its ranks,
+// then the rows and sums of the bins with returns (no more than rays, nor than
+// rows), the sums per beam in the per-beam form.
+int64_t fold_words(const SensorDev& s) {
+    const int64_t most = std::min<int64_t>(s.nr, col_beams_max(s) * s.ne);
+    return 2 * band_count(s) + most * (1 + (s.fold_beams ? col_beams_max(s) : 1));
 }
-int64_t unit_rays_max(const SensorDev& s) { return unit_beams_max(s) * (int64_t)s.ne; }
+
+// Warps of a fold block: four columns, or the beams of one column (up to 16).
+int fold_warps(const SensorDev& s) {
+    return s.fold_beams ? (int)std::max<int64_t>(4, std::min<int64_t>(16, col_beams_max(s))) : 4;
+}
+
+// Rows per block of the row kernel: a whole band of 32, which reads the band's
+// column tables once, while that leaves at least eight blocks an SM; else 16 or 8.
+int rows_per_block(int64_t total_rows, int sm_count) {
+    for (int r : {32, 16})
+        if (total_rows / r >= 8ll * sm_count) return r;
+    return 8;
+}
 
 SensorDev make_sensor(const sonar_sensor& s, uint64_t seed, uint64_t frame, const Tune& t, int fan_w,
                       int fan_h) {
@@ -223,32 +224,18 @@ SensorDev make_sensor(const sonar_sensor& s, uint64_t seed, uint64_t frame, cons
     d.seed_hi = (uint32_t)(seed >> 32);
     d.frame_lo = (uint32_t)frame;
     d.frame_hi = (uint32_t)(frame >> 32);
-    d.cols = t.cols;
-    d.n_tiles = (s.n_az_bins + t.cols - 1) / t.cols;
     const int tb = (t.tb >= 1 && t.tb <= 32 && (t.tb & (t.tb - 1)) == 0) ? t.tb : 8;   // beams per warp tile
     d.tb = tb;
     d.occ = t.occ;
     const int64_t be = 32 / tb;   // ray-cast blocks: one warp on tb beams x be elevations
     d.trace_blocks = (int32_t)(((s.n_beams + tb - 1) / tb) * ((s.n_elev + be - 1) / be));
-    // The per-beam fold when columns hold several beams (n_beams > n_az_bins:
-    // with one beam per column both folds add in the same order, and the
-    // all-warp fold is faster) and its rows fit in shared memory next to the
-    // column block and the list.  The choice depends on the sensor shape alone
-    // (it is made for one column per unit), so every tile shape folds in the
-    // same order; wider units are narrowed until they fit.
-    auto fits = [&](const SensorDev& x) {
-        const int64_t bins = (int64_t)x.nr * x.cols;
-        const int64_t need = bins + unit_beams_max(x) * x.nr + (bins + 31) / 32 + std::min<int64_t>(unit_rays_max(x), bins);
-        return need * (int64_t)sizeof(float) <= (int64_t)kMaxDynSmem;
-    };
-    SensorDev one_col = d;
-    one_col.cols = 1;
-    one_col.n_tiles = s.n_az_bins;
-    d.fold_beams = (s.n_beams > s.n_az_bins && fits(one_col)) ? 1 : 0;
-    while (d.fold_beams && d.cols > 1 && !fits(d)) {
-        d.cols = std::max(1, d.cols / 2);
-        d.n_tiles = (s.n_az_bins + d.cols - 1) / d.cols;
-    }
+    // The per-beam fold when columns hold several beams (n_beams > n_az_bins)
+    // and a column's dense rows, one per beam, would fit 200 KB of shared memory.
+    // The choice depends on the sensor shape alone, so a bin's order of summation
+    // never depends on how the frame is launched.
+    const int64_t beams = col_beams_max(d), dense = (int64_t)d.nr * (1 + beams) + (d.nr + 31) / 32 +
+                                                    std::min<int64_t>(beams * d.ne, d.nr);
+    d.fold_beams = (s.n_beams > s.n_az_bins && dense * (int64_t)sizeof(float) <= 200 * 1024) ? 1 : 0;
     return d;
 }
 
@@ -288,7 +275,7 @@ extern "C" sonar_status sonar_destroy(sonar_ctx_t ctx) {
     cudaDeviceSynchronize();
     for (auto& s : ctx->scenes) free_scene(&s);
     for (Scratch* s : {&ctx->rowmax, &ctx->noised, &ctx->rowinfo, &ctx->partials, &ctx->counters, &ctx->hits,
-                       &ctx->trig})
+                       &ctx->trig, &ctx->vals, &ctx->bands})
         if (s->p) cudaFreeAsync(s->p, 0);
     cudaDeviceSynchronize();
     cudaFree(ctx->d_err);
@@ -372,15 +359,6 @@ extern "C" sonar_status sonar_scene_info(sonar_ctx_t ctx, int32_t id, int64_t ou
 namespace {
 
 
-// Shared memory of a binning block: the column block of the unit, the per-beam
-// rows of the fold if any, a bitmap of the bins with returns, and the list of
-// those bins (no more entries than rays, nor than bins).
-size_t bin_smem(const SensorDev& s) {
-    const int64_t bins = (int64_t)s.nr * s.cols;
-    const int64_t beams = s.fold_beams ? unit_beams_max(s) * s.nr : 0;   // per-beam rows of the fold
-    return (size_t)(bins + beams + (bins + 31) / 32 + std::min<int64_t>(unit_rays_max(s), bins)) * sizeof(float);
-}
-
 // The context's exact-ray table buffer, grown to `entries`; a new buffer holds
 // no tables yet.
 cudaError_t grow_trig(sonar_ctx* ctx, size_t entries, cudaStream_t s) {
@@ -412,10 +390,18 @@ cudaError_t single_trig(sonar_ctx* ctx, const SensorDev& S, cudaStream_t s) {
     return e;
 }
 
-// Trace, bin and noise of one sensor (polar_off = hits_off = rowmax_off = 0).
+// Where a single-sensor call keeps its fold's result: the compact lists, or (no
+// room for them) P of the bins with returns in the polar image itself.
+struct FoldStore {
+    float2* vals = nullptr;
+    uint2* bands = nullptr;
+    float* dense = nullptr;
+};
+
+// Trace, fold, noise and row normalisation of one sensor (all offsets 0).
 sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& sc, const sonar_params* p,
-                            const float* d_theta, int32_t n_mat, sonar_hit* hits, float* noised, float* binned,
-                            uint32_t* gmax, int block, cudaStream_t s) {
+                            const float* d_theta, int32_t n_mat, sonar_hit* hits, const FoldStore& f, float* noised,
+                            float* binned, float* polar, uint32_t* gmax, cudaStream_t s) {
     if (p->normalise == 2) CU(cudaMemsetAsync(gmax, 0, sizeof(uint32_t), s), "cudaMemsetAsync");
     CU(single_trig(ctx, S, s), "trig launch");
     TraceArgs t{};
@@ -425,33 +411,53 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     t.hits = hits;
     t.err = ctx->d_err;
     CU(launch_trace(t, S.trace_blocks, S.occ, s), "trace launch");
-    BinArgs a{};
-    a.n_units = S.n_tiles;
+    if (f.dense) CU(cudaMemsetAsync(f.dense, 0, sizeof(float) * (size_t)S.nr * S.naz, s), "cudaMemsetAsync");
+    FoldArgs a{};
     a.n_mat = n_mat;
+    a.words_per_warp = (int32_t)fold_words(S);
     a.one = S;
     a.one_scene = sc;
     a.theta = d_theta;
-    a.params = *p;
+    a.sigma_sm = p->sigma_sm;
     a.hits = hits;
-    a.noised = noised;
-    a.binned = binned;
-    a.rowmax = gmax;
+    a.vals = f.vals;
+    a.bands = f.bands;
+    a.dense = f.dense;
     a.err = ctx->d_err;
-    CU(launch_bin(a, p->accumulate == 0, S.n_tiles, block, bin_smem(S), s), "binning launch");
+    int warps = fold_warps(S);
+    if (!S.fold_beams)
+        while (warps > 1 && sizeof(uint32_t) * warps * fold_words(S) > kMaxDynSmem) warps /= 2;
+    const size_t smem = sizeof(uint32_t) * fold_words(S) * (S.fold_beams ? 1 : warps);
+    CU(launch_fold(a, S.fold_beams ? S.naz : (S.naz + warps - 1) / warps, 32 * warps, smem, s), "fold launch");
+    RowsArgs r{};
+    r.rows_per_block = rows_per_block(S.nr, ctx->sm_count);
+    r.one = S;
+    r.params = *p;
+    r.vals = f.vals;
+    r.bands = f.bands;
+    r.dense = f.dense;
+    r.noised = noised;
+    r.binned = binned;
+    r.polar = polar;
+    r.gmax = gmax;
+    const bool vec = S.naz % 4 == 0 && aligned16(noised) && aligned16(polar) && aligned16(binned);
+    CU(launch_rows(r, (S.nr + r.rows_per_block - 1) / r.rows_per_block, S.naz, vec, s), "row launch");
     return SONAR_OK;
 }
 
-// Normalisation and fan of one sensor (polar_off = fan_off = rowmax_off = 0).
+// Whole-image normalisation (mode 2) and fan of one sensor (all offsets 0).
 sonar_status single_post(sonar_ctx* ctx, const SensorDev& S, int normalise, const float* noised,
                          const uint32_t* gmax, float* polar, float* fan, cudaStream_t s) {
-    NormArgs n{};
-    n.one = S;
-    n.total_rows = S.nr;
-    n.noised = noised;
-    n.gmax = gmax;
-    n.normalise = normalise;
-    n.polar = polar;
-    CU(launch_norm(n, s), "normalisation launch");
+    if (normalise == 2) {
+        NormArgs n{};
+        n.one = S;
+        n.total_rows = S.nr;
+        n.noised = noised;
+        n.gmax = gmax;
+        n.normalise = normalise;
+        n.polar = polar;
+        CU(launch_norm(n, s), "normalisation launch");
+    }
     if (fan) {
         FanArgs f{};
         f.one = S;
@@ -505,10 +511,12 @@ extern "C" sonar_status sonar_render(sonar_ctx_t ctx, int32_t scene_id, const so
     }
     CU(grow_trig(ctx, (size_t)(S.nb + S.ne), s), "scratch allocation");
     S.trig = (float4*)ctx->trig.p;
-    sonar_status st2 = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, noised,
-                                      out->binned, (uint32_t*)ctx->rowmax.p, t.block, s);
+    CU(grow(ctx->vals, sizeof(float2) * (size_t)S.nb * S.ne, s), "scratch allocation");
+    CU(grow(ctx->bands, sizeof(uint2) * (size_t)band_count(S) * S.naz, s), "scratch allocation");
+    const FoldStore fold{(float2*)ctx->vals.p, (uint2*)ctx->bands.p, nullptr};
+    sonar_status st2 = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, fold,
+                                      noised, out->binned, out->polar, (uint32_t*)ctx->rowmax.p, s);
     if (st2 != SONAR_OK) return st2;
-    (void)npol;
     return single_post(ctx, S, params->normalise, noised, (const uint32_t*)ctx->rowmax.p, out->polar, out->fan, s);
 }
 
@@ -520,9 +528,7 @@ extern "C" sonar_status sonar_fan_resample(sonar_ctx_t ctx, const sonar_sensor* 
     if (!d_polar || !d_fan) return fail(ctx, SONAR_ERR_ARG, "NULL polar or fan");
     if (fan_w < 1 || fan_h < 1) return fail(ctx, SONAR_ERR_ARG, "fan size must be >= 1");
     CU(cudaSetDevice(ctx->device), "cudaSetDevice");
-    Tune t;
-    t.cols = 1;
-    const SensorDev S = make_sensor(*sensor, 0, 0, t, fan_w, fan_h);
+    const SensorDev S = make_sensor(*sensor, 0, 0, Tune{}, fan_w, fan_h);
     FanArgs f{};
     f.one = S;
     f.polar = d_polar;
@@ -601,7 +607,8 @@ struct sonar_batch {
     sonar_ctx* ctx = nullptr;
     std::vector<sonar_batch_item> items;
     std::vector<SensorDev> hs;        // host copy of the descriptors
-    std::vector<Unit> units;          // forward work list (column tiles)
+    std::vector<int4> fold_map;       // per fold block: (sensor, first column, scene, 0)
+    std::vector<int2> rows_map;       // per row-kernel block: (sensor, first row)
     std::vector<AdjUnit> adj_units;   // adjoint work list (ray chunks)
     std::vector<int32_t> fan_prefix;  // fan blocks per sensor, prefix
     std::vector<int32_t> trace_prefix;  // trace blocks per sensor, prefix
@@ -610,9 +617,15 @@ struct sonar_batch {
     int block = 128;
     int trace_occ = 0;
     int adj_chunk = 0;
-    size_t smem1 = 0;
+    size_t fold_smem = 0;
+    int fold_block = 128, fold_words_per_warp = 0;
+    int rows_step = 32, max_naz = 1;
+    bool rows_vec = false;            // every row starts on a 16-byte boundary of a 16-byte aligned image
     SensorDev* d_sens = nullptr;
-    Unit* d_units = nullptr;
+    int4* d_fold_map = nullptr;
+    int2* d_rows_map = nullptr;
+    float2* d_vals = nullptr;         // the fold's values, a slot per ray
+    uint2* d_bands = nullptr;         // the fold's bitmaps
     AdjUnit* d_adj_units = nullptr;
     SceneDev* d_scenes = nullptr;
     int32_t* d_fan_prefix = nullptr;
@@ -641,7 +654,7 @@ struct sonar_batch {
     float* d_noised = nullptr;
     RowInfo* d_rowinfo = nullptr;
     double* d_partials = nullptr;
-    int32_t* d_counters = nullptr;    // [0] phase-1 work, [1] adjoint work
+    int32_t* d_counters = nullptr;    // [1] adjoint work
     int n_mat_cap = 0;
     size_t n_scene_table = 0;         // entries in d_scenes
     // host staging for updates (pinned, double-buffered)
@@ -671,7 +684,8 @@ struct sonar_batch {
 namespace {
 
 void batch_free_device(sonar_batch* b) {
-    for (void* p : {(void*)b->d_sens, (void*)b->d_units, (void*)b->d_adj_units, (void*)b->d_scenes,
+    for (void* p : {(void*)b->d_sens, (void*)b->d_fold_map, (void*)b->d_rows_map, (void*)b->d_vals,
+                    (void*)b->d_bands, (void*)b->d_adj_units, (void*)b->d_scenes,
                     (void*)b->d_fan_prefix, (void*)b->d_trace_prefix, (void*)b->d_trace_map,
                     (void*)b->d_fan_map, (void*)b->d_row_map, (void*)b->d_hits, (void*)b->d_trig, (void*)b->d_trig_stamp,
                     (void*)b->d_rowmax,
@@ -694,7 +708,8 @@ void batch_free_device(sonar_batch* b) {
     b->d_trig = nullptr;
     b->d_trig_stamp = nullptr;
     b->n_mat_cap = 0;
-    b->d_sens = nullptr; b->d_units = nullptr; b->d_adj_units = nullptr; b->d_scenes = nullptr;
+    b->d_fold_map = nullptr; b->d_rows_map = nullptr; b->d_vals = nullptr; b->d_bands = nullptr;
+    b->d_sens = nullptr; b->d_adj_units = nullptr; b->d_scenes = nullptr;
     b->d_fan_prefix = nullptr;
     b->d_rowmax = nullptr; b->d_noised = nullptr; b->d_rowinfo = nullptr; b->d_partials = nullptr;
     b->d_counters = nullptr;
@@ -745,12 +760,14 @@ sonar_status batch_plan(sonar_batch* b) {
     batch_free_device(b);
     const int n = (int)b->items.size();
     b->hs.assign(n, SensorDev{});
-    b->units.clear();
+    b->fold_map.clear();
+    b->rows_map.clear();
     b->adj_units.clear();
     b->fan_prefix.assign(n + 1, 0);
     b->trace_prefix.assign(n + 1, 0);
-    b->smem1 = 0;
-    int64_t rows = 0, polar_end = 0;
+    int64_t rows = 0, polar_end = 0, rays = 0, bands = 0;
+    b->max_naz = 1;
+    b->rows_vec = true;
     std::map<int, int64_t> block_votes;
     for (int k = 0; k < n; ++k) {
         const sonar_batch_item& it = b->items[k];
@@ -761,6 +778,12 @@ sonar_status batch_plan(sonar_batch* b) {
         S.hits_off = it.hits_offset;
         S.fan_off = it.fan_offset;
         S.rowmax_off = rows;
+        S.val_off = rays;
+        S.band_off = bands;
+        rays += (int64_t)S.nb * S.ne;
+        bands += band_count(S) * S.naz;
+        b->max_naz = std::max(b->max_naz, S.naz);
+        b->rows_vec = b->rows_vec && S.naz % 4 == 0 && S.polar_off % 4 == 0;
         rows += S.nr;    // room for mode 1; mode 2 uses the first slot of each sensor
         polar_end = std::max<int64_t>(polar_end, it.polar_offset + (int64_t)S.nr * S.naz);
         b->hs[k] = S;
@@ -768,23 +791,7 @@ sonar_status batch_plan(sonar_batch* b) {
             b->fan_prefix[k] + (S.fan_w > 0 ? tile_squares(S.fan_w, S.fan_h) : 0);
         b->trace_prefix[k + 1] = b->trace_prefix[k] + S.trace_blocks;
         block_votes[t.block] += (int64_t)S.nb * S.ne;
-        for (int tile = 0; tile < S.n_tiles; ++tile) {
-            Unit u;
-            u.sensor = k;
-            u.scene = S.scene;
-            u.c0 = tile * S.cols;
-            u.c1 = std::min(u.c0 + S.cols, S.naz);
-            const int64_t i0 = first_beam_of_col(u.c0, S.nb, S.naz), i1 = first_beam_of_col(u.c1, S.nb, S.naz);
-            u.rays = (int32_t)((i1 - i0) * S.ne);
-            b->units.push_back(u);
-        }
-        b->smem1 = std::max(b->smem1, bin_smem(S));
     }
-    // largest units first: the persistent blocks then finish close together
-    std::stable_sort(b->units.begin(), b->units.end(), [&](const Unit& x, const Unit& y) {
-        return (int64_t)x.rays * 4 + b->hs[x.sensor].nr * (x.c1 - x.c0) / 64 >
-               (int64_t)y.rays * 4 + b->hs[y.sensor].nr * (y.c1 - y.c0) / 64;
-    });
     b->block = 128;
     int64_t best = -1;
     for (auto& kv : block_votes)
@@ -807,6 +814,23 @@ sonar_status batch_plan(sonar_batch* b) {
     }
     b->total_rows = rows;
     b->total_polar = polar_end;
+    // the fold's blocks: the warps that the sensor with most rays wants, fewer
+    // where the columns of some sensor need more shared memory than that
+    int warps = n > 0 ? fold_warps(b->hs[kmost]) : 4;
+    int64_t warp_words = 0, block_words = 0;
+    for (const SensorDev& S : b->hs) (S.fold_beams ? block_words : warp_words) =
+        std::max(S.fold_beams ? block_words : warp_words, fold_words(S));
+    while (warps > 1 && (int64_t)sizeof(uint32_t) * warps * warp_words > (int64_t)kMaxDynSmem) warps /= 2;
+    b->fold_block = 32 * warps;
+    b->fold_words_per_warp = (int)warp_words;
+    b->fold_smem = sizeof(uint32_t) * (size_t)std::max(block_words, warps * warp_words);
+    b->rows_step = rows_per_block(rows, ctx->sm_count);
+    for (int k = 0; k < n; ++k) {
+        const SensorDev& S = b->hs[k];
+        const int step = S.fold_beams ? 1 : warps;
+        for (int c = 0; c < S.naz; c += step) b->fold_map.push_back(make_int4(k, c, S.scene, 0));
+        for (int r = 0; r < S.nr; r += b->rows_step) b->rows_map.push_back(make_int2(k, r));
+    }
     int64_t all_rays = 0;
     for (const SensorDev& S : b->hs) all_rays += (int64_t)S.nb * S.ne;
     b->total_rays = all_rays;
@@ -817,13 +841,16 @@ sonar_status batch_plan(sonar_batch* b) {
             b->adj_units.push_back(AdjUnit{k, (int32_t)r0, (int32_t)std::min<int64_t>(r, r0 + b->adj_chunk),
                                            b->hs[k].scene});
     }
-    const size_t nu = b->units.size(), na = b->adj_units.size();
+    const size_t na = b->adj_units.size();
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void** p, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(p, std::max(bytes, (size_t)16));
     };
     alloc((void**)&b->d_sens, sizeof(SensorDev) * n);
-    alloc((void**)&b->d_units, sizeof(Unit) * nu);
+    alloc((void**)&b->d_fold_map, sizeof(int4) * b->fold_map.size());
+    alloc((void**)&b->d_rows_map, sizeof(int2) * b->rows_map.size());
+    alloc((void**)&b->d_vals, sizeof(float2) * rays);
+    alloc((void**)&b->d_bands, sizeof(uint2) * bands);
     alloc((void**)&b->d_scenes, sizeof(SceneDev) * std::max<size_t>(1, ctx->scenes.size()));
     b->n_scene_table = ctx->scenes.size();
     alloc((void**)&b->d_adj_units, sizeof(AdjUnit) * na);
@@ -977,7 +1004,10 @@ sonar_status batch_plan(sonar_batch* b) {
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch allocation");
     const std::vector<SceneDev> table = scene_table(ctx);
     e = cudaMemcpy(b->d_sens, b->hs.data(), sizeof(SensorDev) * n, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_units, b->units.data(), sizeof(Unit) * nu, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(b->d_fold_map, b->fold_map.data(), sizeof(int4) * b->fold_map.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(b->d_rows_map, b->rows_map.data(), sizeof(int2) * b->rows_map.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !table.empty())
         e = cudaMemcpy(b->d_scenes, table.data(), sizeof(SceneDev) * table.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -1008,12 +1038,6 @@ cudaError_t batch_scratch(sonar_batch* b, const sonar_batch_outputs* out) {
     return e;
 }
 
-int persistent_grid(const sonar_batch* b, int det) {
-    const int per_sm = bin_blocks_per_sm(det, b->block, b->smem1);
-    const int64_t g = std::min<int64_t>((int64_t)b->units.size(), (int64_t)b->ctx->sm_count * per_sm);
-    return (int)std::max<int64_t>(1, g);
-}
-
 // Kernel nodes of a captured graph (-1 if the graph cannot be inspected).
 int kernel_nodes(cudaGraph_t g) {
     size_t n = 0;
@@ -1035,13 +1059,13 @@ void append_bytes(std::vector<unsigned char>& v, const T& x) {
     v.insert(v.end(), p, p + sizeof(T));
 }
 
-// The forward's launches: part 1 up to binning (trig tables, ray cast, binning
-// and noise), part 2 the normalisation and fan, part 0 both.
+// The forward's launches: part 1 up to I~ (trig tables, ray cast, fold, and the
+// row kernel, which also normalises by rows), part 2 the whole-image
+// normalisation and the fan, part 0 both.
 sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const float* d_theta, int32_t n_mat,
                                     const sonar_batch_outputs* out, cudaStream_t s, bool events = false,
                                     int part = 0, bool tables = true) {
     sonar_ctx* ctx = b->ctx;
-    const int det = p->accumulate == 0;
     if (part != 2) {
         if (p->normalise == 2)
             CU(cudaMemsetAsync(b->d_rowmax, 0, sizeof(uint32_t) * b->total_rows, s), "cudaMemsetAsync");
@@ -1057,37 +1081,49 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         t.params = *p;
         t.hits = hits;
         t.err = ctx->d_err;
-        t.zero_word = b->d_counters;   // the binning's work counter, cleared for the launch after
         CU(launch_trace(t, b->trace_prefix.back(), b->trace_occ, s), "batch trace launch");
         if (events) CU(cudaEventRecordWithFlags(b->ev[6], s, cudaEventRecordExternal), "cudaEventRecord");
-        BinArgs a{};
+        FoldArgs a{};
         a.sensors = b->d_sens;
-        a.units = b->d_units;
         a.scenes = b->d_scenes;
-        a.work_counter = b->d_counters;
-        a.n_units = (int32_t)b->units.size();
+        a.block_map = b->d_fold_map;
         a.n_mat = n_mat;
+        a.words_per_warp = b->fold_words_per_warp;
         a.theta = d_theta;
-        a.params = *p;
-        a.noised = out->noised ? out->noised : b->d_noised;
-        a.binned = out->binned;
+        a.sigma_sm = p->sigma_sm;
         a.hits = hits;
-        a.rowmax = b->d_rowmax;
+        a.vals = b->d_vals;
+        a.bands = b->d_bands;
         a.err = ctx->d_err;
-        CU(launch_bin(a, det, persistent_grid(b, det), b->block, b->smem1, s), "batch binning launch");
+        CU(launch_fold(a, (int)b->fold_map.size(), b->fold_block, b->fold_smem, s), "batch fold launch");
+        RowsArgs r{};
+        r.sensors = b->d_sens;
+        r.block_map = b->d_rows_map;
+        r.rows_per_block = b->rows_step;
+        r.params = *p;
+        r.vals = b->d_vals;
+        r.bands = b->d_bands;
+        r.noised = out->noised ? out->noised : b->d_noised;
+        r.binned = out->binned;
+        r.polar = out->polar;
+        r.gmax = b->d_rowmax;
+        const bool vec = b->rows_vec && aligned16(r.noised) && aligned16(r.binned) && aligned16(r.polar);
+        CU(launch_rows(r, (int)b->rows_map.size(), b->max_naz, vec, s), "batch row launch");
         if (events) CU(cudaEventRecordWithFlags(b->ev[1], s, cudaEventRecordExternal), "cudaEventRecord");
     }
     if (part == 1) return SONAR_OK;
-    NormArgs c{};
-    c.sensors = b->d_sens;
-    c.row_map = b->d_row_map;
-    c.n_sensors = (int32_t)b->items.size();
-    c.total_rows = b->total_rows;
-    c.noised = out->noised ? out->noised : b->d_noised;
-    c.gmax = b->d_rowmax;
-    c.normalise = p->normalise;
-    c.polar = out->polar;
-    CU(launch_norm(c, s), "batch normalisation launch");
+    if (p->normalise == 2) {
+        NormArgs c{};
+        c.sensors = b->d_sens;
+        c.row_map = b->d_row_map;
+        c.n_sensors = (int32_t)b->items.size();
+        c.total_rows = b->total_rows;
+        c.noised = out->noised ? out->noised : b->d_noised;
+        c.gmax = b->d_rowmax;
+        c.normalise = p->normalise;
+        c.polar = out->polar;
+        CU(launch_norm(c, s), "batch normalisation launch");
+    }
     if (out->fan) {
         FanArgs f{};
         f.sensors = b->d_sens;
@@ -1185,7 +1221,7 @@ extern "C" sonar_status sonar_batch_update(sonar_batch_t b, const sonar_batch_it
         SensorDev S = b->hs[k];
         scene_moved |= S.scene != items[k].scene_id;
         const sonar_batch_item& it = items[k];
-        const SensorDev fresh = make_sensor(it.sensor, it.seed, it.frame, Tune{S.cols, S.tb, b->block, S.occ},
+        const SensorDev fresh = make_sensor(it.sensor, it.seed, it.frame, Tune{1, S.tb, b->block, S.occ},
                                             it.fan_w, it.fan_h);
         memcpy(S.pos, fresh.pos, sizeof S.pos);
         memcpy(S.rot, fresh.rot, sizeof S.rot);
@@ -1212,13 +1248,14 @@ extern "C" sonar_status sonar_batch_update(sonar_batch_t b, const sonar_batch_it
        "descriptor upload");
     if (scene_moved) {   // the ray-cast map and the work units carry their scene: patch them (rare, pageable copies)
         for (int4& m : b->h_trace_map) m.z = b->hs[m.x].scene;
-        for (Unit& x : b->units) x.scene = b->hs[x.sensor].scene;
+        for (int4& m : b->fold_map) m.z = b->hs[m.x].scene;
         for (AdjUnit& x : b->adj_units) x.scene = b->hs[x.sensor].scene;
         CU(cudaMemcpyAsync(b->d_trace_map, b->h_trace_map.data(), sizeof(int4) * b->h_trace_map.size(),
                            cudaMemcpyHostToDevice, s),
            "trace map upload");
-        CU(cudaMemcpyAsync(b->d_units, b->units.data(), sizeof(Unit) * b->units.size(), cudaMemcpyHostToDevice, s),
-           "unit upload");
+        CU(cudaMemcpyAsync(b->d_fold_map, b->fold_map.data(), sizeof(int4) * b->fold_map.size(),
+                           cudaMemcpyHostToDevice, s),
+           "fold map upload");
         CU(cudaMemcpyAsync(b->d_adj_units, b->adj_units.data(), sizeof(AdjUnit) * b->adj_units.size(),
                            cudaMemcpyHostToDevice, s),
            "unit upload");
@@ -1418,8 +1455,8 @@ extern "C" sonar_status sonar_render_batch_step(sonar_batch_t b, const sonar_par
         b->step = nullptr;
         const float* noised = out->noised ? out->noised : b->d_noised;
         const sonar_hit* hits = out->hits ? out->hits : b->d_hits;
-        // one graph, two branches after binning: the adjoint (which reads I~ and
-        // the hit records only) beside the normalisation and the fan
+        // one graph, two branches after the row kernel: the adjoint (which reads I~
+        // and the hit records only) beside the fan (and whole-image normalisation)
         CU(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "graph capture");
         st = batch_forward_launches(b, p, d_theta, n_mat, out, b->cap, true, 1);
         cudaError_t e = cudaSuccess;
@@ -1458,10 +1495,10 @@ extern "C" sonar_status sonar_batch_info(sonar_batch_t b, int64_t out[5]) {
     if (!b || !out) return SONAR_ERR_ARG;
     int64_t rays = 0;
     for (const SensorDev& S : b->hs) rays += (int64_t)S.nb * S.ne;
-    out[0] = (int64_t)b->units.size();
+    out[0] = (int64_t)b->fold_map.size();
     out[1] = rays;
-    out[2] = persistent_grid(b, 1);
-    out[3] = b->block;
+    out[2] = (int64_t)b->fold_map.size();
+    out[3] = b->fold_block;
     out[4] = b->graphs;
     return SONAR_OK;
 }
@@ -1597,7 +1634,7 @@ extern "C" sonar_status sonar_autotune(sonar_batch_t b, const sonar_params* p, c
         // with default binning shapes
         for (int occ : {0, kTraceCap, kTraceWide, kTraceCap | kTraceWide}) {
             for (int tb : {1, 2, 4, 8, 16, 32}) {
-                ctx->tune[k] = Tune{0, tb, 128, occ};
+                ctx->tune[k] = Tune{1, tb, 128, occ};
                 if ((st = batch_plan(b)) != SONAR_OK) goto restore;
                 if (batch_scratch(b, out) != cudaSuccess) { st = fail(ctx, SONAR_ERR_OOM, "batch scratch"); goto restore; }
                 const float ms = time_batch(b, p, d_theta, n_mat, out, nullptr, nullptr, s, 3, 3);
@@ -1605,31 +1642,24 @@ extern "C" sonar_status sonar_autotune(sonar_batch_t b, const sonar_params* p, c
                 if (ms < best_ms) { best_ms = ms; best.tb = tb; best.occ = occ; }
             }
         }
-        // then columns per binning unit and the binning block size (which also
-        // sets the adjoint's block and ray chunks): forward and, when the caller's
-        // outputs hold the hit records and I~, the adjoint of a constant
-        // upstream gradient too
+        // then the adjoint's block size (which also sets its ray chunks), when the
+        // caller's outputs hold the hit records and I~ that its timing needs: the
+        // forward and the adjoint of a constant upstream gradient
         best_ms = 1e30f;
         const int tb = best.tb, occ = best.occ;
         for (int block : {64, 128, 256}) {
-            for (int cols : {1, 2, 4, 8, 16, 32}) {
-                if (cols > k[3] || (size_t)cols * k[2] * 4 * 65 > kMaxDynSmem * 32) continue;
-                ctx->tune[k] = Tune{cols, tb, block, occ};
-                if ((st = batch_plan(b)) != SONAR_OK) goto restore;
-                if (batch_scratch(b, out) != cudaSuccess) { st = fail(ctx, SONAR_ERR_OOM, "batch scratch"); goto restore; }
-                const float* g = nullptr;
-                if (adj_grad) {
-                    if (cudaMalloc(&b->d_partials, sizeof(double) * b->adj_units.size() * (n_mat + 2)) != cudaSuccess) {
-                        st = fail(ctx, SONAR_ERR_OOM, "batch scratch");
-                        goto restore;
-                    }
-                    b->n_mat_cap = n_mat;
-                    g = adj_grad;
-                }
-                const float ms = time_batch(b, p, d_theta, n_mat, out, g, adj_dtheta, s, 3, 3);
-                if (cudaGetLastError() != cudaSuccess) continue;
-                if (ms < best_ms) { best_ms = ms; best = Tune{cols, tb, block, occ}; }
+            if (!adj_grad) break;
+            ctx->tune[k] = Tune{1, tb, block, occ};
+            if ((st = batch_plan(b)) != SONAR_OK) goto restore;
+            if (batch_scratch(b, out) != cudaSuccess) { st = fail(ctx, SONAR_ERR_OOM, "batch scratch"); goto restore; }
+            if (cudaMalloc(&b->d_partials, sizeof(double) * b->adj_units.size() * (n_mat + 2)) != cudaSuccess) {
+                st = fail(ctx, SONAR_ERR_OOM, "batch scratch");
+                goto restore;
             }
+            b->n_mat_cap = n_mat;
+            const float ms = time_batch(b, p, d_theta, n_mat, out, adj_grad, adj_dtheta, s, 3, 3);
+            if (cudaGetLastError() != cudaSuccess) continue;
+            if (ms < best_ms) { best_ms = ms; best = Tune{1, tb, block, occ}; }
         }
         ctx->tune[k] = best;
     }
@@ -1922,6 +1952,12 @@ extern "C" sonar_status sonar_render_noalloc(sonar_ctx_t ctx, int32_t scene_id, 
     const int64_t hit_words = out->hits ? 0 : 4 * (int64_t)sensor->n_beams * sensor->n_elev;
     const int64_t noised_at = hits_at + (hit_words + 63) / 64 * 64;
     const int64_t need = out->noised ? noised_at : noised_at + npol;
+    // the fold's compact lists (2 words a ray, 2 a column and band of 32 rows)
+    // where the array has room for them too; else it writes P into the polar
+    // image, which holds it until the row kernel overwrites it (same images)
+    const int64_t vals_at = (need + 63) / 64 * 64;
+    const int64_t bands_at = vals_at + (2 * (int64_t)sensor->n_beams * sensor->n_elev + 63) / 64 * 64;
+    const int64_t fold_end = bands_at + 2 * (((int64_t)sensor->n_range_bins + 31) / 32) * sensor->n_az_bins;
     if (need > (int64_t)SONAR_NOALLOC_SCRATCH_WORDS)
         return fail(ctx, SONAR_ERR_ARG, "sonar_render_noalloc: frame needs " + std::to_string(need) +
                                             " scratch words, the fixed scratch holds " +
@@ -1939,8 +1975,15 @@ extern "C" sonar_status sonar_render_noalloc(sonar_ctx_t ctx, int32_t scene_id, 
     S.trig = (float4*)((float*)base + 64);
     // single_forward clears the maximum (the array still holds the previous
     // call's values); hit records and the noised image are fully overwritten
-    st = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, noised, out->binned,
-                        rowmax, t.block, s);
+    FoldStore fold;
+    if (fold_end <= (int64_t)SONAR_NOALLOC_SCRATCH_WORDS) {
+        fold.vals = (float2*)((float*)base + vals_at);
+        fold.bands = (uint2*)((float*)base + bands_at);
+    } else {
+        fold.dense = out->polar;
+    }
+    st = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, fold, noised,
+                        out->binned, out->polar, rowmax, s);
     if (st != SONAR_OK) return st;
     return single_post(ctx, S, params->normalise, noised, rowmax, out->polar, out->fan, s);
 }

@@ -32,16 +32,16 @@ inline SceneDev scene_dev(const SceneStore& s) {
     return SceneDev{s.nodes, s.tris, s.mat_orig, s.root, (int32_t)s.n_tris, s.nodes8};
 }
 
-// Kernel launchers (trace.cu: ray cast and counters; render.cu: binning, noise,
+// Kernel launchers (trace.cu: ray cast and counters; render.cu: fold, noise,
 // normalisation, fan and adjoint; image.cu: Eq. 1 camera; dvl.cu: DVL;
 // probe.cu: L2 read-bandwidth probe).
 void set_kernel_attributes();
 cudaError_t launch_trig(const SensorDev* sensors, const SensorDev& one, int n_sensors, int max_angles,
                         cudaStream_t st);
 cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStream_t st);
-cudaError_t launch_bin(const BinArgs& a, int det, int grid, int block, size_t smem, cudaStream_t st);
-int bin_blocks_per_sm(int det, int block, size_t smem);
-constexpr size_t kMaxDynSmem = 200 * 1024;
+cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st);
+cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st);
+constexpr size_t kMaxDynSmem = 220 * 1024;   // of the 227 KB a block may have, less the static part
 cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, void* out, cudaStream_t st);
 cudaError_t launch_norm(const NormArgs& a, cudaStream_t st);
 cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st);

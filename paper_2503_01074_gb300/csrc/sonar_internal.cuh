@@ -27,7 +27,7 @@ constexpr int kLeafMax = 2;          // triangles per collapsed leaf (a heightfi
 constexpr int kStackMax = 96;        // traversal stack entries (tree height is checked at build)
 constexpr int32_t kEmpty = (int32_t)0x80000000;
 constexpr int kMaxMat = 1024;
-constexpr int kMaxCols = 64;         // azimuth columns per binning unit, at most
+constexpr int kRowsStaged = 8192;    // widest row whose column tables the row kernel keeps in shared memory
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;
 
 __host__ __device__ inline int32_t leaf_handle(int32_t first, int32_t count) {
@@ -60,13 +60,12 @@ struct SensorDev {
     int32_t fan_w, fan_h;
     uint32_t seed_lo, seed_hi, frame_lo, frame_hi;
     int32_t scene;       // index into the scene table
-    int32_t cols;        // binning: azimuth columns per work unit
-    int32_t n_tiles;     // binning work units of this sensor = ceil(naz / cols)
     int32_t tb;          // trace: beams per warp tile (elevations = 32 / tb)
     int32_t occ;         // trace: variant bits kTraceCap, kTraceWide
     int32_t trace_blocks;  // trace: one-warp blocks covering the sensor
-    int32_t fold_beams;  // binning: deterministic fold into per-beam rows (fits in shared memory)
+    int32_t fold_beams;  // fold: per-beam rows (several beams per column, and they fit in shared memory)
     int64_t polar_off, hits_off, fan_off, rowmax_off;
+    int64_t val_off, band_off;   // fold: first value slot (a slot per ray) and first bitmap word pair
     float4* trig;        // float-float sin/cos of the beam azimuths [nb] and elevations [ne]
     uint4* fan_lut;      // per-pixel fan coordinates shared with same-geometry sensors (nullptr: compute)
     uint32_t* trig_stamp;  // batch: per k_trig block, the trig_version its table entries were built for
@@ -76,18 +75,15 @@ struct SensorDev {
     uint32_t pad_;
 };
 
-// A work unit: the azimuth columns [c0, c1) of one sensor, i.e. every ray
-// of the beams that fall into those columns.
-struct Unit {
-    int32_t sensor;
-    int32_t c0, c1;
-    int32_t rays;     // host: orders the work list
-    int32_t scene;    // the sensor's scene (its descriptor is fetched beside the sensor's)
-};
-
 // First beam whose azimuth bin floor((2i+1) naz / (2 nb)) is >= c.
 __host__ __device__ inline int32_t first_beam_of_col(int64_t c, int64_t nb, int64_t naz) {
     // (2i + 1) naz >= 2 nb c  <=>  i >= (2 nb c - naz) / (2 naz)
+    if (nb * naz < (1ll << 29) && c <= naz) {   // 32-bit division (the 64-bit one costs ~4x)
+        const uint32_t p = 2u * (uint32_t)nb * (uint32_t)c, q = (uint32_t)naz;
+        if (p <= q) return 0;
+        const uint32_t i = (p - q + 2u * q - 1u) / (2u * q);
+        return (int32_t)(i < (uint32_t)nb ? i : (uint32_t)nb);
+    }
     const int64_t num = 2 * nb * c - naz;
     if (num <= 0) return 0;
     const int64_t den = 2 * naz;
@@ -139,38 +135,52 @@ __device__ __forceinline__ U4 philox10(U4 c, const PhiloxKey& K) {
 }
 __device__ __forceinline__ U4 philox10(U4 c, uint32_t k0, uint32_t k1) { return philox10(c, philox_key(k0, k1)); }
 
+// Fast division and reciprocal square root of arguments that are never
+// subnormal: the flush-to-zero forms, which skip the rescaling of subnormals
+// (three to four instructions) and agree with the others everywhere else.
+__device__ __forceinline__ float div_normal(float a, float b) {
+    float r;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
 // -2 ln u for u = (x + 1) / 2^32, without branches.  With u = 2^e f and f in
 // [sqrt(1/2), sqrt(2)), ln u = e ln 2 + 2 atanh(z), z = (f - 1) / (f + 1),
 // |z| <= 3 - 2 sqrt(2) < 0.1716, and 2 atanh(z) = 2 z (1 + z^2/3 + ... +
 // z^10/11) to well below FP32 rounding (the next term is < 2^-33 relative).
 // For u >= sqrt(1/2) (e = 0), f - 1 = -(2^32 - 1 - x) / 2^32 is taken from the
-// integer complement, so u close to 1 keeps its relative accuracy.
+// integer complement, so u close to 1 keeps its relative accuracy; only one of
+// x and its complement is converted (conversions run at a quarter of the rate).
+// Adding 1 - sqrt(1/2) to u's bits carries into the exponent exactly where the
+// mantissa is above sqrt(2), so the split into e and f takes no comparison.
 __device__ __forceinline__ float neg2log_u(uint32_t x) {
     const bool upper = x >= 0xB504F333u;   // (x + 1) / 2^32 >= sqrt(1/2)
-    const float u = fmaf((float)x, 0x1p-32f, 0x1p-32f);
-    const uint32_t bits = __float_as_uint(u);
-    float f = __uint_as_float((bits & 0x007FFFFFu) | 0x3F800000u);   // mantissa in [1, 2)
-    int e = (int)(bits >> 23) - 127;
-    const bool fold = f > 1.41421356f;
-    f = fold ? 0.5f * f : f;
-    e = fold ? e + 1 : e;
-    float d = f - 1.0f;                                                // exact
-    d = upper ? -(float)(0xFFFFFFFFu - x) * 0x1p-32f : d;
-    e = upper ? 0 : e;
-    const float z = __fdividef(d, 2.0f + d);
+    const float c = (float)(upper ? ~x : x);
+    const float u = fmaf(c, 0x1p-32f, 0x1p-32f);
+    constexpr uint32_t kRoot = 0x3F3504F4u;   // the least f
+    const uint32_t bits = __float_as_uint(u) + (0x3F800000u - kRoot);
+    const float f = __uint_as_float((bits & 0x007FFFFFu) + kRoot);
+    const float d = upper ? c * -0x1p-32f : f - 1.0f;   // exact
+    // e in [-32, 0]: exact as a float without a conversion instruction
+    const float e = __uint_as_float(0x4B000000u | (bits >> 23)) - 8388735.0f;
+    const float ef = upper ? 0.0f : e;
+    const float z = div_normal(d, 2.0f + d);
     const float z2 = z * z;
     float p = fmaf(z2, 1.0f / 11.0f, 1.0f / 9.0f);
     p = fmaf(z2, p, 1.0f / 7.0f);
     p = fmaf(z2, p, 1.0f / 5.0f);
     p = fmaf(z2, p, 1.0f / 3.0f);
     p = fmaf(z2, p, 1.0f);
-    // e in [-32, 0]: exact as a float without a conversion instruction
-    const float ef = __uint_as_float(0x4B000000u | (uint32_t)(e + 64)) - 8388672.0f;
     return -2.0f * fmaf(ef, 0.693147180559945f, 2.0f * z * p);
 }
 
-// sqrt(v) for v >= 0 from the reciprocal square root (a few ulp).
-__device__ __forceinline__ float sqrt_nonneg(float v) { return v > 0.0f ? v * rsqrtf(v) : 0.0f; }
+// sqrt(v) for v = 0 or v >= 2^-32 (neg2log_u's values) from the reciprocal square root (a few ulp).
+__device__ __forceinline__ float sqrt_nonneg(float v) { return v > 0.0f ? v * rsqrt_normal(v) : 0.0f; }
 
 // The two noise streams of a frame (Eq. 4 and 5), key = seed.  Additive term:
 // Rayleigh(sigma_sa) by inversion of word (bin mod 4) of counter (bin / 4,
@@ -207,6 +217,14 @@ __device__ __forceinline__ void copy_words(T* dst, const T* src, int lane) {
         reinterpret_cast<uint32_t*>(dst)[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
 }
 
+// The same from a kernel's parameter block (one launch parameter per sensor call).
+template <class T>
+__device__ __forceinline__ void copy_param(T* dst, const T* src, int lane) {
+    static_assert(sizeof(T) % 4 == 0, "descriptor of whole words");
+    for (int i = lane; i < (int)(sizeof(T) / 4); i += 32)
+        reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+}
+
 // ---- kernel argument blocks ----
 
 struct TraceCounters {
@@ -229,29 +247,47 @@ struct TraceArgs {
     sonar_hit* hits;            // written unless counting (the caller's buffer or scratch)
     uint32_t* err;
     TraceCounters tc;           // counting launches only
-    int32_t* zero_word;         // cleared for the launch after this one (a work counter), or nullptr
+    int32_t* zero_word;         // cleared for a later launch (the adjoint's work counter), or nullptr
 };
 
-// Binning and noise over column-tile work units.
-struct BinArgs {
+// The fold of the hit records into bins: one warp or block per azimuth column.
+// Its result, per sensor: bands[w * naz + c] = (bitmap of rows 32 w .. 32 w + 31
+// of column c with returns, index of the first one's value), values (P, speckle
+// factor) in row order from the column's first ray slot on.
+struct FoldArgs {
     const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
-    const Unit* units;          // batch: device work list; single: nullptr
     const SceneDev* scenes;     // batch: device table; single: nullptr (use `one_scene`)
-    int32_t* work_counter;      // persistent work list counter (nullptr: unit = blockIdx.x)
-    int32_t n_units;
+    const int4* block_map;      // batch: per block (sensor, first column, its scene, 0)
     int32_t n_mat;
+    int32_t words_per_warp;     // shared memory of a warp's column
     SensorDev one;
     SceneDev one_scene;
     const float* theta;         // (alpha, gain, mu[...])
-    sonar_params params;
+    float sigma_sm;
     const sonar_hit* hits;      // the trace kernel's records
-    float* noised;
-    float* binned;
-    uint32_t* rowmax;           // normalise = 2: ordered-encoded image maximum per sensor
+    float2* vals;
+    uint2* bands;
+    float* dense;               // instead of vals and bands: P of the bins with returns, in an image of zeros
     uint32_t* err;
 };
 
-// Normalisation: one warp per (sensor, range row).
+// Noise and range-wise normalisation: one warp per (sensor, range row).
+struct RowsArgs {
+    const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
+    const int2* block_map;      // batch: per block (sensor, first row)
+    int32_t rows_per_block;     // 8, 16 or 32 (a block's rows lie in one band of 32)
+    SensorDev one;
+    sonar_params params;
+    const float2* vals;
+    const uint2* bands;
+    const float* dense;         // instead of vals and bands (may be `polar` itself)
+    float* noised;
+    float* binned;
+    float* polar;               // normalise = 0 and 1
+    uint32_t* gmax;             // normalise = 2: ordered-encoded image maximum per sensor
+};
+
+// Whole-image normalisation: one warp per pair of range rows.
 struct NormArgs {
     const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
     const int32_t* row_map;     // batch: sensor of each row
