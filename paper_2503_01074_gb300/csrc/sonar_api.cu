@@ -154,14 +154,26 @@ int wide_for_launch(const sonar_ctx* ctx, int64_t blocks) {
     return blocks <= 32ll * ctx->sm_count ? kTraceWide : 0;
 }
 
-// The ray-cast variant of one sensor's own launch (tile tb from its tuning
-// row, variant `occ` of that row): the tree by the launch size, and no
+// The variant of a launch of `blocks` one-warp blocks that no tuning row names:
+// the tree by the launch size, and the 64-register cap (32 resident warps per
+// SM instead of 20, for a few spills) once the launch is at least two waves.
+// Uncapped / capped: 8,192 blocks (1.7 waves) 86.9 / 88.3 us, 65,536 blocks 528 /
+// 432 us, 227,072 blocks of three sensor types 1572 / 1277 us, 262,144 blocks
+// over 33.6 million triangles 2420 / 1994 us.
+int default_variant(const sonar_ctx* ctx, int64_t blocks) {
+    if (const int wide = wide_for_launch(ctx, blocks)) return wide;
+    return blocks >= 64ll * ctx->sm_count ? kTraceCap : 0;
+}
+
+// The ray-cast variant of one sensor's own launch (tile tb, variant `occ` of its
+// tuning row, if it has one): the tree by the launch size, and no
 // register cap for a launch of at most one wave, which cannot use the
 // occupancy that the cap buys.
 int single_variant(const sonar_ctx* ctx, const sonar_sensor& s, int tb, int occ) {
     const int64_t be = 32 / tb;
     const int64_t blocks = ((s.n_beams + tb - 1) / tb) * ((s.n_elev + be - 1) / be);
-    if (wide_for_launch(ctx, blocks)) return kTraceWide;
+    const bool tuned = ctx->tune.count(ShapeKey{s.n_beams, s.n_elev, s.n_range_bins, s.n_az_bins}) != 0;
+    if (!tuned || wide_for_launch(ctx, blocks)) return default_variant(ctx, blocks);
     return occ & ~kTraceWide;
 }
 
@@ -797,8 +809,8 @@ sonar_status batch_plan(sonar_batch* b) {
     for (auto& kv : block_votes)
         if (kv.second > best) { best = kv.second; b->block = kv.first; }
     // the trace launch takes the variant of the sensor shape with most rays; an
-    // untuned shape walks the tree the launch size calls for, and the 8-wide tree
-    // only when every scene of the batch has one
+    // untuned shape the one the launch size calls for; the 8-wide tree only when
+    // every scene of the batch has one
     int64_t most = -1;
     int kmost = 0;
     for (int k = 0; k < n; ++k) {
@@ -808,7 +820,7 @@ sonar_status batch_plan(sonar_batch* b) {
     if (n > 0) {
         const sonar_sensor& ms = b->items[kmost].sensor;
         if (!ctx->tune.count(ShapeKey{ms.n_beams, ms.n_elev, ms.n_range_bins, ms.n_az_bins}))
-            b->trace_occ = (b->trace_occ & ~kTraceWide) | wide_for_launch(ctx, b->trace_prefix[n]);
+            b->trace_occ = default_variant(ctx, b->trace_prefix[n]);
         for (const sonar_batch_item& it : b->items)
             if (!ctx->scenes[it.scene_id].nodes8) b->trace_occ &= ~kTraceWide;
     }
