@@ -534,40 +534,43 @@ __global__ void k_collapse_enqueue(const int32_t* picks, const uint32_t* prefix,
     }
 }
 
-// Writes the W-wide nodes of one level: entry e is node base + e, W / 4
-// halves in the 4-wide layout; its r-th internal child is node base_next +
-// prefix[e] + r.  Empty slots hold an inverted box that no ray enters and the
-// empty handle.
+// Writes the W-wide nodes of one level: entry e is node base + e; its r-th
+// internal child is node base_next + prefix[e] + r.  Empty slots hold a box at
+// +inf that no ray enters and the empty handle.  The 4-wide layout keeps the
+// planes axis by axis, the 8-wide one child by child (sonar_internal.cuh).
 template <int W>
 __global__ void k_collapse_write(const int32_t* picks, const uint32_t* prefix, int64_t nq, int64_t base,
                                  int64_t base_next, const float4* pairs, float4* nodes) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nq) return;
     uint32_t r = prefix[e];
-    for (int half = 0; half < W / 4; ++half) {
-        float lo[3][4], hi[3][4];
-        int32_t hh[4];
-        for (int k = 0; k < 4; ++k) {
-            const int32_t x = picks[W * e + 4 * half + k];
-            if (x < 0) {
-                for (int a = 0; a < 3; ++a) lo[a][k] = hi[a][k] = __int_as_float(0x7F800000);
-                hh[k] = kEmpty;
-                continue;
-            }
-            const float4 l = pairs[2 * (int64_t)x], h = pairs[2 * (int64_t)x + 1];
-            lo[0][k] = l.x; lo[1][k] = l.y; lo[2][k] = l.z;
-            hi[0][k] = h.x; hi[1][k] = h.y; hi[2][k] = h.z;
-            const int32_t c = __float_as_int(l.w);
-            hh[k] = c >= 0 ? (int32_t)(base_next + r++) : c;
-        }
-        float4* o = nodes + 2 * W * (base + e) + 8 * half;
-        for (int a = 0; a < 3; ++a) {   // per axis: (lo, hi) of children 0, 1 | 2, 3
-            o[2 * a] = make_float4(lo[a][0], hi[a][0], lo[a][1], hi[a][1]);
-            o[2 * a + 1] = make_float4(lo[a][2], hi[a][2], lo[a][3], hi[a][3]);
-        }
-        o[6] = make_float4(__int_as_float(hh[0]), __int_as_float(hh[1]), __int_as_float(hh[2]),
-                           __int_as_float(hh[3]));
+    const float inf = __int_as_float(0x7F800000);
+    float4 l[W], h[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        const int32_t x = picks[W * e + k];
+        l[k] = h[k] = make_float4(inf, inf, inf, __int_as_float(kEmpty));
+        if (x < 0) continue;
+        l[k] = pairs[2 * (int64_t)x];
+        h[k] = pairs[2 * (int64_t)x + 1];
+        if (__float_as_int(l[k].w) >= 0) l[k].w = __int_as_float((int32_t)(base_next + r++));
+    }
+    float4* o = nodes + 2 * W * (base + e);
+    if constexpr (W == 4) {
+        o[0] = make_float4(l[0].x, h[0].x, l[1].x, h[1].x);
+        o[1] = make_float4(l[2].x, h[2].x, l[3].x, h[3].x);
+        o[2] = make_float4(l[0].y, h[0].y, l[1].y, h[1].y);
+        o[3] = make_float4(l[2].y, h[2].y, l[3].y, h[3].y);
+        o[4] = make_float4(l[0].z, h[0].z, l[1].z, h[1].z);
+        o[5] = make_float4(l[2].z, h[2].z, l[3].z, h[3].z);
+        o[6] = make_float4(l[0].w, l[1].w, l[2].w, l[3].w);
         o[7] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    } else {
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            o[2 * k] = make_float4(l[k].x, h[k].x, l[k].y, h[k].y);
+            o[2 * k + 1] = make_float4(l[k].z, h[k].z, l[k].w, 0.0f);
+        }
     }
 }
 

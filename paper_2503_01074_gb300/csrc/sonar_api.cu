@@ -154,13 +154,22 @@ int wide_for_launch(const sonar_ctx* ctx, int64_t blocks) {
     return blocks <= 32ll * ctx->sm_count ? kTraceWide : 0;
 }
 
-// The variant of a launch of `blocks` one-warp blocks that no tuning row names:
-// the tree by the launch size, and the 64-register cap (32 resident warps per
+// Several lanes per ray (0: one) for a launch of `blocks` 32-ray tiles, while it is a
+// small part of a wave: the crossings, measured with k_trace_group, lie near 20,000
+// rays (eight lanes against four) and 100,000 rays (four against one).
+int group_lanes(const sonar_ctx* ctx, int64_t blocks) {
+    if (blocks <= 4ll * ctx->sm_count) return kTraceGroup8;
+    return blocks <= 20ll * ctx->sm_count ? kTraceGroup4 : 0;
+}
+
+// The variant of a launch of `blocks` 32-ray tiles that no tuning row names: several
+// lanes per ray for small launches, else the tree by the launch size, and the 64-register cap (32 resident warps per
 // SM instead of 20, for a few spills) once the launch is at least two waves.
 // Uncapped / capped: 8,192 blocks (1.7 waves) 86.9 / 88.3 us, 65,536 blocks 528 /
 // 432 us, 227,072 blocks of three sensor types 1572 / 1277 us, 262,144 blocks
 // over 33.6 million triangles 2420 / 1994 us.
 int default_variant(const sonar_ctx* ctx, int64_t blocks) {
+    if (const int lanes = group_lanes(ctx, blocks)) return kTraceWide | lanes;
     if (const int wide = wide_for_launch(ctx, blocks)) return wide;
     return blocks >= 64ll * ctx->sm_count ? kTraceCap : 0;
 }
@@ -421,6 +430,7 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     t.one_scene = sc;
     t.params = *p;
     t.hits = hits;
+    t.from_last = S.rot[8] > 0.0f;
     t.err = ctx->d_err;
     CU(launch_trace(t, S.trace_blocks, S.occ, s), "trace launch");
     if (f.dense) CU(cudaMemsetAsync(f.dense, 0, sizeof(float) * (size_t)S.nr * S.naz, s), "cudaMemsetAsync");
@@ -580,6 +590,7 @@ extern "C" sonar_status sonar_render_backward(sonar_ctx_t ctx, int32_t scene_id,
         tr.one_scene = scene_dev(ctx->scenes[scene_id]);
         tr.params = *params;
         tr.hits = (sonar_hit*)ctx->hits.p;
+        tr.from_last = S.rot[8] > 0.0f;
         tr.err = ctx->d_err;
         CU(launch_trace(tr, S.trace_blocks, S.occ, s), "trace launch");
         hits = (const sonar_hit*)ctx->hits.p;
@@ -809,7 +820,8 @@ sonar_status batch_plan(sonar_batch* b) {
     for (auto& kv : block_votes)
         if (kv.second > best) { best = kv.second; b->block = kv.first; }
     // the trace launch takes the variant of the sensor shape with most rays; an
-    // untuned shape the one the launch size calls for; the 8-wide tree only when
+    // untuned shape, and a launch small enough for several lanes per ray, the one
+    // the launch size calls for; the 8-wide tree only when
     // every scene of the batch has one
     int64_t most = -1;
     int kmost = 0;
@@ -819,7 +831,8 @@ sonar_status batch_plan(sonar_batch* b) {
     }
     if (n > 0) {
         const sonar_sensor& ms = b->items[kmost].sensor;
-        if (!ctx->tune.count(ShapeKey{ms.n_beams, ms.n_elev, ms.n_range_bins, ms.n_az_bins}))
+        if (!ctx->tune.count(ShapeKey{ms.n_beams, ms.n_elev, ms.n_range_bins, ms.n_az_bins}) ||
+            group_lanes(ctx, b->trace_prefix[n]))
             b->trace_occ = default_variant(ctx, b->trace_prefix[n]);
         for (const sonar_batch_item& it : b->items)
             if (!ctx->scenes[it.scene_id].nodes8) b->trace_occ &= ~kTraceWide;

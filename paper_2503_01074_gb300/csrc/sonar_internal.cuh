@@ -6,9 +6,12 @@
 //               0, 1, [1] of children 2, 3, [2], [3] the same for y, [4], [5] for
 //               z, [6] the 4 child handles, [7] unused.  Empty slots: boxes at +inf
 //               (never entered), kEmpty.
-//   nodes8      8-wide, float4[16] = 256 B per node: two halves in the 4-wide
-//               layout, children 0..3 and 4..7.  Built from the same binary
-//               hierarchy; a handle >= 0 here indexes nodes8.
+//   nodes8      8-wide, float4[16] = 256 B per node: child c is 32 bytes at 32 c,
+//               (lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, handle, 0), one 256-bit load (a
+//               lane of the several-lanes-per-ray walk takes whole children; the
+//               4-wide walk of a ray per thread is 4 % faster axis by axis).
+//               Built from the same binary hierarchy; a handle >= 0 here indexes
+//               nodes8.
 //   handles     int32: >= 0 a node index; < 0 a leaf ~((first << 3) | (count - 1)),
 //               a run of 1..8 triangles in leaf order; kEmpty an empty slot.
 //   triangles   float4[3] per triangle in leaf order (48 B):
@@ -45,9 +48,12 @@ struct SceneDev {
 };
 
 // SensorDev::occ, the ray-cast variant: bit kTraceCap caps registers at 64 so
-// that 32 one-warp blocks fit an SM; bit kTraceWide walks the 8-wide tree.
+// that 32 one-warp blocks fit an SM; bit kTraceWide walks the 8-wide tree, with
+// kTraceGroup8 or kTraceGroup4 by eight or four lanes per ray (chosen by the
+// launch size, never by a tuning row).
 constexpr int kTraceCap = 8;
 constexpr int kTraceWide = 16;
+constexpr int kTraceGroup8 = 32, kTraceGroup4 = 64;
 
 // One sensor of a render, with everything the kernels derive from it.
 struct SensorDev {
@@ -247,6 +253,7 @@ struct TraceArgs {
     sonar_hit* hits;            // written unless counting (the caller's buffer or scratch)
     uint32_t* err;
     TraceCounters tc;           // counting launches only
+    int32_t from_last;          // single: tiles from the last to the first
     int32_t* zero_word;         // cleared for a later launch (the adjoint's work counter), or nullptr
 };
 

@@ -59,15 +59,6 @@ __device__ __forceinline__ void ray_dir_ff(const SensorDev& s, int i, int j, ff 
 }
 
 
-// Two consecutive float4 of a node (32 bytes, 32-byte aligned: nodes are
-// 128-byte lines) in one 256-bit read-only load, so that a node visit takes
-// four load instructions instead of seven.
-__device__ __forceinline__ void ld_node_pair(const float4* p, float4& a, float4& b) {
-    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
-}
-
 // ---------------------------------------------------------------------------
 // closest hit: LBVH walk with a short stack
 // ---------------------------------------------------------------------------
@@ -149,6 +140,27 @@ __device__ __forceinline__ int az_bin(const SensorDev& s, int i) {
 // trace: one ray per thread, hit record out
 // ---------------------------------------------------------------------------
 
+// The hit record of ray (ri, rj) of direction d: `best` the triangle hit (leaf
+// order, -1: none) at distance best_t.
+__device__ __forceinline__ uint4 record_of(const SensorDev& S, const SceneDev& sc, const sonar_params& p, float3 d,
+                                           int ri, int best, float best_t) {
+    uint32_t key = kNoKey, orig = 0xFFFFFFFFu, cosb = 0u;
+    float tr = CUDART_INF_F;
+    if (best >= 0) {
+        const float4* tp = sc.tris + 3 * (int64_t)best;
+        const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
+        const float3 v0 = f3(va.x, va.y, va.z);
+        const float3 n = cross3(sub(f3(vb.x, vb.y, vb.z), v0), sub(f3(vc.x, vc.y, vc.z), v0));
+        const float dn = dot3(d, n) / sqrtf(dot3(n, n));
+        orig = __float_as_uint(vb.w);
+        tr = best_t;
+        cosb = __float_as_uint(p.two_sided ? fabsf(dn) : fmaxf(-dn, 0.0f));
+        const int br = range_bin(S, best_t);
+        if (br >= 0) key = (uint32_t)(br * S.naz + az_bin(S, ri));
+    }
+    return make_uint4(key, orig, __float_as_uint(tr), cosb);
+}
+
 // A float twice, as the packed pair operand of fma.rn.f32x2.
 __device__ __forceinline__ unsigned long long pk2(float v) {
     unsigned long long r;
@@ -214,7 +226,7 @@ __device__ __forceinline__ int32_t child_at(const int32_t (&hs)[W], uint32_t k) 
 // With STATS the kernel also counts node visits and triangle tests and marks
 // the nodes and triangles it touches (records are then not written).
 template <int MINB, bool STATS, int W>
-__global__ void __launch_bounds__(32, MINB) k_trace(TraceArgs a) {
+__global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ TraceArgs a) {
     __shared__ SensorDev S;
     __shared__ SceneDev SC;
     if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by the next launch only
@@ -230,11 +242,9 @@ __global__ void __launch_bounds__(32, MINB) k_trace(TraceArgs a) {
         for (int i = threadIdx.x; i < kCW; i += 32) reinterpret_cast<uint32_t*>(&SC)[i] = __ldg(c_src + i);
         tile = m.y;
     } else {
-        if (threadIdx.x == 0) {
-            S = a.one;
-            SC = a.one_scene;
-        }
-        tile = blockIdx.x;
+        copy_param(&S, &a.one, threadIdx.x);
+        copy_param(&SC, &a.one_scene, threadIdx.x);
+        tile = a.from_last ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     }
     __syncthreads();
     const int tb = S.tb, te = 32 / S.tb;
@@ -283,39 +293,48 @@ __global__ void __launch_bounds__(32, MINB) k_trace(TraceArgs a) {
                 // missed child sorts last as 0xFFFFFFFF
                 uint32_t key[W];
                 int32_t hs[W];
+                // per axis, the (lo, hi) planes of every child
+                float xs[W][2], ys[W][2], zs[W][2];
+                if constexpr (W == 4) {
+                    float4 a0, a1, unused;
+                    ld_node_pair(pn, a0, a1);
+                    xs[0][0] = a0.x; xs[0][1] = a0.y; xs[1][0] = a0.z; xs[1][1] = a0.w;
+                    xs[2][0] = a1.x; xs[2][1] = a1.y; xs[3][0] = a1.z; xs[3][1] = a1.w;
+                    ld_node_pair(pn + 2, a0, a1);
+                    ys[0][0] = a0.x; ys[0][1] = a0.y; ys[1][0] = a0.z; ys[1][1] = a0.w;
+                    ys[2][0] = a1.x; ys[2][1] = a1.y; ys[3][0] = a1.z; ys[3][1] = a1.w;
+                    ld_node_pair(pn + 4, a0, a1);
+                    zs[0][0] = a0.x; zs[0][1] = a0.y; zs[1][0] = a0.z; zs[1][1] = a0.w;
+                    zs[2][0] = a1.x; zs[2][1] = a1.y; zs[3][0] = a1.z; zs[3][1] = a1.w;
+                    ld_node_pair(pn + 6, a0, unused);
+                    hs[0] = __float_as_int(a0.x); hs[1] = __float_as_int(a0.y);
+                    hs[2] = __float_as_int(a0.z); hs[3] = __float_as_int(a0.w);
+                } else {
 #pragma unroll
-                for (int half = 0; half < W / 4; ++half) {   // a 4-wide node, or the halves of an 8-wide one
-                    float4 lx, hx, ly, hy, lz, hz, chf, unused;
-                    ld_node_pair(pn + 8 * half, lx, hx);
-                    ld_node_pair(pn + 8 * half + 2, ly, hy);
-                    ld_node_pair(pn + 8 * half + 4, lz, hz);
-                    ld_node_pair(pn + 8 * half + 6, chf, unused);
-                    hs[4 * half + 0] = __float_as_int(chf.x);
-                    hs[4 * half + 1] = __float_as_int(chf.y);
-                    hs[4 * half + 2] = __float_as_int(chf.z);
-                    hs[4 * half + 3] = __float_as_int(chf.w);
-                    // per axis, the (lo, hi) planes of children 0, 1 | 2, 3
-                    const float lxs[4] = {lx.x, lx.z, hx.x, hx.z}, hxs[4] = {lx.y, lx.w, hx.y, hx.w};
-                    const float lys[4] = {ly.x, ly.z, hy.x, hy.z}, hys[4] = {ly.y, ly.w, hy.y, hy.w};
-                    const float lzs[4] = {lz.x, lz.z, hz.x, hz.z}, hzs[4] = {lz.y, lz.w, hz.y, hz.w};
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float t0, t1;
-                        fma2(lxs[c], hxs[c], ivx, novx, t0, t1);
-                        float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
-                        fma2(lys[c], hys[c], ivy, novy, t0, t1);
-                        lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
-                        fma2(lzs[c], hzs[c], ivz, novz, t0, t1);
-                        lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
-                        // an empty slot's box lies at +inf on every axis: along an axis
-                        // the ray travels in the + direction its entry distance is +inf,
-                        // and if it travels in the - direction along all three its exit
-                        // distance is -inf; the exit is also at most tcut, which is
-                        // finite, so an empty slot never passes and needs no handle check
-                        const bool hit = lo <= hi * 1.0000005f;
-                        key[4 * half + c] =
-                            hit ? ((__float_as_uint(lo) & ~(uint32_t)(W - 1)) | (uint32_t)(4 * half + c)) : 0xFFFFFFFFu;
+                    for (int c = 0; c < W; ++c) {
+                        const Child ch = ld_child(pn + 2 * c);
+                        xs[c][0] = ch.x0; xs[c][1] = ch.x1;
+                        ys[c][0] = ch.y0; ys[c][1] = ch.y1;
+                        zs[c][0] = ch.z0; zs[c][1] = ch.z1;
+                        hs[c] = ch.handle;
                     }
+                }
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    float t0, t1;
+                    fma2(xs[c][0], xs[c][1], ivx, novx, t0, t1);
+                    float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
+                    fma2(ys[c][0], ys[c][1], ivy, novy, t0, t1);
+                    lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
+                    fma2(zs[c][0], zs[c][1], ivz, novz, t0, t1);
+                    lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
+                    // an empty slot's box lies at +inf on every axis: along an axis
+                    // the ray travels in the + direction its entry distance is +inf,
+                    // and if it travels in the - direction along all three its exit
+                    // distance is -inf; the exit is also at most tcut, which is
+                    // finite, so an empty slot never passes and needs no handle check
+                    const bool hit = lo <= hi * 1.0000005f;
+                    key[c] = hit ? ((__float_as_uint(lo) & ~(uint32_t)(W - 1)) | (uint32_t)c) : 0xFFFFFFFFu;
                 }
                 sort_keys<W>(key);
                 int nhit = 0;
@@ -396,22 +415,8 @@ __global__ void __launch_bounds__(32, MINB) k_trace(TraceArgs a) {
             // the ray is finished: its hit record (bin key, triangle, range, incidence)
             live = false;
             if (!STATS) {
-                uint32_t key = kNoKey, orig = 0xFFFFFFFFu, cosb = 0u;
-                float tr = CUDART_INF_F;
-                if (best >= 0) {
-                    const float4* tp = sc.tris + 3 * (int64_t)best;
-                    const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
-                    const float3 v0 = f3(va.x, va.y, va.z);
-                    const float3 n = cross3(sub(f3(vb.x, vb.y, vb.z), v0), sub(f3(vc.x, vc.y, vc.z), v0));
-                    const float dn = dot3(d, n) / sqrtf(dot3(n, n));
-                    orig = __float_as_uint(vb.w);
-                    tr = best_t;
-                    cosb = __float_as_uint(p.two_sided ? fabsf(dn) : fmaxf(-dn, 0.0f));
-                    const int br = range_bin(S, best_t);
-                    if (br >= 0) key = (uint32_t)(br * S.naz + az_bin(S, ri));
-                }
                 *reinterpret_cast<uint4*>(a.hits + S.hits_off + (int64_t)ri * S.ne + rj) =
-                    make_uint4(key, orig, __float_as_uint(tr), cosb);
+                    record_of(S, sc, p, d, ri, best, best_t);
             }
         }
         if (__ballot_sync(0xFFFFFFFFu, live) == 0u) break;
@@ -422,6 +427,257 @@ __global__ void __launch_bounds__(32, MINB) k_trace(TraceArgs a) {
         atomicAdd(a.tc.exact, (unsigned long long)exact_n);
     }
 }
+// Several lanes (G = 8 or 4) per ray, for launches that cannot fill the GPU.
+// Such a launch lasts as long as its longest chain of dependent node visits (a
+// frame of 32,768 rays is a fifth of a wave of k_trace's warps), and there a
+// visit costs its ~300 instructions in a row and waits for the slowest of 32
+// rays.  Here a lane loads and tests 8 / G children of an 8-wide node; the
+// nearest entered child is next (a minimum over the ray's lanes), the others
+// go to the ray's stack in shared memory with their entry distances, and an
+// entry beyond the ray's cut is dropped when it comes up.  Entered leaves are
+// parked by their lanes until every ray of the warp holds one or has nothing
+// left to visit; then the triangles are spread over the ray's lanes, two lanes
+// a leaf.  Every lane keeps the closest of the triangles it tested itself; the
+// ray's cut is the least of them, and the candidates are compared at the end
+// by the same rule as in k_trace (distance, exact decision for near ties), so
+// the records are the same.
+// Bound by the longest rays' chains of visits up to about 20,000 rays, above that
+// by issue (four lanes a ray: 15 us per 32,768 rays, against 24 us by eight and
+// 6.5 us by one lane in a launch that fills the GPU).  Ray cast of one frame, one
+// lane a ray -> four -> eight lanes: 1,024 rays over a plane and a sphere 29.6 ->
+// 17.9 -> 17.1 us; 8,192 rays over a seabed 40.4 -> 22.2 -> 21.0; 16,403 rays to
+// 27 m 140 -> 55 -> 42; 32,768 rays 42.7 -> 29.1 -> 34.5; 65,536 rays (two frames)
+// 57.2 -> 41.6 -> 53.2; 131,072 rays 61.2 -> 71.1 -> 96.5.
+constexpr int kGroupThreads = 64;       // threads per block
+
+template <int G>
+__global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_constant__ TraceArgs a) {
+    constexpr int kRays = kGroupThreads / G;            // rays per block
+    constexpr int kParts = 32 / kRays;                  // blocks per 32-ray tile
+    constexpr int J = 8 / G;                            // children per lane: c, c + G, ...
+    constexpr uint32_t kLanes = (1u << G) - 1u;
+    __shared__ SensorDev S;
+    __shared__ SceneDev SC;
+    __shared__ int s_tile;
+    __shared__ float2 s_stack[kRays][kStackMax];        // (handle bits, entry distance)
+    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
+    if (threadIdx.x < 32) {
+        const int tile = blockIdx.x / kParts;
+        if (a.sensors) {
+            const int4 m = __ldg(a.block_map + tile);
+            copy_words(&S, a.sensors + m.x, threadIdx.x);
+            copy_words(&SC, a.scenes + m.z, threadIdx.x);
+            if (threadIdx.x == 0) s_tile = m.y;
+        } else {
+            copy_param(&S, &a.one, threadIdx.x);
+            copy_param(&SC, &a.one_scene, threadIdx.x);
+            if (threadIdx.x == 0) s_tile = a.from_last ? a.one.trace_blocks - 1 - tile : tile;
+        }
+    }
+    __syncthreads();
+    const int tb = S.tb, te = 32 / tb, tiles_b = (S.nb + tb - 1) / tb;
+    const int ty = s_tile / tiles_b, tx = s_tile - ty * tiles_b;
+    const int group = threadIdx.x / G, c = threadIdx.x & (G - 1);
+    const int l = (blockIdx.x % kParts) * kRays + group;   // the ray within its tile
+    const int ri = tx * tb + l % tb, rj = ty * te + l / tb;
+    const SceneDev& sc = SC;
+    const float tlimit = a.params.clip_tmax ? S.rmax : 3.0e38f;
+    const float3 o = f3(S.pos[0], S.pos[1], S.pos[2]);
+    const bool inside = ri < S.nb && rj < S.ne;
+    const float3 d = inside ? ray_dir32(S, ri, rj) : f3(0.0f, 0.0f, 1.0f);
+    const float tiny = 1e-20f;
+    const float3 inv = f3(1.0f / (fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x)),
+                          1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y)),
+                          1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z)));
+    const float3 oinv = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    const int lane = threadIdx.x & 31, shift = lane & ~(G - 1);
+    const uint32_t mine = kLanes << shift;
+    float2* stack = s_stack[group];
+    int sp = 0, best = -1;
+    uint32_t best_id = 0xFFFFFFFFu;
+    float best_t = tlimit, cut = tlimit;   // this lane's closest; the ray's
+    float node_t = 0.0f;                   // entry distance of `node`
+    int32_t leaf[J], late[J];              // leaves parked by this lane (0: none); `late` came while it held one
+#pragma unroll
+    for (int j = 0; j < J; ++j) leaf[j] = late[j] = 0;
+    int32_t node = inside ? sc.root : kEmpty;
+    if (node < 0 && node != kEmpty) {      // a scene of one leaf
+        if (c == 0) leaf[0] = node;
+        node = kEmpty;
+    }
+    // the ray's 8-bit mask of the children (slot c + G j) whose lanes say yes
+    auto slots = [&](const bool (&yes)[J]) {
+        uint32_t m = 0u;
+#pragma unroll
+        for (int j = 0; j < J; ++j) m |= ((__ballot_sync(0xFFFFFFFFu, yes[j]) >> shift) & kLanes) << (G * j);
+        return m;
+    };
+    for (;;) {
+        int32_t h[J];
+        float lo[J];
+        bool inner[J];
+        uint32_t kmin = 0xFFFFFFFFu;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            h[j] = kEmpty;
+            lo[j] = 0.0f;
+            inner[j] = false;
+        }
+        if (node >= 0) {
+            Child ch[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) ch[j] = ld_child(sc.nodes8 + 16 * (int64_t)node + 2 * (c + G * j));
+            const float tcut = cut * 1.00002f;
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const float x0 = fmaf(ch[j].x0, inv.x, -oinv.x), x1 = fmaf(ch[j].x1, inv.x, -oinv.x);
+                const float y0 = fmaf(ch[j].y0, inv.y, -oinv.y), y1 = fmaf(ch[j].y1, inv.y, -oinv.y);
+                const float z0 = fmaf(ch[j].z0, inv.z, -oinv.z), z1 = fmaf(ch[j].z1, inv.z, -oinv.z);
+                h[j] = ch[j].handle;
+                lo[j] = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fmaxf(fminf(z0, z1), 0.0f));
+                const float hi = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fminf(fmaxf(z0, z1), tcut));
+                const bool enter = lo[j] <= hi * 1.0000005f;   // never an empty slot (see k_trace)
+                inner[j] = enter && h[j] >= 0;
+                if (enter && h[j] < 0) {
+                    if (leaf[j] == 0) leaf[j] = h[j];
+                    else late[j] = h[j];
+                }
+                if (inner[j]) kmin = min(kmin, (__float_as_uint(lo[j]) & ~7u) | (uint32_t)(c + G * j));
+            }
+        }
+#pragma unroll
+        for (int k = 1; k < G; k <<= 1) kmin = min(kmin, __shfl_xor_sync(0xFFFFFFFFu, kmin, k));
+        const uint32_t near = kmin & 7u;   // the slot of the nearest
+        int32_t next = h[0];
+        float next_t = lo[0];
+        if constexpr (J == 2) {
+            if (near >= G) { next = h[1]; next_t = lo[1]; }
+        }
+        next = __shfl_sync(0xFFFFFFFFu, next, shift + (near & (G - 1)));
+        next_t = __shfl_sync(0xFFFFFFFFu, next_t, shift + (near & (G - 1)));
+        const uint32_t entered = slots(inner);
+        if (entered) {
+            const uint32_t others = entered & ~(1u << near);
+            const int n = __popc(others);
+            if (sp + n > kStackMax) {   // cannot happen for a checked height: give up the ray
+                atomicOr(a.err, SONAR_DEVERR_STACK);
+                node = kEmpty;
+                sp = 0;
+#pragma unroll
+                for (int j = 0; j < J; ++j) leaf[j] = late[j] = 0;
+                best = -1;
+                best_t = cut = tlimit;
+            } else {
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const uint32_t slot = (uint32_t)(c + G * j);
+                    if ((others >> slot) & 1u)
+                        stack[sp + __popc(others & ((1u << slot) - 1u))] = make_float2(__int_as_float(h[j]), lo[j]);
+                }
+                sp += n;
+                node = next;
+                node_t = next_t;
+            }
+            __syncwarp(mine);
+        } else {
+            node = kEmpty;
+        }
+        bool has_leaf[J], has_late = false;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            has_leaf[j] = leaf[j] != 0;
+            has_late = has_late || late[j] != 0;
+        }
+        uint32_t parked = slots(has_leaf);
+        const bool waits = (node == kEmpty && sp == 0) || parked != 0u;
+        const bool all_wait = __all_sync(0xFFFFFFFFu, waits), any_late = __any_sync(0xFFFFFFFFu, has_late);
+        if ((all_wait || any_late) && __any_sync(0xFFFFFFFFu, parked != 0u)) {
+            do {
+                uint32_t m = parked;   // this lane's leaf: set bit number c / 2
+                if ((c >> 1) > 0) m &= m - 1;
+                if (G > 4 && (c >> 1) > 1) m &= m - 1;
+                if (G > 4 && (c >> 1) > 2) m &= m - 1;
+                const int slot = (__ffs(m) - 1) & 7;
+                int32_t x = __shfl_sync(0xFFFFFFFFu, leaf[0], shift + (slot & (G - 1)));
+                if constexpr (J == 2) {
+                    const int32_t x1 = __shfl_sync(0xFFFFFFFFu, leaf[1], shift + (slot & (G - 1)));
+                    if (slot >= G) x = x1;
+                }
+                x = ~x;
+                const int32_t first = x >> 3, count = m ? (x & 7) + 1 : 0;
+                for (int k = c & 1; k < count; k += 2) {
+                    const int32_t f = first + k;
+                    if (f >= sc.n_tris) {
+                        atomicOr(a.err, SONAR_DEVERR_INDEX);
+                        break;
+                    }
+                    const float4* tp = sc.tris + 3 * (int64_t)f;
+                    const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
+                    float t;
+                    const int r = mt32(o, d, va, vb, vc, t);
+                    if (r == 0 || (r == 2 && !exact_hit(S, ri, rj, va, vb, vc, &t)) || !(t < tlimit)) continue;
+                    const uint32_t id = __float_as_uint(vb.w);
+                    bool take;
+                    if (best < 0) take = true;
+                    else if (fabsf(t - best_t) <= 2e-5f * fmaxf(t, best_t))
+                        take = exact_closer(S, ri, rj, tp, id, sc.tris + 3 * (int64_t)best, best_id);
+                    else take = t < best_t;
+                    if (take) {
+                        best = f;
+                        best_id = id;
+                        best_t = t;
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < G / 2; ++k) parked &= parked - 1;
+            } while (__any_sync(0xFFFFFFFFu, parked != 0u));
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                leaf[j] = late[j];
+                late[j] = 0;
+            }
+            cut = best_t;
+#pragma unroll
+            for (int k = 1; k < G; k <<= 1) cut = fminf(cut, __shfl_xor_sync(0xFFFFFFFFu, cut, k));
+        }
+        if (node != kEmpty && !(node_t <= cut * 1.00002f)) node = kEmpty;
+        while (node == kEmpty && sp > 0) {   // an entry beyond the cut would fail its box test now
+            const float2 e = stack[--sp];
+            if (e.y <= cut * 1.00002f) {
+                node = __float_as_int(e.x);
+                node_t = e.y;
+            }
+        }
+        bool more = node != kEmpty;
+#pragma unroll
+        for (int j = 0; j < J; ++j) more = more || leaf[j] != 0;
+        if (!__any_sync(0xFFFFFFFFu, more)) break;
+    }
+    // the ray's closest of its lanes' candidates
+#pragma unroll
+    for (int k = 1; k < G; k <<= 1) {
+        const float t2 = __shfl_xor_sync(0xFFFFFFFFu, best_t, k);
+        const int b2 = __shfl_xor_sync(0xFFFFFFFFu, best, k);
+        const uint32_t id2 = __shfl_xor_sync(0xFFFFFFFFu, best_id, k);
+        if (b2 < 0) continue;
+        bool take;
+        if (best < 0) take = true;
+        else if (b2 == best) take = false;
+        else if (fabsf(t2 - best_t) <= 2e-5f * fmaxf(t2, best_t))
+            take = exact_closer(S, ri, rj, sc.tris + 3 * (int64_t)b2, id2, sc.tris + 3 * (int64_t)best, best_id);
+        else take = t2 < best_t;
+        if (take) {
+            best = b2;
+            best_id = id2;
+            best_t = t2;
+        }
+    }
+    if (inside && c == 0)
+        *reinterpret_cast<uint4*>(a.hits + S.hits_off + (int64_t)ri * S.ne + rj) =
+            record_of(S, sc, a.params, d, ri, best, best_t);
+}
+
 // ---------------------------------------------------------------------------
 // counters
 // ---------------------------------------------------------------------------
@@ -453,7 +709,11 @@ cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStre
         // one sensor's launch on a scene without an 8-wide tree walks the 4-wide
         // one (a batch's variant is checked against all its scenes on the host)
         const bool wide = (occupancy & kTraceWide) && (a.sensors || a.one_scene.nodes8);
-        if (wide) {
+        if (wide && (occupancy & kTraceGroup8)) {
+            k_trace_group<8><<<(unsigned)blocks * (32 * 8 / kGroupThreads), kGroupThreads, 0, st>>>(a);
+        } else if (wide && (occupancy & kTraceGroup4)) {
+            k_trace_group<4><<<(unsigned)blocks * (32 * 4 / kGroupThreads), kGroupThreads, 0, st>>>(a);
+        } else if (wide) {
             if (cap) k_trace<32, false, 8><<<blocks, 32, 0, st>>>(a);
             else k_trace<4, false, 8><<<blocks, 32, 0, st>>>(a);
         } else {
