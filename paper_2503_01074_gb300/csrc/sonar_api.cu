@@ -45,6 +45,7 @@ struct sonar_ctx {
     std::vector<bool> alive;
     std::string last_error;
     uint32_t* d_err = nullptr;
+    cudaMemPool_t pool = nullptr;   // scenes and the scratch of their builds
     Scratch rowmax, noised, rowinfo, partials, counters, hits, trig, vals, bands;
     // the exact-ray tables last built by a single-sensor call: their buffer and
     // the angular geometry they hold (beams, elevations, fields of view)
@@ -284,6 +285,24 @@ extern "C" sonar_status sonar_create(int32_t device, sonar_ctx_t* out) {
         delete ctx;
         return SONAR_ERR_OOM;
     }
+    // scenes come from a pool of the context's own, which keeps up to 1 GiB of
+    // freed memory mapped (the scratch of a two-million-triangle build and its
+    // scene) for the next build, and gives the rest back at the next
+    // synchronisation and everything when the context goes
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = 1ull << 30;
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+        cudaFree(ctx->d_err);
+        delete ctx;
+        return SONAR_ERR_CUDA;
+    }
     set_kernel_attributes();
     cudaGetLastError();
     *out = ctx;
@@ -299,6 +318,7 @@ extern "C" sonar_status sonar_destroy(sonar_ctx_t ctx) {
                        &ctx->trig, &ctx->vals, &ctx->bands})
         if (s->p) cudaFreeAsync(s->p, 0);
     cudaDeviceSynchronize();
+    cudaMemPoolDestroy(ctx->pool);
     cudaFree(ctx->d_err);
     delete ctx;
     return SONAR_OK;
@@ -338,8 +358,10 @@ extern "C" sonar_status sonar_scene_upload(sonar_ctx_t ctx, const float* d_verts
     CU(cudaSetDevice(ctx->device), "cudaSetDevice");
     SceneStore s;
     std::string msg;
-    const sonar_status st = build_scene(d_verts, n_verts, d_tris, d_mat, n_tris, (cudaStream_t)stream, &s, &msg);
+    const sonar_status st = build_scene(d_verts, n_verts, d_tris, d_mat, n_tris, ctx->sm_count, ctx->pool,
+                                        (cudaStream_t)stream, &s, &msg);
     if (st != SONAR_OK) {
+        cudaStreamSynchronize((cudaStream_t)stream);   // what was allocated on it is freed on another
         free_scene(&s);
         return fail(ctx, st, msg);
     }

@@ -25,7 +25,8 @@ struct SceneStore {
 };
 
 sonar_status build_scene(const float* verts, int64_t nv, const int32_t* tris, const int32_t* mat,
-                         int64_t nt, cudaStream_t st, SceneStore* out, std::string* msg);
+                         int64_t nt, int sm_count, cudaMemPool_t pool, cudaStream_t st, SceneStore* out,
+                         std::string* msg);
 void free_scene(SceneStore* s);
 
 inline SceneDev scene_dev(const SceneStore& s) {
