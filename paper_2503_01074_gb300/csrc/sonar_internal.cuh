@@ -314,11 +314,11 @@ __host__ __device__ inline int32_t fan_squares(int32_t w, int32_t h) {
     return ((w + kFanSide - 1) / kFanSide) * ((h + kFanSide - 1) / kFanSide);
 }
 // The fan of a sensor that shares no coordinate table (single frames, sensors
-// of unique geometry) goes in smaller squares: one frame's fan is then several
-// blocks per SM instead of about one.
-constexpr int kTileSide = 32;
+// of unique geometry): blocks of kTileCols columns of its left half and their
+// mirror columns, by kTileRows rows (one frame's fan is several blocks per SM).
+constexpr int kTileCols = 32, kTileRows = 16;
 __host__ __device__ inline int32_t tile_squares(int32_t w, int32_t h) {
-    return ((w + kTileSide - 1) / kTileSide) * ((h + kTileSide - 1) / kTileSide);
+    return (((w + 1) / 2 + kTileCols - 1) / kTileCols) * ((h + kTileRows - 1) / kTileRows);
 }
 
 // DVL measurement of n poses (four beams each).
