@@ -16,27 +16,86 @@ namespace {
 // DVL (Sec. III-A-3): four-beam Janus ranges, least-squares velocity, rate
 // ---------------------------------------------------------------------------
 
-// Closest hit along one ray (any origin and direction) by a per-thread walk
-// of the 4-wide hierarchy: certified FP32 Moller-Trumbore, undecided tests
+// The exact decision of an uncertain FP32 test, on the FP32 direction (out of
+// line: rarely needed).
+__device__ __noinline__ bool exact_distance(float3 o, float3 d, float4 a, float4 b, float4 c, float* t) {
+    const float of[3] = {o.x, o.y, o.z};
+    const ff df[3] = {ff{d.x, 0.0f}, ff{d.y, 0.0f}, ff{d.z, 0.0f}};
+    ff D, T;
+    if (!mt_ff(of, df, a, b, c, D, T)) return false;
+    *t = T.hi / D.hi;
+    return true;
+}
+
+// Closest hit along one ray (any origin and direction) by a walk of the 4-wide
+// hierarchy, a lane per ray: certified FP32 Moller-Trumbore, undecided tests
 // decided exactly in float-float on the FP32 direction; ties go to the lower
-// caller index.  Returns the distance (+inf for a miss).
-__device__ float closest_distance(const SceneDev& sc, float3 o, float3 d, float tmax, uint32_t* err) {
-    if (sc.root == kEmpty) return CUDART_INF_F;
+// caller index.  Lanes park a leaf and descend on until every active lane of the
+// warp holds one, as in the sonar's ray cast.  Returns the distance (+inf for a
+// miss, and for a lane without a ray).
+__device__ __forceinline__ float closest_distance(const SceneDev& sc, bool live, float3 o, float3 d, uint32_t* err) {
     const float tiny = 1e-20f;
     const float3 inv = f3(1.0f / (fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x)),
                           1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y)),
                           1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z)));
-    const float3 oinv = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-    const float of[3] = {o.x, o.y, o.z};
-    const ff dff[3] = {ff{d.x, 0.0f}, ff{d.y, 0.0f}, ff{d.z, 0.0f}};
+    const unsigned long long ivx = pk2(inv.x), ivy = pk2(inv.y), ivz = pk2(inv.z);
+    const unsigned long long novx = pk2(-(o.x * inv.x)), novy = pk2(-(o.y * inv.y)), novz = pk2(-(o.z * inv.z));
     int32_t stack[kStackMax];
     int sp = 0;
-    float best_t = tmax;
+    float best_t = 3.0e38f;   // a finite cut keeps empty slots (boxes at +inf) out, see k_trace
     uint32_t best_id = 0xFFFFFFFFu;
-    int32_t node = sc.root;
-    while (node != kEmpty) {
-        if (node < 0) {
-            const int32_t x = ~node;
+    int32_t node = live ? sc.root : kEmpty, leaf = 0;
+    if (node < 0 && node != kEmpty) { leaf = node; node = kEmpty; }
+    while (node != kEmpty || leaf != 0) {
+        while (node >= 0) {
+            const float4* pn = sc.nodes + 8 * (int64_t)node;
+            const float tcut = best_t * 1.00002f;
+            float4 x0, x1, y0, y1, z0, z1, ch, unused;
+            ld_node_pair(pn, x0, x1);
+            ld_node_pair(pn + 2, y0, y1);
+            ld_node_pair(pn + 4, z0, z1);
+            ld_node_pair(pn + 6, ch, unused);
+            const int32_t hs[4] = {__float_as_int(ch.x), __float_as_int(ch.y), __float_as_int(ch.z), __float_as_int(ch.w)};
+            // per axis, the (lo, hi) planes of children 0, 1 | 2, 3
+            const float xs[4][2] = {{x0.x, x0.y}, {x0.z, x0.w}, {x1.x, x1.y}, {x1.z, x1.w}};
+            const float ys[4][2] = {{y0.x, y0.y}, {y0.z, y0.w}, {y1.x, y1.y}, {y1.z, y1.w}};
+            const float zs[4][2] = {{z0.x, z0.y}, {z0.z, z0.w}, {z1.x, z1.y}, {z1.z, z1.w}};
+            uint32_t key[4];
+            int nhit = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float t0, t1;
+                fma2(xs[c][0], xs[c][1], ivx, novx, t0, t1);
+                float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
+                fma2(ys[c][0], ys[c][1], ivy, novy, t0, t1);
+                lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
+                fma2(zs[c][0], zs[c][1], ivz, novz, t0, t1);
+                lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
+                const bool hit = lo <= hi * 1.0000005f;
+                key[c] = hit ? ((__float_as_uint(lo) & ~3u) | (uint32_t)c) : 0xFFFFFFFFu;
+                nhit += hit;
+            }
+            sort_keys<4>(key);
+            if (nhit == 0) {
+                node = sp > 0 ? stack[--sp] : kEmpty;
+            } else {
+                if (sp + nhit - 1 > kStackMax) {   // cannot happen for a checked depth: give up the ray
+                    atomicOr(err, SONAR_DEVERR_STACK);
+                    return CUDART_INF_F;
+                }
+#pragma unroll
+                for (int c = 3; c >= 1; --c)
+                    if (c < nhit) stack[sp++] = child_at<4>(hs, key[c] & 3u);
+                node = child_at<4>(hs, key[0] & 3u);
+            }
+            if (node < 0 && node != kEmpty && leaf == 0) {   // park the leaf, keep descending
+                leaf = node;
+                node = sp > 0 ? stack[--sp] : kEmpty;
+            }
+            if (!__any_sync(__activemask(), leaf == 0)) break;
+        }
+        while (leaf != 0) {
+            const int32_t x = ~leaf;
             const int32_t first = x >> 3, count = (x & 7) + 1;
             for (int k = 0; k < count; ++k) {
                 const int32_t f = first + k;
@@ -48,67 +107,19 @@ __device__ float closest_distance(const SceneDev& sc, float3 o, float3 d, float 
                 const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
                 float t;
                 const int r = mt32(o, d, va, vb, vc, t);
-                if (r == 0) continue;
-                if (r == 2) {
-                    ff D, T;
-                    if (!mt_ff(of, dff, va, vb, vc, D, T)) continue;
-                    t = T.hi / D.hi;
-                }
+                if (r == 0 || (r == 2 && !exact_distance(o, d, va, vb, vc, &t))) continue;
                 const uint32_t id = __float_as_uint(vb.w);
                 if (t < best_t || (t == best_t && id < best_id)) {
                     best_t = t;
                     best_id = id;
                 }
             }
-            node = sp > 0 ? stack[--sp] : kEmpty;
-            continue;
+            leaf = 0;
+            if (node < 0 && node != kEmpty) {   // the next stacked entry is a leaf too
+                leaf = node;
+                node = sp > 0 ? stack[--sp] : kEmpty;
+            }
         }
-        const float4* pn = sc.nodes + 8 * (int64_t)node;
-        const float4 lx = __ldg(pn), hx = __ldg(pn + 1), ly = __ldg(pn + 2), hy = __ldg(pn + 3);
-        const float4 lz = __ldg(pn + 4), hz = __ldg(pn + 5);
-        const int4 ch = __ldg(reinterpret_cast<const int4*>(pn + 6));
-        const float tcut = best_t * 1.00002f;
-        // per axis, the (lo, hi) planes of children 0, 1 | 2, 3
-        const float lxs[4] = {lx.x, lx.z, hx.x, hx.z}, hxs[4] = {lx.y, lx.w, hx.y, hx.w};
-        const float lys[4] = {ly.x, ly.z, hy.x, hy.z}, hys[4] = {ly.y, ly.w, hy.y, hy.w};
-        const float lzs[4] = {lz.x, lz.z, hz.x, hz.z}, hzs[4] = {lz.y, lz.w, hz.y, hz.w};
-        const int32_t hs[4] = {ch.x, ch.y, ch.z, ch.w};
-        uint32_t key[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float t0 = fmaf(lxs[c], inv.x, -oinv.x), t1 = fmaf(hxs[c], inv.x, -oinv.x);
-            float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
-            t0 = fmaf(lys[c], inv.y, -oinv.y); t1 = fmaf(hys[c], inv.y, -oinv.y);
-            lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
-            t0 = fmaf(lzs[c], inv.z, -oinv.z); t1 = fmaf(hzs[c], inv.z, -oinv.z);
-            lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
-            const bool hit = hs[c] != kEmpty && lo <= hi * 1.0000005f;
-            key[c] = hit ? ((__float_as_uint(lo) & ~3u) | (uint32_t)c) : 0xFFFFFFFFu;
-        }
-#define SONAR_USORT(x, y)                                \
-        {                                                \
-            const uint32_t mn = min(key[x], key[y]);     \
-            key[y] = max(key[x], key[y]);                \
-            key[x] = mn;                                 \
-        }
-        SONAR_USORT(0, 1) SONAR_USORT(2, 3) SONAR_USORT(0, 2) SONAR_USORT(1, 3) SONAR_USORT(1, 2)
-#undef SONAR_USORT
-        const int nhit = (key[0] != 0xFFFFFFFFu) + (key[1] != 0xFFFFFFFFu) + (key[2] != 0xFFFFFFFFu) +
-                         (key[3] != 0xFFFFFFFFu);
-        if (nhit == 0) {
-            node = sp > 0 ? stack[--sp] : kEmpty;
-            continue;
-        }
-        if (sp + nhit - 1 > kStackMax) {   // cannot happen for a checked depth: give up the ray
-            atomicOr(err, SONAR_DEVERR_STACK);
-            return CUDART_INF_F;
-        }
-        for (int c = nhit - 1; c >= 1; --c) {
-            const uint32_t k = key[c] & 3u;
-            stack[sp++] = k == 0 ? hs[0] : k == 1 ? hs[1] : k == 2 ? hs[2] : hs[3];
-        }
-        const uint32_t k = key[0] & 3u;
-        node = k == 0 ? hs[0] : k == 1 ? hs[1] : k == 2 ? hs[2] : hs[3];
     }
     return best_id == 0xFFFFFFFFu ? CUDART_INF_F : best_t;
 }
@@ -119,27 +130,29 @@ __device__ __forceinline__ float normal_of(uint32_t a, uint32_t b) {
     return sqrt_nonneg(neg2log_u(a)) * cospif(2.0f * u2);
 }
 
-// Four lanes per pose, lane k casting beam k; the group's first lane fits the
-// velocity by least squares over the valid beams (Cramer's rule on the 3 x 3
-// normal equations) and writes the pose's outputs.
-__global__ void __launch_bounds__(128) k_dvl(DvlArgs a) {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = g >> 2;
-    const int k = (int)(g & 3);
-    const int lane = threadIdx.x & 31, base = lane & ~3;
-    const unsigned grp = 0xFu << base;
+// 32 poses per block, warp k casting beam k of them; then a thread per pose fits
+// the velocity by least squares over the valid beams (Cramer's rule on the 3 x 3
+// normal equations) and writes the pose's outputs.  Consecutive poses are mostly
+// steps of one track, so the rays of a warp are nearly parallel and close, and
+// visit much the same nodes.
+// Bound by issue like the sonar's ray cast.  1M poses (4M beams) over 524,288
+// triangles: 624 us, against 707 us with the four beams of a pose side by side in
+// a warp, scalar plane distances and seven loads a node.
+constexpr int kDvlPoses = 32;
+__global__ void __launch_bounds__(4 * kDvlPoses) k_dvl(const __grid_constant__ DvlArgs a) {
+    __shared__ float s_range[4][kDvlPoses], s_u[4][kDvlPoses];
+    const int k = threadIdx.x / kDvlPoses, q = threadIdx.x & (kDvlPoses - 1);
+    const int64_t p = (int64_t)blockIdx.x * kDvlPoses + q;
     const bool live = p < a.n;
-    float range = CUDART_INF_F, u = 0.0f;
-    bool valid = false;
+    float3 o = f3(0.0f, 0.0f, 0.0f), d = f3(0.0f, 0.0f, 1.0f);
+    float u = 0.0f;
     if (live) {
-        const float* q = a.pose + 12 * p;
-        const float3 o = f3(q[0], q[1], q[2]);
-        const float* R = q + 3;
+        const float* pose = a.pose + 12 * p;
+        o = f3(pose[0], pose[1], pose[2]);
+        const float* R = pose + 3;
         const float bx = a.beam[k][0], by = a.beam[k][1], bz = a.beam[k][2];
-        float3 d = f3(fmaf(R[0], bx, fmaf(R[1], by, R[2] * bz)), fmaf(R[3], bx, fmaf(R[4], by, R[5] * bz)),
-                      fmaf(R[6], bx, fmaf(R[7], by, R[8] * bz)));
-        range = closest_distance(a.scene, o, d, CUDART_INF_F, a.err);
-        valid = range >= a.r_min && range <= a.r_max;
+        d = f3(fmaf(R[0], bx, fmaf(R[1], by, R[2] * bz)), fmaf(R[3], bx, fmaf(R[4], by, R[5] * bz)),
+               fmaf(R[6], bx, fmaf(R[7], by, R[8] * bz)));
         // sensor-frame velocity R^T v and this beam's radial velocity with noise
         const float* vw = a.vel_world + 3 * p;
         const float vs0 = fmaf(R[0], vw[0], fmaf(R[3], vw[1], R[6] * vw[2]));
@@ -149,17 +162,25 @@ __global__ void __launch_bounds__(128) k_dvl(DvlArgs a) {
                               a.seed_lo, a.seed_hi);
         const float w = (k & 1) ? normal_of(x.z, x.w) : normal_of(x.x, x.y);
         u = fmaf(bx, vs0, fmaf(by, vs1, bz * vs2)) + a.sigma_b * w;
-        a.ranges[4 * p + k] = range;
     }
-    const unsigned vm = __ballot_sync(0xFFFFFFFFu, valid);
+    s_range[k][q] = closest_distance(a.scene, live, o, d, a.err);
+    s_u[k][q] = u;
+    __syncthreads();
+    if (!live || k != 0) return;
     float rr[4], uu[4];
+    unsigned bits = 0u;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        rr[j] = __shfl_sync(0xFFFFFFFFu, range, base + j);
-        uu[j] = __shfl_sync(0xFFFFFFFFu, u, base + j);
+        rr[j] = s_range[j][q];
+        uu[j] = s_u[j][q];
+        if (rr[j] >= a.r_min && rr[j] <= a.r_max) bits |= 1u << j;
     }
-    if (!live || k != 0) return;
-    const unsigned bits = (vm & grp) >> base;
+    if ((reinterpret_cast<uintptr_t>(a.ranges) & 15u) == 0) {
+        reinterpret_cast<float4*>(a.ranges)[p] = make_float4(rr[0], rr[1], rr[2], rr[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a.ranges[4 * p + j] = rr[j];
+    }
     const int nvalid = __popc(bits);
     float A[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, y[3] = {0.f, 0.f, 0.f};
     float far = 0.0f;
@@ -196,19 +217,45 @@ __global__ void __launch_bounds__(128) k_dvl(DvlArgs a) {
     a.period[p] = (flags & 16) ? fmaf(a.t1, far, a.t0) : a.t_lost;
 }
 
-// Emission schedule: one thread per vehicle walks its steps (a measurement at
-// step 0, then max(1, ceil(period / dt)) steps after each measurement).
-__global__ void k_dvl_schedule(const float* period, int64_t n_veh, int64_t n_steps, float dt, int32_t* emit) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Emission schedule: one warp per vehicle walks its steps (a measurement at step
+// 0, then max(1, ceil(period / dt)) steps after each measurement), a chunk of
+// steps at a time: the lanes turn the chunk's periods into step counts in shared
+// memory, lane 0 walks those, and the chunk is written as whole rows.
+// 4096 vehicles x 256 steps: 17 us, against 78 us with a thread per vehicle that
+// clears, reads and marks its row alone.
+constexpr int kSchedWarps = 4, kSchedChunk = 256;
+__global__ void __launch_bounds__(32 * kSchedWarps) k_dvl_schedule(const float* period, int64_t n_veh, int64_t n_steps,
+                                                                   float dt, int32_t* emit) {
+    __shared__ int32_t s_next[kSchedWarps][kSchedChunk];
+    __shared__ uint32_t s_bits[kSchedWarps][kSchedChunk / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t v = (int64_t)blockIdx.x * kSchedWarps + warp;
     if (v >= n_veh) return;
     const float* P = period + v * n_steps;
     int32_t* E = emit + v * n_steps;
-    for (int64_t s = 0; s < n_steps; ++s) E[s] = 0;
-    int64_t s = 0;
-    while (s < n_steps) {
-        E[s] = 1;
-        const float q = ceilf(P[s] / dt);
-        s += q >= 1.0f ? (int64_t)q : 1;
+    int64_t at = 0;   // the next measurement (the same in every lane)
+    for (int64_t s0 = 0; s0 < n_steps; s0 += kSchedChunk) {
+        const int count = (int)min((int64_t)kSchedChunk, n_steps - s0);
+        if (lane < kSchedChunk / 32) s_bits[warp][lane] = 0u;
+        if (at < s0 + count) {
+            for (int i = lane; i < count; i += 32) {
+                const float q = ceilf(P[s0 + i] / dt);
+                s_next[warp][i] = q >= 1073741824.0f ? 0 : q >= 1.0f ? (int32_t)q : 1;   // 0: beyond 32 bits
+            }
+            __syncwarp();
+            if (lane == 0) {
+                while (at < s0 + count) {
+                    const int i = (int)(at - s0);
+                    s_bits[warp][i >> 5] |= 1u << (i & 31);
+                    const int32_t step = s_next[warp][i];
+                    at += step > 0 ? step : (int64_t)fminf(ceilf(P[at] / dt), 4.0e18f);
+                }
+            }
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+        }
+        __syncwarp();
+        for (int i = lane; i < count; i += 32) E[s0 + i] = (int32_t)((s_bits[warp][i >> 5] >> (i & 31)) & 1u);
+        __syncwarp();
     }
 }
 
@@ -219,13 +266,15 @@ __global__ void k_dvl_schedule(const float* period, int64_t n_veh, int64_t n_ste
 // ---------------------------------------------------------------------------
 
 cudaError_t launch_dvl(const DvlArgs& a, cudaStream_t st) {
-    if (a.n > 0) k_dvl<<<(unsigned)((4 * a.n + 127) / 128), 128, 0, st>>>(a);
+    if (a.n > 0) k_dvl<<<(unsigned)((a.n + kDvlPoses - 1) / kDvlPoses), 4 * kDvlPoses, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dvl_schedule(const float* period, int64_t n_veh, int64_t n_steps, float dt, int32_t* emit,
                                 cudaStream_t st) {
-    if (n_veh > 0 && n_steps > 0) k_dvl_schedule<<<(unsigned)((n_veh + 127) / 128), 128, 0, st>>>(period, n_veh, n_steps, dt, emit);
+    if (n_veh > 0 && n_steps > 0) 
+        k_dvl_schedule<<<(unsigned)((n_veh + kSchedWarps - 1) / kSchedWarps), 32 * kSchedWarps, 0, st>>>(
+            period, n_veh, n_steps, dt, emit);
     return cudaGetLastError();
 }
 

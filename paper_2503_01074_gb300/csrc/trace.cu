@@ -161,55 +161,6 @@ __device__ __forceinline__ uint4 record_of(const SensorDev& S, const SceneDev& s
     return make_uint4(key, orig, __float_as_uint(tr), cosb);
 }
 
-// A float twice, as the packed pair operand of fma.rn.f32x2.
-__device__ __forceinline__ unsigned long long pk2(float v) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-    return r;
-}
-// (d0, d1) = (a0, a1) * b + c element by element in one packed FP32 FMA
-// (sm_100 and later), each element rounded exactly like fmaf
-__device__ __forceinline__ void fma2(float a0, float a1, unsigned long long b, unsigned long long c, float& d0,
-                                     float& d1) {
-    asm("{\n\t.reg .b64 ra, rd;\n\tmov.b64 ra, {%2, %3};\n\tfma.rn.f32x2 rd, ra, %4, %5;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "l"(b), "l"(c));
-}
-// Sorts W child keys ascending in registers: a 5-comparator network for 4,
-// Batcher's odd-even merge sort (19 comparators) for 8.
-template <int W>
-__device__ __forceinline__ void sort_keys(uint32_t (&key)[W]) {
-#define SONAR_USORT(x, y)                            \
-    {                                                \
-        const uint32_t mn = min(key[x], key[y]);     \
-        key[y] = max(key[x], key[y]);                \
-        key[x] = mn;                                 \
-    }
-    if constexpr (W == 4) {
-        SONAR_USORT(0, 1) SONAR_USORT(2, 3) SONAR_USORT(0, 2) SONAR_USORT(1, 3) SONAR_USORT(1, 2)
-    } else {
-        SONAR_USORT(0, 1) SONAR_USORT(2, 3) SONAR_USORT(4, 5) SONAR_USORT(6, 7)
-        SONAR_USORT(0, 2) SONAR_USORT(1, 3) SONAR_USORT(4, 6) SONAR_USORT(5, 7)
-        SONAR_USORT(1, 2) SONAR_USORT(5, 6)
-        SONAR_USORT(0, 4) SONAR_USORT(1, 5) SONAR_USORT(2, 6) SONAR_USORT(3, 7)
-        SONAR_USORT(2, 4) SONAR_USORT(3, 5)
-        SONAR_USORT(1, 2) SONAR_USORT(3, 4) SONAR_USORT(5, 6)
-    }
-#undef SONAR_USORT
-}
-
-// The handle in slot k (0 <= k < W) of a node's handles held in registers.
-template <int W>
-__device__ __forceinline__ int32_t child_at(const int32_t (&hs)[W], uint32_t k) {
-    if constexpr (W == 4) {
-        return k == 0 ? hs[0] : k == 1 ? hs[1] : k == 2 ? hs[2] : hs[3];
-    } else {
-        const int32_t h01 = (k & 1) ? hs[1] : hs[0], h23 = (k & 1) ? hs[3] : hs[2];
-        const int32_t h45 = (k & 1) ? hs[5] : hs[4], h67 = (k & 1) ? hs[7] : hs[6];
-        const int32_t h03 = (k & 2) ? h23 : h01, h47 = (k & 2) ? h67 : h45;
-        return (k & 4) ? h47 : h03;
-    }
-}
-
 // Each block is one warp on a tile of tb beams x (32 / tb) elevations of one
 // sensor: lane l traces beam i0 + l % tb, elevation j0 + l / tb, so that the
 // warp's rays sample a compact patch of the field of view.  (One-warp blocks
