@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(kThreads) k_mark(int l, BuildState* st, const 
     else mark_level<8>(1, l, st, info, list8, first8);
 }
 
-// Writes wide node e.  Empty slots hold a box at +inf that no ray enters and the
+// Writes wide node e.  Empty slots hold a point at +inf that no ray enters and the
 // empty handle.  The 4-wide layout keeps the planes axis by axis, the 8-wide one
 // child by child (sonar_internal.cuh).
 template <int W>
@@ -625,30 +625,36 @@ __device__ void write_node(int64_t e, const int32_t* list, const int32_t* first_
     const int n = pick_children<W>(list[e], info, side, handle);
     int32_t r = first_child[e];
     const float inf = __int_as_float(0x7F800000);
-    float4 l[W], h[W];
+    // centre and half-width: the half-width rounded up, so that the box only grows
+    float c[3][W], h[3][W];
+    int32_t hs[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-        l[k] = h[k] = make_float4(inf, inf, inf, __int_as_float(kEmpty));
+        c[0][k] = c[1][k] = c[2][k] = inf;
+        h[0][k] = h[1][k] = h[2][k] = 0.0f;
+        hs[k] = kEmpty;
         if (k >= n) continue;
-        l[k] = pairs[2 * (int64_t)side[k]];
-        h[k] = pairs[2 * (int64_t)side[k] + 1];
-        l[k].w = __int_as_float(handle[k] >= 0 ? r++ : handle[k]);
+        const float4 l4 = pairs[2 * (int64_t)side[k]], h4 = pairs[2 * (int64_t)side[k] + 1];
+        const float lo[3] = {l4.x, l4.y, l4.z}, hi[3] = {h4.x, h4.y, h4.z};
+        for (int a = 0; a < 3; ++a) {
+            c[a][k] = 0.5f * lo[a] + 0.5f * hi[a];
+            h[a][k] = fmaxf(__fsub_ru(hi[a], c[a][k]), __fsub_ru(c[a][k], lo[a]));
+        }
+        hs[k] = handle[k] >= 0 ? r++ : handle[k];
     }
     float4* o = nodes + 2 * W * e;
     if constexpr (W == 4) {
-        o[0] = make_float4(l[0].x, h[0].x, l[1].x, h[1].x);
-        o[1] = make_float4(l[2].x, h[2].x, l[3].x, h[3].x);
-        o[2] = make_float4(l[0].y, h[0].y, l[1].y, h[1].y);
-        o[3] = make_float4(l[2].y, h[2].y, l[3].y, h[3].y);
-        o[4] = make_float4(l[0].z, h[0].z, l[1].z, h[1].z);
-        o[5] = make_float4(l[2].z, h[2].z, l[3].z, h[3].z);
-        o[6] = make_float4(l[0].w, l[1].w, l[2].w, l[3].w);
+        for (int a = 0; a < 3; ++a) {
+            o[2 * a] = make_float4(c[a][0], c[a][1], c[a][2], c[a][3]);
+            o[2 * a + 1] = make_float4(h[a][0], h[a][1], h[a][2], h[a][3]);
+        }
+        o[6] = make_float4(__int_as_float(hs[0]), __int_as_float(hs[1]), __int_as_float(hs[2]), __int_as_float(hs[3]));
         o[7] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     } else {
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            o[2 * k] = make_float4(l[k].x, h[k].x, l[k].y, h[k].y);
-            o[2 * k + 1] = make_float4(l[k].z, h[k].z, l[k].w, 0.0f);
+            o[2 * k] = make_float4(c[0][k], h[0][k], c[1][k], h[1][k]);
+            o[2 * k + 1] = make_float4(c[2][k], h[2][k], __int_as_float(hs[k]), 0.0f);
         }
     }
 }

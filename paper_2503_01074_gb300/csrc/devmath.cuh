@@ -129,25 +129,26 @@ __device__ __forceinline__ bool mt_ff(const float o[3], const ff d[3], float4 a,
 }
 
 
-// Two consecutive float4 of a node (32 bytes, 32-byte aligned: nodes are
-// 128-byte lines) in one 256-bit read-only load, so that a 4-wide node takes
-// four load instructions instead of seven.
-__device__ __forceinline__ void ld_node_pair(const float4* p, float4& a, float4& b) {
+// Two consecutive float4 of a 4-wide node (32 bytes, 32-byte aligned: nodes are
+// 128-byte lines) in one 256-bit read-only load, so that a node takes four load
+// instructions instead of seven.
+__device__ __forceinline__ void ld_node_pair(const float4* p, float (&a)[4], float (&b)[4]) {
     asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
         : "l"(p));
 }
 
-// One child of an 8-wide node (32 bytes, 32-byte aligned) in one such load: its box's (lo, hi) planes per axis and its handle.
+// One child of an 8-wide node (32 bytes, 32-byte aligned) in one such load: its
+// box's centre and half-width per axis and its handle.
 struct Child {
-    float x0, x1, y0, y1, z0, z1;
+    float cx, hx, cy, hy, cz, hz;
     int32_t handle;
 };
 __device__ __forceinline__ Child ld_child(const float4* p) {
     Child c;
     float h, unused;
     asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(c.x0), "=f"(c.x1), "=f"(c.y0), "=f"(c.y1), "=f"(c.z0), "=f"(c.z1), "=f"(h), "=f"(unused)
+        : "=f"(c.cx), "=f"(c.hx), "=f"(c.cy), "=f"(c.hy), "=f"(c.cz), "=f"(c.hz), "=f"(h), "=f"(unused)
         : "l"(p));
     c.handle = __float_as_int(h);
     return c;
@@ -193,7 +194,8 @@ __device__ __forceinline__ void sort_keys(uint32_t (&key)[W]) {
 template <int W>
 __device__ __forceinline__ int32_t child_at(const int32_t (&hs)[W], uint32_t k) {
     if constexpr (W == 4) {
-        return k == 0 ? hs[0] : k == 1 ? hs[1] : k == 2 ? hs[2] : hs[3];
+        const int32_t h01 = (k & 1) ? hs[1] : hs[0], h23 = (k & 1) ? hs[3] : hs[2];
+        return (k & 2) ? h23 : h01;
     } else {
         const int32_t h01 = (k & 1) ? hs[1] : hs[0], h23 = (k & 1) ? hs[3] : hs[2];
         const int32_t h45 = (k & 1) ? hs[5] : hs[4], h67 = (k & 1) ? hs[7] : hs[6];

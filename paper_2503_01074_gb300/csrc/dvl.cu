@@ -40,59 +40,66 @@ __device__ __forceinline__ float closest_distance(const SceneDev& sc, bool live,
                           1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z)));
     const unsigned long long ivx = pk2(inv.x), ivy = pk2(inv.y), ivz = pk2(inv.z);
     const unsigned long long novx = pk2(-(o.x * inv.x)), novy = pk2(-(o.y * inv.y)), novz = pk2(-(o.z * inv.z));
-    int32_t stack[kStackMax];
-    int sp = 0;
+    const float3 ainv = f3(fabsf(inv.x), fabsf(inv.y), fabsf(inv.z));
+    int32_t stack[kStackMax + 1];   // above a bottom entry that ends the walk
+    stack[0] = kEmpty;
+    int sp = 1;
     float best_t = 3.0e38f;   // a finite cut keeps empty slots (boxes at +inf) out, see k_trace
     uint32_t best_id = 0xFFFFFFFFu;
     int32_t node = live ? sc.root : kEmpty, leaf = 0;
     if (node < 0 && node != kEmpty) { leaf = node; node = kEmpty; }
-    while (node != kEmpty || leaf != 0) {
-        while (node >= 0) {
-            const float4* pn = sc.nodes + 8 * (int64_t)node;
-            const float tcut = best_t * 1.00002f;
-            float4 x0, x1, y0, y1, z0, z1, ch, unused;
-            ld_node_pair(pn, x0, x1);
-            ld_node_pair(pn + 2, y0, y1);
-            ld_node_pair(pn + 4, z0, z1);
-            ld_node_pair(pn + 6, ch, unused);
-            const int32_t hs[4] = {__float_as_int(ch.x), __float_as_int(ch.y), __float_as_int(ch.z), __float_as_int(ch.w)};
-            // per axis, the (lo, hi) planes of children 0, 1 | 2, 3
-            const float xs[4][2] = {{x0.x, x0.y}, {x0.z, x0.w}, {x1.x, x1.y}, {x1.z, x1.w}};
-            const float ys[4][2] = {{y0.x, y0.y}, {y0.z, y0.w}, {y1.x, y1.y}, {y1.z, y1.w}};
-            const float zs[4][2] = {{z0.x, z0.y}, {z0.z, z0.w}, {z1.x, z1.y}, {z1.z, z1.w}};
-            uint32_t key[4];
-            int nhit = 0;
+    while (__any_sync(0xFFFFFFFFu, node != kEmpty || leaf != 0)) {
+        // descend while some lane has a node to visit and no leaf yet
+        while (__any_sync(0xFFFFFFFFu, node >= 0 && leaf == 0)) {
+            if (node >= 0) {
+                const float4* pn = sc.nodes + 8 * (int64_t)node;
+                const float tcut = best_t * 1.00002f;
+                // centres and half-widths of the children's boxes, handles (see k_trace)
+                float cx[4], hx[4], cy[4], hy[4], cz[4], hz[4], ch[4], none[4];
+                ld_node_pair(pn, cx, hx);
+                ld_node_pair(pn + 2, cy, hy);
+                ld_node_pair(pn + 4, cz, hz);
+                ld_node_pair(pn + 6, ch, none);
+                int32_t hs[4];
+                uint32_t key[4];
+                float tx[4], ty[4], tz[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float t0, t1;
-                fma2(xs[c][0], xs[c][1], ivx, novx, t0, t1);
-                float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
-                fma2(ys[c][0], ys[c][1], ivy, novy, t0, t1);
-                lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
-                fma2(zs[c][0], zs[c][1], ivz, novz, t0, t1);
-                lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
-                const bool hit = lo <= hi * 1.0000005f;
-                key[c] = hit ? ((__float_as_uint(lo) & ~3u) | (uint32_t)c) : 0xFFFFFFFFu;
-                nhit += hit;
-            }
-            sort_keys<4>(key);
-            if (nhit == 0) {
-                node = sp > 0 ? stack[--sp] : kEmpty;
-            } else {
-                if (sp + nhit - 1 > kStackMax) {   // cannot happen for a checked depth: give up the ray
-                    atomicOr(err, SONAR_DEVERR_STACK);
-                    return CUDART_INF_F;
+                for (int c = 0; c < 4; c += 2) {
+                    fma2(cx[c], cx[c + 1], ivx, novx, tx[c], tx[c + 1]);
+                    fma2(cy[c], cy[c + 1], ivy, novy, ty[c], ty[c + 1]);
+                    fma2(cz[c], cz[c + 1], ivz, novz, tz[c], tz[c + 1]);
                 }
 #pragma unroll
-                for (int c = 3; c >= 1; --c)
-                    if (c < nhit) stack[sp++] = child_at<4>(hs, key[c] & 3u);
-                node = child_at<4>(hs, key[0] & 3u);
+                for (int c = 0; c < 4; ++c) {
+                    hs[c] = __float_as_int(ch[c]);
+                    const float lo = fmaxf(fmaxf(fmaf(-hx[c], ainv.x, tx[c]), fmaf(-hy[c], ainv.y, ty[c])),
+                                           fmaxf(fmaf(-hz[c], ainv.z, tz[c]), 0.0f));
+                    const float hi = fminf(fminf(fmaf(hx[c], ainv.x, tx[c]), fmaf(hy[c], ainv.y, ty[c])),
+                                           fminf(fmaf(hz[c], ainv.z, tz[c]), tcut));
+                    const bool hit = lo <= hi * 1.0000005f;
+                    key[c] = hit ? ((__float_as_uint(lo) & ~3u) | (uint32_t)c) : 0xFFFFFFFFu;
+                }
+                sort_keys<4>(key);
+                if (sp + 3 > kStackMax) {   // cannot happen for a checked depth: give up the ray
+                    atomicOr(err, SONAR_DEVERR_STACK);
+                    node = kEmpty;
+                    leaf = 0;
+                    sp = 1;
+                    best_id = 0xFFFFFFFFu;
+                    best_t = 0.0f;
+                } else {
+#pragma unroll
+                    for (int c = 3; c >= 1; --c)
+                        if (key[c] != 0xFFFFFFFFu) stack[sp++] = child_at<4>(hs, key[c] & 3u);
+                    if (key[0] != 0xFFFFFFFFu) node = child_at<4>(hs, key[0] & 3u);
+                    else node = stack[--sp];
+                }
+                if (node < 0 && node != kEmpty && leaf == 0) {   // park the leaf, keep descending
+                    leaf = node;
+                    node = stack[--sp];
+                }
             }
-            if (node < 0 && node != kEmpty && leaf == 0) {   // park the leaf, keep descending
-                leaf = node;
-                node = sp > 0 ? stack[--sp] : kEmpty;
-            }
-            if (!__any_sync(__activemask(), leaf == 0)) break;
+            __syncwarp();
         }
         while (leaf != 0) {
             const int32_t x = ~leaf;
@@ -117,7 +124,7 @@ __device__ __forceinline__ float closest_distance(const SceneDev& sc, bool live,
             leaf = 0;
             if (node < 0 && node != kEmpty) {   // the next stacked entry is a leaf too
                 leaf = node;
-                node = sp > 0 ? stack[--sp] : kEmpty;
+                node = stack[--sp];
             }
         }
     }
@@ -136,8 +143,9 @@ __device__ __forceinline__ float normal_of(uint32_t a, uint32_t b) {
 // steps of one track, so the rays of a warp are nearly parallel and close, and
 // visit much the same nodes.
 // Bound by issue like the sonar's ray cast.  1M poses (4M beams) over 524,288
-// triangles: 624 us, against 707 us with the four beams of a pose side by side in
-// a warp, scalar plane distances and seven loads a node.
+// triangles: 707 us with the four beams of a pose side by side in a warp, scalar
+// plane distances and seven loads a node; 624 us by beams; 444 us with the
+// boxes and the descent in step of k_trace.
 constexpr int kDvlPoses = 32;
 __global__ void __launch_bounds__(4 * kDvlPoses) k_dvl(const __grid_constant__ DvlArgs a) {
     __shared__ float s_range[4][kDvlPoses], s_u[4][kDvlPoses];

@@ -1,17 +1,19 @@
 // Internal device-side definitions of libsonar (GB300, sm_103a).
 //
 // Data layout in HBM
-//   nodes       4-wide, float4[8] = 128 B (one cache line) per node, per axis
-//               two float4 of (lo, hi) plane pairs: [0] (lo.x, hi.x) of children
-//               0, 1, [1] of children 2, 3, [2], [3] the same for y, [4], [5] for
-//               z, [6] the 4 child handles, [7] unused.  Empty slots: boxes at +inf
+//   nodes       4-wide, float4[8] = 128 B (one cache line) per node: per axis the
+//               centres of the four children's boxes and their half-widths (two
+//               float4, one 256-bit load), then [6] the 4 child handles, [7] unused.
+//               A ray's distances to a box's near and far plane are its distance to
+//               the centre plane -+ |1 / d| times the half-width: FMAs, where lo and
+//               hi planes need a minimum and a maximum per axis (and the pipe of
+//               those is the busiest of the walk).  Empty slots: points at +inf
 //               (never entered), kEmpty.
 //   nodes8      8-wide, float4[16] = 256 B per node: child c is 32 bytes at 32 c,
-//               (lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, handle, 0), one 256-bit load (a
-//               lane of the several-lanes-per-ray walk takes whole children; the
-//               4-wide walk of a ray per thread is 4 % faster axis by axis).
-//               Built from the same binary hierarchy; a handle >= 0 here indexes
-//               nodes8.
+//               (centre, half-width) of x, y, z, handle, 0, one 256-bit load (a lane
+//               of the several-lanes-per-ray walk takes whole children; the 4-wide
+//               walk of a ray per lane is 4 % faster axis by axis).  Built from the
+//               same binary hierarchy; a handle >= 0 here indexes nodes8.
 //   handles     int32: >= 0 a node index; < 0 a leaf ~((first << 3) | (count - 1)),
 //               a run of 1..8 triangles in leaf order; kEmpty an empty slot.
 //   triangles   float4[3] per triangle in leaf order (48 B):
@@ -253,6 +255,7 @@ struct TraceArgs {
     sonar_hit* hits;            // written unless counting (the caller's buffer or scratch)
     uint32_t* err;
     TraceCounters tc;           // counting launches only
+    int32_t n_tiles;            // k_trace: 32-ray tiles of the launch
     int32_t from_last;          // single: tiles from the last to the first
     int32_t* zero_word;         // cleared for a later launch (the adjoint's work counter), or nullptr
 };

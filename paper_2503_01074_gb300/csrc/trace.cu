@@ -2,11 +2,12 @@
 //
 // k_trig              float-float sin/cos tables of each sensor's beam azimuths
 //                     and elevations (FP64 once per sensor).
-// k_trace             one ray per thread, warps on compact beam x elevation
+// k_trace             one ray per lane, warps on compact beam x elevation
 //                     patches: ray generation -> closest hit (LBVH walk,
 //                     Moller-Trumbore) -> range/azimuth bin -> 16-byte hit record.
 //                     The STATS variant counts node visits and triangle tests and
 //                     marks the nodes and triangles it touches.
+// k_trace_group       the same with eight or four lanes per ray, for small launches.
 // k_popcount          counts the marked nodes and triangles.
 //
 // Ray casting precision: the walk and the triangle tests run in FP32.  A test
@@ -95,6 +96,65 @@ __device__ __noinline__ bool exact_closer(const SensorDev& s, int i, int j, cons
     return c < 0 || (c == 0 && id_p < id_q);
 }
 
+// The exact test of two triangles along the exact ray of (i, j), by a whole warp:
+// each half takes one (triangles f0 and f1 in leaf order), a lane per component of
+// a vector or per product, the same operations in the same order as mt_ff, so the
+// same bits.  Returns in every lane whether each is hit and its D and T, and the
+// length of the unnormalised direction.  An undecided test falls to about one ray
+// of a 32-ray tile; by its lane alone it took ~750 instructions in a row.
+struct ExactPair {
+    bool hit0, hit1;
+    ff D0, T0, D1, T1;
+    float len;
+};
+__device__ __forceinline__ ff shfl16(ff v, int src) {
+    return ff{__shfl_sync(0xFFFFFFFFu, v.hi, src, 16), __shfl_sync(0xFFFFFFFFu, v.lo, src, 16)};
+}
+__device__ __forceinline__ float axis_of(float4 v, int a) { return a == 0 ? v.x : a == 1 ? v.y : v.z; }
+
+__device__ __noinline__ ExactPair exact_pair(const SensorDev& s, const float4* tris, int i, int j, int f0, int f1) {
+    const int lane = threadIdx.x & 31, l = min(lane & 15, 11), kind = l / 3, ax = l - 3 * kind;
+    const float4* tp = tris + 3 * (int64_t)(lane < 16 ? f0 : f1);
+    const float4 a = __ldg(tp), b = __ldg(tp + 1), c = __ldg(tp + 2);
+    // components: lanes 0-2 e1, 3-5 e2, 6-8 s = o - v0, 9-11 the direction w
+    const ff e = ff_two_sum(kind == 0 ? axis_of(b, ax) : kind == 1 ? axis_of(c, ax) : s.pos[ax], -axis_of(a, ax));
+    const float4 bp = __ldg(s.trig + i), el = __ldg(s.trig + s.nb + j);
+    const ff sp{bp.x, bp.y}, cp{bp.z, bp.w}, st{el.x, el.y}, ct{el.z, el.w};
+    const ff w = ff_add(ff_add(ff_mulf(ff_mul(sp, ct), s.rot[3 * ax]), ff_mulf(ff_mul(cp, ct), s.rot[3 * ax + 1])),
+                        ff_mulf(st, s.rot[3 * ax + 2]));
+    const ff v{kind == 3 ? w.hi : e.hi, kind == 3 ? w.lo : e.lo};
+    // cross products: lanes 0-2 p = w x e2, 3-5 q = s x e1
+    const int y = ax == 2 ? 0 : ax + 1, z = ax == 0 ? 2 : ax - 1;
+    const int ka = kind == 0 ? 9 : 6, kb = kind == 0 ? 3 : 0;
+    const ff ay = shfl16(v, ka + y), bz = shfl16(v, kb + z), az = shfl16(v, ka + z), by = shfl16(v, kb + y);
+    const ff cr = ff_sub(ff_mul(ay, bz), ff_mul(az, by));
+    // dot products, three lanes each: det = e1 p, u = s p, v = w q, t = e2 q
+    const ff x0 = shfl16(v, (kind == 0 ? 0 : kind == 1 ? 6 : kind == 2 ? 9 : 3) + ax);
+    const ff x1 = shfl16(cr, (kind < 2 ? 0 : 3) + ax);
+    const ff m = ff_mul(x0, x1);
+    const ff dot = ff_add(ff_add(shfl16(m, 3 * kind), shfl16(m, 3 * kind + 1)), shfl16(m, 3 * kind + 2));
+    const ff det = shfl16(dot, 0);
+    ff un = shfl16(dot, 3), vn = shfl16(dot, 6), tn = shfl16(dot, 9);
+    const int sg = ff_sign(det);
+    ff D = det;
+    if (sg < 0) { D = ff_neg(det); un = ff_neg(un); vn = ff_neg(vn); tn = ff_neg(tn); }
+    const bool hit = sg != 0 && !(ff_sign(un) < 0 || ff_sign(vn) < 0 || ff_sign(ff_sub(ff_sub(D, un), vn)) < 0 ||
+                                  ff_sign(tn) <= 0);
+    const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+    auto of = [&](float x, int half) { return __shfl_sync(0xFFFFFFFFu, x, 16 * half); };
+    ExactPair r;
+    r.hit0 = hits & 1u;
+    r.hit1 = (hits >> 16) & 1u;
+    r.D0 = ff{of(D.hi, 0), of(D.lo, 0)};
+    r.T0 = ff{of(tn.hi, 0), of(tn.lo, 0)};
+    r.D1 = ff{of(D.hi, 1), of(D.lo, 1)};
+    r.T1 = ff{of(tn.hi, 1), of(tn.lo, 1)};
+    const float w0 = __shfl_sync(0xFFFFFFFFu, w.hi, 0), w1 = __shfl_sync(0xFFFFFFFFu, w.hi, 1),
+                w2 = __shfl_sync(0xFFFFFFFFu, w.hi, 2);
+    r.len = sqrtf(w0 * w0 + w1 * w1 + w2 * w2);
+    return r;
+}
+
 // Float-float sine and cosine tables of the sensor's beam azimuths
 // phi_i = -H/2 + (i + 1/2) H / N_b and elevations theta_j = -V/2 + (j + 1/2) V / N_e
 // (computed in FP64 once per sensor, split into hi + lo floats): trig[i] for
@@ -161,47 +221,59 @@ __device__ __forceinline__ uint4 record_of(const SensorDev& S, const SceneDev& s
     return make_uint4(key, orig, __float_as_uint(tr), cosb);
 }
 
-// Each block is one warp on a tile of tb beams x (32 / tb) elevations of one
-// sensor: lane l traces beam i0 + l % tb, elevation j0 + l / tb, so that the
-// warp's rays sample a compact patch of the field of view.  (One-warp blocks
-// free their slot as soon as their rays are done.)  Records go to their
-// canonical index i * n_elev + j.
+// Each warp takes a tile of tb beams x (32 / tb) elevations of one sensor: lane l
+// traces beam i0 + l % tb, elevation j0 + l / tb, so that the warp's rays sample
+// a compact patch of the field of view.  Records go to their canonical index
+// i * n_elev + j.
 //
 // The walk over the W-wide hierarchy (W = 4, or 8 for launches too small to
 // fill the GPU, where fewer dependent node loads per ray matter more than the
-// extra box tests per visit) is a while-while loop: a lane descends
-// nearest child first, pushing the other entered children; a lane that
-// reaches a leaf parks it and keeps descending until every active lane of the
-// warp holds one, so that the triangle tests run together.  A lane whose ray
-// is finished writes its record at once and idles until the warp is done.
+// extra box tests per visit) is a while-while loop in step: lanes descend nearest
+// child first, pushing the other entered children; a lane that reaches a leaf
+// parks it and keeps descending until no lane is without one, so that the
+// triangle tests run together, and the whole warp settles the undecided ones
+// (exact_pair).  A lane whose ray is finished writes its record at once and
+// idles until the warp is done.
+//
+// Bound by issue, the pipe of comparisons, minima and selections first, with the
+// latency of node loads next (about 62 % of the issue slots, 25 of 32 warps).
+// What that came to, ray cast of 64 frames of 512 x 64 rays / 128 mixed sensors /
+// 32 frames of 1024 x 256 rays over 33.6 million triangles, hit records the same:
+// 432 / 1277 / 1994 us, undecided tests by their lane alone; 426 / 1261 / 1979 by
+// the warp, which also takes the walk from 95 registers to 69; 405 / 1200 / 1882
+// with handles selected by the bits of their slot and no count of entered
+// children; 393 / 1163 / 1838 with a bottom stack entry instead of an empty test
+// and two tiles a block (the block limit is 32 per SM, and two warps share the
+// slot of one); 383 / 1132 / 1791 with boxes as centre and half-width.
 // With STATS the kernel also counts node visits and triangle tests and marks
 // the nodes and triangles it touches (records are then not written).
+constexpr int kTraceWarps = 2;   // tiles per block, each a warp's own
 template <int MINB, bool STATS, int W>
-__global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ TraceArgs a) {
-    __shared__ SensorDev S;
-    __shared__ SceneDev SC;
-    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by the next launch only
-    int tile;
+__global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_constant__ TraceArgs a) {
+    __shared__ SensorDev s_S[kTraceWarps];
+    __shared__ SceneDev s_SC[kTraceWarps];
+    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int tile = blockIdx.x * kTraceWarps + wid;
+    if (tile >= a.n_tiles) return;
+    SensorDev& S = s_S[wid];
+    SceneDev& SC = s_SC[wid];
     if (a.sensors) {
         // the warp copies the sensor and scene descriptors word by word, both at
         // once (the map carries the scene index): one round trip after the map
-        const int4 m = a.block_map[blockIdx.x];
-        const uint32_t* s_src = reinterpret_cast<const uint32_t*>(a.sensors + m.x);
-        const uint32_t* c_src = reinterpret_cast<const uint32_t*>(a.scenes + m.z);
-        constexpr int kSW = (int)(sizeof(SensorDev) / 4), kCW = (int)(sizeof(SceneDev) / 4);
-        for (int i = threadIdx.x; i < kSW; i += 32) reinterpret_cast<uint32_t*>(&S)[i] = __ldg(s_src + i);
-        for (int i = threadIdx.x; i < kCW; i += 32) reinterpret_cast<uint32_t*>(&SC)[i] = __ldg(c_src + i);
+        const int4 m = a.block_map[tile];
+        copy_words(&S, a.sensors + m.x, lane);
+        copy_words(&SC, a.scenes + m.z, lane);
         tile = m.y;
     } else {
-        copy_param(&S, &a.one, threadIdx.x);
-        copy_param(&SC, &a.one_scene, threadIdx.x);
-        tile = a.from_last ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+        copy_param(&S, &a.one, lane);
+        copy_param(&SC, &a.one_scene, lane);
+        if (a.from_last) tile = a.n_tiles - 1 - tile;
     }
-    __syncthreads();
+    __syncwarp();
     const int tb = S.tb, te = 32 / S.tb;
     const int tiles_b = (S.nb + tb - 1) / tb;
     const int ty = tile / tiles_b, tx = tile - ty * tiles_b;
-    const int lane = threadIdx.x;
     const int ri = tx * tb + (lane % tb);
     const int rj = ty * te + lane / tb;
     const SceneDev& sc = SC;
@@ -220,8 +292,10 @@ __global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ Trac
     // (inv, inv) and (-o inv, -o inv) per axis as packed pairs for the box tests
     const unsigned long long ivx = pk2(inv.x), ivy = pk2(inv.y), ivz = pk2(inv.z);
     const unsigned long long novx = pk2(-oinv.x), novy = pk2(-oinv.y), novz = pk2(-oinv.z);
-    int32_t stack[kStackMax];
-    int sp = 0, best = -1;
+    const float3 ainv = f3(fabsf(inv.x), fabsf(inv.y), fabsf(inv.z));
+    int32_t stack[kStackMax + 1];   // above a bottom entry that ends the walk
+    stack[0] = kEmpty;
+    int sp = 1, best = -1;
     uint32_t best_id = 0xFFFFFFFFu;
     float best_t = tlimit;
     uint64_t visits = 0, tests = 0, exact_n = 0;
@@ -231,8 +305,9 @@ __global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ Trac
     if (node < 0 && node != kEmpty) { leaf = node; node = kEmpty; }
     bool live = inside;
     for (;;) {
-        if (live) {
-            while (node >= 0) {
+        // descend while some lane has a node to visit and no leaf yet
+        while (__any_sync(0xFFFFFFFFu, node >= 0 && leaf == 0)) {
+            if (node >= 0) {
                 const float4* pn = W == 4 ? sc.nodes + 8 * (int64_t)node : sc.nodes8 + 16 * (int64_t)node;
                 if (STATS) {
                     ++visits;
@@ -244,42 +319,41 @@ __global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ Trac
                 // missed child sorts last as 0xFFFFFFFF
                 uint32_t key[W];
                 int32_t hs[W];
-                // per axis, the (lo, hi) planes of every child
-                float xs[W][2], ys[W][2], zs[W][2];
+                // per axis, the centre and half-width of every child's box
+                float cx[W], hx[W], cy[W], hy[W], cz[W], hz[W];
                 if constexpr (W == 4) {
-                    float4 a0, a1, unused;
-                    ld_node_pair(pn, a0, a1);
-                    xs[0][0] = a0.x; xs[0][1] = a0.y; xs[1][0] = a0.z; xs[1][1] = a0.w;
-                    xs[2][0] = a1.x; xs[2][1] = a1.y; xs[3][0] = a1.z; xs[3][1] = a1.w;
-                    ld_node_pair(pn + 2, a0, a1);
-                    ys[0][0] = a0.x; ys[0][1] = a0.y; ys[1][0] = a0.z; ys[1][1] = a0.w;
-                    ys[2][0] = a1.x; ys[2][1] = a1.y; ys[3][0] = a1.z; ys[3][1] = a1.w;
-                    ld_node_pair(pn + 4, a0, a1);
-                    zs[0][0] = a0.x; zs[0][1] = a0.y; zs[1][0] = a0.z; zs[1][1] = a0.w;
-                    zs[2][0] = a1.x; zs[2][1] = a1.y; zs[3][0] = a1.z; zs[3][1] = a1.w;
-                    ld_node_pair(pn + 6, a0, unused);
-                    hs[0] = __float_as_int(a0.x); hs[1] = __float_as_int(a0.y);
-                    hs[2] = __float_as_int(a0.z); hs[3] = __float_as_int(a0.w);
+                    ld_node_pair(pn, cx, hx);
+                    ld_node_pair(pn + 2, cy, hy);
+                    ld_node_pair(pn + 4, cz, hz);
+                    float h[4], none[4];
+                    ld_node_pair(pn + 6, h, none);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) hs[c] = __float_as_int(h[c]);
                 } else {
 #pragma unroll
                     for (int c = 0; c < W; ++c) {
                         const Child ch = ld_child(pn + 2 * c);
-                        xs[c][0] = ch.x0; xs[c][1] = ch.x1;
-                        ys[c][0] = ch.y0; ys[c][1] = ch.y1;
-                        zs[c][0] = ch.z0; zs[c][1] = ch.z1;
+                        cx[c] = ch.cx; hx[c] = ch.hx;
+                        cy[c] = ch.cy; hy[c] = ch.hy;
+                        cz[c] = ch.cz; hz[c] = ch.hz;
                         hs[c] = ch.handle;
                     }
                 }
+                // the ray's distance to a box's centre plane, two children at a time
+                float tx[W], ty[W], tz[W];
+#pragma unroll
+                for (int c = 0; c < W; c += 2) {
+                    fma2(cx[c], cx[c + 1], ivx, novx, tx[c], tx[c + 1]);
+                    fma2(cy[c], cy[c + 1], ivy, novy, ty[c], ty[c + 1]);
+                    fma2(cz[c], cz[c + 1], ivz, novz, tz[c], tz[c + 1]);
+                }
 #pragma unroll
                 for (int c = 0; c < W; ++c) {
-                    float t0, t1;
-                    fma2(xs[c][0], xs[c][1], ivx, novx, t0, t1);
-                    float lo = fminf(t0, t1), hi = fmaxf(t0, t1);
-                    fma2(ys[c][0], ys[c][1], ivy, novy, t0, t1);
-                    lo = fmaxf(lo, fminf(t0, t1)); hi = fminf(hi, fmaxf(t0, t1));
-                    fma2(zs[c][0], zs[c][1], ivz, novz, t0, t1);
-                    lo = fmaxf(fmaxf(lo, fminf(t0, t1)), 0.0f); hi = fminf(fminf(hi, fmaxf(t0, t1)), tcut);
-                    // an empty slot's box lies at +inf on every axis: along an axis
+                    const float lo = fmaxf(fmaxf(fmaf(-hx[c], ainv.x, tx[c]), fmaf(-hy[c], ainv.y, ty[c])),
+                                           fmaxf(fmaf(-hz[c], ainv.z, tz[c]), 0.0f));
+                    const float hi = fminf(fminf(fmaf(hx[c], ainv.x, tx[c]), fmaf(hy[c], ainv.y, ty[c])),
+                                           fminf(fmaf(hz[c], ainv.z, tz[c]), tcut));
+                    // an empty slot's box is a point at +inf on every axis: along an axis
                     // the ray travels in the + direction its entry distance is +inf,
                     // and if it travels in the - direction along all three its exit
                     // distance is -inf; the exit is also at most tcut, which is
@@ -288,78 +362,87 @@ __global__ void __launch_bounds__(32, MINB) k_trace(const __grid_constant__ Trac
                     key[c] = hit ? ((__float_as_uint(lo) & ~(uint32_t)(W - 1)) | (uint32_t)c) : 0xFFFFFFFFu;
                 }
                 sort_keys<W>(key);
-                int nhit = 0;
-#pragma unroll
-                for (int c = 0; c < W; ++c) nhit += key[c] != 0xFFFFFFFFu;
-                if (nhit == 0) {
-                    node = sp > 0 ? stack[--sp] : kEmpty;
+                if (sp + W - 1 > kStackMax) {   // cannot happen for a checked height: give up the ray
+                    atomicOr(a.err, SONAR_DEVERR_STACK);
+                    node = kEmpty;
+                    leaf = 0;
+                    sp = 1;
+                    best = -1;
                 } else {
-                    if (sp + nhit - 1 > kStackMax) {   // cannot happen for a checked height: give up the ray
-                        atomicOr(a.err, SONAR_DEVERR_STACK);
-                        node = kEmpty;
-                        leaf = 0;
-                        sp = 0;
-                        best = -1;
-                        break;
-                    }
 #pragma unroll
                     for (int c = W - 1; c >= 1; --c) {
-                        if (c < nhit) stack[sp++] = child_at<W>(hs, key[c] & (uint32_t)(W - 1));
+                        if (key[c] != 0xFFFFFFFFu) stack[sp++] = child_at<W>(hs, key[c] & (uint32_t)(W - 1));
                     }
-                    node = child_at<W>(hs, key[0] & (uint32_t)(W - 1));
+                    if (key[0] != 0xFFFFFFFFu) node = child_at<W>(hs, key[0] & (uint32_t)(W - 1));
+                    else node = stack[--sp];
                 }
                 if (node < 0 && node != kEmpty && leaf == 0) {   // park the leaf, keep descending
                     leaf = node;
-                    node = sp > 0 ? stack[--sp] : kEmpty;
+                    node = stack[--sp];
                 }
-                if (!__any_sync(__activemask(), leaf == 0)) break;
             }
-            while (leaf != 0) {
-                // a run of triangles in leaf order
-                const int32_t x = ~leaf;
-                const int32_t first = x >> 3, count = (x & 7) + 1;
-                for (int k = 0; k < count; ++k) {
-                    const int32_t f = first + k;
+            __syncwarp();
+        }
+        // the triangles of the parked leaves, a triangle of every lane's at a time;
+        // undecided tests and near ties are settled by the whole warp, one after another
+        while (__any_sync(0xFFFFFFFFu, leaf != 0)) {
+            const int32_t x = ~leaf;
+            const int32_t first = x >> 3, count = leaf != 0 ? (x & 7) + 1 : 0;
+            for (int k = 0; __any_sync(0xFFFFFFFFu, k < count); ++k) {
+                const int32_t f = first + k;
+                int r = 0;
+                float t = 0.0f;
+                uint32_t id = 0u;
+                if (k < count) {
                     if (f >= sc.n_tris) {
                         atomicOr(a.err, SONAR_DEVERR_INDEX);
-                        break;
-                    }
-                    const float4* tp = sc.tris + 3 * (int64_t)f;
-                    const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
-                    if (STATS) {
-                        ++tests;
-                        atomicOr(a.tc.tri_bits + (f >> 5), 1u << (f & 31));
-                    }
-                    float t;
-                    const int r = mt32(o, d, va, vb, vc, t);
-                    if (r == 0) continue;
-                    if (r == 2) {
-                        if (STATS) ++exact_n;
-                        if (!exact_hit(S, ri, rj, va, vb, vc, &t)) continue;
-                    }
-                    if (!(t < tlimit)) continue;
-                    const uint32_t id = __float_as_uint(vb.w);
-                    bool take;
-                    if (best < 0) {
-                        take = true;
-                    } else if (fabsf(t - best_t) <= 2e-5f * fmaxf(t, best_t)) {
-                        // near tie: decide on the exact distances, then on the caller's index
-                        if (STATS) ++exact_n;
-                        take = exact_closer(S, ri, rj, tp, id, sc.tris + 3 * (int64_t)best, best_id);
                     } else {
-                        take = t < best_t;
-                    }
-                    if (take) {
-                        best = f;
-                        best_id = id;
-                        best_t = t;
+                        const float4* tp = sc.tris + 3 * (int64_t)f;
+                        const float4 va = __ldg(tp), vb = __ldg(tp + 1), vc = __ldg(tp + 2);
+                        if (STATS) {
+                            ++tests;
+                            atomicOr(a.tc.tri_bits + (f >> 5), 1u << (f & 31));
+                        }
+                        r = mt32(o, d, va, vb, vc, t);
+                        id = __float_as_uint(vb.w);
                     }
                 }
-                leaf = 0;
-                if (node < 0 && node != kEmpty) {   // the next stacked entry is a leaf too
-                    leaf = node;
-                    node = sp > 0 ? stack[--sp] : kEmpty;
+                for (uint32_t m = __ballot_sync(0xFFFFFFFFu, r == 2); m; m &= m - 1) {
+                    const int src = __ffs(m) - 1;
+                    const int fs = __shfl_sync(0xFFFFFFFFu, f, src);
+                    const ExactPair e = exact_pair(S, sc.tris, __shfl_sync(0xFFFFFFFFu, ri, src),
+                                                   __shfl_sync(0xFFFFFFFFu, rj, src), fs, fs);
+                    if (lane == src) {
+                        if (STATS) ++exact_n;
+                        r = e.hit0;
+                        t = (e.T0.hi / e.D0.hi) * e.len;
+                    }
                 }
+                const bool cand = r != 0 && t < tlimit;
+                bool take = cand && (best < 0 || t < best_t);
+                // near tie: decide on the exact distances, then on the caller's index
+                const bool tie = cand && best >= 0 && fabsf(t - best_t) <= 2e-5f * fmaxf(t, best_t);
+                for (uint32_t m = __ballot_sync(0xFFFFFFFFu, tie); m; m &= m - 1) {
+                    const int src = __ffs(m) - 1;
+                    const ExactPair e = exact_pair(S, sc.tris, __shfl_sync(0xFFFFFFFFu, ri, src),
+                                                   __shfl_sync(0xFFFFFFFFu, rj, src), __shfl_sync(0xFFFFFFFFu, f, src),
+                                                   __shfl_sync(0xFFFFFFFFu, best, src));
+                    if (lane == src) {
+                        if (STATS) ++exact_n;
+                        const int c = ff_sign(ff_sub(ff_mul(e.T0, e.D1), ff_mul(e.T1, e.D0)));
+                        take = e.hit0 && (!e.hit1 || c < 0 || (c == 0 && id < best_id));
+                    }
+                }
+                if (take) {
+                    best = f;
+                    best_id = id;
+                    best_t = t;
+                }
+            }
+            leaf = 0;
+            if (node < 0 && node != kEmpty) {   // the next stacked entry is a leaf too
+                leaf = node;
+                node = stack[--sp];
             }
         }
         if (live && node == kEmpty) {
@@ -441,6 +524,7 @@ __global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_
                           1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y)),
                           1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z)));
     const float3 oinv = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    const float3 ainv = f3(fabsf(inv.x), fabsf(inv.y), fabsf(inv.z));
     const int lane = threadIdx.x & 31, shift = lane & ~(G - 1);
     const uint32_t mine = kLanes << shift;
     float2* stack = s_stack[group];
@@ -481,12 +565,13 @@ __global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_
             const float tcut = cut * 1.00002f;
 #pragma unroll
             for (int j = 0; j < J; ++j) {
-                const float x0 = fmaf(ch[j].x0, inv.x, -oinv.x), x1 = fmaf(ch[j].x1, inv.x, -oinv.x);
-                const float y0 = fmaf(ch[j].y0, inv.y, -oinv.y), y1 = fmaf(ch[j].y1, inv.y, -oinv.y);
-                const float z0 = fmaf(ch[j].z0, inv.z, -oinv.z), z1 = fmaf(ch[j].z1, inv.z, -oinv.z);
+                const float tx = fmaf(ch[j].cx, inv.x, -oinv.x), ty = fmaf(ch[j].cy, inv.y, -oinv.y),
+                            tz = fmaf(ch[j].cz, inv.z, -oinv.z);
                 h[j] = ch[j].handle;
-                lo[j] = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fmaxf(fminf(z0, z1), 0.0f));
-                const float hi = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fminf(fmaxf(z0, z1), tcut));
+                lo[j] = fmaxf(fmaxf(fmaf(-ch[j].hx, ainv.x, tx), fmaf(-ch[j].hy, ainv.y, ty)),
+                              fmaxf(fmaf(-ch[j].hz, ainv.z, tz), 0.0f));
+                const float hi = fminf(fminf(fmaf(ch[j].hx, ainv.x, tx), fmaf(ch[j].hy, ainv.y, ty)),
+                                       fminf(fmaf(ch[j].hz, ainv.z, tz), tcut));
                 const bool enter = lo[j] <= hi * 1.0000005f;   // never an empty slot (see k_trace)
                 inner[j] = enter && h[j] >= 0;
                 if (enter && h[j] < 0) {
@@ -664,12 +749,17 @@ cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStre
             k_trace_group<8><<<(unsigned)blocks * (32 * 8 / kGroupThreads), kGroupThreads, 0, st>>>(a);
         } else if (wide && (occupancy & kTraceGroup4)) {
             k_trace_group<4><<<(unsigned)blocks * (32 * 4 / kGroupThreads), kGroupThreads, 0, st>>>(a);
-        } else if (wide) {
-            if (cap) k_trace<32, false, 8><<<blocks, 32, 0, st>>>(a);
-            else k_trace<4, false, 8><<<blocks, 32, 0, st>>>(a);
         } else {
-            if (cap) k_trace<32, false, 4><<<blocks, 32, 0, st>>>(a);
-            else k_trace<4, false, 4><<<blocks, 32, 0, st>>>(a);
+            const unsigned grid = (unsigned)((blocks + kTraceWarps - 1) / kTraceWarps);
+            TraceArgs b = a;
+            b.n_tiles = blocks;
+            if (wide) {
+                if (cap) k_trace<16, false, 8><<<grid, 32 * kTraceWarps, 0, st>>>(b);
+                else k_trace<4, false, 8><<<grid, 32 * kTraceWarps, 0, st>>>(b);
+            } else {
+                if (cap) k_trace<16, false, 4><<<grid, 32 * kTraceWarps, 0, st>>>(b);
+                else k_trace<4, false, 4><<<grid, 32 * kTraceWarps, 0, st>>>(b);
+            }
         }
     }
     return cudaGetLastError();
@@ -685,8 +775,10 @@ cudaError_t launch_stats(const SensorDev& s, const SceneDev& sc, const sonar_par
     a.err = err;
     a.tc = tc;
     if (s.trace_blocks > 0) {
-        if ((s.occ & kTraceWide) && sc.nodes8) k_trace<4, true, 8><<<s.trace_blocks, 32, 0, st>>>(a);
-        else k_trace<4, true, 4><<<s.trace_blocks, 32, 0, st>>>(a);
+        a.n_tiles = s.trace_blocks;
+        const unsigned grid = (unsigned)((s.trace_blocks + kTraceWarps - 1) / kTraceWarps);
+        if ((s.occ & kTraceWide) && sc.nodes8) k_trace<4, true, 8><<<grid, 32 * kTraceWarps, 0, st>>>(a);
+        else k_trace<4, true, 4><<<grid, 32 * kTraceWarps, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
