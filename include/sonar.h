@@ -364,13 +364,13 @@ sonar_status sonar_autotune(sonar_batch_t batch, const sonar_params* params,
  * unused (kept so that saved rows stay valid; >= 1), block the adjoint's threads
  * per block, tb = beams per ray-cast warp (a power of two <= 32; elevations = 32 / tb), occ =
  * the ray-cast variant, a sum of flags: 8 caps its registers at 64 (32
- * one-warp blocks per SM), 16 walks the 8-wide tree instead of the 4-wide one
+ * resident warps per SM), 16 walks the 8-wide tree instead of the 4-wide one
  * (both are built per scene; the hit records are the same either way).  A
- * launch of at most 20 tiles of 32 rays per SM casts every ray with eight or
+ * launch of at most 22 tiles of 32 rays per SM casts every ray with eight or
  * four lanes on the 8-wide tree, whatever its row; a larger batch takes the
- * row's variant; a larger single-sensor call of at most one wave of one-warp
- * blocks (32 per SM) walks the 8-wide tree without the register cap, and one
- * beyond that the 4-wide tree with its row's cap.
+ * row's variant; a larger single-sensor call of at most one wave (32 tiles per
+ * SM) walks the 4-wide tree without the register cap, and one beyond that the
+ * 4-wide tree with its row's cap.
  * Returns the number of entries in *count. */
 sonar_status sonar_tune_get(sonar_ctx_t ctx, int32_t* rows, int32_t cap, int32_t* count);
 

@@ -28,19 +28,35 @@ namespace {
 // fold: the rays of every azimuth column -> the column's bins with returns
 // ---------------------------------------------------------------------------
 
-// The score of a hit record: s = mu[m] cos exp(-2 alpha r) gain (Eq. 2).
-__device__ __forceinline__ float score_of(const FoldArgs& a, const SceneDev& sc, uint4 h, float alpha, float gain) {
-    int m = __ldg(sc.mat_orig + h.y);
+// The score of a hit record of material m: s = mu[m] cos exp(-2 alpha r) gain (Eq. 2).
+__device__ __forceinline__ float score_of(const FoldArgs& a, int m, float r, float cosine, float alpha, float gain) {
     m = m < a.n_mat ? m : a.n_mat - 1;
-    return __ldg(a.theta + 2 + m) * __uint_as_float(h.w) * expf(-2.0f * alpha * __uint_as_float(h.z)) * gain;
+    return __ldg(a.theta + 2 + m) * cosine * expf(-2.0f * alpha * r) * gain;
+}
+
+// Division by naz of multiples of it: a shift by its trailing zeros and a
+// multiplication by the inverse of its odd part modulo 2^32 (Newton's iteration
+// doubles the correct low bits, from 5).
+struct ExactDiv {
+    uint32_t naz, inv;
+    int shift;
+};
+__device__ __forceinline__ ExactDiv exact_div(uint32_t naz) {
+    const int shift = __ffs((int)naz) - 1;
+    const uint32_t odd = naz >> shift;
+    uint32_t x = (odd * 3u) ^ 2u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x *= 2u - odd * x;
+    return ExactDiv{naz, x, shift};
 }
 
 // Range row of a record of azimuth column `col`, or -1: no return, or a
 // corrupt record (reported in the error word).
-__device__ __forceinline__ int row_of(const FoldArgs& a, const SensorDev& S, const SceneDev& sc, uint4 h, int col) {
-    if (h.x == kNoKey) return -1;
-    const uint32_t row = h.x / (uint32_t)S.naz;
-    if (row >= (uint32_t)S.nr || h.x - row * (uint32_t)S.naz != (uint32_t)col || h.y >= (uint32_t)sc.n_tris) {
+__device__ __forceinline__ int row_of(const FoldArgs& a, const ExactDiv& div, uint32_t nr, uint32_t n_tris,
+                                      uint32_t key, uint32_t tri, uint32_t col) {
+    if (key == kNoKey) return -1;
+    const uint32_t row = ((key - col) >> div.shift) * div.inv;
+    if (row >= nr || row * div.naz + col != key || tri >= n_tris) {
         atomicOr(a.err, SONAR_DEVERR_INDEX);
         return -1;
     }
@@ -89,13 +105,67 @@ __device__ __forceinline__ void fold_step(float* acc, float* scores, int idx, fl
 
 // A finished bin (rank k of its column): P and the speckle factor 0.5 + w_sm
 // of Eq. 3, compactly; or P into the image itself where no scratch holds them.
-__device__ __forceinline__ void put_bin(const FoldArgs& a, const SensorDev& S, const PhiloxKey& K, int64_t first, int k,
-                                        int row, int col, float P) {
+__device__ __forceinline__ void put_bin(const FoldArgs& a, const SensorDev& S, int64_t first, int k, int row, int col,
+                                        float P) {
     const uint32_t b = (uint32_t)row * (uint32_t)S.naz + (uint32_t)col;
     if (a.dense) {
         a.dense[S.polar_off + b] = P;
     } else {
-        a.vals[S.val_off + first + k] = make_float2(P, 0.5f + gauss_of(bin_draws(b, S, K), a.sigma_sm));
+        a.vals[S.val_off + first + k] = make_float2(P, 0.5f + gauss_of(philox10(U4{b, S.frame_lo, 0u, S.frame_hi}, S.seed_lo, S.seed_hi), a.sigma_sm));
+    }
+}
+
+constexpr int kFoldAhead = 2;   // chunks of 32 rays whose loads are issued together
+
+// Marks the rows of rays first, first + step, ... (step a multiple of 32) of a
+// column's n records.
+__device__ __forceinline__ void mark_rows(const FoldArgs& a, const ExactDiv& div, const SensorDev& S,
+                                          const SceneDev& sc, const sonar_hit* H, uint32_t n, uint32_t first, uint32_t step,
+                                          int col, uint32_t* bits) {
+    for (uint32_t j = first; j < n; j += kFoldAhead * step) {
+        uint2 h[kFoldAhead];   // key, triangle
+#pragma unroll
+        for (int u = 0; u < kFoldAhead; ++u)
+            h[u] = j + u * step < n ? __ldg(reinterpret_cast<const uint2*>(H + j + u * step)) : make_uint2(kNoKey, 0u);
+#pragma unroll
+        for (int u = 0; u < kFoldAhead; ++u) {
+            const int row = row_of(a, div, S.nr, sc.n_tris, h[u].x, h[u].y, col);
+            if (row >= 0) atomicOr(bits + (row >> 5), 1u << (row & 31));
+        }
+    }
+}
+
+// Sums the scores of n consecutive records, in order, at the ranks of their rows
+// (one warp): the records of several chunks, then their materials, are loaded
+// together, so that a chunk does not wait for both in turn.
+__device__ __forceinline__ void sum_rows(const FoldArgs& a, const ExactDiv& div, const SensorDev& S,
+                                         const SceneDev& sc, const sonar_hit* H, uint32_t n, int col,
+                                         const uint32_t* bits, const uint32_t* pre, int* rows, float* acc,
+                                         float* scores, float alpha, float gain, int lane) {
+    for (uint32_t jb = 0; jb < n; jb += 32 * kFoldAhead) {
+        uint4 h[kFoldAhead];
+#pragma unroll
+        for (int u = 0; u < kFoldAhead; ++u)
+            h[u] = jb + 32 * u + lane < n ? __ldg(reinterpret_cast<const uint4*>(H + jb + 32 * u + lane))
+                                          : make_uint4(kNoKey, 0u, 0u, 0u);
+        int row[kFoldAhead], mat[kFoldAhead];
+#pragma unroll
+        for (int u = 0; u < kFoldAhead; ++u) {
+            row[u] = row_of(a, div, S.nr, sc.n_tris, h[u].x, h[u].y, col);
+            mat[u] = row[u] >= 0 ? __ldg(sc.mat_orig + h[u].y) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kFoldAhead; ++u) {
+            if (jb + 32 * u >= n) break;
+            int idx = -1;
+            float score = 0.0f;
+            if (row[u] >= 0) {
+                idx = bit_rank(bits, pre, row[u]);
+                rows[idx] = row[u];   // every writer of a rank writes the same row
+                score = score_of(a, mat[u], __uint_as_float(h[u].z), __uint_as_float(h[u].w), alpha, gain);
+            }
+            fold_step(acc, scores, idx, score, lane);
+        }
     }
 }
 
@@ -112,13 +182,15 @@ __device__ __forceinline__ void put_bin(const FoldArgs& a, const SensorDev& S, c
 // per range bin, and no pass over all bins is left here.
 //
 // Bound by the latency of its dependent steps (record, material, rank, sum),
-// which the resident columns hide.  Measured, this kernel and k_rows against the
-// binning kernel over dense column blocks and the normalisation pass that they
-// replace: 64 frames of 512 x 64 rays into 1000 x 512 bins 48 + 98 us against
-// 231 + 43 us (132 + 43 us with hand-picked units); 32 frames of 1024 x 256
-// rays into 4000 x 1024 bins 148 + 410 us against 1122 + 153 us; one frame of
-// 3000 x 460 rays into 350 x 220 bins 42 + 6 us against 462 + 5 us.
-__global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a) {
+// which the resident columns hide (40 registers: 48 warps an SM), and by issue where
+// columns hold many rays.  Measured, this kernel and k_rows against the binning
+// kernel over dense column blocks and the normalisation pass that they replace:
+// 64 frames of 512 x 64 rays into 1000 x 512 bins 39 + 90 us against 231 + 43 us
+// (132 + 43 us with hand-picked units); 32 frames of 1024 x 256 rays into 4000 x
+// 1024 bins 474 us together against 1122 + 153; one frame of 3000 x 460 rays into
+// 350 x 220 bins 39 + 6 us against 462 + 5.  Rows by exact division instead of a
+// general one, fewer registers and two chunks of loads at a time were 17 % of it.
+__global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArgs a) {
     extern __shared__ __align__(16) uint32_t fold_smem[];
     __shared__ SensorDev S;
     __shared__ SceneDev SC;
@@ -139,15 +211,15 @@ __global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a
     }
     __syncthreads();
     const float alpha = __ldg(a.theta), gain = __ldg(a.theta + 1);
-    const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
+    const ExactDiv div = exact_div((uint32_t)S.naz);
     const int ne = S.ne, nwords = (S.nr + 31) >> 5;
     const int col = s_col + (S.fold_beams ? 0 : warp);
     if (col >= S.naz) return;   // whole warps only (the last block of a sensor)
     const int i0 = first_beam_of_col(col, S.nb, S.naz), i1 = first_beam_of_col(col + 1, S.nb, S.naz);
     const int64_t first = (int64_t)i0 * ne;          // the column's first ray, and its first value slot
-    const int64_t n = (int64_t)(i1 - i0) * ne;
+    const int n = (i1 - i0) * ne;                    // a sensor's rays fit 31 bits
     const sonar_hit* H = a.hits + S.hits_off + first;
-    const int most = (int)min((int64_t)S.nr, n);     // bins with returns, at most
+    const int most = min(S.nr, n);                   // bins with returns, at most
     if (!S.fold_beams) {
         uint32_t* bits = fold_smem + (int64_t)warp * a.words_per_warp;
         uint32_t* pre = bits + nwords;
@@ -155,29 +227,13 @@ __global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a
         int* rows = reinterpret_cast<int*>(acc + most);
         for (int w = lane; w < nwords; w += 32) bits[w] = 0u;
         __syncwarp();
-        for (int64_t j = lane; j < n; j += 32) {
-            const int row = row_of(a, S, SC, __ldg(reinterpret_cast<const uint4*>(H + j)), col);
-            if (row >= 0) atomicOr(bits + (row >> 5), 1u << (row & 31));
-        }
+        mark_rows(a, div, S, SC, H, n, lane, 32, col, bits);
         __syncwarp();
         const int nd = bit_prefix(bits, pre, nwords, lane);
         for (int k = lane; k < nd; k += 32) acc[k] = 0.0f;
         __syncwarp();
-        for (int64_t jb = 0; jb < n; jb += 32) {
-            int idx = -1;
-            float score = 0.0f;
-            if (jb + lane < n) {
-                const uint4 h = __ldg(reinterpret_cast<const uint4*>(H + jb + lane));
-                const int row = row_of(a, S, SC, h, col);
-                if (row >= 0) {
-                    idx = bit_rank(bits, pre, row);
-                    rows[idx] = row;
-                    score = score_of(a, SC, h, alpha, gain);
-                }
-            }
-            fold_step(acc, s_scores[warp], idx, score, lane);
-        }
-        for (int k = lane; k < nd; k += 32) put_bin(a, S, K, first, k, rows[k], col, acc[k]);
+        sum_rows(a, div, S, SC, H, n, col, bits, pre, rows, acc, s_scores[warp], alpha, gain, lane);
+        for (int k = lane; k < nd; k += 32) put_bin(a, S, first, k, rows[k], col, acc[k]);
         if (a.bands)
             for (int w = lane; w < nwords; w += 32)
                 a.bands[S.band_off + (int64_t)w * S.naz + col] = make_uint2(bits[w], (uint32_t)first + pre[w]);
@@ -192,10 +248,7 @@ __global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a
     float* acc = reinterpret_cast<float*>(rows + most);   // [nbeam][nd]
     for (int w = tid; w < nwords; w += nt) bits[w] = 0u;
     __syncthreads();
-    for (int64_t j = tid; j < n; j += nt) {
-        const int row = row_of(a, S, SC, __ldg(reinterpret_cast<const uint4*>(H + j)), col);
-        if (row >= 0) atomicOr(bits + (row >> 5), 1u << (row & 31));
-    }
+    mark_rows(a, div, S, SC, H, n, tid, nt, col, bits);
     __syncthreads();
     if (warp == 0) {
         const int total = bit_prefix(bits, pre, nwords, lane);
@@ -205,27 +258,14 @@ __global__ void __launch_bounds__(512) k_fold(const __grid_constant__ FoldArgs a
     const int nd = s_n;
     for (int k = tid; k < nbeam * nd; k += nt) acc[k] = 0.0f;
     __syncthreads();
-    for (int bb = warp; bb < nbeam; bb += nw) {
-        for (int jb = 0; jb < ne; jb += 32) {
-            int idx = -1;
-            float score = 0.0f;
-            if (jb + lane < ne) {
-                const uint4 h = __ldg(reinterpret_cast<const uint4*>(H + (int64_t)bb * ne + jb + lane));
-                const int row = row_of(a, S, SC, h, col);
-                if (row >= 0) {
-                    idx = bit_rank(bits, pre, row);
-                    rows[idx] = row;   // every writer of a rank writes the same row
-                    score = score_of(a, SC, h, alpha, gain);
-                }
-            }
-            fold_step(acc + bb * nd, s_scores[warp], idx, score, lane);
-        }
-    }
+    for (int bb = warp; bb < nbeam; bb += nw)
+        sum_rows(a, div, S, SC, H + (int64_t)bb * ne, ne, col, bits, pre, rows, acc + bb * nd, s_scores[warp], alpha, gain,
+                 lane);
     __syncthreads();
     for (int k = tid; k < nd; k += nt) {
         float P = 0.0f;
         for (int bb = 0; bb < nbeam; ++bb) P += acc[bb * nd + k];
-        put_bin(a, S, K, first, k, rows[k], col, P);
+        put_bin(a, S, first, k, rows[k], col, P);
     }
     if (a.bands)
         for (int w = tid; w < nwords; w += nt)
@@ -279,9 +319,11 @@ __device__ __forceinline__ float div_by(float v, float m, float y) {
 // (wider rows, and the dense form of the fold's result): I~ is written, then read
 // back by the same lanes and divided.
 //
-// Bound by instruction issue (about 80 per bin, most of them the logarithm and a
-// quarter of a Philox block): 64 frames of 1000 x 512 bins in 98 us, 2.7 TB/s of
-// stores.  The 262 MB that it writes would take 39 us.
+// Bound by instruction issue (about 75 per bin, most of them the logarithm and a
+// quarter of a Philox block): 64 frames of 1000 x 512 bins in 92 us, 2.8 TB/s of
+// stores (the 262 MB that it writes would take 39 us); 125 us with an IEEE division,
+// two integer conversions and general square roots and divisions per bin.  32 rows
+// a block: 16 take 4 to 8 % longer, 8 up to 25 % (the column tables are read again).
 template <int REG, bool VEC>
 __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_constant__ RowsArgs a) {
     extern __shared__ __align__(16) uint32_t rows_smem[];
@@ -328,19 +370,21 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
         if (row >= nr) break;
         const uint32_t b0 = (uint32_t)row * (uint32_t)naz;
         const int sh = VEC ? 0 : (int)(b0 & 3u), nq = (sh + naz + 3) >> 2;
-        const int64_t off = S.polar_off + (int64_t)b0 - sh;   // of the first quad's first bin
+        const int64_t off = S.polar_off + (int64_t)b0 - sh + 4 * lane;   // of the lane's first quad's first bin
         const float rc = fmaf(small_u2f((uint32_t)row) + 0.5f, dr, S.rmin);
-        const uint32_t bit = 1u << (row & 31);
-        // the four bins of quad q: I~ in v, P in p
-        auto quad = [&](int q, float (&v)[4], float (&p)[4]) {
+        const uint32_t bit = 1u << (row & 31), below = bit - 1u;
+        // The four bins of the lane's k-th quad (quad q = lane + 32 k of the row, at
+        // 128 k elements from the first): I~ in v, P in p.
+        auto quad = [&](int k, float (&v)[4], float (&p)[4]) {
+            const int q = lane + 32 * k;
             float2 ret[4];
             float pt[4];
             uint2 w[4];
             if (VEC && staged) {   // 16-byte shared-memory reads
-                const float4 p4 = *reinterpret_cast<const float4*>(pat + 4 * q);
+                const float4 p4 = reinterpret_cast<const float4*>(pat)[q];
                 pt[0] = p4.x; pt[1] = p4.y; pt[2] = p4.z; pt[3] = p4.w;
-                const uint4 w0 = *reinterpret_cast<const uint4*>(mask + 4 * q);
-                const uint4 w1 = *reinterpret_cast<const uint4*>(mask + 4 * q + 2);
+                const uint4 w0 = reinterpret_cast<const uint4*>(mask)[2 * q];
+                const uint4 w1 = reinterpret_cast<const uint4*>(mask)[2 * q + 1];
                 w[0] = make_uint2(w0.x, w0.y); w[1] = make_uint2(w0.z, w0.w);
                 w[2] = make_uint2(w1.x, w1.y); w[3] = make_uint2(w1.z, w1.w);
             }
@@ -351,7 +395,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                 if (VEC || (c >= 0 && c < naz)) {
                     if (!(VEC && staged)) pt[j] = staged ? pat[c] : pattern_of(S, c, da, inv_sphi);
                     if (dense) {
-                        ret[j].x = a.dense[off + 4 * q + j];
+                        ret[j].x = a.dense[off + 128 * k + j];
                         w[j].x = 0u;
                     } else if (!(VEC && staged)) {
                         w[j] = staged ? mask[c] : __ldg(bands + c);
@@ -363,7 +407,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
             if ((w[0].x | w[1].x | w[2].x | w[3].x) & bit) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (w[j].x & bit) ret[j] = __ldg(vals + w[j].y + __popc(w[j].x & (bit - 1u)));
+                    if (w[j].x & bit) ret[j] = __ldg(vals + (w[j].y + __popc(w[j].x & below)));
             }
             const U4 x = additive_words((b0 >> 2) + (uint32_t)q, flo, fhi, K);
             const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
@@ -389,74 +433,76 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                 for (int j = 0; j < 4; ++j) v[j] = v[j] == -CUDART_INF_F ? most : v[j];
             }
         };
-        auto store = [&](float* to, int q, const float (&v)[4]) {
+        auto store = [&](float* to, int k, const float (&v)[4]) {   // `to`: the image at `off`
             if (VEC) {
-                *reinterpret_cast<float4*>(to + off + 4 * q) = make_float4(v[0], v[1], v[2], v[3]);
+                reinterpret_cast<float4*>(to)[32 * k] = make_float4(v[0], v[1], v[2], v[3]);
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int c = 4 * q - sh + j;
-                    if (c >= 0 && c < naz) to[off + 4 * q + j] = v[j];
+                    const int c = 4 * (lane + 32 * k) - sh + j;
+                    if (c >= 0 && c < naz) to[128 * k + j] = v[j];
                 }
             }
         };
+        float* const noised = a.noised + off;
+        float* const polar = a.polar + off;
+        const int nk = (nq - lane + 31) >> 5;   // the lane's quads
         float m = -CUDART_INF_F;
         if constexpr (REG > 0) {
             float v[REG][4];
+            float least = CUDART_INF_F;
 #pragma unroll
             for (int k = 0; k < REG; ++k) {
-                const int q = lane + 32 * k;
-                if (q < nq) {
+                if (k < nk) {
                     float p[4];
-                    quad(q, v[k], p);
-                    if (a.binned) store(a.binned, q, p);
-                    store(a.noised, q, v[k]);
-                } else {
-                    v[k][0] = v[k][1] = v[k][2] = v[k][3] = -CUDART_INF_F;
+                    quad(k, v[k], p);
+                    if (a.binned) store(a.binned + off, k, p);
+                    store(noised, k, v[k]);
+                    m = fmaxf(m, fmaxf(fmaxf(v[k][0], v[k][1]), fmaxf(v[k][2], v[k][3])));
+                    least = fminf(least, fminf(fminf(v[k][0], v[k][1]), fminf(v[k][2], v[k][3])));
                 }
             }
-#pragma unroll
-            for (int k = 0; k < REG; ++k) m = fmaxf(m, fmaxf(fmaxf(v[k][0], v[k][1]), fmaxf(v[k][2], v[k][3])));
             for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-            if (mode != 2) {
-                // the row's values are the additive term (positive) and more unless a
-                // reflectivity is negative: the general division is the exception
-                bool plain = mode == 1 && m >= 0x1p-60f && m <= 0x1p60f;
-#pragma unroll
-                for (int k = 0; k < REG; ++k) {
-                    const float least = fminf(fminf(v[k][0], v[k][1]), fminf(v[k][2], v[k][3]));
-                    plain = plain && (least >= 0x1p-100f || lane + 32 * k >= nq);
-                }
+            // the row's values are the additive term (positive) and more unless a
+            // reflectivity is negative: the general division is the exception
+            if (__all_sync(0xFFFFFFFFu, least >= 0x1p-100f && m >= 0x1p-60f && m <= 0x1p60f) && mode == 1) {
                 const float y = 1.0f / m;
 #pragma unroll
                 for (int k = 0; k < REG; ++k) {
-                    const int q = lane + 32 * k;
-                    if (q < nq) {
+                    if (k < nk) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            v[k][j] = plain ? div_by(v[k][j], m, y) : norm_value(v[k][j], m, mode);
-                        store(a.polar, q, v[k]);
+                        for (int j = 0; j < 4; ++j) v[k][j] = div_by(v[k][j], m, y);
+                        store(polar, k, v[k]);
+                    }
+                }
+            } else if (mode != 2) {
+#pragma unroll
+                for (int k = 0; k < REG; ++k) {
+                    if (k < nk) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[k][j] = norm_value(v[k][j], m, mode);
+                        store(polar, k, v[k]);
                     }
                 }
             }
         } else {
-            for (int q = lane; q < nq; q += 32) {
+            for (int k = 0; k < nk; ++k) {
                 float v[4], p[4];
-                quad(q, v, p);
-                if (a.binned) store(a.binned, q, p);
-                store(a.noised, q, v);
+                quad(k, v, p);
+                if (a.binned) store(a.binned + off, k, p);
+                store(noised, k, v);
                 m = fmaxf(m, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
             }
             for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
             if (mode != 2) {
-                for (int q = lane; q < nq; q += 32) {
+                for (int k = 0; k < nk; ++k) {
                     float v[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int c = 4 * q - sh + j;
-                        v[j] = VEC || (c >= 0 && c < naz) ? norm_value(a.noised[off + 4 * q + j], m, mode) : 0.0f;
+                        const int c = 4 * (lane + 32 * k) - sh + j;
+                        v[j] = VEC || (c >= 0 && c < naz) ? norm_value(noised[128 * k + j], m, mode) : 0.0f;
                     }
-                    store(a.polar, q, v);
+                    store(polar, k, v);
                 }
             }
         }
@@ -657,6 +703,9 @@ __device__ __forceinline__ uint4 fan_coord(const SensorDev& s, int64_t pix) {
                       __float_as_uint(col.w));
 }
 
+// The same out of line, for kernels that read a table and need it rarely.
+__device__ __noinline__ uint4 fan_coord_apart(const SensorDev& s, int64_t pix) { return fan_coord(s, pix); }
+
 // The bilinear value at q = bin (ia, ja), dn and dj bins to the next row and
 // column (explicit roundings: the table and the direct path give the same bits).
 __device__ __forceinline__ float fan_bilinear(const float* q, uint32_t dn, uint32_t dj, float wr, float wa) {
@@ -732,7 +781,7 @@ __global__ void __launch_bounds__(256) k_fan_tiles(const __grid_constant__ FanAr
 // one thread reads a pixel's table entry once and resamples that pixel for up
 // to kFanGroup frames (a frame whose geometry no longer matches the table
 // computes its own coordinates).
-__global__ void __launch_bounds__(256) k_fan_group(FanGroupArgs a) {
+__global__ void __launch_bounds__(256, 8) k_fan_group(const __grid_constant__ FanGroupArgs a) {
     __shared__ SensorDev M[kFanGroup];
     __shared__ int4 s_m;
     __shared__ int s_w, s_h;
@@ -764,11 +813,11 @@ __global__ void __launch_bounds__(256) k_fan_group(FanGroupArgs a) {
         const int v = v0 + k;
         if (v >= h) break;
         const int64_t pix = (int64_t)v * w + u;
-        const uint4 c = lut ? __ldg(lut + pix) : fan_coord(M[0], pix);
+        const uint4 c = lut ? __ldg(lut + pix) : fan_coord_apart(M[0], pix);
 #pragma unroll
         for (int q = 0; q < kFanGroup; ++q) {
             if (q < nm) {
-                const uint4 cq = M[q].fan_lut ? c : fan_coord(M[q], pix);
+                const uint4 cq = M[q].fan_lut ? c : fan_coord_apart(M[q], pix);
                 // the fan is never re-read by the step: streaming stores leave L2
                 // to the polar images and the coordinate table
                 __stcs(a.fan + M[q].fan_off + pix, fan_blend(cq, a.polar + M[q].polar_off));

@@ -24,7 +24,7 @@ struct Tune {
     int cols = 1;     // kept for saved rows: the fold takes one azimuth column per warp
     int tb = 0;       // tracing: beams per warp tile, elevations = 32 / tb (0: derive)
     int block = 128;  // adjoint: threads per block (which also sets its ray chunks)
-    int occ = 0;      // tracing variant: kTraceCap caps registers at 64 (32 one-warp blocks per SM),
+    int occ = 0;      // tracing variant: kTraceCap caps registers at 64 (32 warps per SM),
                       // kTraceWide walks the 8-wide tree
 };
 
@@ -147,43 +147,35 @@ Tune tune_for(const sonar_ctx* ctx, const sonar_sensor& s) {
     return t;
 }
 
-// The tree a ray-cast launch of `blocks` one-warp blocks walks: the 8-wide one
-// when the launch is at most one wave (32 resident blocks per SM), where a
-// ray's chain of dependent node loads sets the time, else the 4-wide one,
-// which costs fewer instructions per ray once the SMs have warps to switch to.
-int wide_for_launch(const sonar_ctx* ctx, int64_t blocks) {
-    return blocks <= 32ll * ctx->sm_count ? kTraceWide : 0;
-}
-
-// Several lanes per ray (0: one) for a launch of `blocks` 32-ray tiles, while it is a
+// Several lanes per ray (0: one) for a launch of `tiles` 32-ray tiles, while it is a
 // small part of a wave: the crossings, measured with k_trace_group, lie near 20,000
-// rays (eight lanes against four) and 100,000 rays (four against one).
-int group_lanes(const sonar_ctx* ctx, int64_t blocks) {
-    if (blocks <= 4ll * ctx->sm_count) return kTraceGroup8;
-    return blocks <= 20ll * ctx->sm_count ? kTraceGroup4 : 0;
+// rays (eight lanes against four) and 105,000 rays (four against one).
+int group_lanes(const sonar_ctx* ctx, int64_t tiles) {
+    if (tiles <= 4ll * ctx->sm_count) return kTraceGroup8;
+    return tiles <= 22ll * ctx->sm_count ? kTraceGroup4 : 0;
 }
 
-// The variant of a launch of `blocks` 32-ray tiles that no tuning row names: several
-// lanes per ray for small launches, else the tree by the launch size, and the 64-register cap (32 resident warps per
-// SM instead of 20, for a few spills) once the launch is at least two waves.
-// Uncapped / capped: 8,192 blocks (1.7 waves) 86.9 / 88.3 us, 65,536 blocks 528 /
-// 432 us, 227,072 blocks of three sensor types 1572 / 1277 us, 262,144 blocks
-// over 33.6 million triangles 2420 / 1994 us.
-int default_variant(const sonar_ctx* ctx, int64_t blocks) {
-    if (const int lanes = group_lanes(ctx, blocks)) return kTraceWide | lanes;
-    if (const int wide = wide_for_launch(ctx, blocks)) return wide;
-    return blocks >= 64ll * ctx->sm_count ? kTraceCap : 0;
+// The variant of a launch of `tiles` 32-ray tiles that no tuning row names: several
+// lanes per ray on the 8-wide tree for small launches, else a lane per ray on the
+// 4-wide one, capped at 64 registers (32 resident warps per SM instead of 28)
+// once the launch is at least two waves.  Uncapped / capped / on the 8-wide tree:
+// 4,096 tiles 56.5 / 57.6 / 62.1 us, 8,192 tiles of shorter rays 77.9 / 79.8 / 96.1
+// us, 65,536 tiles 395 / 383 / 607 us, 227,072 tiles of three sensor types 1159 /
+// 1132 / 1817 us.
+int default_variant(const sonar_ctx* ctx, int64_t tiles) {
+    if (const int lanes = group_lanes(ctx, tiles)) return kTraceWide | lanes;
+    return tiles >= 64ll * ctx->sm_count ? kTraceCap : 0;
 }
 
 // The ray-cast variant of one sensor's own launch (tile tb, variant `occ` of its
-// tuning row, if it has one): the tree by the launch size, and no
-// register cap for a launch of at most one wave, which cannot use the
-// occupancy that the cap buys.
+// tuning row, if it has one): a launch of at most one wave takes the default of
+// its size (tuning rows are made by batches), a larger one the 4-wide tree with
+// its row's cap.
 int single_variant(const sonar_ctx* ctx, const sonar_sensor& s, int tb, int occ) {
     const int64_t be = 32 / tb;
-    const int64_t blocks = ((s.n_beams + tb - 1) / tb) * ((s.n_elev + be - 1) / be);
+    const int64_t tiles = ((s.n_beams + tb - 1) / tb) * ((s.n_elev + be - 1) / be);
     const bool tuned = ctx->tune.count(ShapeKey{s.n_beams, s.n_elev, s.n_range_bins, s.n_az_bins}) != 0;
-    if (!tuned || wide_for_launch(ctx, blocks)) return default_variant(ctx, blocks);
+    if (!tuned || tiles <= 32ll * ctx->sm_count) return default_variant(ctx, tiles);
     return occ & ~kTraceWide;
 }
 

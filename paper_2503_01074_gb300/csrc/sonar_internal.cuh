@@ -50,7 +50,7 @@ struct SceneDev {
 };
 
 // SensorDev::occ, the ray-cast variant: bit kTraceCap caps registers at 64 so
-// that 32 one-warp blocks fit an SM; bit kTraceWide walks the 8-wide tree, with
+// that 32 warps fit an SM; bit kTraceWide walks the 8-wide tree, with
 // kTraceGroup8 or kTraceGroup4 by eight or four lanes per ray (chosen by the
 // launch size, never by a tuning row).
 constexpr int kTraceCap = 8;
@@ -70,7 +70,7 @@ struct SensorDev {
     int32_t scene;       // index into the scene table
     int32_t tb;          // trace: beams per warp tile (elevations = 32 / tb)
     int32_t occ;         // trace: variant bits kTraceCap, kTraceWide
-    int32_t trace_blocks;  // trace: one-warp blocks covering the sensor
+    int32_t trace_blocks;  // trace: 32-ray tiles covering the sensor
     int32_t fold_beams;  // fold: per-beam rows (several beams per column, and they fit in shared memory)
     int64_t polar_off, hits_off, fan_off, rowmax_off;
     int64_t val_off, band_off;   // fold: first value slot (a slot per ray) and first bitmap word pair
@@ -141,7 +141,18 @@ __device__ __forceinline__ U4 philox10(U4 c, const PhiloxKey& K) {
     }
     return c;
 }
-__device__ __forceinline__ U4 philox10(U4 c, uint32_t k0, uint32_t k1) { return philox10(c, philox_key(k0, k1)); }
+// With the round keys as running sums: two additions a round for twenty registers
+// less, where draws are few.
+__device__ __forceinline__ U4 philox10(U4 c, uint32_t k0, uint32_t k1) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0};
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return c;
+}
 
 // Fast division and reciprocal square root of arguments that are never
 // subnormal: the flush-to-zero forms, which skip the rescaling of subnormals
@@ -173,18 +184,21 @@ __device__ __forceinline__ float neg2log_u(uint32_t x) {
     constexpr uint32_t kRoot = 0x3F3504F4u;   // the least f
     const uint32_t bits = __float_as_uint(u) + (0x3F800000u - kRoot);
     const float f = __uint_as_float((bits & 0x007FFFFFu) + kRoot);
-    const float d = upper ? c * -0x1p-32f : f - 1.0f;   // exact
+    // powers of two are carried along rather than multiplied in at the end (they
+    // scale every rounding alike, so no bit changes): d4 = -4 d (exact), y = -4 z,
+    // y^2 = 16 z^2, the k-th coefficient over 16^k
+    const float d4 = upper ? c * 0x1p-30f : fmaf(f, -4.0f, 4.0f);
     // e in [-32, 0]: exact as a float without a conversion instruction
     const float e = __uint_as_float(0x4B000000u | (bits >> 23)) - 8388735.0f;
     const float ef = upper ? 0.0f : e;
-    const float z = div_normal(d, 2.0f + d);
-    const float z2 = z * z;
-    float p = fmaf(z2, 1.0f / 11.0f, 1.0f / 9.0f);
-    p = fmaf(z2, p, 1.0f / 7.0f);
-    p = fmaf(z2, p, 1.0f / 5.0f);
-    p = fmaf(z2, p, 1.0f / 3.0f);
-    p = fmaf(z2, p, 1.0f);
-    return -2.0f * fmaf(ef, 0.693147180559945f, 2.0f * z * p);
+    const float y = div_normal(d4, fmaf(d4, -0.25f, 2.0f));
+    const float y2 = y * y;
+    float p = fmaf(y2, 0x1p-20f * (1.0f / 11.0f), 0x1p-16f * (1.0f / 9.0f));
+    p = fmaf(y2, p, 0x1p-12f * (1.0f / 7.0f));
+    p = fmaf(y2, p, 0x1p-8f * (1.0f / 5.0f));
+    p = fmaf(y2, p, 0x1p-4f * (1.0f / 3.0f));
+    p = fmaf(y2, p, 1.0f);
+    return fmaf(ef, -2.0f * 0.693147180559945f, y * p);
 }
 
 // sqrt(v) for v = 0 or v >= 2^-32 (neg2log_u's values) from the reciprocal square root (a few ulp).
@@ -243,11 +257,11 @@ struct TraceCounters {
     uint32_t* tri_bits;             // touched triangles (bitmap)
 };
 
-// Ray casting: one-warp blocks of 32 rays.
+// Ray casting: tiles of 32 rays.
 struct TraceArgs {
     const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
     const SceneDev* scenes;     // batch: device table; single: nullptr (use `one_scene`)
-    const int4* block_map;      // batch: per block (sensor, tile of that sensor, its scene, 0)
+    const int4* block_map;      // batch: per tile (sensor, tile of that sensor, its scene, 0)
     int32_t n_sensors;
     SensorDev one;
     SceneDev one_scene;
