@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
     __shared__ SceneDev SC;
     __shared__ int s_col, s_n;
     __shared__ float s_scores[16][32];
+    let_next_start();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     if (warp == 0) {
         if (a.sensors) {
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
     const int n = (i1 - i0) * ne;                    // a sensor's rays fit 31 bits
     const sonar_hit* H = a.hits + S.hits_off + first;
     const int most = min(S.nr, n);                   // bins with returns, at most
+    wait_for_previous();   // the hit records
     if (!S.fold_beams) {
         uint32_t* bits = fold_smem + (int64_t)warp * a.words_per_warp;
         uint32_t* pre = bits + nwords;
@@ -329,6 +331,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
     extern __shared__ __align__(16) uint32_t rows_smem[];
     __shared__ SensorDev S;
     __shared__ int s_row0;
+    let_next_start();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (warp == 0) {
         // the rows run from the last sensor back to the first, so that the first
@@ -355,10 +358,12 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
     float* pat = reinterpret_cast<float*>(rows_smem);
     uint2* mask = reinterpret_cast<uint2*>(rows_smem + ((naz + 3) & ~3));
     if (staged) {
-        for (int c = tid; c < naz; c += blockDim.x) {
-            pat[c] = pattern_of(S, c, da, inv_sphi);
-            if (!dense) mask[c] = __ldg(bands + c);
-        }
+        for (int c = tid; c < naz; c += blockDim.x) pat[c] = pattern_of(S, c, da, inv_sphi);
+    }
+    wait_for_previous();   // the fold's bitmaps and values
+    if (staged) {
+        if (!dense)
+            for (int c = tid; c < naz; c += blockDim.x) mask[c] = bands[c];
         __syncthreads();
     }
     const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
@@ -582,7 +587,9 @@ __device__ __forceinline__ void norm_row(const NormArgs& a, int64_t g, int lane)
 // loads are issued before either reduction (4 KB in flight per warp); other
 // rows go one at a time (in registers up to 1024 aligned bins, else in two
 // passes).
-__global__ void __launch_bounds__(256, 4) k_norm_rows(NormArgs a) {
+__global__ void __launch_bounds__(256, 4) k_norm_rows(const __grid_constant__ NormArgs a) {
+    let_next_start();
+    wait_for_previous();
     constexpr int kV = 4;   // float4 per lane: rows of up to 512 bins
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -734,6 +741,7 @@ __device__ __forceinline__ float fan_blend(uint4 c, const float* P) {
 __global__ void __launch_bounds__(256) k_fan_tiles(const __grid_constant__ FanArgs a) {
     __shared__ SensorDev S;
     __shared__ int s_sq;
+    let_next_start();
     if (threadIdx.x < 32) {
         if (a.block_map) {
             const int2 m = __ldg(a.block_map + blockIdx.x);
@@ -755,6 +763,7 @@ __global__ void __launch_bounds__(256) k_fan_tiles(const __grid_constant__ FanAr
     float* F = a.fan + S.fan_off;
     const int um = w - 1 - u;   // the mirror pixel (u itself in the middle of an odd width)
     const float x = fan_x(g, um);
+    wait_for_previous();   // the normalised image
 #pragma unroll
     for (int k = 0; k < kTileRows; k += 256 / kTileCols) {
         const int v = v0 + k;
@@ -863,6 +872,7 @@ __global__ void __launch_bounds__(256) k_fan_lut(FanLutArgs a) {
 __global__ void k_adj_rows(const SensorDev* sensors, const int32_t* row_map, SensorDev one, int n_sensors,
                            int64_t total, int mode, const float* noised, const float* grad, RowInfo* info,
                            int32_t* zero_word) {
+    let_next_start();
     const int lane = threadIdx.x & 31;
     if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0;   // the gather's work counter
     __shared__ float s_m[32];
@@ -1000,7 +1010,7 @@ __global__ void k_adj_rows(const SensorDev* sensors, const int32_t* row_map, Sen
 // thread then in a fixed tree); k_adj_final adds the rows in a fixed order.
 // A unit holds a few hundred rays: its sums are FP32 (float-float across
 // lanes), its row of partials FP64.
-__global__ void __launch_bounds__(512) k_adjoint(AdjArgs a) {
+__global__ void __launch_bounds__(512) k_adjoint(const __grid_constant__ AdjArgs a) {
     extern __shared__ double slab_d[];   // [n_warps][n_mat] (FP32 sums; sized in doubles by the host)
     float* slab = reinterpret_cast<float*>(slab_d);
     __shared__ SensorDev S;
@@ -1008,6 +1018,7 @@ __global__ void __launch_bounds__(512) k_adjoint(AdjArgs a) {
     __shared__ AdjUnit U;
     __shared__ int s_unit;
     __shared__ ff s_ag[2][32];
+    let_next_start();
     const int tid = threadIdx.x, nt = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const int nm = a.n_mat, nq = nm + 2;
@@ -1032,14 +1043,17 @@ __global__ void __launch_bounds__(512) k_adjoint(AdjArgs a) {
             copy_words(&SC, a.scenes + un.scene, lane);
             if (lane == 0) U = un;
         }
+        if (!a.units && warp == 0) {
+            copy_param(&S, &a.one, lane);
+            copy_param(&SC, &a.one_scene, lane);
+        }
         if (!a.units && tid == 0) {
-            S = a.one;
-            SC = a.one_scene;
             U.sensor = 0;
             U.r0 = u * a.chunk;
             U.r1 = min(U.r0 + a.chunk, a.one.nb * a.one.ne);
         }
         for (int k = tid; k < nw * nm; k += nt) slab[k] = 0.0f;
+        wait_for_previous();   // the row terms
         __syncthreads();
         const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
         float acc_a = 0.0f, acc_g = 0.0f;
@@ -1116,6 +1130,7 @@ __global__ void __launch_bounds__(512) k_adjoint(AdjArgs a) {
 __global__ void __launch_bounds__(256) k_adj_final(const double* partials, int n_units, int nq, float* dtheta) {
     __shared__ double red[256];
     const int q = blockIdx.x;
+    wait_for_previous();   // the partial sums
     double v = 0.0;
     for (int u = threadIdx.x; u < n_units; u += 256) v += partials[(int64_t)u * nq + q];
     red[threadIdx.x] = v;
@@ -1139,30 +1154,23 @@ void set_kernel_attributes() {
     cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
 }
 
-cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
-    if (grid > 0) k_fold<<<grid, block, smem, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st, bool early) {
+    return grid > 0 ? launch_kernel(k_fold, grid, block, smem, st, early, a) : cudaSuccess;
 }
 
 // The row kernel for rows of up to `naz` bins: in registers up to 512 and up to
 // 1024 bins, else written and read back.  `vec`: 16-byte stores (every row of
 // every sensor starts on a 16-byte boundary of each image).
-cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st) {
+cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st, bool early) {
     if (grid <= 0) return cudaSuccess;
     // a row whose first bin is not a multiple of 4 may need one quad more
     const int reach = vec ? naz : naz + 3;
     const size_t smem = naz <= kRowsStaged ? ((size_t)((naz + 3) & ~3) + 2 * (size_t)naz) * sizeof(uint32_t) : 0;
-    if (reach <= 512 && !a.dense) {
-        if (vec) k_rows<4, true><<<grid, 256, smem, st>>>(a);
-        else k_rows<4, false><<<grid, 256, smem, st>>>(a);
-    } else if (reach <= 1024 && !a.dense) {
-        if (vec) k_rows<8, true><<<grid, 256, smem, st>>>(a);
-        else k_rows<8, false><<<grid, 256, smem, st>>>(a);
-    } else {
-        if (vec) k_rows<0, true><<<grid, 256, smem, st>>>(a);
-        else k_rows<0, false><<<grid, 256, smem, st>>>(a);
-    }
-    return cudaGetLastError();
+    if (reach <= 512 && !a.dense)
+        return launch_kernel(vec ? k_rows<4, true> : k_rows<4, false>, grid, 256, smem, st, early, a);
+    if (reach <= 1024 && !a.dense)
+        return launch_kernel(vec ? k_rows<8, true> : k_rows<8, false>, grid, 256, smem, st, early, a);
+    return launch_kernel(vec ? k_rows<0, true> : k_rows<0, false>, grid, 256, smem, st, early, a);
 }
 
 cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, void* out, cudaStream_t st) {
@@ -1172,15 +1180,13 @@ cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_norm(const NormArgs& a, cudaStream_t st) {
+cudaError_t launch_norm(const NormArgs& a, cudaStream_t st, bool early) {
     const int64_t threads = ((a.total_rows + 1) / 2) * 32;   // a warp per pair of rows
-    k_norm_rows<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(k_norm_rows, (unsigned)((threads + 255) / 256), 256, 0, st, early, a);
 }
 
-cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st) {
-    if (blocks > 0) k_fan_tiles<<<blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool early) {
+    return blocks > 0 ? launch_kernel(k_fan_tiles, blocks, 256, 0, st, early, a) : cudaSuccess;
 }
 
 cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st) {
@@ -1208,12 +1214,12 @@ cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st) {
-    k_adjoint<<<grid, block, smem, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,
+                           bool early, bool early_final) {
+    const cudaError_t e = launch_kernel(k_adjoint, grid, block, smem, st, early, a);
     if (e != cudaSuccess) return e;
-    k_adj_final<<<a.n_mat + 2, 256, 0, st>>>(a.partials, a.n_units, a.n_mat + 2, dtheta);
-    return cudaGetLastError();
+    return launch_kernel(k_adj_final, a.n_mat + 2, 256, 0, st, early_final, (const double*)a.partials, (int)a.n_units,
+                         (int)(a.n_mat + 2), dtheta);
 }
 
 int adjoint_blocks_per_sm(int block, size_t smem) {

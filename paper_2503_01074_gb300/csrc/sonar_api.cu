@@ -408,20 +408,28 @@ cudaError_t grow_trig(sonar_ctx* ctx, size_t entries, cudaStream_t s) {
 // build skips the launch (calls on a context are stream-ordered); while the
 // stream is being captured into a graph the launch is always recorded, so that
 // a replay rebuilds the tables it reads.
-cudaError_t single_trig(sonar_ctx* ctx, const SensorDev& S, cudaStream_t s) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(s, &cap);
-    if (e != cudaSuccess) return e;
-    if (cap == cudaStreamCaptureStatusNone && ctx->trig_at == S.trig && ctx->trig_nb == S.nb && ctx->trig_ne == S.ne &&
+cudaError_t single_trig(sonar_ctx* ctx, const SensorDev& S, bool capturing, cudaStream_t s) {
+    if (!capturing && ctx->trig_at == S.trig && ctx->trig_nb == S.nb && ctx->trig_ne == S.ne &&
         ctx->trig_hfov == S.hfov && ctx->trig_vfov == S.vfov)
         return cudaSuccess;
-    e = launch_trig(nullptr, S, 1, S.nb + S.ne, s);
-    const bool keep = e == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    const cudaError_t e = launch_trig(nullptr, S, 1, S.nb + S.ne, s);
+    const bool keep = e == cudaSuccess && !capturing;
     ctx->trig_at = keep ? S.trig : nullptr;
     ctx->trig_nb = S.nb;
     ctx->trig_ne = S.ne;
     ctx->trig_hfov = S.hfov;
     ctx->trig_vfov = S.vfov;
+    return e;
+}
+
+// Whether the stream is being captured into a graph.  A single-sensor call's later
+// kernels are launched early (programmatic dependent launch) only when it is not, so
+// that their setup overlaps the kernel before: 32.5 -> 28.8 us a frame of 1,024
+// rays, 51.6 -> 42.0 us one of 32,768.
+cudaError_t is_capturing(cudaStream_t s, bool* capturing) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    *capturing = cap != cudaStreamCaptureStatusNone;
     return e;
 }
 
@@ -436,9 +444,9 @@ struct FoldStore {
 // Trace, fold, noise and row normalisation of one sensor (all offsets 0).
 sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& sc, const sonar_params* p,
                             const float* d_theta, int32_t n_mat, sonar_hit* hits, const FoldStore& f, float* noised,
-                            float* binned, float* polar, uint32_t* gmax, cudaStream_t s) {
+                            float* binned, float* polar, uint32_t* gmax, bool capturing, cudaStream_t s) {
     if (p->normalise == 2) CU(cudaMemsetAsync(gmax, 0, sizeof(uint32_t), s), "cudaMemsetAsync");
-    CU(single_trig(ctx, S, s), "trig launch");
+    CU(single_trig(ctx, S, capturing, s), "trig launch");
     TraceArgs t{};
     t.one = S;
     t.one_scene = sc;
@@ -464,7 +472,9 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     if (!S.fold_beams)
         while (warps > 1 && sizeof(uint32_t) * warps * fold_words(S) > kMaxDynSmem) warps /= 2;
     const size_t smem = sizeof(uint32_t) * fold_words(S) * (S.fold_beams ? 1 : warps);
-    CU(launch_fold(a, S.fold_beams ? S.naz : (S.naz + warps - 1) / warps, 32 * warps, smem, s), "fold launch");
+    CU(launch_fold(a, S.fold_beams ? S.naz : (S.naz + warps - 1) / warps, 32 * warps, smem, s,
+                   !capturing && !f.dense),
+       "fold launch");
     RowsArgs r{};
     r.rows_per_block = rows_per_block(S.nr, ctx->sm_count);
     r.one = S;
@@ -477,13 +487,14 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     r.polar = polar;
     r.gmax = gmax;
     const bool vec = S.naz % 4 == 0 && aligned16(noised) && aligned16(polar) && aligned16(binned);
-    CU(launch_rows(r, (S.nr + r.rows_per_block - 1) / r.rows_per_block, S.naz, vec, s), "row launch");
+    CU(launch_rows(r, (S.nr + r.rows_per_block - 1) / r.rows_per_block, S.naz, vec, s, !capturing),
+       "row launch");
     return SONAR_OK;
 }
 
 // Whole-image normalisation (mode 2) and fan of one sensor (all offsets 0).
 sonar_status single_post(sonar_ctx* ctx, const SensorDev& S, int normalise, const float* noised,
-                         const uint32_t* gmax, float* polar, float* fan, cudaStream_t s) {
+                         const uint32_t* gmax, float* polar, float* fan, bool capturing, cudaStream_t s) {
     if (normalise == 2) {
         NormArgs n{};
         n.one = S;
@@ -492,14 +503,14 @@ sonar_status single_post(sonar_ctx* ctx, const SensorDev& S, int normalise, cons
         n.gmax = gmax;
         n.normalise = normalise;
         n.polar = polar;
-        CU(launch_norm(n, s), "normalisation launch");
+        CU(launch_norm(n, s, !capturing), "normalisation launch");
     }
     if (fan) {
         FanArgs f{};
         f.one = S;
         f.polar = polar;
         f.fan = fan;
-        CU(launch_fan_tiles(f, tile_squares(S.fan_w, S.fan_h), s), "fan launch");
+        CU(launch_fan_tiles(f, tile_squares(S.fan_w, S.fan_h), s, !capturing), "fan launch");
     }
     return SONAR_OK;
 }
@@ -550,10 +561,13 @@ extern "C" sonar_status sonar_render(sonar_ctx_t ctx, int32_t scene_id, const so
     CU(grow(ctx->vals, sizeof(float2) * (size_t)S.nb * S.ne, s), "scratch allocation");
     CU(grow(ctx->bands, sizeof(uint2) * (size_t)band_count(S) * S.naz, s), "scratch allocation");
     const FoldStore fold{(float2*)ctx->vals.p, (uint2*)ctx->bands.p, nullptr};
+    bool capturing = false;
+    CU(is_capturing(s, &capturing), "capture status");
     sonar_status st2 = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, fold,
-                                      noised, out->binned, out->polar, (uint32_t*)ctx->rowmax.p, s);
+                                      noised, out->binned, out->polar, (uint32_t*)ctx->rowmax.p, capturing, s);
     if (st2 != SONAR_OK) return st2;
-    return single_post(ctx, S, params->normalise, noised, (const uint32_t*)ctx->rowmax.p, out->polar, out->fan, s);
+    return single_post(ctx, S, params->normalise, noised, (const uint32_t*)ctx->rowmax.p, out->polar, out->fan, capturing,
+                       s);
 }
 
 extern "C" sonar_status sonar_fan_resample(sonar_ctx_t ctx, const sonar_sensor* sensor, const float* d_polar,
@@ -592,13 +606,15 @@ extern "C" sonar_status sonar_render_backward(sonar_ctx_t ctx, int32_t scene_id,
     SensorDev S = make_sensor(*sensor, seed, frame, t, 0, 0);
     const int groups = params->normalise == 1 ? S.nr : 1;
     CU(grow(ctx->rowinfo, sizeof(RowInfo) * groups, s), "scratch allocation");
+    bool capturing = false;
+    CU(is_capturing(s, &capturing), "capture status");
     const sonar_hit* hits = d_hits;
     if (!hits) {   // recompute the hit records with the ray-cast kernel (bitwise the forward's)
         CU(grow_trig(ctx, (size_t)(S.nb + S.ne), s), "scratch allocation");
         CU(grow(ctx->hits, sizeof(sonar_hit) * (size_t)S.nb * S.ne, s), "scratch allocation");
         S.trig = (float4*)ctx->trig.p;
         S.occ = single_variant(ctx, *sensor, S.tb, S.occ);
-        CU(single_trig(ctx, S, s), "trig launch");
+        CU(single_trig(ctx, S, capturing, s), "trig launch");
         TraceArgs tr{};
         tr.one = S;
         tr.one_scene = scene_dev(ctx->scenes[scene_id]);
@@ -632,7 +648,8 @@ extern "C" sonar_status sonar_render_backward(sonar_ctx_t ctx, int32_t scene_id,
     a.partials = (double*)ctx->partials.p;
     a.err = ctx->d_err;
     const size_t smem = sizeof(double) * (t.block / 32) * n_mat;
-    CU(launch_adjoint(a, n_units, t.block, smem, d_dtheta, s), "adjoint launch");
+    CU(launch_adjoint(a, n_units, t.block, smem, d_dtheta, s, !capturing && params->normalise != 0, !capturing),
+       "adjoint launch");
     return SONAR_OK;
 }
 
@@ -2021,8 +2038,10 @@ extern "C" sonar_status sonar_render_noalloc(sonar_ctx_t ctx, int32_t scene_id, 
     } else {
         fold.dense = out->polar;
     }
+    bool capturing = false;
+    CU(is_capturing(s, &capturing), "capture status");
     st = single_forward(ctx, S, scene_dev(ctx->scenes[scene_id]), params, d_theta, n_mat, hits, fold, noised,
-                        out->binned, out->polar, rowmax, s);
+                        out->binned, out->polar, rowmax, capturing, s);
     if (st != SONAR_OK) return st;
-    return single_post(ctx, S, params->normalise, noised, rowmax, out->polar, out->fan, s);
+    return single_post(ctx, S, params->normalise, noised, rowmax, out->polar, out->fan, capturing, s);
 }

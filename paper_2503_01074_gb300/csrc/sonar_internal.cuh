@@ -247,6 +247,13 @@ __device__ __forceinline__ void copy_param(T* dst, const T* src, int lane) {
         reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
 }
 
+// Programmatic dependent launch: a kernel launched with `early` (sonar_host.h) may
+// start once every block of the kernel before it has started and said so; it sets
+// itself up from its parameters and waits here for the whole of that kernel before
+// it touches what kernels write.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- kernel argument blocks ----
 
 struct TraceCounters {

@@ -252,6 +252,7 @@ template <int MINB, bool STATS, int W>
 __global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_constant__ TraceArgs a) {
     __shared__ SensorDev s_S[kTraceWarps];
     __shared__ SceneDev s_SC[kTraceWarps];
+    let_next_start();
     if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int tile = blockIdx.x * kTraceWarps + wid;
@@ -494,6 +495,7 @@ __global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_
     __shared__ SceneDev SC;
     __shared__ int s_tile;
     __shared__ float2 s_stack[kRays][kStackMax];        // (handle bits, entry distance)
+    let_next_start();
     if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     if (threadIdx.x < 32) {
         const int tile = blockIdx.x / kParts;
