@@ -795,6 +795,7 @@ __global__ void __launch_bounds__(256, 8) k_fan_group(const __grid_constant__ Fa
     __shared__ int4 s_m;
     __shared__ int s_w, s_h;
     __shared__ const uint4* s_lut;
+    let_next_start();
     if (threadIdx.x == 0) {
         s_m = a.block_map[blockIdx.x];
         const SensorDev& o = a.sensors[s_m.x];
@@ -810,6 +811,7 @@ __global__ void __launch_bounds__(256, 8) k_fan_group(const __grid_constant__ Fa
         reinterpret_cast<uint32_t*>(M)[i] =
             reinterpret_cast<const uint32_t*>(a.sensors + a.members[s_m.z + q])[i - q * kWords];
     }
+    wait_for_previous();   // the normalised images and the table
     __syncthreads();
     const int w = s_w, h = s_h;
     const int sx = (w + kFanSide - 1) / kFanSide;
@@ -839,7 +841,10 @@ __global__ void __launch_bounds__(256, 8) k_fan_group(const __grid_constant__ Fa
 // pixels).  A block whose stamp already holds the owner's fan_version has
 // nothing to do: the table depends on the fan geometry only, and the host bumps
 // the version whenever an update changes it.
-__global__ void __launch_bounds__(256) k_fan_lut(FanLutArgs a) {
+// The tables depend on nothing that the kernels before it in a forward write, so it
+// works first and waits last (the kernel after it waits for this one alone).
+__global__ void __launch_bounds__(256) k_fan_lut(const __grid_constant__ FanLutArgs a) {
+    let_next_start();
     __shared__ SensorDev S;
     __shared__ int s_blk;
     __shared__ uint4* s_lut;
@@ -850,7 +855,10 @@ __global__ void __launch_bounds__(256) k_fan_lut(FanLutArgs a) {
         s_lut = a.luts[m.x];
     }
     __syncthreads();
-    if (S.fan_stamp && S.fan_stamp[s_blk] == S.fan_version) return;   // block-uniform
+    if (S.fan_stamp && S.fan_stamp[s_blk] == S.fan_version) {   // block-uniform
+        wait_for_previous();
+        return;
+    }
     const int64_t base = (int64_t)s_blk * kFanTile;
     const int64_t n = (int64_t)S.fan_w * S.fan_h;
 #pragma unroll 1
@@ -860,6 +868,7 @@ __global__ void __launch_bounds__(256) k_fan_lut(FanLutArgs a) {
     }
     // the entries are read by later launches only, which see both them and the stamp
     if (threadIdx.x == 0 && S.fan_stamp) S.fan_stamp[s_blk] = S.fan_version;
+    wait_for_previous();
 }
 
 // ---------------------------------------------------------------------------
@@ -873,6 +882,7 @@ __global__ void k_adj_rows(const SensorDev* sensors, const int32_t* row_map, Sen
                            int64_t total, int mode, const float* noised, const float* grad, RowInfo* info,
                            int32_t* zero_word) {
     let_next_start();
+    wait_for_previous();
     const int lane = threadIdx.x & 31;
     if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0;   // the gather's work counter
     __shared__ float s_m[32];
@@ -1025,6 +1035,7 @@ __global__ void __launch_bounds__(512) k_adjoint(const __grid_constant__ AdjArgs
     const float alpha = __ldg(a.theta), gain = __ldg(a.theta + 1);
     const int mode = a.params.normalise;
     int next_u = 0;   // thread 0: the unit taken ahead
+    wait_for_previous();   // the row terms, the work counter
     for (int iter = 0;; ++iter) {
         int u;
         if (a.work_counter) {
@@ -1053,7 +1064,6 @@ __global__ void __launch_bounds__(512) k_adjoint(const __grid_constant__ AdjArgs
             U.r1 = min(U.r0 + a.chunk, a.one.nb * a.one.ne);
         }
         for (int k = tid; k < nw * nm; k += nt) slab[k] = 0.0f;
-        wait_for_previous();   // the row terms
         __syncthreads();
         const PhiloxKey K = philox_key(S.seed_lo, S.seed_hi);
         float acc_a = 0.0f, acc_g = 0.0f;
@@ -1189,29 +1199,21 @@ cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool
     return blocks > 0 ? launch_kernel(k_fan_tiles, blocks, 256, 0, st, early, a) : cudaSuccess;
 }
 
-cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st) {
-    if (blocks > 0) k_fan_group<<<blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st, bool early) {
+    return blocks > 0 ? launch_kernel(k_fan_group, blocks, 256, 0, st, early, a) : cudaSuccess;
 }
 
-cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st) {
-    if (blocks > 0) k_fan_lut<<<blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, bool early) {
+    return blocks > 0 ? launch_kernel(k_fan_lut, blocks, 256, 0, st, early, a) : cudaSuccess;
 }
 
 cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one, int n_sensors,
                             int64_t total_groups, int normalise, const float* noised,
-                            const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st) {
-    if (normalise == 1) {
-        const int64_t threads = total_groups * 32;
-        k_adj_rows<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(sensors, row_map, one, n_sensors,
-                                                                      total_groups, 1, noised, grad, info,
-                                                                      zero_word);
-    } else if (normalise == 2) {
-        k_adj_rows<<<(unsigned)total_groups, 1024, 0, st>>>(sensors, row_map, one, n_sensors, total_groups, 2,
-                                                            noised, grad, info, zero_word);
-    }
-    return cudaGetLastError();
+                            const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early) {
+    if (normalise == 0) return cudaSuccess;
+    const int64_t blocks = normalise == 1 ? (total_groups * 32 + 255) / 256 : total_groups;
+    return launch_kernel(k_adj_rows, (unsigned)blocks, normalise == 1 ? 256 : 1024, 0, st, early, sensors, row_map, one,
+                         n_sensors, total_groups, normalise, noised, grad, info, zero_word);
 }
 
 cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,

@@ -720,6 +720,8 @@ struct sonar_batch {
     cudaStream_t cap = nullptr;
     cudaStream_t side = nullptr;      // the adjoint branch of the combined step graph
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+    cudaStream_t mark[2] = {};        // the phase events of the forward and of the adjoint, beside the kernels
+    cudaEvent_t mark_ev = nullptr;
     cudaGraphExec_t fwd = nullptr, bwd = nullptr, step = nullptr;
     // the forward without the two table kernels (exact-ray sin/cos, fan
     // coordinates), replayed while the tables are known to be current: no
@@ -1115,6 +1117,22 @@ void append_bytes(std::vector<unsigned char>& v, const T& x) {
     v.insert(v.end(), p, p + sizeof(T));
 }
 
+// Records phase event `ev` after what stream `s` (being captured) holds so far, on
+// a branch of its own: the next kernel then follows the last one directly, and
+// may start early.
+cudaError_t mark_phase(sonar_batch* b, cudaStream_t mark, cudaEvent_t ev, cudaStream_t s) {
+    cudaError_t e = cudaEventRecord(b->mark_ev, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(mark, b->mark_ev, 0);
+    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev, mark, cudaEventRecordExternal);
+    return e;
+}
+
+// Joins the branch of phase events back into the captured stream.
+cudaError_t join_marks(sonar_batch* b, cudaStream_t mark, cudaStream_t s) {
+    const cudaError_t e = cudaEventRecord(b->mark_ev, mark);
+    return e == cudaSuccess ? cudaStreamWaitEvent(s, b->mark_ev, 0) : e;
+}
+
 // The forward's launches: part 1 up to I~ (trig tables, ray cast, fold, and the
 // row kernel, which also normalises by rows), part 2 the whole-image
 // normalisation and the fan, part 0 both.
@@ -1126,7 +1144,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         if (p->normalise == 2)
             CU(cudaMemsetAsync(b->d_rowmax, 0, sizeof(uint32_t) * b->total_rows, s), "cudaMemsetAsync");
         sonar_hit* hits = out->hits ? out->hits : b->d_hits;   // scratch allocated by the caller, outside capture
-        if (events) CU(cudaEventRecordWithFlags(b->ev[0], s, cudaEventRecordExternal), "cudaEventRecord");
+        if (events) CU(mark_phase(b, b->mark[0], b->ev[0], s), "cudaEventRecord");
         if (tables)
             CU(launch_trig(b->d_sens, SensorDev{}, (int)b->items.size(), b->max_angles, s), "batch trig launch");
         TraceArgs t{};
@@ -1137,8 +1155,8 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         t.params = *p;
         t.hits = hits;
         t.err = ctx->d_err;
-        CU(launch_trace(t, b->trace_prefix.back(), b->trace_occ, s), "batch trace launch");
-        if (events) CU(cudaEventRecordWithFlags(b->ev[6], s, cudaEventRecordExternal), "cudaEventRecord");
+        CU(launch_trace(t, b->trace_prefix.back(), b->trace_occ, s, tables), "batch trace launch");
+        if (events) CU(mark_phase(b, b->mark[0], b->ev[6], s), "cudaEventRecord");
         FoldArgs a{};
         a.sensors = b->d_sens;
         a.scenes = b->d_scenes;
@@ -1151,7 +1169,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         a.vals = b->d_vals;
         a.bands = b->d_bands;
         a.err = ctx->d_err;
-        CU(launch_fold(a, (int)b->fold_map.size(), b->fold_block, b->fold_smem, s), "batch fold launch");
+        CU(launch_fold(a, (int)b->fold_map.size(), b->fold_block, b->fold_smem, s, true), "batch fold launch");
         RowsArgs r{};
         r.sensors = b->d_sens;
         r.block_map = b->d_rows_map;
@@ -1164,8 +1182,8 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         r.polar = out->polar;
         r.gmax = b->d_rowmax;
         const bool vec = b->rows_vec && aligned16(r.noised) && aligned16(r.binned) && aligned16(r.polar);
-        CU(launch_rows(r, (int)b->rows_map.size(), b->max_naz, vec, s), "batch row launch");
-        if (events) CU(cudaEventRecordWithFlags(b->ev[1], s, cudaEventRecordExternal), "cudaEventRecord");
+        CU(launch_rows(r, (int)b->rows_map.size(), b->max_naz, vec, s, true), "batch row launch");
+        if (events) CU(mark_phase(b, b->mark[0], b->ev[1], s), "cudaEventRecord");
     }
     if (part == 1) return SONAR_OK;
     if (p->normalise == 2) {
@@ -1178,7 +1196,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         c.gmax = b->d_rowmax;
         c.normalise = p->normalise;
         c.polar = out->polar;
-        CU(launch_norm(c, s), "batch normalisation launch");
+        CU(launch_norm(c, s, true), "batch normalisation launch");
     }
     if (out->fan) {
         FanArgs f{};
@@ -1190,14 +1208,14 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         if (b->lut_blocks > 0) {
             if (tables) {
                 FanLutArgs l{b->d_sens, b->d_lut_map, b->d_luts};
-                CU(launch_fan_lut(l, b->lut_blocks, s), "batch fan table launch");
+                CU(launch_fan_lut(l, b->lut_blocks, s, true), "batch fan table launch");
             }
             FanGroupArgs g{b->d_sens, b->d_group_map, b->d_members, out->polar, out->fan};
-            CU(launch_fan_group(g, b->group_blocks, s), "batch grouped fan launch");
+            CU(launch_fan_group(g, b->group_blocks, s, true), "batch grouped fan launch");
         }
-        CU(launch_fan_tiles(f, b->fan_blocks, s), "batch fan launch");
+        CU(launch_fan_tiles(f, b->fan_blocks, s, true), "batch fan launch");
     }
-    if (events) CU(cudaEventRecordWithFlags(b->ev[2], s, cudaEventRecordExternal), "cudaEventRecord");
+    if (events) CU(mark_phase(b, b->mark[0], b->ev[2], s), "cudaEventRecord");
     return SONAR_OK;
 }
 
@@ -1223,6 +1241,9 @@ extern "C" sonar_status sonar_batch_create(sonar_ctx_t ctx, const sonar_batch_it
     }
     if (st == SONAR_OK && e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (st == SONAR_OK && e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+    for (int k = 0; k < 2 && st == SONAR_OK && e == cudaSuccess; ++k)
+        e = cudaStreamCreateWithFlags(&b->mark[k], cudaStreamNonBlocking);
+    if (st == SONAR_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&b->mark_ev, cudaEventDisableTiming);
     if (st == SONAR_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming);
     if (st == SONAR_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join_ev, cudaEventDisableTiming);
     for (int k = 0; k < 7 && st == SONAR_OK && e == cudaSuccess; ++k) e = cudaEventCreate(&b->ev[k]);
@@ -1347,8 +1368,10 @@ extern "C" sonar_status sonar_render_batch(sonar_batch_t b, const sonar_params* 
         exec = nullptr;
         CU(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "graph capture");
         st = batch_forward_launches(b, p, d_theta, n_mat, out, b->cap, true, 0, !lean);
+        const cudaError_t ej = join_marks(b, b->mark[0], b->cap);
         cudaGraph_t g = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+        cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+        if (e == cudaSuccess) e = ej;
         if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
         CU(e, "graph capture");
         (lean ? b->fwd_lean_kernels : b->fwd_kernels) = kernel_nodes(g);
@@ -1372,11 +1395,12 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
                                      const float* grad, const float* noised, const sonar_hit* hits, float* dtheta,
                                      cudaStream_t s, bool events = false) {
     sonar_ctx* ctx = b->ctx;
+    bool cast = false;   // a kernel of this call precedes the row terms
     // the gather's work counter is cleared by a kernel before it (the ray cast
     // of recomputed records, the row terms), else by a memset
     if (hits && p->normalise == 0)
         CU(cudaMemsetAsync(b->d_counters + 1, 0, sizeof(int32_t), s), "cudaMemsetAsync");
-    if (events) CU(cudaEventRecordWithFlags(b->ev[3], s, cudaEventRecordExternal), "cudaEventRecord");
+    if (events) CU(mark_phase(b, b->mark[1], b->ev[3], s), "cudaEventRecord");
     if (!hits) {   // recompute the hit records with the ray-cast kernel into the batch scratch
         CU(launch_trig(b->d_sens, SensorDev{}, (int)b->items.size(), b->max_angles, s), "batch trig launch");
         TraceArgs tr{};
@@ -1388,15 +1412,16 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
         tr.hits = b->d_hits;
         tr.err = ctx->d_err;
         tr.zero_word = b->d_counters + 1;
-        CU(launch_trace(tr, b->trace_prefix.back(), b->trace_occ, s), "batch trace launch");
+        CU(launch_trace(tr, b->trace_prefix.back(), b->trace_occ, s, true), "batch trace launch");
         hits = b->d_hits;
+        cast = true;
     }
     if (p->normalise != 0)
         CU(launch_adj_rows(b->d_sens, b->d_row_map, SensorDev{}, (int)b->items.size(),
                            p->normalise == 1 ? b->total_rows : (int64_t)b->items.size(), p->normalise, noised,
-                           grad, b->d_rowinfo, b->d_counters + 1, s),
+                           grad, b->d_rowinfo, b->d_counters + 1, s, cast),
            "batch adjoint rows");
-    if (events) CU(cudaEventRecordWithFlags(b->ev[4], s, cudaEventRecordExternal), "cudaEventRecord");
+    if (events) CU(mark_phase(b, b->mark[1], b->ev[4], s), "cudaEventRecord");
     AdjArgs a{};
     a.sensors = b->d_sens;
     a.units = b->d_adj_units;
@@ -1416,8 +1441,8 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
     const int per_sm = adjoint_blocks_per_sm(b->block, smem);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)b->adj_units.size(),
                                                                     (int64_t)ctx->sm_count * per_sm));
-    CU(launch_adjoint(a, grid, b->block, smem, dtheta, s), "batch adjoint launch");
-    if (events) CU(cudaEventRecordWithFlags(b->ev[5], s, cudaEventRecordExternal), "cudaEventRecord");
+    CU(launch_adjoint(a, grid, b->block, smem, dtheta, s, cast || p->normalise != 0, true), "batch adjoint launch");
+    if (events) CU(mark_phase(b, b->mark[1], b->ev[5], s), "cudaEventRecord");
     return SONAR_OK;
 }
 
@@ -1458,8 +1483,10 @@ extern "C" sonar_status sonar_render_batch_backward(sonar_batch_t b, const sonar
         b->bwd = nullptr;
         CU(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "graph capture");
         st = batch_backward_launches(b, p, d_theta, n_mat, d_grad, d_noised, d_hits, d_dtheta, b->cap, true);
+        const cudaError_t ej = join_marks(b, b->mark[1], b->cap);
         cudaGraph_t g = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+        cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+        if (e == cudaSuccess) e = ej;
         if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
         CU(e, "graph capture");
         b->bwd_kernels = kernel_nodes(g);
@@ -1529,16 +1556,20 @@ extern "C" sonar_status sonar_render_batch_step(sonar_batch_t b, const sonar_par
             const cudaError_t e1 = cudaEventRecord(b->join_ev, b->side);
             const cudaError_t e2 = e1 == cudaSuccess ? cudaStreamWaitEvent(b->cap, b->join_ev, 0) : e1;
             if (e == cudaSuccess) e = e2;
+            const cudaError_t e4 = join_marks(b, b->mark[1], b->cap);
+            if (e == cudaSuccess) e = e4;
         }
+        const cudaError_t e5 = join_marks(b, b->mark[0], b->cap);
+        if (e == cudaSuccess) e = e5;
         cudaGraph_t g = nullptr;
         const cudaError_t e3 = cudaStreamEndCapture(b->cap, &g);
         if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
         if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(ctx, e, "graph fork"); }
         CU(e3, "graph capture");
         b->step_kernels = kernel_nodes(g);
-        const cudaError_t e4 = cudaGraphInstantiate(&b->step, g, 0);
+        const cudaError_t e6 = cudaGraphInstantiate(&b->step, g, 0);
         cudaGraphDestroy(g);
-        CU(e4, "graph instantiation");
+        CU(e6, "graph instantiation");
         b->step_key = key;
         ++b->graphs;
     }
@@ -1599,6 +1630,9 @@ extern "C" sonar_status sonar_batch_destroy(sonar_batch_t b) {
     }
     if (b->cap) cudaStreamDestroy(b->cap);
     if (b->side) cudaStreamDestroy(b->side);
+    for (cudaStream_t& m : b->mark)
+        if (m) cudaStreamDestroy(m);
+    if (b->mark_ev) cudaEventDestroy(b->mark_ev);
     if (b->fork_ev) cudaEventDestroy(b->fork_ev);
     if (b->join_ev) cudaEventDestroy(b->join_ev);
     delete b;

@@ -54,20 +54,20 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
 }
 cudaError_t launch_trig(const SensorDev* sensors, const SensorDev& one, int n_sensors, int max_angles,
                         cudaStream_t st);
-cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStream_t st);
+cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStream_t st, bool early = false);
 // `early`: the launch may overlap the end of the launch before it on the stream, which
-// must be a kernel (a single-sensor call's own; not while capturing).
+// must be one of these kernels (see wait_for_previous).
 cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st, bool early = false);
 cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st, bool early = false);
 constexpr size_t kMaxDynSmem = 220 * 1024;   // of the 227 KB a block may have, less the static part
 cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, void* out, cudaStream_t st);
 cudaError_t launch_norm(const NormArgs& a, cudaStream_t st, bool early = false);
 cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool early = false);
-cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st);
-cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st);
+cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, bool early = false);
+cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st, bool early = false);
 cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one, int n_sensors,
                             int64_t total_groups, int normalise, const float* noised,
-                            const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st);
+                            const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early = false);
 // `early` for the gather, and `early_final` for the final sum after it.
 cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,
                            bool early = false, bool early_final = false);

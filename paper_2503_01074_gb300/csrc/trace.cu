@@ -160,6 +160,7 @@ __device__ __noinline__ ExactPair exact_pair(const SensorDev& s, const float4* t
 // (computed in FP64 once per sensor, split into hi + lo floats): trig[i] for
 // beams, trig[N_b + j] for elevations, each (sin hi, sin lo, cos hi, cos lo).
 __global__ void k_trig(const SensorDev* sensors, SensorDev one) {
+    let_next_start();
     const SensorDev& s = sensors ? sensors[blockIdx.y] : one;
     // a batch block whose entries were built for the sensor's current fields of
     // view has nothing to do (block-uniform; only later launches read the table)
@@ -253,7 +254,6 @@ __global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_c
     __shared__ SensorDev s_S[kTraceWarps];
     __shared__ SceneDev s_SC[kTraceWarps];
     let_next_start();
-    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int tile = blockIdx.x * kTraceWarps + wid;
     if (tile >= a.n_tiles) return;
@@ -272,6 +272,8 @@ __global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_c
         if (a.from_last) tile = a.n_tiles - 1 - tile;
     }
     __syncwarp();
+    wait_for_previous();   // the exact-ray tables
+    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     const int tb = S.tb, te = 32 / S.tb;
     const int tiles_b = (S.nb + tb - 1) / tb;
     const int ty = tile / tiles_b, tx = tile - ty * tiles_b;
@@ -496,7 +498,6 @@ __global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_
     __shared__ int s_tile;
     __shared__ float2 s_stack[kRays][kStackMax];        // (handle bits, entry distance)
     let_next_start();
-    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     if (threadIdx.x < 32) {
         const int tile = blockIdx.x / kParts;
         if (a.sensors) {
@@ -510,6 +511,8 @@ __global__ void __launch_bounds__(kGroupThreads, 12) k_trace_group(const __grid_
             if (threadIdx.x == 0) s_tile = a.from_last ? a.one.trace_blocks - 1 - tile : tile;
         }
     }
+    wait_for_previous();   // the exact-ray tables
+    if (a.zero_word && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_word = 0;   // read by a later launch only
     __syncthreads();
     const int tb = S.tb, te = 32 / tb, tiles_b = (S.nb + tb - 1) / tb;
     const int ty = s_tile / tiles_b, tx = s_tile - ty * tiles_b;
@@ -741,30 +744,21 @@ cudaError_t launch_trig(const SensorDev* sensors, const SensorDev& one, int n_se
     return cudaGetLastError();
 }
 
-cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStream_t st) {
-    if (blocks > 0) {
-        const bool cap = occupancy & kTraceCap;
-        // one sensor's launch on a scene without an 8-wide tree walks the 4-wide
-        // one (a batch's variant is checked against all its scenes on the host)
-        const bool wide = (occupancy & kTraceWide) && (a.sensors || a.one_scene.nodes8);
-        if (wide && (occupancy & kTraceGroup8)) {
-            k_trace_group<8><<<(unsigned)blocks * (32 * 8 / kGroupThreads), kGroupThreads, 0, st>>>(a);
-        } else if (wide && (occupancy & kTraceGroup4)) {
-            k_trace_group<4><<<(unsigned)blocks * (32 * 4 / kGroupThreads), kGroupThreads, 0, st>>>(a);
-        } else {
-            const unsigned grid = (unsigned)((blocks + kTraceWarps - 1) / kTraceWarps);
-            TraceArgs b = a;
-            b.n_tiles = blocks;
-            if (wide) {
-                if (cap) k_trace<16, false, 8><<<grid, 32 * kTraceWarps, 0, st>>>(b);
-                else k_trace<4, false, 8><<<grid, 32 * kTraceWarps, 0, st>>>(b);
-            } else {
-                if (cap) k_trace<16, false, 4><<<grid, 32 * kTraceWarps, 0, st>>>(b);
-                else k_trace<4, false, 4><<<grid, 32 * kTraceWarps, 0, st>>>(b);
-            }
-        }
-    }
-    return cudaGetLastError();
+cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStream_t st, bool early) {
+    if (blocks <= 0) return cudaSuccess;
+    const bool cap = occupancy & kTraceCap;
+    // one sensor's launch on a scene without an 8-wide tree walks the 4-wide
+    // one (a batch's variant is checked against all its scenes on the host)
+    const bool wide = (occupancy & kTraceWide) && (a.sensors || a.one_scene.nodes8);
+    if (wide && (occupancy & kTraceGroup8))
+        return launch_kernel(k_trace_group<8>, (unsigned)blocks * (32 * 8 / kGroupThreads), kGroupThreads, 0, st, early, a);
+    if (wide && (occupancy & kTraceGroup4))
+        return launch_kernel(k_trace_group<4>, (unsigned)blocks * (32 * 4 / kGroupThreads), kGroupThreads, 0, st, early, a);
+    TraceArgs b = a;
+    b.n_tiles = blocks;
+    return launch_kernel(wide ? (cap ? k_trace<16, false, 8> : k_trace<4, false, 8>)
+                              : (cap ? k_trace<16, false, 4> : k_trace<4, false, 4>),
+                         (unsigned)((blocks + kTraceWarps - 1) / kTraceWarps), 32 * kTraceWarps, 0, st, early, b);
 }
 
 cudaError_t launch_stats(const SensorDev& s, const SceneDev& sc, const sonar_params& p,
