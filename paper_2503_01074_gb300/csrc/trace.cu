@@ -245,7 +245,8 @@ __device__ __forceinline__ uint4 record_of(const SensorDev& S, const SceneDev& s
 // with handles selected by the bits of their slot and no count of entered
 // children; 393 / 1163 / 1838 with a bottom stack entry instead of an empty test
 // and two tiles a block (the block limit is 32 per SM, and two warps share the
-// slot of one); 383 / 1132 / 1791 with boxes as centre and half-width.
+// slot of one); 383 / 1132 / 1791 with boxes as centre and half-width; 360 / 998 /
+// 1686 on a hierarchy over the triangles' box centres.
 // With STATS the kernel also counts node visits and triangle tests and marks
 // the nodes and triangles it touches (records are then not written).
 constexpr int kTraceWarps = 2;   // tiles per block, each a warp's own
@@ -484,7 +485,9 @@ __global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_c
 // lane a ray -> four -> eight lanes: 1,024 rays over a plane and a sphere 29.6 ->
 // 17.9 -> 17.1 us; 8,192 rays over a seabed 40.4 -> 22.2 -> 21.0; 16,403 rays to
 // 27 m 140 -> 55 -> 42; 32,768 rays 42.7 -> 29.1 -> 34.5; 65,536 rays (two frames)
-// 57.2 -> 41.6 -> 53.2; 131,072 rays 61.2 -> 71.1 -> 96.5.
+// 57.2 -> 41.6 -> 53.2; 131,072 rays 61.2 -> 71.1 -> 96.5 (all on a hierarchy over
+// centroids; over box centres the first three are 15.0 by eight lanes, 18.8 by four
+// and 37.0 by eight).
 constexpr int kGroupThreads = 64;       // threads per block
 
 template <int G>
