@@ -486,8 +486,7 @@ __global__ void __launch_bounds__(32 * kTraceWarps, MINB) k_trace(const __grid_c
 // 17.9 -> 17.1 us; 8,192 rays over a seabed 40.4 -> 22.2 -> 21.0; 16,403 rays to
 // 27 m 140 -> 55 -> 42; 32,768 rays 42.7 -> 29.1 -> 34.5; 65,536 rays (two frames)
 // 57.2 -> 41.6 -> 53.2; 131,072 rays 61.2 -> 71.1 -> 96.5 (all on a hierarchy over
-// centroids; over box centres the first three are 15.0 by eight lanes, 18.8 by four
-// and 37.0 by eight).
+// centroids; over box centres the first three are 15.0, 18.8 and 37.0 as launched).
 constexpr int kGroupThreads = 64;       // threads per block
 
 template <int G>
