@@ -789,12 +789,15 @@ __global__ void __launch_bounds__(256) k_fan_tiles(const __grid_constant__ FanAr
 // The fan of the frames that share one coordinate table, in the same squares:
 // one thread reads a pixel's table entry once and resamples that pixel for up
 // to kFanGroup frames (a frame whose geometry no longer matches the table
-// computes its own coordinates).  Waits for the table (16 bytes a pixel, read once
-// from HBM) and then for the frames' rows, so the entry of a thread's next row is
-// asked for before this row's frames; it has the registers for that at six blocks an
-// SM.  64 frames of 1024 x 576: 131 us with eight blocks and no entry ahead, now 126
-// (22 % of it are the 151 MB written); 32 frames of 512 x 288 are the same either way.
-__global__ void __launch_bounds__(256, 6) k_fan_group(const __grid_constant__ FanGroupArgs a) {
+// computes its own coordinates).  Bound by the latency of the table (16 bytes a
+// pixel, read once from HBM) and of the frames' rows behind it: a thread takes two
+// rows of two frames at a time, sixteen gathers in flight, and has asked for its next
+// two table entries before.  That takes 64 registers, four blocks an SM, and is
+// faster than more blocks with fewer gathers each (one pixel of one frame at a time,
+// eight blocks -> this): 64 frames of 1024 x 576 131 -> 110 us (151 MB written, 131 MB
+// read), 32 frames of 512 x 288 24 -> 14.  Four rows, four frames or squares of 32
+// are slower by 5 to 30 %.
+__global__ void __launch_bounds__(256, 4) k_fan_group(const __grid_constant__ FanGroupArgs a) {
     __shared__ SensorDev M[kFanGroup];
     __shared__ int4 s_m;
     __shared__ int s_w, s_h;
@@ -823,25 +826,66 @@ __global__ void __launch_bounds__(256, 6) k_fan_group(const __grid_constant__ Fa
     const int v0 = (s_m.y / sx) * kFanSide + (threadIdx.x / kFanSide);
     if (u >= w) return;
     const uint4* lut = s_lut;
-    constexpr int kStep = 256 / kFanSide;
-    uint4 ahead = make_uint4(0u, 0u, 0u, 0u);   // the table entry of the next row, on its way during this one
-    if (lut && v0 < h) ahead = __ldg(lut + (int64_t)v0 * w + u);
-#pragma unroll 1
-    for (int k = 0; k < kFanSide; k += kStep) {
-        const int v = v0 + k;
-        if (v >= h) break;
-        const int64_t pix = (int64_t)v * w + u;
-        const uint4 c = lut ? ahead : fan_coord_apart(M[0], pix);
-        if (lut && v + kStep < h) ahead = __ldg(lut + pix + (int64_t)kStep * w);
+    constexpr int kStep = 256 / kFanSide, kRows = 2;
+    bool shared = lut != nullptr;   // every frame here goes by the table
+    const float* P[kFanGroup];
+    float* F[kFanGroup];
 #pragma unroll
-        for (int q = 0; q < kFanGroup; ++q) {
-            if (q < nm) {
-                const uint4 cq = M[q].fan_lut ? c : fan_coord_apart(M[q], pix);
-                // the fan is never re-read by the step: streaming stores leave L2
-                // to the polar images and the coordinate table
-                __stcs(a.fan + M[q].fan_off + pix, fan_blend(cq, a.polar + M[q].polar_off));
+    for (int q = 0; q < kFanGroup; ++q) {
+        const SensorDev& m = M[q < nm ? q : 0];
+        shared = shared && m.fan_lut != nullptr;
+        P[q] = a.polar + m.polar_off;
+        F[q] = a.fan + m.fan_off;
+    }
+    // the fan is never re-read by the step: streaming stores leave L2 to the polar
+    // images and the coordinate table
+    if (!shared) {
+#pragma unroll 1
+        for (int v = v0; v < min(v0 + kFanSide, h); v += kStep) {
+            const int64_t pix = (int64_t)v * w + u;
+            for (int q = 0; q < nm; ++q) {
+                const uint4 c = lut && M[q].fan_lut ? __ldg(lut + pix) : fan_coord_apart(M[q], pix);
+                __stcs(a.fan + M[q].fan_off + pix, fan_blend(c, a.polar + M[q].polar_off));
             }
         }
+        return;
+    }
+    const uint4 outside = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+    uint4 ahead[kRows];   // the table's entries of the next rows, on their way during these
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+        ahead[r] = v0 + r * kStep < h ? __ldg(lut + (int64_t)(v0 + r * kStep) * w + u) : outside;
+#pragma unroll 1
+    for (int k = 0; k < kFanSide; k += kRows * kStep) {
+        const int v = v0 + k;
+        if (v >= h) break;
+        const int64_t pix = (int64_t)v * w + u, step = (int64_t)kStep * w;
+        uint4 c[kRows];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            c[r] = ahead[r];
+            ahead[r] = v + (r + kRows) * kStep < h ? __ldg(lut + pix + (r + kRows) * step) : outside;
+        }
+        // every gather before the first store: the compiler must not move a load
+        // above a store that might alias it
+        float value[kRows][kFanGroup];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            const bool in = c[r].x != 0xFFFFFFFFu;   // else the image's first bin is read and dropped
+            const uint32_t at = in ? c[r].x : 0u, dn = c[r].y >> 1, dj = c[r].y & 1u;
+#pragma unroll
+            for (int q = 0; q < kFanGroup; ++q) {
+                const float x = fan_bilinear(P[q] + at, dn, dj, __uint_as_float(c[r].z), __uint_as_float(c[r].w));
+                value[r][q] = in ? x : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+            if (v + r * kStep < h) {
+#pragma unroll
+                for (int q = 0; q < kFanGroup; ++q)
+                    if (q < nm) __stcs(F[q] + pix + r * step, value[r][q]);
+            }
     }
 }
 
