@@ -737,8 +737,10 @@ __device__ __forceinline__ float fan_blend(uint4 c, const float* P) {
 // A pixel out of range needs no bearing.
 // Bound by issue: 128 fans of unlike geometry (132 million pixels) 790 -> 428 us
 // against a pixel per coordinate computation (and two integer divisions more),
-// one 1024 x 576 fan 9.1 -> 6.7 us.
-__global__ void __launch_bounds__(256) k_fan_tiles(const __grid_constant__ FanArgs a) {
+// 397 with all 64 warps of an SM (32 registers instead of 40; both rows' gathers
+// before the first store, which takes more of them: 407); one 1024 x 576 fan 9.1 ->
+// 6.7 us.
+__global__ void __launch_bounds__(256, 8) k_fan_tiles(const __grid_constant__ FanArgs a) {
     __shared__ SensorDev S;
     __shared__ int s_sq;
     let_next_start();
