@@ -720,8 +720,8 @@ def run_ours(args):
     e2e = None
     # algorithmic bytes per frame (the per-kernel figures of the design notes):
     # the ray cast reads the nodes (128 B 4-wide, 256 B 8-wide) and triangles
-    # (48 B) its rays touch and writes a 16-byte record per ray; binning reads the records and
-    # writes I~; the normalisation + fan reads I~, writes N and the fan image
+    # (48 B) its rays touch and writes a 16-byte record per ray; the fold reads the records and
+    # the row kernel writes I~ and N; the fan reads N, writes the fan image
     # and reads the shared coordinate table (16 B a pixel, once per launch);
     # the adjoint reads I~ and G per bin, the records and a G gather per ray
     alg = 0
@@ -733,8 +733,8 @@ def run_ours(args):
         tests += st["tests"]
         exact += st["exact_tests"]
     nbin, npx, nray = base.n_range_bins * base.n_az_bins, base.fan_w * base.fan_h, base.n_rays
-    bytes_frame = {"trace": alg / B, "bin_noise": nray * 16 + nbin * 4,
-                   "normalise_fan": nbin * 8 + npx * 4 + npx * 16 / B,
+    bytes_frame = {"trace": alg / B, "bin_noise": nray * 16 + nbin * 8,
+                   "normalise_fan": nbin * 4 + npx * 4 + npx * 16 / B,
                    "adjoint_rows": nbin * 8, "adjoint_gather": nray * 20}
     fwd_bytes = bytes_frame["trace"] + bytes_frame["bin_noise"] + bytes_frame["normalise_fan"]
     adj_bytes = bytes_frame["adjoint_rows"] + bytes_frame["adjoint_gather"]
@@ -1019,8 +1019,8 @@ def run_ours(args):
                 "kernel": "k_trace (ray generation + LBVH walk + Moller-Trumbore + bin key)",
                 "avg_launch_ms": trace_ms, "algorithmic_bytes_per_launch": int(alg),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback"}
-    # the binning kernel streams hit records in and I~ out: its own figure
-    bin_bytes = B * (base.n_rays * 16 + base.n_range_bins * base.n_az_bins * 4)
+    # the fold and row kernels stream hit records in, I~ and N out: their own figure
+    bin_bytes = B * (base.n_rays * 16 + base.n_range_bins * base.n_az_bins * 8)
     extras["bin_noise_GBps"] = bin_bytes / (bin_ms / 1000.0) / 1e9
     extras["node4_visits_per_ray"] = visits / (B * base.n_rays)
     extras["tri_tests_per_ray"] = tests / (B * base.n_rays)

@@ -73,7 +73,7 @@ __device__ __forceinline__ float3 load_v(const float* v, int32_t i) {
 // lie a third of a cell apart, which paired triangles of different cells.  Ray cast
 // of 64 frames of 32,768 rays by centroids -> by box centres 383 -> 360 us, of 32
 // frames of 8,192 rays 79 -> 66, of 7.3 million rays of three sensor types 1132 ->
-// 998, of 16 frames of 262,144 rays over 33.6 million triangles 1791 -> 1686.
+// 998, of 32 frames of 262,144 rays over 33.6 million triangles 1791 -> 1686.
 __device__ __forceinline__ float3 box_centre(float3 p, float3 q, float3 r) {
     return make_float3(0.5f * fminf(p.x, fminf(q.x, r.x)) + 0.5f * fmaxf(p.x, fmaxf(q.x, r.x)),
                        0.5f * fminf(p.y, fminf(q.y, r.y)) + 0.5f * fmaxf(p.y, fmaxf(q.y, r.y)),

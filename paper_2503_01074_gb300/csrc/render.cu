@@ -8,8 +8,8 @@
 //                     maximum and N = I~ / max; writes I~ and N, reads neither.
 // k_norm_rows         whole-image normalisation only: N = I~ / max.
 // k_fan_*             fan resample of the normalised image: per-pixel polar
-//                     coordinate tables, then bilinear gathers for up to 8
-//                     frames per table read.
+//                     coordinate tables, then bilinear gathers for two frames
+//                     per table read.
 // adjoint             per-group (row) Jacobian terms, then a per-ray gather of
 //                     dL/dP into (dalpha, dgain, dmu) over ray chunks, and a
 //                     fixed-order final reduction (deterministic).

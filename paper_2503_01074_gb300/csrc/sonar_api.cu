@@ -159,9 +159,9 @@ int group_lanes(const sonar_ctx* ctx, int64_t tiles) {
 // lanes per ray on the 8-wide tree for small launches, else a lane per ray on the
 // 4-wide one, capped at 64 registers (32 resident warps per SM instead of 28)
 // once the launch is at least two waves.  Uncapped / capped / on the 8-wide tree:
-// 4,096 tiles 56.5 / 57.6 / 62.1 us, 8,192 tiles of shorter rays 77.9 / 79.8 / 96.1
-// us, 65,536 tiles 395 / 383 / 607 us, 227,072 tiles of three sensor types 1159 /
-// 1132 / 1817 us.
+// 4,096 tiles 56.1 / 56.4 / 59.8 us, 8,192 tiles of shorter rays 63.8 / 66.1 / 80.4
+// us, 65,536 tiles 372 / 362 / 573 us, 227,072 tiles of three sensor types 1027 /
+// 999 / 1625 us.
 int default_variant(const sonar_ctx* ctx, int64_t tiles) {
     if (const int lanes = group_lanes(ctx, tiles)) return kTraceWide | lanes;
     return tiles >= 64ll * ctx->sm_count ? kTraceCap : 0;
