@@ -930,81 +930,88 @@ __global__ void __launch_bounds__(256) k_fan_lut(const __grid_constant__ FanLutA
 // ---------------------------------------------------------------------------
 
 // Group terms of the normalisation Jacobian: m, argmax (lowest index on
-// ties) and c = sum G I~ / m^2.  Mode 1: one warp per range row; mode 2: one
-// block per sensor image.
-__global__ void k_adj_rows(const SensorDev* sensors, const int32_t* row_map, SensorDev one, int n_sensors,
-                           int64_t total, int mode, const float* noised, const float* grad, RowInfo* info,
-                           int32_t* zero_word) {
+// ties) and c = sum G I~ / m^2, one warp per range row, or per `per_warp` of them
+// one after another.
+// Bound by HBM, and by what a warp waits for between rows: the place of its row (two
+// dependent loads), its bins, the reduction.  So every load of up to 512 bins is
+// issued before the first compare, and what follows (the row's next 512 bins, the
+// next row) is asked for before the reduction.  128,000 rows of 1024 bins 192 -> 157
+// us (6.7 TB/s), 64,000 rows of 512 bins 55 -> 53 (57 with a row per warp); more
+// warps of fewer registers spill.
+__global__ void __launch_bounds__(256, 4) k_adj_rows(const SensorDev* sensors, const int32_t* row_map, SensorDev one,
+                                                  int64_t total, int per_warp, const float* noised, const float* grad,
+                                                  RowInfo* info, int32_t* zero_word) {
     let_next_start();
     wait_for_previous();
     const int lane = threadIdx.x & 31;
     if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0;   // the gather's work counter
-    __shared__ float s_m[32];
-    __shared__ int s_a[32];
-    __shared__ ff s_d[32];
-    if (mode == 1) {
-        const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        if (g >= total) return;
-        const SensorDev& s = sensors ? sensors[row_map[g]] : one;
-        const int row = (int)(g - s.rowmax_off);
-        const float* In = noised + s.polar_off + (int64_t)row * s.naz;
-        const float* G = grad + s.polar_off + (int64_t)row * s.naz;
+    const int64_t g0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+    float4 xs[4], ys[4];   // 512 bins of I~ and G, each lane's vectors
+    int naz = 0, row = 0;
+    int64_t off = 0;
+    bool vec = false;
+    auto place = [&](int64_t g) {
+        const SensorDev& s = sensors ? sensors[__ldg(row_map + g)] : one;
+        naz = s.naz;
+        row = (int)(g - s.rowmax_off);
+        off = s.polar_off + (int64_t)row * naz;
+        vec = ((s.polar_off | naz) & 3) == 0;
+    };
+    auto ask = [&](int j0) {   // bins j0 .. j0 + 511 of the row
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = j0 + 4 * (lane + 32 * k);
+            if (j < naz) {   // I~ is not read again by the adjoint: evict first, keep G in L2
+                xs[k] = __ldcs(reinterpret_cast<const float4*>(noised + off + j));
+                ys[k] = __ldg(reinterpret_cast<const float4*>(grad + off + j));
+            }
+        }
+    };
+    if (g0 < total) {
+        place(g0);
+        if (vec) ask(0);
+    }
+    for (int64_t g = g0; g < g0 + per_warp && g < total; ++g) {
+        const bool more = g + 1 < g0 + per_warp && g + 1 < total;
+        const int base = row * naz;
         float m = -CUDART_INF_F;
         int am = 0x7FFFFFFF;
         float dl = 0.0f;                      // per-lane partial of sum G I~ (few terms)
-        if (((s.polar_off | s.naz) & 3) == 0 && s.naz <= 512) {
-            // 16-byte rows of up to 512 bins: every load of the row (I~ and G) is
-            // issued before the first compare, then each lane takes its 4
-            // consecutive bins per vector in index order
-            const float4* In4 = reinterpret_cast<const float4*>(In);
-            const float4* G4 = reinterpret_cast<const float4*>(G);
-            const int n4 = s.naz >> 2;
-            float4 xs[4], ys[4];
+        if (vec) {
+            // what follows is asked for as soon as these bins are taken: the row's
+            // next 512, or the next row, on its way during the reduction
+#pragma unroll 1
+            for (int j0 = 0, n = naz; j0 < n; j0 += 512) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int q = lane + 32 * k;
-                if (q < n4) {
-                    xs[k] = __ldcs(In4 + q);   // I~ is not read again by the adjoint: evict first, keep G in L2
-                    ys[k] = __ldg(G4 + q);
+                for (int k = 0; k < 4; ++k) {
+                    const int j = j0 + 4 * (lane + 32 * k);
+                    if (j >= n) continue;
+                    const float4 x = xs[k], y = ys[k];   // four consecutive bins, in index order
+                    if (x.x > m) { m = x.x; am = j; }
+                    if (x.y > m) { m = x.y; am = j + 1; }
+                    if (x.z > m) { m = x.z; am = j + 2; }
+                    if (x.w > m) { m = x.w; am = j + 3; }
+                    dl = fmaf(y.x, x.x, dl);
+                    dl = fmaf(y.y, x.y, dl);
+                    dl = fmaf(y.z, x.z, dl);
+                    dl = fmaf(y.w, x.w, dl);
+                }
+                if (j0 + 512 < n) {
+                    ask(j0 + 512);
+                } else if (more) {
+                    place(g + 1);
+                    if (vec) ask(0);
                 }
             }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int q = lane + 32 * k;
-                if (q >= n4) continue;
-                const float4 x = xs[k], y = ys[k];
-                const int j = q << 2;
-                if (x.x > m) { m = x.x; am = j; }
-                if (x.y > m) { m = x.y; am = j + 1; }
-                if (x.z > m) { m = x.z; am = j + 2; }
-                if (x.w > m) { m = x.w; am = j + 3; }
-                dl = fmaf(y.x, x.x, dl);
-                dl = fmaf(y.y, x.y, dl);
-                dl = fmaf(y.z, x.z, dl);
-                dl = fmaf(y.w, x.w, dl);
-            }
-        } else if (((s.polar_off | s.naz) & 3) == 0) {
-            // wider 16-byte rows: each lane takes 4 consecutive bins per load, in index order
-            const float4* In4 = reinterpret_cast<const float4*>(In);
-            const float4* G4 = reinterpret_cast<const float4*>(G);
-#pragma unroll 4
-            for (int q = lane; q < (s.naz >> 2); q += 32) {
-                const float4 x = __ldcs(In4 + q), y = __ldg(G4 + q);
-                const int j = q << 2;
-                if (x.x > m) { m = x.x; am = j; }
-                if (x.y > m) { m = x.y; am = j + 1; }
-                if (x.z > m) { m = x.z; am = j + 2; }
-                if (x.w > m) { m = x.w; am = j + 3; }
-                dl = fmaf(y.x, x.x, dl);
-                dl = fmaf(y.y, x.y, dl);
-                dl = fmaf(y.z, x.z, dl);
-                dl = fmaf(y.w, x.w, dl);
-            }
         } else {
-            for (int j = lane; j < s.naz; j += 32) {
-                const float x = In[j];
+            for (int j = lane; j < naz; j += 32) {
+                const float x = noised[off + j];
                 if (x > m) { m = x; am = j; }
-                dl = fmaf(G[j], x, dl);
+                dl = fmaf(grad[off + j], x, dl);
+            }
+            if (more) {
+                place(g + 1);
+                if (vec) ask(0);
             }
         }
         // lane partials added across the warp in float-float (error-free
@@ -1022,47 +1029,59 @@ __global__ void k_adj_rows(const SensorDev* sensors, const int32_t* row_map, Sen
             r.m = m;
             r.valid = m > 0.0f;
             r.c = r.valid ? (__fadd_rn(dot.hi, dot.lo) / m) / m : 0.0f;
-            r.arg = row * s.naz + am;
+            r.arg = base + am;
             info[g] = r;
         }
-    } else {
-        const int si = blockIdx.x;
-        if (si >= total) return;
-        const SensorDev& s = sensors ? sensors[si] : one;
-        const int64_t n = (int64_t)s.nr * s.naz;
-        const float* In = noised + s.polar_off;
-        const float* G = grad + s.polar_off;
-        float m = -CUDART_INF_F;
-        int am = 0x7FFFFFFF;
-        ff dot{0.0f, 0.0f};   // float-float: products exact (FMA), sums error-free
-        for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-            const float x = In[j], y = G[j];
-            if (x > m) { m = x; am = (int)j; }
-            const float p = __fmul_rn(y, x);
-            dot = ff_add(dot, ff{p, fmaf(y, x, -p)});
+    }
+}
+
+// The same for whole images: one block per image.
+__global__ void __launch_bounds__(1024) k_adj_images(const SensorDev* sensors, SensorDev one, int64_t total,
+                                                     const float* noised, const float* grad, RowInfo* info,
+                                                     int32_t* zero_word) {
+    let_next_start();
+    wait_for_previous();
+    const int lane = threadIdx.x & 31;
+    if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0;   // the gather's work counter
+    __shared__ float s_m[32];
+    __shared__ int s_a[32];
+    __shared__ ff s_d[32];
+    const int si = blockIdx.x;
+    if (si >= total) return;
+    const SensorDev& s = sensors ? sensors[si] : one;
+    const int64_t n = (int64_t)s.nr * s.naz;
+    const float* In = noised + s.polar_off;
+    const float* G = grad + s.polar_off;
+    float m = -CUDART_INF_F;
+    int am = 0x7FFFFFFF;
+    ff dot{0.0f, 0.0f};   // float-float: products exact (FMA), sums error-free
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        const float x = In[j], y = G[j];
+        if (x > m) { m = x; am = (int)j; }
+        const float p = __fmul_rn(y, x);
+        dot = ff_add(dot, ff{p, fmaf(y, x, -p)});
+    }
+    for (int o = 16; o; o >>= 1) {
+        const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o);
+        const int a2 = __shfl_xor_sync(0xFFFFFFFFu, am, o);
+        if (m2 > m || (m2 == m && a2 < am)) { m = m2; am = a2; }
+        const ff d2{__shfl_xor_sync(0xFFFFFFFFu, dot.hi, o), __shfl_xor_sync(0xFFFFFFFFu, dot.lo, o)};
+        dot = ff_add(dot, d2);
+    }
+    const int w = threadIdx.x >> 5;
+    if (lane == 0) { s_m[w] = m; s_a[w] = am; s_d[w] = dot; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
+            if (s_m[k] > m || (s_m[k] == m && s_a[k] < am)) { m = s_m[k]; am = s_a[k]; }
+            dot = ff_add(dot, s_d[k]);
         }
-        for (int o = 16; o; o >>= 1) {
-            const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o);
-            const int a2 = __shfl_xor_sync(0xFFFFFFFFu, am, o);
-            if (m2 > m || (m2 == m && a2 < am)) { m = m2; am = a2; }
-            const ff d2{__shfl_xor_sync(0xFFFFFFFFu, dot.hi, o), __shfl_xor_sync(0xFFFFFFFFu, dot.lo, o)};
-            dot = ff_add(dot, d2);
-        }
-        const int w = threadIdx.x >> 5;
-        if (lane == 0) { s_m[w] = m; s_a[w] = am; s_d[w] = dot; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
-                if (s_m[k] > m || (s_m[k] == m && s_a[k] < am)) { m = s_m[k]; am = s_a[k]; }
-                dot = ff_add(dot, s_d[k]);
-            }
-            RowInfo r;
-            r.m = m;
-            r.valid = m > 0.0f;
-            r.c = r.valid ? (__fadd_rn(dot.hi, dot.lo) / m) / m : 0.0f;
-            r.arg = am;
-            info[s.rowmax_off] = r;
-        }
+        RowInfo r;
+        r.m = m;
+        r.valid = m > 0.0f;
+        r.c = r.valid ? (__fadd_rn(dot.hi, dot.lo) / m) / m : 0.0f;
+        r.arg = am;
+        info[s.rowmax_off] = r;
     }
 }
 
@@ -1261,13 +1280,19 @@ cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, boo
     return blocks > 0 ? launch_kernel(k_fan_lut, blocks, 256, 0, st, early, a) : cudaSuccess;
 }
 
-cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one, int n_sensors,
+cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one,
                             int64_t total_groups, int normalise, const float* noised,
                             const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early) {
     if (normalise == 0) return cudaSuccess;
-    const int64_t blocks = normalise == 1 ? (total_groups * 32 + 255) / 256 : total_groups;
-    return launch_kernel(k_adj_rows, (unsigned)blocks, normalise == 1 ? 256 : 1024, 0, st, early, sensors, row_map, one,
-                         n_sensors, total_groups, normalise, noised, grad, info, zero_word);
+    if (normalise != 1)
+        return launch_kernel(k_adj_images, (unsigned)total_groups, 1024, 0, st, early, sensors, one, total_groups, noised,
+                             grad, info, zero_word);
+    // two rows a warp once the launch is four waves or so (32 warps on each of 152 SMs);
+    // four are no faster
+    const int per_warp = total_groups >= 20000 ? 2 : 1;
+    const int64_t warps = (total_groups + per_warp - 1) / per_warp;
+    return launch_kernel(k_adj_rows, (unsigned)((warps + 7) / 8), 256, 0, st, early, sensors, row_map, one, total_groups,
+                         per_warp, noised, grad, info, zero_word);
 }
 
 cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,

@@ -631,7 +631,7 @@ extern "C" sonar_status sonar_render_backward(sonar_ctx_t ctx, int32_t scene_id,
     const int n_units = (int)((rays + chunk - 1) / chunk);
     CU(grow(ctx->partials, sizeof(double) * (size_t)n_units * nq, s), "scratch allocation");
     if (params->normalise != 0)
-        CU(launch_adj_rows(nullptr, nullptr, S, 1, groups, params->normalise, d_noised, d_grad_polar,
+        CU(launch_adj_rows(nullptr, nullptr, S, groups, params->normalise, d_noised, d_grad_polar,
                            (RowInfo*)ctx->rowinfo.p, nullptr, s),
            "adjoint row launch");
     AdjArgs a{};
@@ -1417,7 +1417,7 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
         cast = true;
     }
     if (p->normalise != 0)
-        CU(launch_adj_rows(b->d_sens, b->d_row_map, SensorDev{}, (int)b->items.size(),
+        CU(launch_adj_rows(b->d_sens, b->d_row_map, SensorDev{},
                            p->normalise == 1 ? b->total_rows : (int64_t)b->items.size(), p->normalise, noised,
                            grad, b->d_rowinfo, b->d_counters + 1, s, cast),
            "batch adjoint rows");

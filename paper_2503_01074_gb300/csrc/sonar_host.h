@@ -65,7 +65,7 @@ cudaError_t launch_norm(const NormArgs& a, cudaStream_t st, bool early = false);
 cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool early = false);
 cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, bool early = false);
 cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st, bool early = false);
-cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one, int n_sensors,
+cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one,
                             int64_t total_groups, int normalise, const float* noised,
                             const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early = false);
 // `early` for the gather, and `early_final` for the final sum after it.
