@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
     const int mode = a.params.normalise;
     const bool dense = REG == 0 && a.dense;
     const uint2* bands = a.bands + S.band_off + (int64_t)(row0 >> 5) * naz;
-    const bool staged = REG > 0 || naz <= kRowsStaged;
+    const bool staged = REG > 0 || naz <= kRowsStaged;   // the launch has room for every such sensor
     float* pat = reinterpret_cast<float*>(rows_smem);
     uint2* mask = reinterpret_cast<uint2*>(rows_smem + ((naz + 3) & ~3));
     if (staged) {
@@ -1242,13 +1242,15 @@ cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cud
 }
 
 // The row kernel for rows of up to `naz` bins: in registers up to 512 and up to
-// 1024 bins, else written and read back.  `vec`: 16-byte stores (every row of
+// 1024 bins, else written and read back.  `staged`: the widest of the launch's
+// sensors whose column tables are staged (no wider than kRowsStaged; 0: none), which
+// may be a narrower one than the widest.  `vec`: 16-byte stores (every row of
 // every sensor starts on a 16-byte boundary of each image).
-cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st, bool early) {
+cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, int staged, bool vec, cudaStream_t st, bool early) {
     if (grid <= 0) return cudaSuccess;
     // a row whose first bin is not a multiple of 4 may need one quad more
     const int reach = vec ? naz : naz + 3;
-    const size_t smem = naz <= kRowsStaged ? ((size_t)((naz + 3) & ~3) + 2 * (size_t)naz) * sizeof(uint32_t) : 0;
+    const size_t smem = ((size_t)((staged + 3) & ~3) + 2 * (size_t)staged) * sizeof(uint32_t);
     if (reach <= 512 && !a.dense)
         return launch_kernel(vec ? k_rows<4, true> : k_rows<4, false>, grid, 256, smem, st, early, a);
     if (reach <= 1024 && !a.dense)

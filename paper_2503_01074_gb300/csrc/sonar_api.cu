@@ -213,6 +213,9 @@ int rows_per_block(int64_t total_rows, int sm_count) {
     return 8;
 }
 
+// Azimuth bins of a sensor whose column tables the row kernel keeps in shared memory, or 0.
+int staged_naz(const SensorDev& s) { return s.naz <= kRowsStaged ? s.naz : 0; }
+
 SensorDev make_sensor(const sonar_sensor& s, uint64_t seed, uint64_t frame, const Tune& t, int fan_w,
                       int fan_h) {
     SensorDev d{};
@@ -487,7 +490,7 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     r.polar = polar;
     r.gmax = gmax;
     const bool vec = S.naz % 4 == 0 && aligned16(noised) && aligned16(polar) && aligned16(binned);
-    CU(launch_rows(r, (S.nr + r.rows_per_block - 1) / r.rows_per_block, S.naz, vec, s, !capturing),
+    CU(launch_rows(r, (S.nr + r.rows_per_block - 1) / r.rows_per_block, S.naz, staged_naz(S), vec, s, !capturing),
        "row launch");
     return SONAR_OK;
 }
@@ -674,6 +677,7 @@ struct sonar_batch {
     size_t fold_smem = 0;
     int fold_block = 128, fold_words_per_warp = 0;
     int rows_step = 32, max_naz = 1;
+    int max_staged_naz = 0;           // the widest sensor whose column tables the row kernel stages (0: none)
     bool rows_vec = false;            // every row starts on a 16-byte boundary of a 16-byte aligned image
     SensorDev* d_sens = nullptr;
     int4* d_fold_map = nullptr;
@@ -823,6 +827,7 @@ sonar_status batch_plan(sonar_batch* b) {
     b->trace_prefix.assign(n + 1, 0);
     int64_t rows = 0, polar_end = 0, rays = 0, bands = 0;
     b->max_naz = 1;
+    b->max_staged_naz = 0;
     b->rows_vec = true;
     std::map<int, int64_t> block_votes;
     for (int k = 0; k < n; ++k) {
@@ -839,6 +844,7 @@ sonar_status batch_plan(sonar_batch* b) {
         rays += (int64_t)S.nb * S.ne;
         bands += band_count(S) * S.naz;
         b->max_naz = std::max(b->max_naz, S.naz);
+        b->max_staged_naz = std::max(b->max_staged_naz, staged_naz(S));
         b->rows_vec = b->rows_vec && S.naz % 4 == 0 && S.polar_off % 4 == 0;
         rows += S.nr;    // room for mode 1; mode 2 uses the first slot of each sensor
         polar_end = std::max<int64_t>(polar_end, it.polar_offset + (int64_t)S.nr * S.naz);
@@ -1182,7 +1188,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         r.polar = out->polar;
         r.gmax = b->d_rowmax;
         const bool vec = b->rows_vec && aligned16(r.noised) && aligned16(r.binned) && aligned16(r.polar);
-        CU(launch_rows(r, (int)b->rows_map.size(), b->max_naz, vec, s, true), "batch row launch");
+        CU(launch_rows(r, (int)b->rows_map.size(), b->max_naz, b->max_staged_naz, vec, s, true), "batch row launch");
         if (events) CU(mark_phase(b, b->mark[0], b->ev[1], s), "cudaEventRecord");
     }
     if (part == 1) return SONAR_OK;

@@ -58,7 +58,8 @@ cudaError_t launch_trace(const TraceArgs& a, int blocks, int occupancy, cudaStre
 // `early`: the launch may overlap the end of the launch before it on the stream, which
 // must be one of these kernels (see wait_for_previous).
 cudaError_t launch_fold(const FoldArgs& a, int grid, int block, size_t smem, cudaStream_t st, bool early = false);
-cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, bool vec, cudaStream_t st, bool early = false);
+cudaError_t launch_rows(const RowsArgs& a, int grid, int naz, int staged, bool vec, cudaStream_t st,
+                        bool early = false);
 constexpr size_t kMaxDynSmem = 220 * 1024;   // of the 227 KB a block may have, less the static part
 cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, void* out, cudaStream_t st);
 cudaError_t launch_norm(const NormArgs& a, cudaStream_t st, bool early = false);
