@@ -1,7 +1,8 @@
 // LBVH construction for the sonar geometry query (OceanSim Sec. III-A-2:
 // the scene is queried by ray casting; this builds the acceleration structure).
 //
-//   1. validate + bounds of box centres grid-stride, one set of atomics per block
+//   1. validate + bounds              of box centres and of vertices; grid-stride, one set
+//                                     of atomics per block
 //   2. Morton codes                   63-bit keys (21 bits per axis) of triangles' box centres
 //   3. radix sort                     stable LSD, 8-bit digits, three launches a digit
 //   4. Karras hierarchy               one thread per internal node (Karras, HPG 2012)
@@ -41,7 +42,9 @@ constexpr int kLevels = 32;   // (3 kLevels + 1 > kStackMax): a deeper 4-wide tr
 struct BuildState {
     uint32_t flags;        // 1: index out of range, 2: negative material, 4: non-finite vertex
     int32_t max_mat;
-    uint32_t lo[3], hi[3]; // ordered-encoded bounds of the box centres
+    // ordered-encoded bounds: of the box centres (the Morton grid), of the triangles'
+    // vertices (the padding)
+    uint32_t lo[3], hi[3], vlo[3], vhi[3];
     int32_t height;        // of the binary hierarchy
     int32_t level[2][kLevels + 1];   // wide nodes per level of the 4-wide and 8-wide tree
 };
@@ -49,7 +52,7 @@ struct BuildState {
 __global__ void k_build_init(BuildState* st, int32_t* list4, int32_t* list8) {
     const int t = threadIdx.x;
     if (t < kLevels + 1) st->level[0][t] = st->level[1][t] = t == 0 ? 1 : 0;
-    if (t < 3) { st->lo[t] = 0xFFFFFFFFu; st->hi[t] = 0u; }
+    if (t < 3) { st->lo[t] = st->vlo[t] = 0xFFFFFFFFu; st->hi[t] = st->vhi[t] = 0u; }
     if (t == 0) {
         st->flags = 0u;
         st->max_mat = -1;
@@ -59,7 +62,7 @@ __global__ void k_build_init(BuildState* st, int32_t* list4, int32_t* list8) {
 }
 
 // ---------------------------------------------------------------------------
-// 1. validation and bounds of the box centres
+// 1. validation and bounds of the box centres and vertices
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ float3 load_v(const float* v, int32_t i) {
@@ -82,20 +85,23 @@ __device__ __forceinline__ float3 box_centre(float3 p, float3 q, float3 r) {
 
 __global__ void __launch_bounds__(kThreads) k_validate(const float* verts, int64_t nv, const int32_t* tris,
                                                        const int32_t* mat, int64_t nt, BuildState* st) {
-    __shared__ uint32_t s_lo[3], s_hi[3], s_flags;
+    // bounds 0-2 of the box centres, 3-5 of the vertices
+    __shared__ uint32_t s_lo[6], s_hi[6], s_flags;
     __shared__ int32_t s_mat;
-    if (threadIdx.x < 3) { s_lo[threadIdx.x] = 0xFFFFFFFFu; s_hi[threadIdx.x] = 0u; }
+    if (threadIdx.x < 6) { s_lo[threadIdx.x] = 0xFFFFFFFFu; s_hi[threadIdx.x] = 0u; }
     if (threadIdx.x == 0) { s_flags = 0; s_mat = -1; }
     __syncthreads();
-    uint32_t lo[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, hi[3] = {0u, 0u, 0u}, flags = 0u;
-    int32_t most = -1;
+    uint32_t lo[6], hi[6], flags = 0u;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) { lo[k] = 0xFFFFFFFFu; hi[k] = 0u; }
+    int32_t most_mat = -1;
     for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < nt; t += (int64_t)gridDim.x * kThreads) {
         const int32_t a = tris[3 * t], b = tris[3 * t + 1], c = tris[3 * t + 2];
         uint32_t f = 0;
         if (a < 0 || b < 0 || c < 0 || a >= nv || b >= nv || c >= nv) f |= 1u;
         const int32_t m = mat[t];
         if (m < 0) f |= 2u;
-        most = max(most, m);
+        most_mat = max(most_mat, m);
         if (!f) {
             const float3 p = load_v(verts, a), q = load_v(verts, b), r = load_v(verts, c);
             const bool fin = isfinite(p.x) && isfinite(p.y) && isfinite(p.z) && isfinite(q.x) &&
@@ -105,31 +111,35 @@ __global__ void __launch_bounds__(kThreads) k_validate(const float* verts, int64
                 f |= 4u;
             } else {
                 const float3 g = box_centre(p, q, r);
-                const uint32_t e[3] = {ord_enc(g.x), ord_enc(g.y), ord_enc(g.z)};
+                const float most[6] = {g.x, g.y, g.z, fmaxf(p.x, fmaxf(q.x, r.x)), fmaxf(p.y, fmaxf(q.y, r.y)),
+                                       fmaxf(p.z, fmaxf(q.z, r.z))};
+                const float least[6] = {g.x, g.y, g.z, fminf(p.x, fminf(q.x, r.x)), fminf(p.y, fminf(q.y, r.y)),
+                                        fminf(p.z, fminf(q.z, r.z))};
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    lo[k] = min(lo[k], e[k]);
-                    hi[k] = max(hi[k], e[k]);
+                for (int k = 0; k < 6; ++k) {
+                    lo[k] = min(lo[k], ord_enc(least[k]));
+                    hi[k] = max(hi[k], ord_enc(most[k]));
                 }
             }
         }
         flags |= f;
     }
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 6; ++k) {
         lo[k] = __reduce_min_sync(0xFFFFFFFFu, lo[k]);
         hi[k] = __reduce_max_sync(0xFFFFFFFFu, hi[k]);
     }
     flags = __reduce_or_sync(0xFFFFFFFFu, flags);
-    most = __reduce_max_sync(0xFFFFFFFFu, most);
+    most_mat = __reduce_max_sync(0xFFFFFFFFu, most_mat);
     if ((threadIdx.x & 31) == 0) {
-        for (int k = 0; k < 3; ++k) { atomicMin(&s_lo[k], lo[k]); atomicMax(&s_hi[k], hi[k]); }
+        for (int k = 0; k < 6; ++k) { atomicMin(&s_lo[k], lo[k]); atomicMax(&s_hi[k], hi[k]); }
         if (flags) atomicOr(&s_flags, flags);
-        atomicMax(&s_mat, most);
+        atomicMax(&s_mat, most_mat);
     }
     __syncthreads();
-    if (threadIdx.x < 3) {
-        atomicMin(&st->lo[threadIdx.x], s_lo[threadIdx.x]);
-        atomicMax(&st->hi[threadIdx.x], s_hi[threadIdx.x]);
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        atomicMin(k < 3 ? &st->lo[k] : &st->vlo[k - 3], s_lo[k]);
+        atomicMax(k < 3 ? &st->hi[k] : &st->vhi[k - 3], s_hi[k]);
     }
     if (threadIdx.x == 0) {
         if (s_flags) atomicOr(&st->flags, s_flags);
@@ -138,15 +148,18 @@ __global__ void __launch_bounds__(kThreads) k_validate(const float* verts, int64
 }
 
 // Box padding: covers the difference between the FP32 traversal ray and the
-// exact ray, so that the FP32 box test never culls an exact hit.
+// exact ray, so that the FP32 box test never culls an exact hit.  That difference
+// grows with the coordinates and the ranges in the scene, so the padding follows the
+// vertices: a few coarse triangles about one middle (a seabed quad) would leave the
+// bounds of their centres as small as the object between them.
 __device__ __forceinline__ float box_pad(const BuildState* st) {
     float ext = 0.0f, mag = 0.0f;
     for (int a = 0; a < 3; ++a) {
-        const float l = ord_dec(st->lo[a]), h = ord_dec(st->hi[a]);
+        const float l = ord_dec(st->vlo[a]), h = ord_dec(st->vhi[a]);
         ext = fmaxf(ext, __fsub_rn(h, l));
         mag = fmaxf(mag, fmaxf(fabsf(l), fabsf(h)));
     }
-    return fmaxf(__fmul_rn(1e-5f, __fadd_rn(ext, mag)), 1e-6f);
+    return fmaxf(__fmul_rn(1e-5f, fminf(__fadd_rn(ext, mag), 3.0e38f)), 1e-6f);   // finite at any extent
 }
 
 // ---------------------------------------------------------------------------
