@@ -432,10 +432,13 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                     }
                 }
             }
-            if (!VEC) {   // bins over the row's ends: no part in its maximum (nor in the least value)
-                const float most = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+            if (!VEC) {   // bins over the row's ends (by column: a bin may be -inf): no part in its maximum
+                const float most = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));   // (nor in the least value)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = v[j] == -CUDART_INF_F ? most : v[j];
+                for (int j = 0; j < 4; ++j) {
+                    const int c = 4 * q - sh + j;
+                    if (c < 0 || c >= naz) v[j] = most;
+                }
             }
         };
         auto store = [&](float* to, int k, const float (&v)[4]) {   // `to`: the image at `off`

@@ -1,5 +1,5 @@
-"""The row kernel (noise, range-wise normalisation) in launches that its widest
-sensor alone does not describe.
+"""The row kernel (noise, range-wise normalisation): launches that its widest
+sensor alone does not describe, and bins that are not finite.
 """
 import math
 
@@ -48,3 +48,31 @@ def test_widths_on_both_sides_of_the_staged_limit(env, widths, mode):
     b.close()
     st, bits = son.check()
     assert st == 0 and bits == 0
+
+
+# rows in registers and written back, with 16-byte vectors and without, quads over their ends
+@pytest.mark.parametrize("naz", [64, 61, 62, 513, 516, 1021, 1030, 1032])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("value", [-math.inf, math.inf, math.nan])
+def test_bins_that_are_not_finite(env, naz, mode, value):
+    """A reflectivity of +-inf or NaN (a fit that diverges) stays in the bins that it
+    reaches, and its neighbours keep the values that they have without it: a bin
+    without such a return is what a render with that material at zero gives."""
+    son, mu, sid = env
+    sp, prm = spec(64, 32, 60, naz), RenderParams(normalise=mode)
+    bad, zero = np.array(mu, np.float32), np.array(mu, np.float32)
+    bad[0], zero[0] = value, 0.0
+    out = son.render(sid, sp, son.theta(0.05, 1.0, bad), prm, 3, 4, fan=False, binned=True)
+    ref = son.render(sid, sp, son.theta(0.05, 1.0, zero), prm, 3, 4, fan=False, binned=True)
+    torch.cuda.synchronize()
+    P, I, N = (out[k].cpu().numpy() for k in ("binned", "noised", "polar"))
+    hit = ~np.isfinite(P)
+    assert hit.any() and not hit.all()
+    assert np.array_equal(I[hit], P[hit], equal_nan=True)
+    assert np.array_equal(I[~hit], ref["noised"].cpu().numpy()[~hit])
+    # the maximum passes over NaN; a row or image whose maximum is not positive is not divided
+    finite = np.where(np.isnan(I), -np.inf, I)
+    top = {0: np.ones(1, np.float32), 1: finite.max(1, keepdims=True), 2: finite.max()}[mode]
+    with np.errstate(invalid="ignore"):
+        want = np.where(top > 0, I / top, I)
+    assert np.array_equal(N, want, equal_nan=True)
