@@ -126,7 +126,7 @@ __device__ __forceinline__ void mark_rows(const FoldArgs& a, const ExactDiv& div
         uint2 h[kFoldAhead];   // key, triangle
 #pragma unroll
         for (int u = 0; u < kFoldAhead; ++u)
-            h[u] = j + u * step < n ? __ldg(reinterpret_cast<const uint2*>(H + j + u * step)) : make_uint2(kNoKey, 0u);
+            h[u] = j + u * step < n ? *reinterpret_cast<const uint2*>(H + j + u * step) : make_uint2(kNoKey, 0u);
 #pragma unroll
         for (int u = 0; u < kFoldAhead; ++u) {
             const int row = row_of(a, div, S.nr, sc.n_tris, h[u].x, h[u].y, col);
@@ -146,7 +146,7 @@ __device__ __forceinline__ void sum_rows(const FoldArgs& a, const ExactDiv& div,
         uint4 h[kFoldAhead];
 #pragma unroll
         for (int u = 0; u < kFoldAhead; ++u)
-            h[u] = jb + 32 * u + lane < n ? __ldg(reinterpret_cast<const uint4*>(H + jb + 32 * u + lane))
+            h[u] = jb + 32 * u + lane < n ? *reinterpret_cast<const uint4*>(H + jb + 32 * u + lane)
                                           : make_uint4(kNoKey, 0u, 0u, 0u);
         int row[kFoldAhead], mat[kFoldAhead];
 #pragma unroll
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                         ret[j].x = a.dense[off + 128 * k + j];
                         w[j].x = 0u;
                     } else if (!(VEC && staged)) {
-                        w[j] = staged ? mask[c] : __ldg(bands + c);
+                        w[j] = staged ? mask[c] : bands[c];
                     }
                 } else {
                     w[j].x = 0u;
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
             if ((w[0].x | w[1].x | w[2].x | w[3].x) & bit) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (w[j].x & bit) ret[j] = __ldg(vals + (w[j].y + __popc(w[j].x & below)));
+                    if (w[j].x & bit) ret[j] = vals[w[j].y + __popc(w[j].x & below)];
             }
             const U4 x = additive_words((b0 >> 2) + (uint32_t)q, flo, fhi, K);
             const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
@@ -553,7 +553,7 @@ __device__ __forceinline__ void norm_row(const NormArgs& a, int64_t g, int lane)
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int q = lane + 32 * k;
-            v[k] = q < n4 ? __ldg(In4 + q) : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+            v[k] = q < n4 ? In4[q] : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
         }
         if (a.normalise == 1) {
             m = -CUDART_INF_F;
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(256, 4) k_norm_rows(const __grid_constant__ No
 #pragma unroll
         for (int k = 0; k < kV; ++k) {
             const int q = lane + 32 * k;
-            v[r][k] = q < n4[r] ? __ldg(In4 + q)
+            v[r][k] = q < n4[r] ? In4[q]
                                 : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
         }
     }
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(256, 4) k_fan_group(const __grid_constant__ Fa
         for (int v = v0; v < min(v0 + kFanSide, h); v += kStep) {
             const int64_t pix = (int64_t)v * w + u;
             for (int q = 0; q < nm; ++q) {
-                const uint4 c = lut && M[q].fan_lut ? __ldg(lut + pix) : fan_coord_apart(M[q], pix);
+                const uint4 c = lut && M[q].fan_lut ? lut[pix] : fan_coord_apart(M[q], pix);
                 __stcs(a.fan + M[q].fan_off + pix, fan_blend(c, a.polar + M[q].polar_off));
             }
         }
@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(256, 4) k_fan_group(const __grid_constant__ Fa
     uint4 ahead[kRows];   // the table's entries of the next rows, on their way during these
 #pragma unroll
     for (int r = 0; r < kRows; ++r)
-        ahead[r] = v0 + r * kStep < h ? __ldg(lut + (int64_t)(v0 + r * kStep) * w + u) : outside;
+        ahead[r] = v0 + r * kStep < h ? lut[(int64_t)(v0 + r * kStep) * w + u] : outside;
 #pragma unroll 1
     for (int k = 0; k < kFanSide; k += kRows * kStep) {
         const int v = v0 + k;
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(256, 4) k_fan_group(const __grid_constant__ Fa
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
             c[r] = ahead[r];
-            ahead[r] = v + (r + kRows) * kStep < h ? __ldg(lut + pix + (r + kRows) * step) : outside;
+            ahead[r] = v + (r + kRows) * kStep < h ? lut[pix + (r + kRows) * step] : outside;
         }
         // every gather before the first store: the compiler must not move a load
         // above a store that might alias it
@@ -1149,7 +1149,7 @@ __global__ void __launch_bounds__(512) k_adjoint(const __grid_constant__ AdjArgs
             int mat = 0;
             float v_mu = 0.0f;
             if (r < U.r1) {
-                const uint4 h = __ldg(reinterpret_cast<const uint4*>(a.hits + S.hits_off + r));
+                const uint4 h = *reinterpret_cast<const uint4*>(a.hits + S.hits_off + r);
                 const uint32_t key = h.x, orig = h.y;
                 const float rr = __uint_as_float(h.z), cf = __uint_as_float(h.w);
                 if (key != kNoKey) {

@@ -251,6 +251,10 @@ __device__ __forceinline__ void copy_param(T* dst, const T* src, int lane) {
 // start once every block of the kernel before it has started and said so; it sets
 // itself up from its parameters and waits here for the whole of that kernel before
 // it touches what kernels write.  Without the launch attribute both do nothing.
+// What a kernel before it in the chain writes (records, values, bitmaps, images,
+// tables) is read by plain loads: the read-only path (__ldg, ld.global.nc) is for data
+// that nothing writes while the kernel lives, and such a load may be moved above the
+// wait.  Descriptors, maps, theta, scenes and a caller's gradient are such data.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -51,7 +51,7 @@ __device__ __forceinline__ float3 ray_dir32(const SensorDev& s, int i, int j) {
 // decisions below only use signs and ratios, which a positive scale leaves
 // unchanged.
 __device__ __forceinline__ void ray_dir_ff(const SensorDev& s, int i, int j, ff w[3]) {
-    const float4 bp = __ldg(s.trig + i), el = __ldg(s.trig + s.nb + j);
+    const float4 bp = s.trig[i], el = s.trig[s.nb + j];
     const ff sp{bp.x, bp.y}, cp{bp.z, bp.w}, st{el.x, el.y}, ct{el.z, el.w};
     const ff ds[3] = {ff_mul(sp, ct), ff_mul(cp, ct), st};
     for (int a = 0; a < 3; ++a)
@@ -118,7 +118,7 @@ __device__ __noinline__ ExactPair exact_pair(const SensorDev& s, const float4* t
     const float4 a = __ldg(tp), b = __ldg(tp + 1), c = __ldg(tp + 2);
     // components: lanes 0-2 e1, 3-5 e2, 6-8 s = o - v0, 9-11 the direction w
     const ff e = ff_two_sum(kind == 0 ? axis_of(b, ax) : kind == 1 ? axis_of(c, ax) : s.pos[ax], -axis_of(a, ax));
-    const float4 bp = __ldg(s.trig + i), el = __ldg(s.trig + s.nb + j);
+    const float4 bp = s.trig[i], el = s.trig[s.nb + j];
     const ff sp{bp.x, bp.y}, cp{bp.z, bp.w}, st{el.x, el.y}, ct{el.z, el.w};
     const ff w = ff_add(ff_add(ff_mulf(ff_mul(sp, ct), s.rot[3 * ax]), ff_mulf(ff_mul(cp, ct), s.rot[3 * ax + 1])),
                         ff_mulf(st, s.rot[3 * ax + 2]));
