@@ -743,6 +743,18 @@ struct sonar_batch {
 
 namespace {
 
+// Drops every captured graph: the next call of each kind captures its launches anew.
+void drop_graphs(sonar_batch* b) {
+    for (cudaGraphExec_t* g : {&b->fwd, &b->fwd_lean, &b->bwd, &b->step}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
+    b->fwd_key.clear();
+    b->fwd_lean_key.clear();
+    b->bwd_key.clear();
+    b->step_key.clear();
+}
+
 void batch_free_device(sonar_batch* b) {
     for (void* p : {(void*)b->d_sens, (void*)b->d_fold_map, (void*)b->d_rows_map, (void*)b->d_vals,
                     (void*)b->d_bands, (void*)b->d_adj_units, (void*)b->d_scenes,
@@ -773,15 +785,7 @@ void batch_free_device(sonar_batch* b) {
     b->d_fan_prefix = nullptr;
     b->d_rowmax = nullptr; b->d_noised = nullptr; b->d_rowinfo = nullptr; b->d_partials = nullptr;
     b->d_counters = nullptr;
-    if (b->fwd) cudaGraphExecDestroy(b->fwd);
-    if (b->fwd_lean) cudaGraphExecDestroy(b->fwd_lean);
-    if (b->bwd) cudaGraphExecDestroy(b->bwd);
-    if (b->step) cudaGraphExecDestroy(b->step);
-    b->fwd = b->fwd_lean = b->bwd = b->step = nullptr;
-    b->fwd_key.clear();
-    b->fwd_lean_key.clear();
-    b->bwd_key.clear();
-    b->step_key.clear();
+    drop_graphs(b);
     b->trig_current = b->lut_current = false;
 }
 
@@ -1291,10 +1295,7 @@ extern "C" sonar_status sonar_batch_update(sonar_batch_t b, const sonar_batch_it
         cudaFree(b->d_scenes);
         b->d_scenes = d;
         b->n_scene_table = table.size();
-        if (b->fwd) cudaGraphExecDestroy(b->fwd);
-        if (b->fwd_lean) cudaGraphExecDestroy(b->fwd_lean);
-        if (b->bwd) cudaGraphExecDestroy(b->bwd);
-        b->fwd = b->fwd_lean = b->bwd = nullptr;
+        drop_graphs(b);   // they hold the old table's address
     }
     const int slot = b->stage_next;
     b->stage_next ^= 1;
