@@ -672,7 +672,8 @@ struct sonar_batch {
     int64_t total_rays = 0;
     int64_t total_rows = 0, total_polar = 0;
     int block = 128;
-    int trace_occ = 0;
+    int plan_occ = 0;                 // the ray-cast variant of the plan
+    int trace_occ = 0;                // the one launched: the plan's, as far as the items' scenes allow
     int adj_chunk = 0;
     size_t fold_smem = 0;
     int fold_block = 128, fold_words_per_warp = 0;
@@ -880,6 +881,7 @@ sonar_status batch_plan(sonar_batch* b) {
         for (const sonar_batch_item& it : b->items)
             if (!ctx->scenes[it.scene_id].nodes8) b->trace_occ &= ~kTraceWide;
     }
+    b->plan_occ = b->trace_occ;
     b->total_rows = rows;
     b->total_polar = polar_end;
     // the fold's blocks: the warps that the sensor with most rays wants, fewer
@@ -1296,6 +1298,18 @@ extern "C" sonar_status sonar_batch_update(sonar_batch_t b, const sonar_batch_it
         b->d_scenes = d;
         b->n_scene_table = table.size();
         drop_graphs(b);   // they hold the old table's address
+    }
+    // an item may go to a scene whose 8-wide tree was too deep to keep: the launches then
+    // walk the 4-wide trees, until an update leads away from it again.  (A scene of
+    // one leaf has no nodes to walk, and needs no tree.)
+    int occ = b->plan_occ;
+    for (int k = 0; k < n; ++k) {
+        const SceneStore& sc = ctx->scenes[items[k].scene_id];
+        if (sc.root >= 0 && !sc.nodes8) occ &= ~kTraceWide;
+    }
+    if (occ != b->trace_occ) {
+        b->trace_occ = occ;
+        drop_graphs(b);
     }
     const int slot = b->stage_next;
     b->stage_next ^= 1;

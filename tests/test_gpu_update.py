@@ -60,3 +60,54 @@ def test_step_after_an_update_to_a_scene_uploaded_since(son):
     b.close()
     st, bits = son.check()
     assert st == 0 and bits == 0
+
+
+def deep_scene():
+    """Clusters in seven octants of every cube, the eighth halved again, 18 times: an
+    8-wide tree of more levels than its walk's stack takes, a 4-wide one that fits."""
+    r = np.random.default_rng(0)
+    tris = []
+    for level in range(18):
+        side = 8.0 * 0.5 ** level
+        for q in range(1, 8):
+            corner = np.array([q & 1, q >> 1 & 1, q >> 2 & 1]) * side / 2
+            for _ in range(4):
+                x = corner + side / 2 * (0.2 + 0.6 * r.random(3))
+                tris.append(x + 0.15 * side * (r.random((3, 3)) - 0.5))
+    v = np.array(tris).reshape(-1, 3).astype(np.float32) + np.float32([-2.0, 1.0, -2.0])
+    return S.Mesh(v, np.arange(len(v), dtype=np.int32).reshape(-1, 3), np.zeros(len(tris), np.int32))
+
+
+@pytest.mark.parametrize("variant", [None, 16])
+@pytest.mark.parametrize("n", [3, 300])
+def test_update_to_a_scene_without_an_8_wide_tree(son, variant, n):
+    """A batch planned for the 8-wide trees (several lanes per ray, or by its tuning
+    row) walks the 4-wide ones once an item's scene has no other, and its own again
+    after; the records do not depend on the tree."""
+    theta, prm = son.theta(0.05, 1.0, MU), RenderParams()
+    wide, deep, one = (son.upload_mesh(m) for m in (S.tiny_scene()[0], deep_scene(), S.random_soup(2, 5)))
+    info = son.scene_info(deep)
+    assert info["bytes"] == 52 * info["n_tris"] + 128 * info["n_pairs"]   # no 8-wide nodes
+    spec = S.SensorSpec(np.zeros(3, np.float32), S.pose_matrix(0.1, math.radians(15)), 64, 32, 100, 64,
+                        math.radians(100.0), math.radians(40.0), 0.5, 20.0)
+    if variant is not None:
+        son.tune_set([[64, 32, 100, 64, 1, 8, 128, variant]])
+    alone = {}
+    b = son.batch(frames(wide, n, spec))
+    grad = torch.randn(b.n_polar, generator=torch.Generator().manual_seed(2)).to(son.device)
+    for sids in ([wide], [wide, deep], [deep], [one, wide], [one, deep], [wide]):
+        items = [(sids[k % len(sids)],) + it[1:] for k, it in enumerate(frames(wide, n, spec))]
+        b.update(items)
+        step(b, theta, prm, grad)
+        d = b.backward(theta, prm, grad, hits=False).clone()
+        torch.cuda.synchronize()
+        assert torch.isfinite(d).all()
+        for k in {0, 1, n - 1}:
+            sid, sp, seed, frame = items[k]
+            if (sid, k) not in alone:
+                alone[sid, k] = son.render(sid, sp, theta, prm, seed, frame, hits=True)["hits"].clone()
+            assert torch.equal(b.view(k)["hits"], alone[sid, k]), (sids, k)
+    assert (alone[deep, 1][:, 1] >= 0).any()
+    b.close()
+    st, bits = son.check()
+    assert st == 0 and bits == 0
