@@ -543,7 +543,7 @@ __device__ __forceinline__ void norm_row(const NormArgs& a, int64_t g, int lane)
     const float* In = a.noised + s.polar_off + (int64_t)row * naz;
     float* out = a.polar + s.polar_off + (int64_t)row * naz;
     float m = 0.0f;
-    if (((s.polar_off | naz) & 3) == 0 && naz <= 1024) {
+    if (a.vec && ((s.polar_off | naz) & 3) == 0 && naz <= 1024) {
         // 16-byte rows of up to 1024 bins: the row stays in registers between
         // the maximum and the division (one read of I~)
         const int n4 = naz >> 2;
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(256, 4) k_norm_rows(const __grid_constant__ No
         if (g >= a.total_rows) continue;
         const SensorDev& s = a.sensors ? a.sensors[a.row_map[g]] : a.one;
         const int naz = s.naz;
-        if (((s.polar_off | naz) & 3) != 0 || naz > 32 * 4 * kV) continue;
+        if (!a.vec || ((s.polar_off | naz) & 3) != 0 || naz > 32 * 4 * kV) continue;
         const int64_t off = s.polar_off + (int64_t)(g - s.rowmax_off) * naz;
         const float4* In4 = reinterpret_cast<const float4*>(a.noised + off);
         out4[r] = reinterpret_cast<float4*>(a.polar + off);
@@ -942,8 +942,8 @@ __global__ void __launch_bounds__(256) k_fan_lut(const __grid_constant__ FanLutA
 // us (6.7 TB/s), 64,000 rows of 512 bins 55 -> 53 (57 with a row per warp); more
 // warps of fewer registers spill.
 __global__ void __launch_bounds__(256, 4) k_adj_rows(const SensorDev* sensors, const int32_t* row_map, SensorDev one,
-                                                  int64_t total, int per_warp, const float* noised, const float* grad,
-                                                  RowInfo* info, int32_t* zero_word) {
+                                                  int64_t total, int per_warp, int aligned, const float* noised,
+                                                  const float* grad, RowInfo* info, int32_t* zero_word) {
     let_next_start();
     wait_for_previous();
     const int lane = threadIdx.x & 31;
@@ -958,7 +958,7 @@ __global__ void __launch_bounds__(256, 4) k_adj_rows(const SensorDev* sensors, c
         naz = s.naz;
         row = (int)(g - s.rowmax_off);
         off = s.polar_off + (int64_t)row * naz;
-        vec = ((s.polar_off | naz) & 3) == 0;
+        vec = aligned && ((s.polar_off | naz) & 3) == 0;
     };
     auto ask = [&](int j0) {   // bins j0 .. j0 + 511 of the row
 #pragma unroll
@@ -1286,7 +1286,7 @@ cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, boo
 }
 
 cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one,
-                            int64_t total_groups, int normalise, const float* noised,
+                            int64_t total_groups, int normalise, bool aligned, const float* noised,
                             const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early) {
     if (normalise == 0) return cudaSuccess;
     if (normalise != 1)
@@ -1297,7 +1297,7 @@ cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, co
     const int per_warp = total_groups >= 20000 ? 2 : 1;
     const int64_t warps = (total_groups + per_warp - 1) / per_warp;
     return launch_kernel(k_adj_rows, (unsigned)((warps + 7) / 8), 256, 0, st, early, sensors, row_map, one, total_groups,
-                         per_warp, noised, grad, info, zero_word);
+                         per_warp, (int)aligned, noised, grad, info, zero_word);
 }
 
 cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,

@@ -505,6 +505,7 @@ sonar_status single_post(sonar_ctx* ctx, const SensorDev& S, int normalise, cons
         n.noised = noised;
         n.gmax = gmax;
         n.normalise = normalise;
+        n.vec = aligned16(noised) && aligned16(polar);
         n.polar = polar;
         CU(launch_norm(n, s, !capturing), "normalisation launch");
     }
@@ -634,7 +635,8 @@ extern "C" sonar_status sonar_render_backward(sonar_ctx_t ctx, int32_t scene_id,
     const int n_units = (int)((rays + chunk - 1) / chunk);
     CU(grow(ctx->partials, sizeof(double) * (size_t)n_units * nq, s), "scratch allocation");
     if (params->normalise != 0)
-        CU(launch_adj_rows(nullptr, nullptr, S, groups, params->normalise, d_noised, d_grad_polar,
+        CU(launch_adj_rows(nullptr, nullptr, S, groups, params->normalise,
+                           aligned16(d_noised) && aligned16(d_grad_polar), d_noised, d_grad_polar,
                            (RowInfo*)ctx->rowinfo.p, nullptr, s),
            "adjoint row launch");
     AdjArgs a{};
@@ -1207,6 +1209,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         c.noised = out->noised ? out->noised : b->d_noised;
         c.gmax = b->d_rowmax;
         c.normalise = p->normalise;
+        c.vec = aligned16(c.noised) && aligned16(out->polar);
         c.polar = out->polar;
         CU(launch_norm(c, s, true), "batch normalisation launch");
     }
@@ -1439,8 +1442,8 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
     }
     if (p->normalise != 0)
         CU(launch_adj_rows(b->d_sens, b->d_row_map, SensorDev{},
-                           p->normalise == 1 ? b->total_rows : (int64_t)b->items.size(), p->normalise, noised,
-                           grad, b->d_rowinfo, b->d_counters + 1, s, cast),
+                           p->normalise == 1 ? b->total_rows : (int64_t)b->items.size(), p->normalise,
+                           aligned16(noised) && aligned16(grad), noised, grad, b->d_rowinfo, b->d_counters + 1, s, cast),
            "batch adjoint rows");
     if (events) CU(mark_phase(b, b->mark[1], b->ev[4], s), "cudaEventRecord");
     AdjArgs a{};

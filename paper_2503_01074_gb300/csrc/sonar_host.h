@@ -67,8 +67,9 @@ cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool
 cudaError_t launch_fan_lut(const FanLutArgs& a, int blocks, cudaStream_t st, bool early = false);
 cudaError_t launch_fan_group(const FanGroupArgs& a, int blocks, cudaStream_t st, bool early = false);
 cudaError_t launch_adj_rows(const SensorDev* sensors, const int32_t* row_map, const SensorDev& one,
-                            int64_t total_groups, int normalise, const float* noised,
+                            int64_t total_groups, int normalise, bool aligned, const float* noised,
                             const float* grad, RowInfo* info, int32_t* zero_word, cudaStream_t st, bool early = false);
+// `aligned`: I~ and G start on 16-byte boundaries (their rows then may, and are read as vectors where they do).
 // `early` for the gather, and `early_final` for the final sum after it.
 cudaError_t launch_adjoint(const AdjArgs& a, int grid, int block, size_t smem, float* dtheta, cudaStream_t st,
                            bool early = false, bool early_final = false);

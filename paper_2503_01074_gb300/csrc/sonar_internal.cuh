@@ -332,6 +332,7 @@ struct NormArgs {
     const float* noised;
     const uint32_t* gmax;       // normalise = 2: ordered-encoded image maximum at rowmax_off
     int32_t normalise;
+    int32_t vec;                // both images start on a 16-byte boundary
     float* polar;
 };
 

@@ -76,3 +76,58 @@ def test_bins_that_are_not_finite(env, naz, mode, value):
     with np.errstate(invalid="ignore"):
         want = np.where(top > 0, I / top, I)
     assert np.array_equal(N, want, equal_nan=True)
+
+
+def off_by_one(n, like=None):
+    """n floats that start four bytes past a 16-byte boundary."""
+    v = torch.zeros(n + 1, device="cuda")[1:]
+    assert v.data_ptr() % 16 == 4
+    return v if like is None else v.copy_(like.reshape(-1))
+
+
+# rows in registers by pairs and alone, in two passes, no multiple of 4; one and two rows per warp of the adjoint
+@pytest.mark.parametrize("nr,naz", [(60, 64), (41, 512), (33, 516), (20, 1024), (20, 1028), (30, 61), (7000, 64)])
+@pytest.mark.parametrize("mode", [1, 2])
+def test_images_off_the_16_byte_boundary(env, nr, naz, mode):
+    """Images and gradients may start at any float.  Forward: the same images, bit for
+    bit.  Adjoint: the same gradient, since one nonzero element of G per row (per
+    image with whole-image normalisation) leaves no order of summation in its row terms."""
+    son, mu, sid = env
+    theta, prm = son.theta(0.05, 1.3, mu), RenderParams(normalise=mode)
+    items = [(sid, spec(64, 16, nr, naz).replace_pose((0.1 * k, 0.0, 0.0), S.pose_matrix(0.1, math.radians(40.0))), 5, k)
+             for k in range(3)]
+    _, sp, seed, frame = items[0]
+    n = nr * naz
+    rng = np.random.default_rng(1)
+    G = np.zeros((3, nr, naz), np.float32)
+    for k in range(3):
+        for row in range(nr) if mode == 1 else (int(rng.integers(nr)),):
+            G[k, row, rng.integers(naz)] = rng.uniform(0.5, 2.0)
+    G = torch.from_numpy(G).to(son.device)
+
+    one = son.render(sid, sp, theta, prm, seed, frame, hits=True, fan=False)
+    views = {key: off_by_one(n).view(nr, naz) for key in ("polar", "noised")}
+    got = son.render(sid, sp, theta, prm, seed, frame, hits=True, fan=False, outputs=dict(views))
+    assert torch.equal(got["polar"], one["polar"]) and torch.equal(got["noised"], one["noised"])
+    d = son.backward(sid, sp, theta, prm, seed, frame, G[0].contiguous(), one["noised"], one["hits"])
+    for g, x in ((off_by_one(n, G[0]), one["noised"]), (G[0].contiguous(), views["noised"]),
+                 (off_by_one(n, G[0]), views["noised"])):
+        assert torch.equal(son.backward(sid, sp, theta, prm, seed, frame, g.view(nr, naz), x, one["hits"]), d)
+
+    b, c = son.batch(items), son.batch(items)
+    c.polar, c.noised = off_by_one(3 * n), off_by_one(3 * n)
+    grads = []
+    for x, g in ((b, G.reshape(-1)), (c, off_by_one(3 * n, G))):
+        x.render(theta, prm, fan=False)
+        grads.append(x.backward(theta, prm, g).clone())
+        grads.append(x.step(theta, prm, g, fan=False).clone())
+    torch.cuda.synchronize()
+    assert torch.equal(b.polar, c.polar) and torch.equal(b.noised, c.noised)
+    assert torch.isfinite(grads[0]).all()
+    if mode == 1:   # one element of a whole image may lie where nothing returned
+        assert grads[0].abs().max() > 0
+    assert all(torch.equal(g, grads[0]) for g in grads[1:])
+    b.close()
+    c.close()
+    st, bits = son.check()
+    assert st == 0 and bits == 0
