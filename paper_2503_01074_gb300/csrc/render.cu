@@ -904,15 +904,17 @@ __global__ void __launch_bounds__(256) k_fan_lut(const __grid_constant__ FanLutA
     let_next_start();
     __shared__ SensorDev S;
     __shared__ int s_blk;
+    __shared__ bool s_current;
     __shared__ uint4* s_lut;
     if (threadIdx.x == 0) {
         const int2 m = a.block_map[blockIdx.x];
         S = a.sensors[m.x];
         s_blk = m.y;
         s_lut = a.luts[m.x];
+        s_current = S.fan_stamp && S.fan_stamp[m.y] == S.fan_version;   // read once for all (see k_trig)
     }
     __syncthreads();
-    if (S.fan_stamp && S.fan_stamp[s_blk] == S.fan_version) {   // block-uniform
+    if (s_current) {
         wait_for_previous();
         return;
     }

@@ -160,11 +160,15 @@ __device__ __noinline__ ExactPair exact_pair(const SensorDev& s, const float4* t
 // (computed in FP64 once per sensor, split into hi + lo floats): trig[i] for
 // beams, trig[N_b + j] for elevations, each (sin hi, sin lo, cos hi, cos lo).
 __global__ void k_trig(const SensorDev* sensors, SensorDev one) {
+    __shared__ bool s_current;
     let_next_start();
     const SensorDev& s = sensors ? sensors[blockIdx.y] : one;
     // a batch block whose entries were built for the sensor's current fields of
-    // view has nothing to do (block-uniform; only later launches read the table)
-    if (s.trig_stamp && s.trig_stamp[blockIdx.x] == s.trig_version) return;
+    // view has nothing to do (only later launches read the table).  One thread reads
+    // the stamp for all: a warp that read it after it was written would skip its entries
+    if (threadIdx.x == 0) s_current = s.trig_stamp && s.trig_stamp[blockIdx.x] == s.trig_version;
+    __syncthreads();
+    if (s_current) return;
     if (s.trig_stamp && threadIdx.x == 0) s.trig_stamp[blockIdx.x] = s.trig_version;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= s.nb + s.ne) return;

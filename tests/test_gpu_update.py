@@ -111,3 +111,32 @@ def test_update_to_a_scene_without_an_8_wide_tree(son, variant, n):
     b.close()
     st, bits = son.check()
     assert st == 0 and bits == 0
+
+
+def test_tables_follow_every_change_of_the_fields_of_view(son):
+    """Changes of the fields of view one after another: every block of the exact-ray and
+    of the fan coordinate tables is built whole each time (a block whose stamp is
+    current has nothing to do, and no warp of it may see the stamp of its own build)."""
+    theta, prm = son.theta(0.05, 1.0, MU), RenderParams()
+    sid = son.upload_mesh(S.random_soup(3000, 9))
+    base = S.SensorSpec(np.zeros(3, np.float32), S.pose_matrix(0.1, math.radians(15)), 200, 90, 64, 128,
+                        math.radians(90.0), math.radians(40.0), 0.5, 20.0, 211, 130)
+    n = 16   # all alike: one shared fan table
+    b = son.batch(frames(sid, n, base))
+    for k in range(12):
+        spec = base.replace_pose(base.pos, base.rot)
+        if k % 4 != 3:   # the last of four is the one before: nothing to rebuild
+            spec.hfov, spec.vfov = base.hfov * (1.0 - 0.02 * k), base.vfov * (1.0 - 0.015 * k)
+        else:
+            spec.hfov, spec.vfov = last.hfov, last.vfov
+        last = spec
+        items = frames(sid, n, spec)
+        b.update(items)
+        b.render(theta, prm)
+        torch.cuda.synchronize()
+        for q in (0, n // 2, n - 1):
+            _, sp, seed, frame = items[q]
+            one = son.render(sid, sp, theta, prm, seed, frame, hits=True, fan=True)
+            got = b.view(q)
+            assert all(torch.equal(one[key], got[key]) for key in ("hits", "polar", "fan")), (k, q)
+    b.close()
