@@ -64,7 +64,10 @@ sonar_status fail(sonar_ctx* ctx, sonar_status st, const std::string& msg) {
     return st;
 }
 
+// The runtime keeps a failed call's error until it is read, and the next launch that
+// looks (cudaGetLastError) would report it again: taken here, where it is reported.
 sonar_status cuda_fail(sonar_ctx* ctx, cudaError_t e, const char* what) {
+    cudaGetLastError();
     return fail(ctx, e == cudaErrorMemoryAllocation ? SONAR_ERR_OOM : SONAR_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -1131,6 +1134,13 @@ void append_bytes(std::vector<unsigned char>& v, const T& x) {
     v.insert(v.end(), p, p + sizeof(T));
 }
 
+// The end of a capture whose launches failed with `st`, already reported.
+sonar_status capture_failed(cudaGraph_t g, sonar_status st) {
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();   // what ending the broken capture left
+    return st;
+}
+
 // Records phase event `ev` after what stream `s` (being captured) holds so far, on
 // a branch of its own: the next kernel then follows the last one directly, and
 // may start early.
@@ -1396,7 +1406,7 @@ extern "C" sonar_status sonar_render_batch(sonar_batch_t b, const sonar_params* 
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(b->cap, &g);
         if (e == cudaSuccess) e = ej;
-        if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
+        if (st != SONAR_OK) return capture_failed(g, st);
         CU(e, "graph capture");
         (lean ? b->fwd_lean_kernels : b->fwd_kernels) = kernel_nodes(g);
         const cudaError_t e2 = cudaGraphInstantiate(&exec, g, 0);
@@ -1511,7 +1521,7 @@ extern "C" sonar_status sonar_render_batch_backward(sonar_batch_t b, const sonar
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(b->cap, &g);
         if (e == cudaSuccess) e = ej;
-        if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
+        if (st != SONAR_OK) return capture_failed(g, st);
         CU(e, "graph capture");
         b->bwd_kernels = kernel_nodes(g);
         const cudaError_t e2 = cudaGraphInstantiate(&b->bwd, g, 0);
@@ -1587,8 +1597,8 @@ extern "C" sonar_status sonar_render_batch_step(sonar_batch_t b, const sonar_par
         if (e == cudaSuccess) e = e5;
         cudaGraph_t g = nullptr;
         const cudaError_t e3 = cudaStreamEndCapture(b->cap, &g);
-        if (st != SONAR_OK) { if (g) cudaGraphDestroy(g); return st; }
-        if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(ctx, e, "graph fork"); }
+        if (st != SONAR_OK) return capture_failed(g, st);
+        if (e != cudaSuccess) return capture_failed(g, cuda_fail(ctx, e, "graph fork"));
         CU(e3, "graph capture");
         b->step_kernels = kernel_nodes(g);
         const cudaError_t e6 = cudaGraphInstantiate(&b->step, g, 0);
