@@ -350,7 +350,8 @@ sonar_status sonar_batch_destroy(sonar_batch_t batch);
  * fastest per sensor shape (n_beams, n_elev, n_range_bins, n_az_bins) in the
  * context's tuning cache; later sonar_batch_create and sonar_render calls use
  * it.  Stage 1 times the forward launches over the ray-cast warp tiles (beams
- * x elevations per warp) and register variants; stage 2, when `out` holds hit
+ * x elevations per warp) and variants (a batch small enough for several lanes per
+ * ray, whose launches go by none of these, keeps flag 8); stage 2, when `out` holds hit
  * records and I~, times the adjoint's block size on the forward launches plus
  * the adjoint of a constant upstream gradient.  Each candidate scores the best of 3 rounds
  * of 3 passes.  Runs on `stream` and synchronises it; allocates and frees its

@@ -1760,6 +1760,11 @@ extern "C" sonar_status sonar_autotune(sonar_batch_t b, const sonar_params* p, c
             for (int tb : {1, 2, 4, 8, 16, 32}) {
                 ctx->tune[k] = Tune{1, tb, 128, occ};
                 if ((st = batch_plan(b)) != SONAR_OK) goto restore;
+                // a launch small enough for several lanes per ray does not go by the row's
+                // variant: four equal launches would leave it to noise.  The row, which
+                // later and larger batches of the shape go by, keeps the variant that
+                // those default to
+                if (occ != kTraceCap && group_lanes(ctx, b->trace_prefix.back())) continue;
                 if (batch_scratch(b, out) != cudaSuccess) { st = fail(ctx, SONAR_ERR_OOM, "batch scratch"); goto restore; }
                 const float ms = time_batch(b, p, d_theta, n_mat, out, nullptr, nullptr, s, 3, 3);
                 if (cudaGetLastError() != cudaSuccess) continue;
