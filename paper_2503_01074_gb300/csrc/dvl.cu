@@ -229,8 +229,7 @@ __global__ void __launch_bounds__(4 * kDvlPoses) k_dvl(const __grid_constant__ D
 // 0, then max(1, ceil(period / dt)) steps after each measurement), a chunk of
 // steps at a time: the lanes turn the chunk's periods into step counts in shared
 // memory, lane 0 walks those, and the chunk is written as whole rows.
-// 4096 vehicles x 256 steps: 17 us, against 78 us with a thread per vehicle that
-// clears, reads and marks its row alone.
+// 4096 vehicles x 256 steps: 17 us, against 78 us with a thread per vehicle (below).
 constexpr int kSchedWarps = 4, kSchedChunk = 256;
 __global__ void __launch_bounds__(32 * kSchedWarps) k_dvl_schedule(const float* period, int64_t n_veh, int64_t n_steps,
                                                                    float dt, int32_t* emit) {
@@ -267,6 +266,31 @@ __global__ void __launch_bounds__(32 * kSchedWarps) k_dvl_schedule(const float* 
     }
 }
 
+// The same, a thread per vehicle that clears, walks and marks its row alone: short
+// schedules of many vehicles, where a warp per vehicle leaves most of its lanes idle.
+// Bound by the chain of a row's loads, then by its scattered stores.
+__global__ void __launch_bounds__(128) k_dvl_schedule_short(const float* period, int64_t n_veh, int64_t n_steps,
+                                                            float dt, int32_t* emit) {
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n_veh) return;
+    const float* P = period + v * n_steps;
+    int32_t* E = emit + v * n_steps;
+    for (int64_t s = 0; s < n_steps; ++s) E[s] = 0;
+    for (int64_t s = 0; s < n_steps;) {
+        E[s] = 1;
+        const float q = ceilf(P[s] / dt);
+        s += q >= 1.0f ? (int64_t)fminf(q, 4.0e18f) : 1;
+    }
+}
+
+// Which of the two: measured by warps -> by threads, periods of 1, 4 and 20 steps:
+// 1,048,576 vehicles x 1 step 150 -> 12, 151 -> 12, 151 -> 11 us; x 16 413 -> 140, 205 ->
+// 92, 156 -> 80; x 48 1017 -> 577, 396 -> 358, 250 -> 323; x 64 1280 -> 844, 458 -> 445, 269 ->
+// 389; 100,000 x 32 70 -> 50, 29 -> 28, 19 -> 23; 32,768 x 48 37 -> 25, 16 -> 15, 10 -> 14;
+// 4,096 x 32 by warps 7, by threads 14 with every step a measurement (one
+// row's chain of loads).
+constexpr int64_t kShortSteps = 48, kShortVehicles = 32768;
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -280,7 +304,9 @@ cudaError_t launch_dvl(const DvlArgs& a, cudaStream_t st) {
 
 cudaError_t launch_dvl_schedule(const float* period, int64_t n_veh, int64_t n_steps, float dt, int32_t* emit,
                                 cudaStream_t st) {
-    if (n_veh > 0 && n_steps > 0) 
+    if (n_veh >= kShortVehicles && n_steps <= kShortSteps && n_steps > 0)
+        k_dvl_schedule_short<<<(unsigned)((n_veh + 127) / 128), 128, 0, st>>>(period, n_veh, n_steps, dt, emit);
+    else if (n_veh > 0 && n_steps > 0)
         k_dvl_schedule<<<(unsigned)((n_veh + kSchedWarps - 1) / kSchedWarps), 32 * kSchedWarps, 0, st>>>(
             period, n_veh, n_steps, dt, emit);
     return cudaGetLastError();
