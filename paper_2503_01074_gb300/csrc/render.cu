@@ -319,7 +319,8 @@ __device__ __forceinline__ float div_by(float v, float m, float y) {
 // REG > 0: a row of up to 128 REG bins stays in registers between its maximum
 // and the division, so I~ and N are written and nothing is read back; REG = 0
 // (wider rows, and the dense form of the fold's result): I~ is written, then read
-// back by the same lanes and divided.
+// back by the same lanes and divided.  Where such rows are few, a block's warps share
+// one (rows_per_block 1): a warp alone takes some 10 ns a bin, 95 us for 8192.
 //
 // Bound by instruction issue (about 75 per bin, most of them the logarithm and a
 // quarter of a Philox block): 64 frames of 1000 x 512 bins in 92 us, 2.8 TB/s of
@@ -331,8 +332,11 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
     extern __shared__ __align__(16) uint32_t rows_smem[];
     __shared__ SensorDev S;
     __shared__ int s_row0;
+    __shared__ float s_top[8];
     let_next_start();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool shared_row = REG == 0 && a.rows_per_block == 1;   // by all warps of the block
+    const int q0 = shared_row ? warp : 0, dq = shared_row ? 8 : 1;   // a lane's quads: q0, q0 + dq, ...
     if (warp == 0) {
         // the rows run from the last sensor back to the first, so that the first
         // sensors' N is the last written and the fan finds it in L2
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
     const uint32_t flo = S.frame_lo, fhi = S.frame_hi;
     const float2* vals = a.vals + S.val_off;
     float image_max = -CUDART_INF_F;
-    for (int r = warp; r < a.rows_per_block; r += 8) {
+    for (int r = shared_row ? 0 : warp; r < a.rows_per_block; r += 8) {
         const int row = row0 + r;
         if (row >= nr) break;
         const uint32_t b0 = (uint32_t)row * (uint32_t)naz;
@@ -494,7 +498,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                 }
             }
         } else {
-            for (int k = 0; k < nk; ++k) {
+            for (int k = q0; k < nk; k += dq) {
                 float v[4], p[4];
                 quad(k, v, p);
                 if (a.binned) store(a.binned + off, k, p);
@@ -502,8 +506,14 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
                 m = fmaxf(m, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
             }
             for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            if (shared_row) {
+                if (lane == 0) s_top[warp] = m;
+                __syncthreads();   // the block has one row, and all its warps are here
+#pragma unroll
+                for (int w = 0; w < 8; ++w) m = fmaxf(m, s_top[w]);
+            }
             if (mode != 2) {
-                for (int k = 0; k < nk; ++k) {
+                for (int k = q0; k < nk; k += dq) {
                     float v[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {

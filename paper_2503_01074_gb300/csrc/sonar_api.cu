@@ -209,8 +209,12 @@ int fold_warps(const SensorDev& s) {
 }
 
 // Rows per block of the row kernel: a whole band of 32, which reads the band's
-// column tables once, while that leaves at least eight blocks an SM; else 16 or 8.
-int rows_per_block(int64_t total_rows, int sm_count) {
+// column tables once, while that leaves at least eight blocks an SM; else 16 or 8.  A
+// launch of few rows, some of them wider than a warp's registers hold, takes a block
+// a row: a frame of 1 x 8192 bins 94 -> 35 us, 9 x 9000 some 95 -> 35, 500 x 1100 30 -> 29, 500 x
+// 20000 231 -> 82; 1000 x 1100 would take 35 instead of 31.
+int rows_per_block(int64_t total_rows, int max_naz, int sm_count) {
+    if (max_naz > 1024 && total_rows < 4ll * sm_count) return 1;
     for (int r : {32, 16})
         if (total_rows / r >= 8ll * sm_count) return r;
     return 8;
@@ -482,7 +486,7 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
                    !capturing && !f.dense),
        "fold launch");
     RowsArgs r{};
-    r.rows_per_block = rows_per_block(S.nr, ctx->sm_count);
+    r.rows_per_block = rows_per_block(S.nr, S.naz, ctx->sm_count);
     r.one = S;
     r.params = *p;
     r.vals = f.vals;
@@ -899,7 +903,7 @@ sonar_status batch_plan(sonar_batch* b) {
     b->fold_block = 32 * warps;
     b->fold_words_per_warp = (int)warp_words;
     b->fold_smem = sizeof(uint32_t) * (size_t)std::max(block_words, warps * warp_words);
-    b->rows_step = rows_per_block(rows, ctx->sm_count);
+    b->rows_step = rows_per_block(rows, b->max_naz, ctx->sm_count);
     for (int k = 0; k < n; ++k) {
         const SensorDev& S = b->hs[k];
         const int step = S.fold_beams ? 1 : warps;

@@ -310,7 +310,8 @@ struct FoldArgs {
 struct RowsArgs {
     const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
     const int2* block_map;      // batch: per block (sensor, first row)
-    int32_t rows_per_block;     // 8, 16 or 32 (a block's rows lie in one band of 32)
+    int32_t rows_per_block;     // 8, 16 or 32 (a block's rows lie in one band of 32), or 1:
+                                // few rows of more than 1024 bins, a block on each
     SensorDev one;
     sonar_params params;
     const float2* vals;

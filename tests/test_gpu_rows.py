@@ -1,5 +1,5 @@
 """The row kernel (noise, range-wise normalisation): launches that its widest
-sensor alone does not describe, and bins that are not finite.
+sensor alone does not describe, bins that are not finite, rows that a block shares.
 """
 import math
 
@@ -131,3 +131,23 @@ def test_images_off_the_16_byte_boundary(env, nr, naz, mode):
     c.close()
     st, bits = son.check()
     assert st == 0 and bits == 0
+
+
+# a block a row, its last quads of fewer than a warp's or a block's: below and above the limit of four rows per SM
+@pytest.mark.parametrize("nr,naz", [(1, 1025), (1, 1028), (3, 4095), (33, 1151), (9, 8192), (2, 8193), (607, 1030), (609, 1032)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_rows_shared_by_a_block(env, nr, naz, mode):
+    """The same rows in a batch that has too many for a block each (a warp a row)."""
+    son, mu, sid = env
+    theta, prm = son.theta(0.05, 1.3, mu), RenderParams(normalise=mode)
+    sp = spec(50, 12, nr, naz)
+    one = son.render(sid, sp, theta, prm, 3, 4, hits=True, fan=False, binned=True)
+    b = son.batch([(sid, sp, 3, 4)] + [(sid, spec(1, 1, 700, 2), 3, 4)])
+    b.render(theta, prm, fan=False, binned=True)
+    torch.cuda.synchronize()
+    got = b.view(0)
+    for key in ("hits", "binned", "noised", "polar"):
+        assert torch.equal(one[key], got[key]), key
+    top = {0: torch.ones(1, device=son.device), 1: one["noised"].amax(1, keepdim=True), 2: one["noised"].max()}[mode]
+    assert torch.equal(one["polar"], one["noised"] / top)
+    b.close()
