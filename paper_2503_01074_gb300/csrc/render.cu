@@ -292,6 +292,7 @@ __device__ __forceinline__ float pattern_of(const SensorDev& S, int col, float d
     return 0.5f * expf(-pc * pc * inv_sphi);
 }
 
+// A bin of a row or image of maximum m (which is not divided where it is not positive).
 __device__ __forceinline__ float norm_value(float In, float m, int mode) {
     return (mode != 0 && m > 0.0f) ? In / m : In;
 }
@@ -542,122 +543,91 @@ __global__ void __launch_bounds__(256) k_philox_words(const uint4* ctr, int64_t 
 }
 
 // ---------------------------------------------------------------------------
-// phase 2a: range-wise normalisation, one warp per (sensor, range row)
+// phase 2a: whole-image normalisation
 // ---------------------------------------------------------------------------
 
-// One row: its maximum over azimuth and N = I~ / max (any alignment and width).
-__device__ __forceinline__ void norm_row(const NormArgs& a, int64_t g, int lane) {
-    const SensorDev& s = a.sensors ? a.sensors[a.row_map[g]] : a.one;
-    const int row = (int)(g - s.rowmax_off);
-    const int naz = s.naz;
-    const float* In = a.noised + s.polar_off + (int64_t)row * naz;
-    float* out = a.polar + s.polar_off + (int64_t)row * naz;
-    float m = 0.0f;
-    if (a.vec && ((s.polar_off | naz) & 3) == 0 && naz <= 1024) {
-        // 16-byte rows of up to 1024 bins: the row stays in registers between
-        // the maximum and the division (one read of I~)
-        const int n4 = naz >> 2;
-        const float4* In4 = reinterpret_cast<const float4*>(In);
-        float4* out4 = reinterpret_cast<float4*>(out);
-        float4 v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int q = lane + 32 * k;
-            v[k] = q < n4 ? In4[q] : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
-        }
-        if (a.normalise == 1) {
-            m = -CUDART_INF_F;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) m = fmaxf(fmaxf(m, fmaxf(v[k].x, v[k].y)), fmaxf(v[k].z, v[k].w));
-            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        } else if (a.normalise == 2) {
-            m = ord_dec(a.gmax[s.rowmax_off]);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int q = lane + 32 * k;
-            if (q < n4)
-                out4[q] = make_float4(norm_value(v[k].x, m, a.normalise), norm_value(v[k].y, m, a.normalise),
-                                      norm_value(v[k].z, m, a.normalise), norm_value(v[k].w, m, a.normalise));
-        }
-        return;
-    }
-    if (a.normalise == 1) {
-        m = -CUDART_INF_F;
-        for (int j = lane; j < naz; j += 32) m = fmaxf(m, In[j]);
-        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    } else if (a.normalise == 2) {
-        m = ord_dec(a.gmax[s.rowmax_off]);
-    }
-    for (int j = lane; j < naz; j += 32) out[j] = norm_value(In[j], m, a.normalise);
-}
-
-// One warp per pair of adjacent range rows, the pairs from the last to the
-// first: the binning kernel wrote the last sensors' I~ last, so the first rows
-// read here are still in L2, and the first sensors' N, written last, are in L2
-// when the fan starts on them.  A row of 16-byte-aligned bins, at most 512 of
-// them, stays in registers between its maximum and the division, and both rows'
-// loads are issued before either reduction (4 KB in flight per warp); other
-// rows go one at a time (in registers up to 1024 aligned bins, else in two
-// passes).
+// N = I~ / max of the image, rows of up to 1024 16-byte-aligned bins: one warp per pair
+// of adjacent rows, the pairs from the last to the first (the row kernel went the same
+// way, so the first rows, written last, are in L2, and so is N for the fan).  Rows of up
+// to 512 bins are loaded both before either is stored (4 KB in flight per warp), wider
+// ones go one after the other.
 __global__ void __launch_bounds__(256, 4) k_norm_rows(const __grid_constant__ NormArgs a) {
     let_next_start();
-    wait_for_previous();
-    constexpr int kV = 4;   // float4 per lane: rows of up to 512 bins
+    wait_for_previous();   // I~ and its maximum
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t pairs = (a.total_rows + 1) >> 1;
     if (t >= pairs) return;
     const int64_t g0 = 2 * (pairs - 1 - t);
-    float4 v[2][kV];
-    float4* out4[2] = {nullptr, nullptr};
+    const int rows = (int)min((int64_t)2, a.total_rows - g0);
+    float4 v[8];
+    const float4* in[2];
+    float4* out[2];
     int n4[2] = {0, 0};
-    bool fast[2] = {false, false};
-    int64_t rowmax_off[2] = {0, 0};
+    float m[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int64_t g = g0 + r;
-        if (g >= a.total_rows) continue;
-        const SensorDev& s = a.sensors ? a.sensors[a.row_map[g]] : a.one;
-        const int naz = s.naz;
-        if (!a.vec || ((s.polar_off | naz) & 3) != 0 || naz > 32 * 4 * kV) continue;
-        const int64_t off = s.polar_off + (int64_t)(g - s.rowmax_off) * naz;
-        const float4* In4 = reinterpret_cast<const float4*>(a.noised + off);
-        out4[r] = reinterpret_cast<float4*>(a.polar + off);
-        n4[r] = naz >> 2;
-        fast[r] = true;
-        rowmax_off[r] = s.rowmax_off;
+        if (r >= rows) continue;
+        const SensorDev& s = a.sensors ? a.sensors[a.row_map[g0 + r]] : a.one;
+        const int64_t off = s.polar_off + (g0 + r - s.rowmax_off) * s.naz;
+        in[r] = reinterpret_cast<const float4*>(a.noised + off);
+        out[r] = reinterpret_cast<float4*>(a.polar + off);
+        n4[r] = s.naz >> 2;
+        m[r] = ord_dec(a.gmax[s.rowmax_off]);
+    }
+    auto divided = [](float4 x, float top) {
+        return make_float4(norm_value(x.x, top, 2), norm_value(x.y, top, 2), norm_value(x.z, top, 2), norm_value(x.w, top, 2));
+    };
+    if (max(n4[0], n4[1]) <= 128) {
 #pragma unroll
-        for (int k = 0; k < kV; ++k) {
-            const int q = lane + 32 * k;
-            v[r][k] = q < n4[r] ? In4[q]
-                                : make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+        for (int k = 0; k < 8; ++k) {
+            const int r = k >> 2, q = lane + 32 * (k & 3);
+            if (q < n4[r]) v[k] = in[r][q];
         }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int r = k >> 2, q = lane + 32 * (k & 3);
+            if (q < n4[r]) out[r][q] = divided(v[k], m[r]);
+        }
+        return;
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int64_t g = g0 + r;
-        if (g >= a.total_rows) continue;
-        if (!fast[r]) {
-            norm_row(a, g, lane);
-            continue;
-        }
-        float m = 0.0f;
-        if (a.normalise == 1) {
-            m = -CUDART_INF_F;
 #pragma unroll
-            for (int k = 0; k < kV; ++k) m = fmaxf(fmaxf(m, fmaxf(v[r][k].x, v[r][k].y)), fmaxf(v[r][k].z, v[r][k].w));
-            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        } else if (a.normalise == 2) {
-            m = ord_dec(a.gmax[rowmax_off[r]]);
-        }
+        for (int k = 0; k < 8; ++k)
+            if (lane + 32 * k < n4[r]) v[k] = in[r][lane + 32 * k];
 #pragma unroll
-        for (int k = 0; k < kV; ++k) {
-            const int q = lane + 32 * k;
-            if (q < n4[r])
-                out4[r][q] = make_float4(norm_value(v[r][k].x, m, a.normalise), norm_value(v[r][k].y, m, a.normalise),
-                                         norm_value(v[r][k].z, m, a.normalise), norm_value(v[r][k].w, m, a.normalise));
-        }
+        for (int k = 0; k < 8; ++k)
+            if (lane + 32 * k < n4[r]) out[r][lane + 32 * k] = divided(v[k], m[r]);
+    }
+}
+
+// The same for rows of any width and alignment: one warp per run of 512 bins of a row
+// (every a.runs-th run of it).  A frame of 50 x 20000 bins 523 us with a warp per pair
+// of rows, 46 with this; 64 frames of 1000 x 511 333 -> 245; 64 frames of 1000 x 512, which
+// the kernel above takes, 175 there and 184 here.
+__global__ void __launch_bounds__(256) k_norm_runs(const __grid_constant__ NormArgs a) {
+    let_next_start();
+    wait_for_previous();   // I~ and its maximum
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (t >= a.total_rows * a.runs) return;
+    const int64_t g = a.total_rows - 1 - t / a.runs;
+    const SensorDev& s = a.sensors ? a.sensors[a.row_map[g]] : a.one;
+    const int naz = s.naz;
+    const int64_t off = s.polar_off + (g - s.rowmax_off) * naz;
+    const float* In = a.noised + off;
+    float* out = a.polar + off;
+    const float m = ord_dec(a.gmax[s.rowmax_off]);
+#pragma unroll 1
+    for (int64_t j = 512 * (t % a.runs) + lane; j < naz; j += 512ll * a.runs) {
+        float v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (j + 32 * k < naz) v[k] = In[j + 32 * k];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (j + 32 * k < naz) out[j + 32 * k] = norm_value(v[k], m, 2);
     }
 }
 
@@ -1281,8 +1251,8 @@ cudaError_t launch_philox(const void* ctr, int64_t n, uint32_t k0, uint32_t k1, 
 }
 
 cudaError_t launch_norm(const NormArgs& a, cudaStream_t st, bool early) {
-    const int64_t threads = ((a.total_rows + 1) / 2) * 32;   // a warp per pair of rows
-    return launch_kernel(k_norm_rows, (unsigned)((threads + 255) / 256), 256, 0, st, early, a);
+    const int64_t warps = a.runs ? a.total_rows * a.runs : (a.total_rows + 1) / 2;
+    return launch_kernel(a.runs ? k_norm_runs : k_norm_rows, (unsigned)((warps + 7) / 8), 256, 0, st, early, a);
 }
 
 cudaError_t launch_fan_tiles(const FanArgs& a, int blocks, cudaStream_t st, bool early) {

@@ -223,6 +223,15 @@ int rows_per_block(int64_t total_rows, int max_naz, int sm_count) {
 // Azimuth bins of a sensor whose column tables the row kernel keeps in shared memory, or 0.
 int staged_naz(const SensorDev& s) { return s.naz <= kRowsStaged ? s.naz : 0; }
 
+// Warps per row of the whole-image normalisation: none (a warp per pair of rows) where
+// every row is up to 1024 bins on 16-byte boundaries, else one for every 512 bins of the
+// widest row, as far as a launch of 2^24 warps goes.
+int norm_runs(int max_naz, int64_t total_rows, bool vec) {
+    if (vec && max_naz <= 1024) return 0;
+    const int64_t runs = ((int64_t)max_naz + 511) / 512;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(runs, (1ll << 24) / total_rows));
+}
+
 SensorDev make_sensor(const sonar_sensor& s, uint64_t seed, uint64_t frame, const Tune& t, int fan_w,
                       int fan_h) {
     SensorDev d{};
@@ -511,8 +520,7 @@ sonar_status single_post(sonar_ctx* ctx, const SensorDev& S, int normalise, cons
         n.total_rows = S.nr;
         n.noised = noised;
         n.gmax = gmax;
-        n.normalise = normalise;
-        n.vec = aligned16(noised) && aligned16(polar);
+        n.runs = norm_runs(S.naz, S.nr, S.naz % 4 == 0 && aligned16(noised) && aligned16(polar));
         n.polar = polar;
         CU(launch_norm(n, s, !capturing), "normalisation launch");
     }
@@ -1222,8 +1230,7 @@ sonar_status batch_forward_launches(sonar_batch* b, const sonar_params* p, const
         c.total_rows = b->total_rows;
         c.noised = out->noised ? out->noised : b->d_noised;
         c.gmax = b->d_rowmax;
-        c.normalise = p->normalise;
-        c.vec = aligned16(c.noised) && aligned16(out->polar);
+        c.runs = norm_runs(b->max_naz, b->total_rows, b->rows_vec && aligned16(c.noised) && aligned16(out->polar));
         c.polar = out->polar;
         CU(launch_norm(c, s, true), "batch normalisation launch");
     }

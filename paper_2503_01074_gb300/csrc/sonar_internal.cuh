@@ -323,7 +323,7 @@ struct RowsArgs {
     uint32_t* gmax;             // normalise = 2: ordered-encoded image maximum per sensor
 };
 
-// Whole-image normalisation: one warp per pair of range rows.
+// Whole-image normalisation: one warp per pair of range rows, or per run of bins of a row.
 struct NormArgs {
     const SensorDev* sensors;   // batch: device array; single: nullptr (use `one`)
     const int32_t* row_map;     // batch: sensor of each row
@@ -331,9 +331,8 @@ struct NormArgs {
     int64_t total_rows;         // sum of n_range_bins over the sensors
     SensorDev one;
     const float* noised;
-    const uint32_t* gmax;       // normalise = 2: ordered-encoded image maximum at rowmax_off
-    int32_t normalise;
-    int32_t vec;                // both images start on a 16-byte boundary
+    const uint32_t* gmax;       // ordered-encoded image maximum at rowmax_off
+    int32_t runs;               // warps per row; 0: rows of up to 1024 aligned bins, a warp per pair
     float* polar;
 };
 
