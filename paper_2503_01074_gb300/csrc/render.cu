@@ -171,7 +171,8 @@ __device__ __forceinline__ void sum_rows(const FoldArgs& a, const ExactDiv& div,
 
 // One warp per azimuth column (sensors with at most one beam per column, and
 // those whose per-beam rows do not fit in shared memory), or one block per
-// column with its warps on the column's beams (S.fold_beams).
+// column (S.fold_block): its warps on the column's beams (S.fold_beams), or, where few
+// columns hold many rays, all of them in pass 1 and one in pass 2.
 //
 // Only the bins that a ray lands in (about 6 % of them) are stored: pass 1 marks
 // the column's rows with returns in a bitmap, a prefix over its words ranks
@@ -207,14 +208,14 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
         } else {
             copy_param(&S, &a.one, lane);
             copy_param(&SC, &a.one_scene, lane);
-            if (lane == 0) s_col = blockIdx.x * (a.one.fold_beams ? 1 : nw);
+            if (lane == 0) s_col = blockIdx.x * (a.one.fold_block ? 1 : nw);
         }
     }
     __syncthreads();
     const float alpha = __ldg(a.theta), gain = __ldg(a.theta + 1);
     const ExactDiv div = exact_div((uint32_t)S.naz);
     const int ne = S.ne, nwords = (S.nr + 31) >> 5;
-    const int col = s_col + (S.fold_beams ? 0 : warp);
+    const int col = s_col + (S.fold_block ? 0 : warp);
     if (col >= S.naz) return;   // whole warps only (the last block of a sensor)
     const int i0 = first_beam_of_col(col, S.nb, S.naz), i1 = first_beam_of_col(col + 1, S.nb, S.naz);
     const int64_t first = (int64_t)i0 * ne;          // the column's first ray, and its first value slot
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
     const sonar_hit* H = a.hits + S.hits_off + first;
     const int most = min(S.nr, n);                   // bins with returns, at most
     wait_for_previous();   // the hit records
-    if (!S.fold_beams) {
+    if (!S.fold_block) {
         uint32_t* bits = fold_smem + (int64_t)warp * a.words_per_warp;
         uint32_t* pre = bits + nwords;
         float* acc = reinterpret_cast<float*>(pre + nwords);
@@ -241,13 +242,13 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
                 a.bands[S.band_off + (int64_t)w * S.naz + col] = make_uint2(bits[w], (uint32_t)first + pre[w]);
         return;
     }
-    // per-beam form: each beam sums its own rows in elevation order, a bin then
-    // adds its column's beams in beam order
-    const int nbeam = i1 - i0, nt = blockDim.x;
+    // block form: each part (a beam, in elevation order; or the whole column) sums its own
+    // rows, a bin then adds its column's parts in order
+    const int parts = S.fold_beams ? i1 - i0 : 1, len = S.fold_beams ? ne : n, nt = blockDim.x;
     uint32_t* bits = fold_smem;
     uint32_t* pre = bits + nwords;
     int* rows = reinterpret_cast<int*>(pre + nwords);
-    float* acc = reinterpret_cast<float*>(rows + most);   // [nbeam][nd]
+    float* acc = reinterpret_cast<float*>(rows + most);   // [parts][nd]
     for (int w = tid; w < nwords; w += nt) bits[w] = 0u;
     __syncthreads();
     mark_rows(a, div, S, SC, H, n, tid, nt, col, bits);
@@ -258,15 +259,15 @@ __global__ void __launch_bounds__(512, 3) k_fold(const __grid_constant__ FoldArg
     }
     __syncthreads();
     const int nd = s_n;
-    for (int k = tid; k < nbeam * nd; k += nt) acc[k] = 0.0f;
+    for (int k = tid; k < parts * nd; k += nt) acc[k] = 0.0f;
     __syncthreads();
-    for (int bb = warp; bb < nbeam; bb += nw)
-        sum_rows(a, div, S, SC, H + (int64_t)bb * ne, ne, col, bits, pre, rows, acc + bb * nd, s_scores[warp], alpha, gain,
+    for (int p = warp; p < parts; p += nw)
+        sum_rows(a, div, S, SC, H + (int64_t)p * len, len, col, bits, pre, rows, acc + p * nd, s_scores[warp], alpha, gain,
                  lane);
     __syncthreads();
     for (int k = tid; k < nd; k += nt) {
         float P = 0.0f;
-        for (int bb = 0; bb < nbeam; ++bb) P += acc[bb * nd + k];
+        for (int p = 0; p < parts; ++p) P += acc[p * nd + k];
         put_bin(a, S, first, k, rows[k], col, P);
     }
     if (a.bands)
@@ -604,8 +605,8 @@ __global__ void __launch_bounds__(256, 4) k_norm_rows(const __grid_constant__ No
 
 // The same for rows of any width and alignment: one warp per run of 512 bins of a row
 // (every a.runs-th run of it).  A frame of 50 x 20000 bins 523 us with a warp per pair
-// of rows, 46 with this; 64 frames of 1000 x 511 333 -> 245; 64 frames of 1000 x 512, which
-// the kernel above takes, 175 there and 184 here.
+// of rows, 46 with this; 64 frames of 1000 x 511 333 -> 242; 64 frames of 1000 x 512, which
+// the kernel above takes, 171 there and 184 here.
 __global__ void __launch_bounds__(256) k_norm_runs(const __grid_constant__ NormArgs a) {
     let_next_start();
     wait_for_previous();   // I~ and its maximum

@@ -203,9 +203,21 @@ int64_t fold_words(const SensorDev& s) {
     return 2 * band_count(s) + most * (1 + (s.fold_beams ? col_beams_max(s) : 1));
 }
 
-// Warps of a fold block: four columns, or the beams of one column (up to 16).
+// Whether a sensor's columns take a block each in a launch of `columns` columns, also
+// without per-beam rows (the sums are the same either way): few columns of many rays,
+// whose rows the block's warps then mark together.  Frames, a warp a column -> a block:
+// 256 columns of 1024 rays into 100 range bins 165 -> 91 us; 64 of 4096 310 -> 167; 4 of 1024 into
+// 8000 57 -> 45, of 16,384 468 -> 366; fewer rays a column gain nothing, and 512 columns of
+// 4096 in a batch take 456 instead of 418.
+bool fold_by_block(const SensorDev& s, int64_t columns) {
+    return s.fold_beams || (columns <= 256 && col_beams_max(s) * s.ne >= 1024);
+}
+
+// Warps of a fold block: four columns; or the beams of one column, up to 16; or 16 to mark
+// the rows of one column.
 int fold_warps(const SensorDev& s) {
-    return s.fold_beams ? (int)std::max<int64_t>(4, std::min<int64_t>(16, col_beams_max(s))) : 4;
+    if (!s.fold_block) return 4;
+    return s.fold_beams ? (int)std::max<int64_t>(4, std::min<int64_t>(16, col_beams_max(s))) : 16;
 }
 
 // Rows per block of the row kernel: a whole band of 32, which reads the band's
@@ -269,6 +281,7 @@ SensorDev make_sensor(const sonar_sensor& s, uint64_t seed, uint64_t frame, cons
     const int64_t beams = col_beams_max(d), dense = (int64_t)d.nr * (1 + beams) + (d.nr + 31) / 32 +
                                                     std::min<int64_t>(beams * d.ne, d.nr);
     d.fold_beams = (s.n_beams > s.n_az_bins && dense * (int64_t)sizeof(float) <= 200 * 1024) ? 1 : 0;
+    d.fold_block = d.fold_beams;
     return d;
 }
 
@@ -488,10 +501,10 @@ sonar_status single_forward(sonar_ctx* ctx, const SensorDev& S, const SceneDev& 
     a.dense = f.dense;
     a.err = ctx->d_err;
     int warps = fold_warps(S);
-    if (!S.fold_beams)
+    if (!S.fold_block)
         while (warps > 1 && sizeof(uint32_t) * warps * fold_words(S) > kMaxDynSmem) warps /= 2;
-    const size_t smem = sizeof(uint32_t) * fold_words(S) * (S.fold_beams ? 1 : warps);
-    CU(launch_fold(a, S.fold_beams ? S.naz : (S.naz + warps - 1) / warps, 32 * warps, smem, s,
+    const size_t smem = sizeof(uint32_t) * fold_words(S) * (S.fold_block ? 1 : warps);
+    CU(launch_fold(a, S.fold_block ? S.naz : (S.naz + warps - 1) / warps, 32 * warps, smem, s,
                    !capturing && !f.dense),
        "fold launch");
     RowsArgs r{};
@@ -563,6 +576,7 @@ extern "C" sonar_status sonar_render(sonar_ctx_t ctx, int32_t scene_id, const so
     CU(cudaSetDevice(ctx->device), "cudaSetDevice");
     const Tune t = single_tune(ctx, *sensor);
     SensorDev S = make_sensor(*sensor, seed, frame, t, out->fan ? out->fan_w : 0, out->fan ? out->fan_h : 0);
+    S.fold_block = fold_by_block(S, S.naz);
     const int64_t npol = (int64_t)S.nr * S.naz;
     float* noised = out->noised;
     if (!noised) {
@@ -901,12 +915,15 @@ sonar_status batch_plan(sonar_batch* b) {
     b->plan_occ = b->trace_occ;
     b->total_rows = rows;
     b->total_polar = polar_end;
+    int64_t columns = 0;
+    for (const SensorDev& S : b->hs) columns += S.naz;
+    for (SensorDev& S : b->hs) S.fold_block = fold_by_block(S, columns);
     // the fold's blocks: the warps that the sensor with most rays wants, fewer
     // where the columns of some sensor need more shared memory than that
     int warps = n > 0 ? fold_warps(b->hs[kmost]) : 4;
     int64_t warp_words = 0, block_words = 0;
-    for (const SensorDev& S : b->hs) (S.fold_beams ? block_words : warp_words) =
-        std::max(S.fold_beams ? block_words : warp_words, fold_words(S));
+    for (const SensorDev& S : b->hs) (S.fold_block ? block_words : warp_words) =
+        std::max(S.fold_block ? block_words : warp_words, fold_words(S));
     while (warps > 1 && (int64_t)sizeof(uint32_t) * warps * warp_words > (int64_t)kMaxDynSmem) warps /= 2;
     b->fold_block = 32 * warps;
     b->fold_words_per_warp = (int)warp_words;
@@ -914,7 +931,7 @@ sonar_status batch_plan(sonar_batch* b) {
     b->rows_step = rows_per_block(rows, b->max_naz, ctx->sm_count);
     for (int k = 0; k < n; ++k) {
         const SensorDev& S = b->hs[k];
-        const int step = S.fold_beams ? 1 : warps;
+        const int step = S.fold_block ? 1 : warps;
         for (int c = 0; c < S.naz; c += step) b->fold_map.push_back(make_int4(k, c, S.scene, 0));
         for (int r = 0; r < S.nr; r += b->rows_step) b->rows_map.push_back(make_int2(k, r));
     }
@@ -2112,6 +2129,7 @@ extern "C" sonar_status sonar_render_noalloc(sonar_ctx_t ctx, int32_t scene_id, 
     float* noised = out->noised ? out->noised : (float*)base + noised_at;
     const Tune t = single_tune(ctx, *sensor);
     SensorDev S = make_sensor(*sensor, seed, frame, t, out->fan ? out->fan_w : 0, out->fan ? out->fan_h : 0);
+    S.fold_block = fold_by_block(S, S.naz);
     S.trig = (float4*)((float*)base + 64);
     // single_forward clears the maximum (the array still holds the previous
     // call's values); hit records and the noised image are fully overwritten

@@ -72,6 +72,7 @@ struct SensorDev {
     int32_t occ;         // trace: variant bits kTraceCap, kTraceWide
     int32_t trace_blocks;  // trace: 32-ray tiles covering the sensor
     int32_t fold_beams;  // fold: per-beam rows (several beams per column, and they fit in shared memory)
+    int32_t fold_block;  // fold: a block per column (per-beam rows, or few columns of many rays)
     int64_t polar_off, hits_off, fan_off, rowmax_off;
     int64_t val_off, band_off;   // fold: first value slot (a slot per ray) and first bitmap word pair
     float4* trig;        // float-float sin/cos of the beam azimuths [nb] and elevations [ne]

@@ -151,3 +151,25 @@ def test_rows_shared_by_a_block(env, nr, naz, mode):
     top = {0: torch.ones(1, device=son.device), 1: one["noised"].amax(1, keepdim=True), 2: one["noised"].max()}[mode]
     assert torch.equal(one["polar"], one["noised"] / top)
     b.close()
+
+
+# columns of 1023 to 2560 rays, beams that do not divide evenly, more rows than a block keeps per beam
+@pytest.mark.parametrize("nb,ne,nr,naz", [(11, 93, 70, 1), (64, 64, 9000, 4), (255, 1024, 100, 255), (500, 20, 8000, 7),
+                                          (2050, 5, 6000, 9), (31, 33, 40, 31)])
+def test_fold_by_blocks_and_by_warps(env, nb, ne, nr, naz):
+    """Few columns of many rays are folded by a block each, in a batch of more columns by
+    a warp each: the same sums, bit for bit."""
+    son, mu, sid = env
+    theta, prm = son.theta(0.05, 1.3, mu), RenderParams()
+    sp = spec(nb, ne, nr, naz)
+    one = son.render(sid, sp, theta, prm, 3, 4, hits=True, fan=False, binned=True)
+    for others in ([], [(sid, spec(3, 2, 5, 300), 3, 4)]):
+        b = son.batch([(sid, sp, 3, 4)] + others)
+        b.render(theta, prm, fan=False, binned=True)
+        torch.cuda.synchronize()
+        got = b.view(0)
+        for key in ("hits", "binned", "noised", "polar"):
+            assert torch.equal(one[key], got[key]), (key, len(others))
+        b.close()
+    st, bits = son.check()
+    assert st == 0 and bits == 0
