@@ -298,8 +298,9 @@ __device__ __forceinline__ float norm_value(float In, float m, int mode) {
     return (mode != 0 && m > 0.0f) ? In / m : In;
 }
 
-// v / m correctly rounded, given y = 1 / m correctly rounded, for v >= 2^-100
-// and 2^-60 <= m <= 2^60 (nothing under- or overflows): v y is within two ulp,
+// v / m correctly rounded, given y = 1 / m correctly rounded, for 2^-60 <= v <= m
+// <= 2^60 (the quotient is at least 2^-120, a residual's last bit at least 2^-106:
+// nothing under- or overflows): v y is within two ulp,
 // one residual step brings it within one, and a second one rounds correctly
 // (P. Markstein, IBM J. Res. Dev. 34(1), 1990).  Five FMA-pipe operations,
 // against nine and two on the quarter-rate unit for the general division.
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(256, REG == 4 ? 3 : 2) k_rows(const __grid_con
             for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
             // the row's values are the additive term (positive) and more unless a
             // reflectivity is negative: the general division is the exception
-            if (__all_sync(0xFFFFFFFFu, least >= 0x1p-100f && m >= 0x1p-60f && m <= 0x1p60f) && mode == 1) {
+            if (__all_sync(0xFFFFFFFFu, least >= 0x1p-60f && m <= 0x1p60f) && mode == 1) {
                 const float y = 1.0f / m;
 #pragma unroll
                 for (int k = 0; k < REG; ++k) {

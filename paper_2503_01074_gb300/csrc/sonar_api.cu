@@ -744,7 +744,7 @@ struct sonar_batch {
     float* d_noised = nullptr;
     RowInfo* d_rowinfo = nullptr;
     double* d_partials = nullptr;
-    int32_t* d_counters = nullptr;    // [1] adjoint work
+    int32_t* d_counter = nullptr;     // adjoint work
     int n_mat_cap = 0;
     size_t n_scene_table = 0;         // entries in d_scenes
     // host staging for updates (pinned, double-buffered)
@@ -793,7 +793,7 @@ void batch_free_device(sonar_batch* b) {
                     (void*)b->d_fan_prefix, (void*)b->d_trace_prefix, (void*)b->d_trace_map,
                     (void*)b->d_fan_map, (void*)b->d_row_map, (void*)b->d_hits, (void*)b->d_trig, (void*)b->d_trig_stamp,
                     (void*)b->d_rowmax,
-                    (void*)b->d_noised, (void*)b->d_rowinfo, (void*)b->d_partials, (void*)b->d_counters,
+                    (void*)b->d_noised, (void*)b->d_rowinfo, (void*)b->d_partials, (void*)b->d_counter,
                     (void*)b->d_fan_lut, (void*)b->d_luts, (void*)b->d_lut_map, (void*)b->d_group_map,
                     (void*)b->d_members, (void*)b->d_fan_stamp})
         if (p) cudaFree(p);
@@ -816,7 +816,7 @@ void batch_free_device(sonar_batch* b) {
     b->d_sens = nullptr; b->d_adj_units = nullptr; b->d_scenes = nullptr;
     b->d_fan_prefix = nullptr;
     b->d_rowmax = nullptr; b->d_noised = nullptr; b->d_rowinfo = nullptr; b->d_partials = nullptr;
-    b->d_counters = nullptr;
+    b->d_counter = nullptr;
     drop_graphs(b);
     b->trig_current = b->lut_current = false;
 }
@@ -1104,7 +1104,7 @@ sonar_status batch_plan(sonar_batch* b) {
     }
     alloc((void**)&b->d_rowmax, sizeof(uint32_t) * rows);
     alloc((void**)&b->d_rowinfo, sizeof(RowInfo) * rows);
-    alloc((void**)&b->d_counters, sizeof(int32_t) * 4);
+    alloc((void**)&b->d_counter, sizeof(int32_t));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch allocation");
     const std::vector<SceneDev> table = scene_table(ctx);
     e = cudaMemcpy(b->d_sens, b->hs.data(), sizeof(SensorDev) * n, cudaMemcpyHostToDevice);
@@ -1461,7 +1461,7 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
     // the gather's work counter is cleared by a kernel before it (the ray cast
     // of recomputed records, the row terms), else by a memset
     if (hits && p->normalise == 0)
-        CU(cudaMemsetAsync(b->d_counters + 1, 0, sizeof(int32_t), s), "cudaMemsetAsync");
+        CU(cudaMemsetAsync(b->d_counter, 0, sizeof(int32_t), s), "cudaMemsetAsync");
     if (events) CU(mark_phase(b, b->mark[1], b->ev[3], s), "cudaEventRecord");
     if (!hits) {   // recompute the hit records with the ray-cast kernel into the batch scratch
         CU(launch_trig(b->d_sens, SensorDev{}, (int)b->items.size(), b->max_angles, s), "batch trig launch");
@@ -1473,7 +1473,7 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
         tr.params = *p;
         tr.hits = b->d_hits;
         tr.err = ctx->d_err;
-        tr.zero_word = b->d_counters + 1;
+        tr.zero_word = b->d_counter;
         CU(launch_trace(tr, b->trace_prefix.back(), b->trace_occ, s, true), "batch trace launch");
         hits = b->d_hits;
         cast = true;
@@ -1481,14 +1481,14 @@ sonar_status batch_backward_launches(sonar_batch* b, const sonar_params* p, cons
     if (p->normalise != 0)
         CU(launch_adj_rows(b->d_sens, b->d_row_map, SensorDev{},
                            p->normalise == 1 ? b->total_rows : (int64_t)b->items.size(), p->normalise,
-                           aligned16(noised) && aligned16(grad), noised, grad, b->d_rowinfo, b->d_counters + 1, s, cast),
+                           aligned16(noised) && aligned16(grad), noised, grad, b->d_rowinfo, b->d_counter, s, cast),
            "batch adjoint rows");
     if (events) CU(mark_phase(b, b->mark[1], b->ev[4], s), "cudaEventRecord");
     AdjArgs a{};
     a.sensors = b->d_sens;
     a.units = b->d_adj_units;
     a.scenes = b->d_scenes;
-    a.work_counter = b->d_counters + 1;
+    a.work_counter = b->d_counter;
     a.n_units = (int32_t)b->adj_units.size();
     a.chunk = b->adj_chunk;
     a.n_mat = n_mat;

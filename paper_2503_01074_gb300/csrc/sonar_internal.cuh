@@ -218,9 +218,6 @@ __device__ __forceinline__ U4 additive_words(uint32_t quad, uint32_t frame_lo, u
 __device__ __forceinline__ U4 bin_draws(uint32_t bin, const SensorDev& s, const PhiloxKey& K) {
     return philox10(U4{bin, s.frame_lo, 0u, s.frame_hi}, K);
 }
-__device__ __forceinline__ uint32_t word_of(const U4& x, uint32_t j) {
-    return j == 0 ? x.x : j == 1 ? x.y : j == 2 ? x.z : x.w;
-}
 __device__ __forceinline__ float rayleigh_of(uint32_t word, float sigma_sa) {
     return sigma_sa * sqrt_nonneg(neg2log_u(word));
 }
