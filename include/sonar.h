@@ -132,7 +132,9 @@ typedef struct {
 const char* sonar_version(void);
 
 /* Creates a context on CUDA device `device` (which becomes current for the
- * calling thread).  *out receives the handle. */
+ * calling thread).  *out receives the handle.  The context keeps up to 1 GiB of
+ * freed scene and build memory mapped for its next scenes, until it is
+ * destroyed. */
 sonar_status sonar_create(int32_t device, sonar_ctx_t* out);
 
 /* Synchronises the device, frees every scene, batch and scratch buffer the
@@ -263,8 +265,9 @@ typedef struct {
 /* Plans a batch: validates the items, lists the blocks of every launch (ray-cast
  * tiles, azimuth columns, bands of range rows, fan squares; launch shapes from
  * the autotuner's cache when it has an entry for the sensor shape, defaults
- * otherwise), allocates the batch's scratch and uploads the descriptors
- * (synchronous).  n_items >= 1. */
+ * otherwise), allocates the batch's scratch (among it 8 bytes a ray, and 8 per
+ * azimuth column and 32 range bins) and uploads the descriptors (synchronous).
+ * n_items >= 1. */
 sonar_status sonar_batch_create(sonar_ctx_t ctx, const sonar_batch_item* items,
                                 int32_t n_items, sonar_batch_t* out);
 
