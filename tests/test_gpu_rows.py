@@ -163,13 +163,17 @@ def test_fold_by_blocks_and_by_warps(env, nb, ne, nr, naz):
     theta, prm = son.theta(0.05, 1.3, mu), RenderParams()
     sp = spec(nb, ne, nr, naz)
     one = son.render(sid, sp, theta, prm, 3, 4, hits=True, fan=False, binned=True)
-    for others in ([], [(sid, spec(3, 2, 5, 300), 3, 4)]):
+    light = (sid, spec(5, 3, 40, 1), 3, 4)   # in a launch with the blocks, by warps of a block of 16
+    for others in ([], [light], [(sid, spec(3, 2, 5, 300), 3, 4)]):
         b = son.batch([(sid, sp, 3, 4)] + others)
         b.render(theta, prm, fan=False, binned=True)
         torch.cuda.synchronize()
         got = b.view(0)
         for key in ("hits", "binned", "noised", "polar"):
             assert torch.equal(one[key], got[key]), (key, len(others))
+        if others and others[0] is light:
+            small = son.render(sid, light[1], theta, prm, 3, 4, hits=True, fan=False, binned=True)
+            assert all(torch.equal(small[key], b.view(1)[key]) for key in ("hits", "binned", "noised", "polar"))
         b.close()
     st, bits = son.check()
     assert st == 0 and bits == 0
